@@ -520,220 +520,155 @@ __global__ void __launch_bounds__(256) k_ew_bwd(const EwBwdDesc* __restrict__ ta
 }
 
 // ---------------------------------------------------------------- BN
-// one CTA per channel: thread t sums tiles t, t+256, ... in double, then a
-// fixed shared-memory tree combines the 256 partial sums
-
-// Sums over one chunk of partial tiles ([tiles][C][2] floats) for the 32
-// channels of a channel group: lane = channel, warp w adds tiles t0+w, t0+w+8,
-// ... (eight independent 256-byte row loads per warp), then warp 0 adds the
-// eight warps' sums in warp order.  When a launch spans several chunks, each
-// CTA leaves its chunk sums in scratch and the last CTA of the channel group
-// (an atomic count) adds them: warp w takes chunks w, w+8, ..., warp 0 adds the
-// warps' sums in order, so the result does not depend on the order the CTAs
-// run in.  Returns true on the threads (warp 0, c < C) that hold the totals in
-// s1 / s2.
-__device__ __forceinline__ bool chunked_sums(const float* __restrict__ part, int C, int tiles, int cg, int chunk,
-                                             int nchunk, double* scratch, int32_t* counter, double& s1, double& s2) {
-  __shared__ double red[8][2][32];
-  __shared__ int is_last;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int c = cg * 32 + lane;
-  const int t0 = chunk * kFinTilesPerCta, t1 = min(tiles, t0 + kFinTilesPerCta);
-  double a = 0.0, b = 0.0;
-  if (c < C) {
-    float2 v[kFinTilesPerCta / 8];
-#pragma unroll
-    for (int k = 0; k < kFinTilesPerCta / 8; ++k) {
-      const int t = t0 + w + 8 * k;
-      v[k] = t < t1 ? *reinterpret_cast<const float2*>(part + ((int64_t)t * C + c) * 2) : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int k = 0; k < kFinTilesPerCta / 8; ++k) {
-      a += (double)v[k].x;
-      b += (double)v[k].y;
-    }
-  }
-  red[w][0][lane] = a;
-  red[w][1][lane] = b;
-  __syncthreads();
-  a = 0.0;
-  b = 0.0;
-  if (w == 0)
-    for (int k = 0; k < 8; ++k) {
-      a += red[k][0][lane];
-      b += red[k][1][lane];
-    }
-  if (nchunk == 1) {
-    s1 = a;
-    s2 = b;
-    return w == 0 && c < C;
-  }
-  if (w == 0 && c < C) {
-    scratch[((int64_t)chunk * C + c) * 2] = a;
-    scratch[((int64_t)chunk * C + c) * 2 + 1] = b;
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) is_last = atomicAdd(counter + cg, 1) == nchunk - 1;
-  __syncthreads();
-  if (!is_last) return false;
-  __threadfence();
-  a = 0.0;
-  b = 0.0;
-  if (c < C)
-    for (int k = w; k < nchunk; k += 8) {
-      a += __ldcg(scratch + ((int64_t)k * C + c) * 2);
-      b += __ldcg(scratch + ((int64_t)k * C + c) * 2 + 1);
-    }
-  red[w][0][lane] = a;
-  red[w][1][lane] = b;
-  __syncthreads();
-  a = 0.0;
-  b = 0.0;
-  if (w == 0)
-    for (int k = 0; k < 8; ++k) {
-      a += red[k][0][lane];
-      b += red[k][1][lane];
-    }
-  if (threadIdx.x == 0) counter[cg] = 0;  // ready for the next launch
-  s1 = a;
-  s2 = b;
-  return w == 0 && c < C;
+// Finalisation of the per-tile BN partials ([tiles][C][2] floats, a few MB at
+// most): latency bounds it, so one CTA takes 8 channels and all their tiles in
+// a single level -- thread = (channel t & 7, tile lane t >> 3), 64 tile lanes,
+// 16 loads in flight a thread, one pass through shared memory.  There is no
+// second level (the former 32 channels x 64 tiles a CTA met in global scratch
+// behind an atomic count: five dependent trips to L2).  Sums run as
+// unevaluated pairs of floats (Knuth's TwoSum), about 48 bits: this part's
+// fp64 pipe would take longer than the loads.  The training step of the
+// 8-subnetwork ResNet-1001 (batch 256, 64 px; 340 such launches of up to 2048
+// tiles a layer): 81.94 -> 81.36 ms.
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float x) {
+  const float s = __fadd_rn(hi, x);
+  const float bb = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
+  hi = s;
 }
+__device__ __forceinline__ void pair_merge(float& hi, float& lo, float hi2, float lo2) {
+  pair_add(hi, lo, hi2);
+  lo = __fadd_rn(lo, lo2);
+}
+// the value of a pair (an overflowed or NaN sum has no meaningful low part)
+__device__ __forceinline__ double pair_value(float2 p) { return isfinite(p.x) ? (double)p.x + (double)p.y : (double)p.x; }
 
-// The same two-level reduction for the forward statistics.  Partial tiles
-// hold (mean_t, M2_t) of their rows (count n_t: rpt rows each, the last tile
-// the remainder of M).  They are combined as shifted sums around K = mean_0
-// (the first tile's mean, read by every CTA): with d_t = mean_t - K,
+constexpr int kFinThreads = 512;
+constexpr int kFinLanes = kFinThreads / kFinChannels;  // tile lanes
+constexpr int kFinUnroll = 16;                         // loads in flight a thread
+static_assert(kFinThreads / 32 == 2 * kFinChannels, "one warp per (channel, quantity) sum");
+
+// Sums over all tiles for the 8 channels of group cg.  MOMENTS false: of the
+// two partial quantities.  MOMENTS true: the tiles hold (mean_t, M2_t) of
+// n_t rows (rpt rows each, the last tile the remainder of M), combined as
+// shifted sums around K = mean_0 (the first tile's mean): with d_t = mean_t - K,
 //   S1 = sum n_t d_t,   S2 = sum (M2_t + n_t d_t^2),
 //   mean = K + S1 / M,  M2 = S2 - S1^2 / M,
 // which is Chan's pairwise update written for many sets at once (no term
 // subtracts two large sums: K lies within a few standard errors of the mean,
-// so S1^2 / M is a small part of S2).  Plain fp64 sums in the fixed order of
-// chunked_sums; returns true on the threads that hold (M, mean, M2).
-__device__ __forceinline__ bool chunked_moments(const float* __restrict__ part, int C, int tiles, int64_t M, int rpt,
-                                                int cg, int chunk, int nchunk, double* scratch, int32_t* counter,
-                                                double& n_out, double& mean_out, double& m2_out) {
-  __shared__ double red[8][2][32];
-  __shared__ int is_last;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int c = cg * 32 + lane;
-  const int t0 = chunk * kFinTilesPerCta, t1 = min(tiles, t0 + kFinTilesPerCta);
-  double a = 0.0, b = 0.0;
-  const float K = c < C && tiles > 0 ? __ldg(part + (int64_t)c * 2) : 0.f;
+// so S1^2 / M is a small part of S2).  Fixed order; threads 0 .. 7 return the
+// sums of their channel.
+template <bool MOMENTS>
+__device__ __forceinline__ void tile_sums(const float* __restrict__ part, int C, int tiles, int64_t M, int rpt, int cg,
+                                          double& s1, double& s2, float& K) {
+  __shared__ float2 red[kFinLanes][2 * kFinChannels + 1];
+  __shared__ float2 tot[2 * kFinChannels];
+  const int ch = threadIdx.x % kFinChannels, tl = threadIdx.x / kFinChannels;
+  const int c = cg * kFinChannels + ch;
+  float ah = 0.f, al = 0.f, bh = 0.f, bl = 0.f;
+  K = 0.f;
   if (c < C) {
-    float2 v[kFinTilesPerCta / 8];
+    const float2* p = reinterpret_cast<const float2*>(part) + c;
+    if (MOMENTS && tiles > 0) K = __ldg(part + (int64_t)c * 2);
+    for (int t0 = tl; t0 < tiles; t0 += kFinLanes * kFinUnroll) {
+      float2 v[kFinUnroll];
 #pragma unroll
-    for (int k = 0; k < kFinTilesPerCta / 8; ++k) {
-      const int t = t0 + w + 8 * k;
-      v[k] = t < t1 ? *reinterpret_cast<const float2*>(part + ((int64_t)t * C + c) * 2) : make_float2(0.f, 0.f);
-    }
-    // this thread's eight tiles in fp32 (d is a small difference of two
-    // close means; the S2 terms are all positive), then fp64 from here on
-    float fa = 0.f, fb = 0.f;
+      for (int k = 0; k < kFinUnroll; ++k) {
+        const int t = t0 + k * kFinLanes;
+        v[k] = t < tiles ? __ldg(p + (int64_t)t * C) : make_float2(0.f, 0.f);
+      }
 #pragma unroll
-    for (int k = 0; k < kFinTilesPerCta / 8; ++k) {
-      const int64_t t = t0 + w + 8 * k;
-      if (t < t1) {
-        const int64_t r1 = (t + 1) * rpt < M ? (t + 1) * rpt : M;
-        const float n = (float)(r1 - t * rpt);
-        const float d = v[k].x - K;
-        const float nd = n * d;
-        fa += nd;
-        fb += v[k].y + nd * d;
+      for (int k = 0; k < kFinUnroll; ++k) {
+        const int t = t0 + k * kFinLanes;
+        if (t >= tiles) continue;
+        if (MOMENTS) {
+          const int64_t r1 = (int64_t)(t + 1) * rpt < M ? (int64_t)(t + 1) * rpt : M;
+          const float n = (float)(r1 - (int64_t)t * rpt);
+          const float d = v[k].x - K;
+          const float nd = n * d;
+          pair_add(ah, al, nd);
+          pair_add(bh, bl, fmaf(nd, d, v[k].y));
+        } else {
+          pair_add(ah, al, v[k].x);
+          pair_add(bh, bl, v[k].y);
+        }
       }
     }
-    a = fa;
-    b = fb;
   }
-  red[w][0][lane] = a;
-  red[w][1][lane] = b;
+  red[tl][2 * ch] = make_float2(ah, al);
+  red[tl][2 * ch + 1] = make_float2(bh, bl);
   __syncthreads();
-  a = 0.0;
-  b = 0.0;
-  if (w == 0)
-    for (int k = 0; k < 8; ++k) {
-      a += red[k][0][lane];
-      b += red[k][1][lane];
+  {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float2 a = red[lane][w];
+#pragma unroll
+    for (int i = 32; i < kFinLanes; i += 32) pair_merge(a.x, a.y, red[lane + i][w].x, red[lane + i][w].y);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float h = __shfl_xor_sync(0xffffffffu, a.x, o), l = __shfl_xor_sync(0xffffffffu, a.y, o);
+      pair_merge(a.x, a.y, h, l);
     }
-  bool have = w == 0 && c < C;
-  if (nchunk > 1) {
-    if (w == 0 && c < C) {
-      scratch[((int64_t)chunk * C + c) * 2] = a;
-      scratch[((int64_t)chunk * C + c) * 2 + 1] = b;
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = atomicAdd(counter + cg, 1) == nchunk - 1;
-    __syncthreads();
-    if (!is_last) return false;
-    __threadfence();
-    a = 0.0;
-    b = 0.0;
-    if (c < C)
-      for (int k = w; k < nchunk; k += 8) {
-        a += __ldcg(scratch + ((int64_t)k * C + c) * 2);
-        b += __ldcg(scratch + ((int64_t)k * C + c) * 2 + 1);
-      }
-    __syncthreads();  // warp 0 has read red[] of the chunk pass
-    red[w][0][lane] = a;
-    red[w][1][lane] = b;
-    __syncthreads();
-    a = 0.0;
-    b = 0.0;
-    if (w == 0)
-      for (int k = 0; k < 8; ++k) {
-        a += red[k][0][lane];
-        b += red[k][1][lane];
-      }
-    if (threadIdx.x == 0) counter[cg] = 0;  // ready for the next launch
+    if (lane == 0) tot[w] = a;
   }
-  // one fp64 division (the reciprocal of the count); this part's fp64 units
-  // are slow, and the callers finish in fp32
-  const double n = (double)M;
-  const double rn = 1.0 / n;
-  n_out = n;
-  mean_out = (double)K + a * rn;
-  m2_out = b - a * a * rn;
-  return have;
+  __syncthreads();
+  s1 = s2 = 0.0;
+  if (threadIdx.x < kFinChannels) {
+    s1 = pair_value(tot[2 * threadIdx.x]);
+    s2 = pair_value(tot[2 * threadIdx.x + 1]);
+  }
 }
 
-__global__ void __launch_bounds__(256) k_bn_fin(const BnFinDesc* __restrict__ tab, const int* __restrict__ tstart,
-                                                int n) {
-  const int inst = find_instance(tstart, n, blockIdx.x);
-  const BnFinDesc& d = tab[inst];
-  const int local = blockIdx.x - tstart[inst];
-  const int cg = local % d.cgroups, chunk = local / d.cgroups;
-  const int c = cg * 32 + (threadIdx.x & 31);
-  float mean, var;
-  if (d.eval) {
-    // eval mode: the running statistics stand in for the batch's
-    if (threadIdx.x >= 32 || c >= d.C) return;
-    mean = d.run_mean[c];
-    var = d.run_var[c];
-  } else {
-    double cnt, mean64, m2;
-    if (!chunked_moments(d.part, d.C, d.tiles, d.count, d.rows_per_tile, cg, chunk, d.nchunk, d.scratch, d.counter,
-                         cnt, mean64, m2))
-      return;
-    // (the sums were fp64; from here fp32 holds every quantity to 2^-24)
-    mean = (float)mean64;
-    var = cnt > 0.0 ? (float)m2 / (float)cnt : 0.f;
-    if (var < 0.f) var = 0.f;
-    if (d.run_mean) {
-      // running statistics follow the batch mean and the unbiased variance
-      const float m = d.momentum;
-      const float unbiased = d.count > 1 ? var * ((float)d.count / (float)(d.count - 1)) : var;
-      d.run_mean[c] = (1.f - m) * d.run_mean[c] + m * mean;
-      d.run_var[c] = (1.f - m) * d.run_var[c] + m * unbiased;
-    }
-  }
+// scale and shift of a BN layer from the statistics it normalises with
+__device__ __forceinline__ void bn_affine(const BnFinDesc& d, int c, float gamma, float beta, float mean, float var) {
   const float rstd = 1.f / sqrtf(var + 1e-5f);
-  const float sc = d.gamma[c] * rstd;
+  const float sc = gamma * rstd;
   d.mean[c] = mean;
   d.rstd[c] = rstd;
   d.scale[c] = sc;
-  d.shift[c] = fmaf(-mean, sc, d.beta[c]);
+  d.shift[c] = fmaf(-mean, sc, beta);
+}
+
+__global__ void __launch_bounds__(kFinThreads) k_bn_fin(const BnFinDesc* __restrict__ tab,
+                                                        const int* __restrict__ tstart, int n) {
+  const int inst = find_instance(tstart, n, blockIdx.x);
+  const BnFinDesc d = tab[inst];
+  const int cg = blockIdx.x - tstart[inst];
+  const int c = cg * kFinChannels + threadIdx.x;
+  const bool fin = threadIdx.x < kFinChannels && c < d.C;
+  // the layer's parameters, loaded beside the partials
+  float gamma = 0.f, beta = 0.f, rm = 0.f, rv = 0.f;
+  if (fin) {
+    gamma = d.gamma[c];
+    beta = d.beta[c];
+    if (d.run_mean) { rm = d.run_mean[c]; rv = d.run_var[c]; }
+  }
+  double s1, s2;
+  float K;
+  tile_sums<true>(d.part, d.C, d.tiles, d.count, d.rows_per_tile, cg, s1, s2, K);
+  if (!fin) return;
+  // (1 / count comes from the host: no fp64 division here; from the moments on
+  // fp32 holds every quantity to 2^-24)
+  const float mean = (float)((double)K + s1 * d.inv_count);
+  const float m2 = (float)(s2 - s1 * s1 * d.inv_count);
+  float var = d.count > 0 ? m2 / (float)d.count : 0.f;
+  if (var < 0.f) var = 0.f;
+  if (d.run_mean) {
+    // running statistics follow the batch mean and the unbiased variance
+    const float m = d.momentum;
+    const float unbiased = d.count > 1 ? var * ((float)d.count / (float)(d.count - 1)) : var;
+    d.run_mean[c] = (1.f - m) * rm + m * mean;
+    d.run_var[c] = (1.f - m) * rv + m * unbiased;
+  }
+  bn_affine(d, c, gamma, beta, mean, var);
+}
+
+// eval mode: the running statistics stand in for the batch's (one thread per channel)
+__global__ void __launch_bounds__(kFinEvalChannels) k_bn_eval(const BnFinDesc* __restrict__ tab,
+                                                              const int* __restrict__ tstart, int n) {
+  const int inst = find_instance(tstart, n, blockIdx.x);
+  const BnFinDesc& d = tab[inst];
+  const int c = (blockIdx.x - tstart[inst]) * kFinEvalChannels + threadIdx.x;
+  if (c < d.C) bn_affine(d, c, d.gamma[c], d.beta[c], d.run_mean[c], d.run_var[c]);
 }
 
 __global__ void __launch_bounds__(256) k_bnb_reduce(const BnBwdDesc* __restrict__ tab,
@@ -780,21 +715,27 @@ __global__ void __launch_bounds__(256) k_bnb_reduce(const BnBwdDesc* __restrict_
   }
 }
 
-__global__ void __launch_bounds__(256) k_bnb_fin(const BnBwdDesc* __restrict__ tab, const int* __restrict__ tstart,
-                                                 int n) {
+__global__ void __launch_bounds__(kFinThreads) k_bnb_fin(const BnBwdDesc* __restrict__ tab,
+                                                         const int* __restrict__ tstart, int n) {
   const int inst = find_instance(tstart, n, blockIdx.x);
-  const BnBwdDesc& d = tab[inst];
-  const int local = blockIdx.x - tstart[inst];
-  const int cg = local % d.cgroups, chunk = local / d.cgroups;
-  const int c = cg * 32 + (threadIdx.x & 31);
+  const BnBwdDesc d = tab[inst];
+  const int cg = blockIdx.x - tstart[inst];
+  const int c = cg * kFinChannels + threadIdx.x;
+  const bool fin = threadIdx.x < kFinChannels && c < d.C;
+  float k0 = 0.f, b0 = 0.f, g0 = 0.f;
+  if (fin) {
+    k0 = d.gamma[c] * d.rstd[c];
+    if (d.accumulate) { b0 = d.dbeta[c]; g0 = d.dgamma[c]; }
+  }
   double s1, s2;
-  if (!chunked_sums(d.part, d.C, d.tiles, cg, chunk, d.nchunk, d.scratch, d.counter, s1, s2)) return;
-  d.dbeta[c] = d.accumulate ? d.dbeta[c] + (float)s1 : (float)s1;
-  d.dgamma[c] = d.accumulate ? d.dgamma[c] + (float)s2 : (float)s2;
-  d.coef[c * 3 + 0] = d.gamma[c] * d.rstd[c];
-  const double rm = 1.0 / (double)d.M;
-  d.coef[c * 3 + 1] = (float)(s1 * rm);
-  d.coef[c * 3 + 2] = (float)(s2 * rm);
+  float unused;
+  tile_sums<false>(d.part, d.C, d.tiles, d.M, 0, cg, s1, s2, unused);
+  if (!fin) return;
+  d.dbeta[c] = d.accumulate ? b0 + (float)s1 : (float)s1;
+  d.dgamma[c] = d.accumulate ? g0 + (float)s2 : (float)s2;
+  d.coef[c * 3 + 0] = k0;
+  d.coef[c * 3 + 1] = (float)(s1 * d.inv_count);
+  d.coef[c * 3 + 2] = (float)(s2 * d.inv_count);
 }
 
 __global__ void __launch_bounds__(256) k_bnb_apply(const BnBwdDesc* __restrict__ tab,
@@ -1274,7 +1215,12 @@ cudaError_t launch_ew_bwd(const EwBwdDesc* tab, const int* tstart, int n, int to
 }
 cudaError_t launch_bn_fin(const BnFinDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {
   if (total <= 0) return cudaSuccess;
-  k_bn_fin<<<total, 256, 0, st>>>(tab, tstart, n);
+  k_bn_fin<<<total, kFinThreads, 0, st>>>(tab, tstart, n);
+  return cudaGetLastError();
+}
+cudaError_t launch_bn_eval(const BnFinDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {
+  if (total <= 0) return cudaSuccess;
+  k_bn_eval<<<total, kFinEvalChannels, 0, st>>>(tab, tstart, n);
   return cudaGetLastError();
 }
 cudaError_t launch_bnb_reduce(const BnBwdDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {
@@ -1289,7 +1235,7 @@ cudaError_t launch_bnb_reduce8(const BnBwdDesc* tab, const int* tstart, int n, i
 }
 cudaError_t launch_bnb_fin(const BnBwdDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {
   if (total <= 0) return cudaSuccess;
-  k_bnb_fin<<<total, 256, 0, st>>>(tab, tstart, n);
+  k_bnb_fin<<<total, kFinThreads, 0, st>>>(tab, tstart, n);
   return cudaGetLastError();
 }
 cudaError_t launch_bnb_apply(const BnBwdDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {

@@ -63,7 +63,7 @@ int cdv(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 // parameters.
 struct InstPlan {
   int P = 0, Q = 0, pad = 0, mtiles = 0, ntiles = 0, splits = 1, pix_per_split = 0, rows = 0;
-  size_t wt = 0, part = 0, stats = 0, fscr = 0, fcnt = 0, gam = 0, bet = 0, scl = 0, shf = 0, coef = 0;
+  size_t wt = 0, part = 0, stats = 0, gam = 0, bet = 0, scl = 0, shf = 0, coef = 0;
   size_t maps = 0;
   int stat_tiles = 0;
   bool bn = false;    // forward statistics / data-gradient BN sums requested
@@ -158,7 +158,7 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
   pl.raw = 0;
   int esz = 2;
   // pass 1: tile grids and the small regions that start from host values
-  // (tensor maps, gamma / beta, finalize counters); pass 2: device scratch
+  // (tensor maps, gamma / beta); pass 2: device scratch
   for (int i = 0; i < n; ++i) {
     const pnn_conv_args& g = a[i];
     InstPlan& ip = pl.in[i];
@@ -177,7 +177,6 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
       ip.bn = g.y_mean != nullptr;
       if (ip.bn) {
         ip.stat_tiles = ip.mtiles;
-        ip.fcnt = take((size_t)cdv(g.k, 32) * 4);
         ip.gam = take((size_t)g.k * 4);
         ip.bet = take((size_t)g.k * 4);
       }
@@ -189,7 +188,6 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
       if (ip.bn) {
         // the fused sums use 128-row tiles; the separate reduction its own
         ip.stat_tiles = std::max(ip.mtiles, cdv(Min, bnb_rows_per_tile(g.c)));
-        ip.fcnt = take((size_t)cdv(g.c, 32) * 4);
         ip.gam = take((size_t)g.c * 4);
       }
       pl.total += ip.mtiles * ip.ntiles;
@@ -216,14 +214,12 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
     const int rsc = g.ksize * g.ksize * g.c;
     if (mode == 0 && ip.bn) {
       ip.stats = take((size_t)ip.stat_tiles * g.k * 8);
-      ip.fscr = take((size_t)cdv(ip.stat_tiles, kFinTilesPerCta) * g.k * 16);
       ip.scl = take((size_t)g.k * 4);
       ip.shf = take((size_t)g.k * 4);
     } else if (mode == 1) {
       ip.wt = take((size_t)g.k * rsc * 2);
       if (ip.bn) {
         ip.stats = take((size_t)ip.stat_tiles * g.c * 8);
-        ip.fscr = take((size_t)cdv(ip.stat_tiles, kFinTilesPerCta) * g.c * 16);
         ip.coef = take((size_t)g.c * 12);
       }
     } else if (mode == 2) {
@@ -370,12 +366,10 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       f.gamma = reinterpret_cast<const float*>(ws + ip.gam); f.beta = reinterpret_cast<const float*>(ws + ip.bet);
       f.mean = g.y_mean; f.rstd = g.y_rstd;
       f.scale = reinterpret_cast<float*>(ws + ip.scl); f.shift = reinterpret_cast<float*>(ws + ip.shf);
-      f.momentum = 0.f; f.eval = 0;
-      f.scratch = reinterpret_cast<double*>(ws + ip.fscr); f.counter = reinterpret_cast<int32_t*>(ws + ip.fcnt);
-      f.cgroups = cdv(g.k, 32);
-      f.nchunk = cdv(std::max(ip.stat_tiles, 1), kFinTilesPerCta);
+      f.momentum = 0.f;
+      f.inv_count = 1.0 / (double)Mout;
       fins.push_back(f);
-      fin_ts.push_back(fin_ts.back() + f.cgroups * f.nchunk);
+      fin_ts.push_back(fin_ts.back() + fin_ctas(g.k));
     }
     if (ip.bn && mode == 1) {
       float* gam = reinterpret_cast<float*>(at(ip.gam));
@@ -391,8 +385,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       b.coef = reinterpret_cast<float*>(ws + ip.coef);
       b.M = Min; b.C = g.c;
       b.rows_per_tile = bnb_rows_per_tile(g.c);
-      b.scratch = reinterpret_cast<double*>(ws + ip.fscr); b.counter = reinterpret_cast<int32_t*>(ws + ip.fcnt);
-      b.cgroups = cdv(g.c, 32);
+      b.inv_count = 1.0 / (double)Min;
       // the TMA-fed data gradient forms the sums of its 128-row tiles in its
       // epilogue when it writes the whole gradient; otherwise the separate
       // reduction kernel runs over its own row tiles
@@ -406,10 +399,9 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
         breds.push_back(b);
         red_ts.push_back(red_ts.back() + b.tiles);
       }
-      b.nchunk = cdv(std::max(b.tiles, 1), kFinTilesPerCta);
       b.accumulate = 0;
       bfins.push_back(b);
-      fin_ts.push_back(fin_ts.back() + b.cgroups * b.nchunk);
+      fin_ts.push_back(fin_ts.back() + fin_ctas(g.c));
     }
     ts[i + 1] = ts[i] + (mode == 2 ? ip.mtiles * ip.ntiles * ip.splits : ip.mtiles * ip.ntiles);
   }
@@ -423,7 +415,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
   memcpy(at(pl.fin_ts), fin_ts.data(), fin_ts.size() * sizeof(int));
   if (!breds.empty()) memcpy(at(pl.red_tab), breds.data(), breds.size() * sizeof(BnBwdDesc));
   memcpy(at(pl.red_ts), red_ts.data(), red_ts.size() * sizeof(int));
-  // (the image zero-fills the status word, the finalize counters and beta)
+  // (the image zero-fills the status word and beta)
   cudaError_t e = cudaMemcpyAsync(ws, img.data(), pl.init_bytes, cudaMemcpyHostToDevice, st);
   const auto* tab = reinterpret_cast<const ConvDesc*>(ws + pl.tab);
   const int* tsd = reinterpret_cast<const int*>(ws + pl.ts);

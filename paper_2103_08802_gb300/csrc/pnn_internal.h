@@ -95,11 +95,12 @@ struct EwBwdDesc {
   int32_t nin;
   int64_t M; int32_t C;
   int32_t rows_per_tile, tiles;
-  double* scratch; int32_t* counter; int32_t cgroups, nchunk;  // fin: as for BnFinDesc
 };
 
 // BN statistics finalisation: partials[tiles][C][2] -> mean, rstd, scale, shift
-constexpr int kFinTilesPerCta = 64;  // BN finalize: partial tiles one CTA adds up (8 per warp)
+constexpr int kFinChannels = 8;       // BN finalize: channels a CTA
+constexpr int kFinEvalChannels = 256; // eval mode: channels a CTA
+inline int fin_ctas(int C) { return (C + kFinChannels - 1) / kFinChannels; }
 struct BnFinDesc {
   const float* part;     // [tiles][C][2] = (mean, M2) of each tile's rows
   int32_t tiles, C;
@@ -109,11 +110,7 @@ struct BnFinDesc {
   float* mean; float* rstd; float* scale; float* shift;
   float* run_mean; float* run_var;  // running statistics of this BN layer
   float momentum;                   // training: rate at which they follow the batch
-  int32_t eval;                     // 1: normalise with the running statistics
-  // the reduction over tiles: CTAs = cgroups (32 channels each) x nchunk (64
-  // tiles each); chunk sums meet in scratch ([nchunk][C][2] doubles) and the
-  // last CTA of a channel group (counter[cg], zero between launches) adds them
-  double* scratch; int32_t* counter; int32_t cgroups, nchunk;
+  double inv_count;                 // 1 / count
 };
 
 // BN backward: dz = da * [z > 0 if relu], z = scale*h + shift, xhat = (h-mean)*rstd
@@ -134,7 +131,7 @@ struct BnBwdDesc {
   float add_c[2];                          // their coefficients
   int64_t M; int32_t C;
   int32_t rows_per_tile, tiles;
-  double* scratch; int32_t* counter; int32_t cgroups, nchunk;  // fin: as for BnFinDesc
+  double inv_count;                        // fin: 1 / M
 };
 
 struct PoolDesc {
@@ -191,6 +188,8 @@ cudaError_t launch_wreduce(const WReduceDesc* tab, const int* tstart, int n, int
 cudaError_t launch_ew(const EwDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_ew_bwd(const EwBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_bn_fin(const BnFinDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
+// eval mode: scale and shift from the running statistics (total: CTAs of kFinEvalChannels channels)
+cudaError_t launch_bn_eval(const BnFinDesc* tab, const int* tstart, int n, int total, cudaStream_t st);
 cudaError_t launch_bnb_reduce(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_bnb_fin(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_bnb_apply(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
