@@ -1,0 +1,830 @@
+// Grouped 1x1 stride-1 convolutions of the bottleneck stacks, forward and data
+// gradient, on the 5th-generation tensor cores: the layers whose channel
+// counts are so small (16 .. 256) that what the epilogue and the operand
+// transform execute per element decides the time, not the MMA.
+//
+//   forward  y[m][n]  = res[m][n] + sum_k act(x)[m][k] * W[n][k],  bf16, and the BN statistics of y
+//   dgrad    dx[m][n] (+)= sum_k dy[m][k] * Wt[n][k],  fp32, and the BN-backward sums of the BN in front
+//
+// One persistent CTA per SM walks the launch's items (an m-tile of 128 rows
+// times a run of N units of BN = 64, 32 or 16 columns).  Roles:
+//   producer    one thread: TMA boxes of raw A rows (a k-step: <= 64 channels)
+//               into the raw ring, and per (k-step, unit) the weight box and
+//               the unit's second operand X -- the residual (forward) or the
+//               BN input h (data gradient) -- into the unit ring;
+//   transform   T warps: raw rows -> BN scale/shift + ReLU (forward) -> bf16
+//               operand, 128-byte-swizzled K-major.  A thread keeps one
+//               8-channel chunk, so its scale and shift stay in registers;
+//               packed fp32 pairs;
+//   MMA         one thread, four accumulators of BN columns;
+//   epilogue    groups of four warps (one per TMEM lane quarter), unit by unit:
+//               the accumulator in one or two wide TMEM loads, X from shared
+//               memory, the output staged in one swizzled tile per warp and
+//               stored by TMA, the column sums from the staged tile with two
+//               columns a lane.
+// Against the per-16-column epilogue with residual rows gathered from global
+// memory and scalar column sums (k_tc_conv.cu), an output element costs about
+// a sixth of the instructions.  Bound by HBM latency and bandwidth, about half
+// of the copy rate: grouped launches of the 8-subnetwork ResNet-1001 (batch
+// 256, 64 px), before -> now: expand forward (16 -> 64 channels + residual +
+// statistics) 218 -> 107 us, reduce forward 117 -> 81, reduce data gradient
+// (+ BN-backward sums) 165 -> 136, expand data gradient 109 -> 98.
+// Every wait is bounded (2 s); on expiry the CTA records status 3, stops,
+// drains its copies and MMAs (bounded) and frees its TMEM.
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "pnn.h"
+#include "pnn_internal.h"
+#include "tc_ptx.cuh"
+
+namespace pnn {
+namespace {
+
+using namespace tc;
+
+enum { FWD = 0, DGRAD = 1 };
+constexpr int kRows = 128;
+constexpr int kOpBytes = kRows * 128;      // one k-step's A operand (64 bf16 a row)
+constexpr int kUnitB = 64 * 128;           // a unit's weight box: up to 64 rows x 64 bf16
+constexpr int kMaxRing = 4;
+constexpr int kAcc = 4;                    // TMEM accumulators of 64 columns
+constexpr int kAccCols = 64;
+constexpr int kSmemBudget = 227 * 1024;
+constexpr int kRedBytes = 2 * 4 * 64 * 8;  // per epilogue group: [2][4 warps][64 columns] pairs
+
+// W = 1 (forward, every instance one k-step and N >= 64): the epilogue does
+// most of the work, 2 transform + 12 epilogue warps; else 6 + 8.
+template <int MODE, int W>
+struct Roles {
+  static constexpr int kT = W ? 2 : 6;
+  static constexpr int kE = W ? 12 : 8;
+  static constexpr int kProducer = 0, kMma = 1, kT0 = 2, kE0 = 2 + kT;
+  static constexpr int kThreads = 32 * (2 + kT + kE);
+  static constexpr int kGroups = kE / 4;
+  // per-warp output staging: forward one 32 x 64 bf16 tile, data gradient two of 32 x 32 fp32
+  static constexpr int kStage = MODE == FWD ? 4096 : 8192;
+};
+static_assert(Roles<FWD, 0>::kE0 % 4 == 0 && Roles<FWD, 1>::kE0 % 4 == 0, "epilogue groups start at a TMEM lane quarter");
+
+struct Shared {
+  uint64_t raw_full[kMaxRing], raw_empty[kMaxRing];
+  uint64_t op_full[kMaxRing], op_empty[kMaxRing];
+  uint64_t u_full[kMaxRing], u_empty[kMaxRing];
+  uint64_t tfull[kAcc], tempty[kAcc];
+  uint64_t drain;
+  uint32_t tmem;
+  int abort_flag;
+  float scale[kPwMaxC], shift[kPwMaxC];
+};
+
+// ring depths for a launch: raw and unit slot bytes follow from its instances
+struct Rings {
+  int nr, no, nu, rawb, ub;
+};
+__host__ __device__ inline int rings_bytes(const Rings& r) { return r.nr * r.rawb + r.no * kOpBytes + r.nu * r.ub; }
+
+template <int MODE, int W>
+constexpr int fixed_bytes() {
+  return 1024 + (int)sizeof(Shared) + Roles<MODE, W>::kE * Roles<MODE, W>::kStage + Roles<MODE, W>::kGroups * kRedBytes;
+}
+template <int MODE, int W>
+bool plan_rings(int rawb, int xb, Rings& r) {
+  r = Rings{2, 2, 2, rawb, kUnitB + xb};
+  const int avail = kSmemBudget - fixed_bytes<MODE, W>();
+  if (rings_bytes(r) > avail) return false;
+  // deepen the unit ring, then the raw ring, while they fit
+  for (int* n : {&r.nu, &r.nr, &r.nu, &r.nr}) {
+    if (*n >= kMaxRing) continue;
+    ++*n;
+    if (rings_bytes(r) > avail) --*n;
+  }
+  return true;
+}
+
+// position in a ring of n slots and the parity of its current lap
+struct Cursor {
+  int n, s;
+  uint32_t ph;
+  __device__ __forceinline__ explicit Cursor(int slots) : n(slots), s(0), ph(0) {}
+  __device__ __forceinline__ void next() {
+    if (++s == n) { s = 0; ph ^= 1; }
+  }
+};
+
+__device__ __forceinline__ uint64_t pk2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 un2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// the two bf16 of a word as an fp32 pair
+__device__ __forceinline__ uint64_t bf2(uint32_t w) {
+  return pk2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+__device__ __forceinline__ uint32_t pack2(uint64_t v) {
+  const float2 f = un2(v);
+  return pack_bf16(f.x, f.y);
+}
+// max(v, 0) of both bf16 (a NaN becomes 0, as fmaxf(v, 0) makes it)
+__device__ __forceinline__ uint32_t relu2(uint32_t w) {
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(w), "r"(0u));
+  return r;
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,"
+      "%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+// wait for this thread's TMEM loads; the registers pass through, so no use of
+// them can be scheduled before it
+template <int N>
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[N]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < N; i += 8)
+    asm volatile("" : "+r"(r[i]), "+r"(r[i + 1]), "+r"(r[i + 2]), "+r"(r[i + 3]), "+r"(r[i + 4]), "+r"(r[i + 5]),
+                      "+r"(r[i + 6]), "+r"(r[i + 7]));
+}
+
+// Walks the items of one CTA (blockIdx.x, + gridDim.x, ...).  Instances are
+// found by stepping forward, so an item costs no division and no descriptor
+// reload unless the instance changes.
+struct Walk {
+  int item, total, ninst, inst, t0, t1;  // instance inst owns items t0 .. t1 - 1
+  int tm, tn;                            // m-tile and N item within the instance
+  bool fresh;                            // the instance changed with this item
+  const ConvDesc* d;
+  __device__ __forceinline__ Walk(const ConvDesc* tab, const int* ts, int n, int tot) {
+    item = blockIdx.x;
+    total = tot;
+    ninst = n;
+    inst = -1;
+    t0 = 0;
+    t1 = 0;
+    tm = tn = 0;
+    fresh = false;
+    d = nullptr;
+    settle(tab, ts);
+  }
+  __device__ __forceinline__ bool more() const { return item < total; }
+  __device__ __forceinline__ void settle(const ConvDesc* tab, const int* ts) {
+    if (item >= total) return;
+    if (item >= t1) {
+      do {
+        ++inst;
+        t0 = t1;
+        t1 = __ldg(ts + inst + 1);
+      } while (item >= t1);
+      d = tab + inst;
+      tm = item - t0;
+      tn = 0;
+      fresh = true;
+    } else {
+      tm += gridDim.x;
+      fresh = false;
+    }
+    const int mt = __ldg(&d->mtiles);
+    while (tm >= mt) { tm -= mt; ++tn; }
+  }
+  __device__ __forceinline__ void next(const ConvDesc* tab, const int* ts) {
+    item += gridDim.x;
+    settle(tab, ts);
+  }
+};
+
+// what the roles need of an instance
+struct Geo {
+  int rows, ncols, kt, nkt, bn, spi, nsub;  // GEMM M, N, K; k-steps; unit columns; units an item, in all
+};
+template <int MODE>
+__device__ __forceinline__ Geo geo(const ConvDesc* d) {
+  Geo g;
+  g.rows = d->B * d->H * d->W;
+  g.ncols = MODE == FWD ? d->K : d->C;
+  g.kt = MODE == FWD ? d->C : d->K;
+  g.nkt = (g.kt + 63) >> 6;
+  g.bn = pw_unit_cols(g.ncols);
+  g.nsub = g.ncols / g.bn;
+  g.spi = d->ntile_w / g.bn;
+  return g;
+}
+
+// whether a unit has a second operand: the residual (forward), the BN input
+// of the sums (data gradient)
+template <int MODE>
+__device__ __forceinline__ bool has_x(const ConvDesc* d) {
+  return MODE == FWD ? d->res != nullptr : d->bnb_part != nullptr;
+}
+
+// ------------------------------------------------------------ transform
+// Rows of one k-step: raw [128][cw] (bf16 or fp32, dense) -> bf16 operand.
+// Thread t of NT takes chunk t % nch (8 channels) of rows t / nch, + NT / nch ...
+template <bool XBF, bool BN, int NT>
+__device__ __forceinline__ void transform_rows(const uint8_t* __restrict__ raw, uint8_t* __restrict__ op, int lgn, int t,
+                                               const float* __restrict__ scs, const float* __restrict__ sfs, int relu) {
+  const int nch = 1 << lgn, cc = t & (nch - 1);
+  const int rpitch = nch * (XBF ? 16 : 32);
+  uint64_t sc[4], sf[4];
+  if (BN) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float2 a = *reinterpret_cast<const float2*>(scs + cc * 8 + 2 * i);
+      const float2 b = *reinterpret_cast<const float2*>(sfs + cc * 8 + 2 * i);
+      sc[i] = pk2(a.x, a.y);
+      sf[i] = pk2(b.x, b.y);
+    }
+  }
+  const int step = NT >> lgn;
+  const uint8_t* src = raw + cc * (XBF ? 16 : 32);
+  // two rows a turn: both rows' loads first
+  for (int r = t >> lgn; r < kRows; r += 2 * step) {
+    const bool two = r + step < kRows;
+    uint4 q[2][XBF ? 1 : 2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      if (e && !two) continue;
+#pragma unroll
+      for (int w = 0; w < (XBF ? 1 : 2); ++w)
+        q[e][w] = *reinterpret_cast<const uint4*>(src + (r + e * step) * rpitch + 16 * w);
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      if (e && !two) continue;
+      uint32_t o[4];
+      if (XBF) {
+        const uint32_t w[4] = {q[e][0].x, q[e][0].y, q[e][0].z, q[e][0].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          o[i] = BN ? pack2(fma2(sc[i], bf2(w[i]), sf[i])) : w[i];
+          if (BN && relu) o[i] = relu2(o[i]);
+        }
+      } else {
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(&q[e][0]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint64_t v = pk2(__uint_as_float(w[2 * i]), __uint_as_float(w[2 * i + 1]));
+          o[i] = BN ? pack2(fma2(sc[i], v, sf[i])) : pack2(v);
+          if (BN && relu) o[i] = relu2(o[i]);
+        }
+      }
+      *reinterpret_cast<uint4*>(op + swz(r + e * step, cc)) = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+  }
+}
+
+// ------------------------------------------------------------ epilogue
+// byte offset of 16-byte chunk j of a row in a TMA-swizzled tile of PITCH-byte rows
+template <int PITCH>
+__device__ __forceinline__ uint32_t swp(int row, int j) {
+  if (PITCH == 128) return (uint32_t)(row * 128 + ((j ^ (row & 7)) << 4));
+  if (PITCH == 64) return (uint32_t)(row * 64 + ((j ^ ((row >> 1) & 3)) << 4));
+  return (uint32_t)(row * 32 + ((j ^ ((row >> 2) & 1)) << 4));
+}
+
+struct EpiState {
+  float2* red;  // this group's [2][4][64] pairs
+  int rbuf;     // which half the next unit uses
+  int bar;      // the group's named barrier
+};
+
+// The four warps' column pairs of a unit -> the tile's partial: forward (mean,
+// M2) merged in order, data gradient plain sums.  Every warp of the group
+// calls it (ok: its own values are valid); one barrier, the halves of red
+// alternate.
+template <int MODE, int BN>
+__device__ __forceinline__ void merge_partials(EpiState& es, bool ok, int q, int lane, int rows, int m0, float* part) {
+  float2* red = es.red + es.rbuf * 256;
+  es.rbuf ^= 1;
+  asm volatile("bar.sync %0, 128;" ::"r"(es.bar) : "memory");
+  const int j = q * 32 + lane;
+  if (j < BN && ok) {
+    float a, b;
+    if (MODE == FWD) {
+      float n = 0.f;
+      a = b = 0.f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int nq = min(32, max(0, rows - (m0 + 32 * i)));
+        const float2 v = red[i * 64 + j];
+        chan_merge(n, a, b, (float)nq, v.x, v.y);
+      }
+    } else {
+      const float2 v0 = red[j], v1 = red[64 + j], v2 = red[128 + j], v3 = red[192 + j];
+      a = v0.x + v1.x + v2.x + v3.x;
+      b = v0.y + v1.y + v2.y + v3.y;
+    }
+    *reinterpret_cast<float2*>(part + 2 * j) = make_float2(a, b);
+  }
+}
+
+// (mean, M2) of the columns of a staged bf16 tile [32][BN] over its first
+// nvalid rows: lane = column pair l % (BN/2) of rows (l / (BN/2)) + RG i, two
+// passes (the sums, then the squared deviations from the warp mean)
+template <int BN, bool FULL>
+__device__ __forceinline__ void staged_moments(const uint8_t* st, int lane, int nvalid, float2* out) {
+  constexpr int PITCH = BN * 2, PAIRS = BN / 2, RG = 32 / PAIRS, IT = 32 / RG;
+  const int p = lane % PAIRS, g = lane / PAIRS;
+  uint32_t w[IT];
+#pragma unroll
+  for (int i = 0; i < IT; ++i)
+    w[i] = *reinterpret_cast<const uint32_t*>(st + swp<PITCH>(RG * i + g, p >> 2) + (p & 3) * 4);
+  uint64_t s[2] = {0ull, 0ull};
+#pragma unroll
+  for (int i = 0; i < IT; ++i) {
+    if (!FULL && RG * i + g >= nvalid) w[i] = 0u;
+    s[i & 1] = add2(s[i & 1], bf2(w[i]));
+  }
+  float2 sum = un2(add2(s[0], s[1]));
+#pragma unroll
+  for (int o = PAIRS; o < 32; o <<= 1) {
+    sum.x += __shfl_xor_sync(0xffffffffu, sum.x, o);
+    sum.y += __shfl_xor_sync(0xffffffffu, sum.y, o);
+  }
+  const float n = (float)nvalid;
+  const float mx = FULL ? sum.x * 0.03125f : (nvalid > 0 ? sum.x / n : 0.f);
+  const float my = FULL ? sum.y * 0.03125f : (nvalid > 0 ? sum.y / n : 0.f);
+  const uint64_t neg = pk2(-mx, -my);
+  s[0] = s[1] = 0ull;
+#pragma unroll
+  for (int i = 0; i < IT; ++i) {
+    const uint64_t d = add2(bf2(w[i]), neg);
+    if (FULL || RG * i + g < nvalid) s[i & 1] = fma2(d, d, s[i & 1]);
+  }
+  float2 m2 = un2(add2(s[0], s[1]));
+#pragma unroll
+  for (int o = PAIRS; o < 32; o <<= 1) {
+    m2.x += __shfl_xor_sync(0xffffffffu, m2.x, o);
+    m2.y += __shfl_xor_sync(0xffffffffu, m2.y, o);
+  }
+  if (g == 0) *reinterpret_cast<float4*>(out + 2 * p) = make_float4(mx, m2.x, my, m2.y);
+}
+
+// Forward unit: accumulator + residual -> bf16 -> staging -> TMA store, statistics.
+template <int BN>
+__device__ __forceinline__ void unit_fwd(const ConvDesc* d, uint32_t tacc, int q, int lane, int rows, int m0, int n0,
+                                         const uint8_t* x, uint8_t* st, float2* redw, uint32_t tempty, uint32_t uempty,
+                                         bool res, bool stats) {
+  uint32_t a[BN];
+#pragma unroll
+  for (int j = 0; j < BN; j += 32) {
+    if (BN >= 32) tmem_ld32(tacc + j, a + j);
+    else tmem_ld16_nowait(tacc + j, a + j);
+  }
+  tmem_wait_ld(a);
+  fence_before();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(tempty);
+  constexpr int PITCH = BN * 2;
+  uint32_t o[BN / 2];
+  if (res) {
+#pragma unroll
+    for (int j = 0; j < BN / 8; ++j) {
+      const uint4 r = *reinterpret_cast<const uint4*>(x + swp<PITCH>(q * 32 + lane, j));
+      const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int c = 8 * j + 2 * i;
+        o[4 * j + i] = pack2(add2(pk2(__uint_as_float(a[c]), __uint_as_float(a[c + 1])), bf2(w[i])));
+      }
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < BN / 2; ++i) o[i] = pack_bf16(__uint_as_float(a[2 * i]), __uint_as_float(a[2 * i + 1]));
+  }
+  // the store issued from this tile for the previous unit must have read it,
+  // and every lane must be done with its statistics
+  if (lane == 0) bulk_wait_read<0>();
+  __syncwarp();
+  if (res && lane == 0) mbar_arrive(uempty);  // X has been read
+#pragma unroll
+  for (int j = 0; j < BN / 8; ++j)
+    *reinterpret_cast<uint4*>(st + swp<PITCH>(lane, j)) = make_uint4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
+  fence_proxy_async();
+  __syncwarp();
+  const int nvalid = min(32, max(0, rows - (m0 + q * 32)));
+  if (lane == 0 && nvalid > 0) {
+    tma_store_2d(d->tma_y, n0, m0 + q * 32, smem_u32(st));
+    bulk_commit();
+  }
+  if (stats) {
+    if (nvalid == 32) staged_moments<BN, true>(st, lane, 32, redw);
+    else staged_moments<BN, false>(st, lane, nvalid, redw);
+  }
+}
+
+// BN-backward sums of HC columns of a staged dX tile [32][HC] fp32 with the
+// unit's h tile [128][BN] bf16: g = dX masked by the ReLU of the forward BN
+// output, xhat = (h - mean) * rstd; (sum g, sum g xhat) over the valid rows.
+template <int BN, bool FULL>
+__device__ __forceinline__ void staged_bn_sums(const uint8_t* st, const uint8_t* h, int c0, const ConvDesc* d, int n0, int q,
+                                               int lane, int nvalid, float2* out) {
+  constexpr int HC = BN < 32 ? BN : 32;
+  constexpr int PAIRS = HC / 2, RG = 32 / PAIRS, IT = 32 / RG;
+  const int p = lane % PAIRS, g = lane / PAIRS;
+  const int c = n0 + c0 + 2 * p;
+  const float2 scv = __ldg(reinterpret_cast<const float2*>(d->x.scale + c));
+  const float2 shv = __ldg(reinterpret_cast<const float2*>(d->x.shift + c));
+  const float2 muv = __ldg(reinterpret_cast<const float2*>(d->bn_mean + c));
+  const float2 rsv = __ldg(reinterpret_cast<const float2*>(d->bn_rstd + c));
+  const uint64_t sc = pk2(scv.x, scv.y), sh = pk2(shv.x, shv.y), nmu = pk2(-muv.x, -muv.y), rs = pk2(rsv.x, rsv.y);
+  const bool relu = d->x.relu != 0;
+  uint64_t s1 = 0ull, s2 = 0ull;
+#pragma unroll
+  for (int i = 0; i < IT; ++i) {
+    // rows r and r + 4 of 128-byte h rows fall into different halves of the banks
+    const int r = BN == 64 ? (i & 3) + 8 * (i >> 2) + 4 * g : RG * i + g;
+    const int hc = c0 / 2 + p;
+    const uint32_t hw =
+        *reinterpret_cast<const uint32_t*>(h + swp<BN * 2>(q * 32 + r, hc >> 2) + (hc & 3) * 4);
+    const float2 dv = *reinterpret_cast<const float2*>(st + swp<HC * 4>(r, p >> 1) + (p & 1) * 8);
+    const uint64_t hv = bf2(hw);
+    const float2 z = un2(fma2(sc, hv, sh));
+    const bool in = FULL || r < nvalid;
+    const uint64_t gv = pk2(in && (!relu || z.x > 0.f) ? dv.x : 0.f, in && (!relu || z.y > 0.f) ? dv.y : 0.f);
+    const uint64_t xh = mul2(add2(hv, nmu), rs);
+    s1 = add2(s1, gv);
+    // (a row past the end adds nothing: its h may be anything)
+    if (in) s2 = fma2(gv, xh, s2);
+  }
+  float2 a = un2(s1), b = un2(s2);
+#pragma unroll
+  for (int o = PAIRS; o < 32; o <<= 1) {
+    a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+    a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+    b.x += __shfl_xor_sync(0xffffffffu, b.x, o);
+    b.y += __shfl_xor_sync(0xffffffffu, b.y, o);
+  }
+  if (g == 0) *reinterpret_cast<float4*>(out + c0 + 2 * p) = make_float4(a.x, b.x, a.y, b.y);
+}
+
+// Data-gradient unit: accumulator -> fp32 staging -> TMA store or reduce-add, BN-backward sums.
+template <int BN>
+__device__ __forceinline__ void unit_dgrad(const ConvDesc* d, uint32_t tacc, int q, int lane, int rows, int m0, int n0,
+                                           const uint8_t* h, uint8_t* stage, int& sbuf, float2* redw, uint32_t tempty,
+                                           uint32_t uempty, bool stats, bool acc) {
+  constexpr int HC = BN < 32 ? BN : 32;
+  const int nvalid = min(32, max(0, rows - (m0 + q * 32)));
+#pragma unroll
+  for (int c0 = 0; c0 < BN; c0 += HC) {
+    uint32_t a[HC];
+    if (HC == 32) tmem_ld32(tacc + c0, a);
+    else tmem_ld16_nowait(tacc + c0, a);
+    tmem_wait_ld(a);
+    if (c0 + HC >= BN) {
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tempty);
+    }
+    // the store issued from this buffer two turns ago must have read it
+    if (lane == 0) bulk_wait_read<1>();
+    __syncwarp();
+    uint8_t* st = stage + sbuf * 4096;
+    sbuf ^= 1;
+#pragma unroll
+    for (int j = 0; j < HC / 4; ++j)
+      *reinterpret_cast<uint4*>(st + swp<HC * 4>(lane, j)) = make_uint4(a[4 * j], a[4 * j + 1], a[4 * j + 2], a[4 * j + 3]);
+    fence_proxy_async();
+    __syncwarp();
+    if (lane == 0 && nvalid > 0) {
+      if (acc) tma_reduce_add_2d(d->tma_y, n0 + c0, m0 + q * 32, smem_u32(st));
+      else tma_store_2d(d->tma_y, n0 + c0, m0 + q * 32, smem_u32(st));
+      bulk_commit();
+    }
+    if (stats) {
+      if (nvalid == 32) staged_bn_sums<BN, true>(st, h, c0, d, n0, q, lane, 32, redw);
+      else staged_bn_sums<BN, false>(st, h, c0, d, n0, q, lane, nvalid, redw);
+    }
+  }
+  __syncwarp();
+  if (stats && lane == 0) mbar_arrive(uempty);  // h has been read
+}
+
+template <int MODE, int W>
+__device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int ninst,
+                                        int total, const Rings& rg, int32_t* status) {
+  using R = Roles<MODE, W>;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw0 = smem_u32(smem_raw);
+  const uint32_t base = (raw0 + 1023u) & ~1023u;
+  uint8_t* const gbase = smem_raw + (base - raw0);
+  // [raw ring | operand ring | unit ring | output staging | reduction | Shared]
+  const int off_op = rg.nr * rg.rawb;
+  const int off_u = off_op + rg.no * kOpBytes;
+  const int off_st = off_u + rg.nu * rg.ub;
+  uint8_t* const stage0 = gbase + off_st;
+  uint8_t* const red0 = stage0 + R::kE * R::kStage;
+  Shared& sh = *reinterpret_cast<Shared*>(red0 + R::kGroups * kRedBytes);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kMaxRing; ++s) {
+      mbar_init(smem_u32(&sh.raw_full[s]), 1);
+      mbar_init(smem_u32(&sh.raw_empty[s]), R::kT);
+      mbar_init(smem_u32(&sh.op_full[s]), R::kT);
+      mbar_init(smem_u32(&sh.op_empty[s]), 1);
+      mbar_init(smem_u32(&sh.u_full[s]), 1);
+      // the MMA's commit and the readers of X: the unit's four epilogue warps, or (no X) the MMA thread for them
+      mbar_init(smem_u32(&sh.u_empty[s]), 1 + 4);
+    }
+    for (int b = 0; b < kAcc; ++b) {
+      mbar_init(smem_u32(&sh.tfull[b]), 1);
+      mbar_init(smem_u32(&sh.tempty[b]), 4);
+    }
+    mbar_init(smem_u32(&sh.drain), 1);
+    sh.abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == R::kMma) tmem_alloc(smem_u32(&sh.tmem), kAcc * kAccCols);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = sh.tmem;
+  volatile int* abort_flag = &sh.abort_flag;
+
+  if (warp == R::kProducer) {
+    // ================================================= TMA producer
+    if (lane == 0) {
+      Cursor cr(rg.nr), cu(rg.nu);
+      uint32_t ka = 0, u = 0;  // k-steps and units issued
+      bool ok = true;
+      for (Walk w(tab, ts, ninst, total); w.more() && ok; w.next(tab, ts)) {
+        const ConvDesc* d = w.d;
+        const Geo g = geo<MODE>(d);
+        const void* ma = d->tma_a;
+        const void* mb = d->tma_b;
+        const void* mx = has_x<MODE>(d) ? d->tma_x : nullptr;
+        const int m0 = w.tm * kRows, sub0 = w.tn * g.spi, sub1 = min(g.nsub, sub0 + g.spi);
+        const uint32_t abytes = (uint32_t)(kRows * min(g.kt, 64) * (MODE == FWD && d->x.dt == DT_BF16 ? 2 : 4));
+        for (int kt = 0; kt < g.nkt && ok; ++kt) {
+          if (!mbar_wait(smem_u32(&sh.raw_empty[cr.s]), cr.ph ^ 1, abort_flag)) { ok = false; break; }
+          const uint32_t full = smem_u32(&sh.raw_full[cr.s]);
+          mbar_expect_tx(full, abytes);
+          tma_load_2d(base + cr.s * rg.rawb, ma, kt * 64, m0, full);
+          cr.next();
+          ++ka;
+          for (int sub = sub0; sub < sub1; ++sub) {
+            if (!mbar_wait(smem_u32(&sh.u_empty[cu.s]), cu.ph ^ 1, abort_flag)) { ok = false; break; }
+            const uint32_t uf = smem_u32(&sh.u_full[cu.s]);
+            const uint32_t slot = base + off_u + cu.s * rg.ub;
+            const bool x = mx != nullptr && kt == g.nkt - 1;
+            mbar_expect_tx(uf, (uint32_t)(g.bn * 128 + (x ? kRows * g.bn * 2 : 0)));
+            tma_load_2d(slot, mb, kt * 64, sub * g.bn, uf);
+            if (x) tma_load_2d(slot + kUnitB, mx, sub * g.bn, m0, uf);
+            cu.next();
+            ++u;
+          }
+        }
+      }
+      if (!ok) { sh.abort_flag = 1; atomicExch(status, 3); }
+      // the copies of the last slots issued must land before the CTA exits
+      for (uint32_t i = ka > (uint32_t)rg.nr ? ka - rg.nr : 0; i < ka; ++i)
+        mbar_wait_drain(smem_u32(&sh.raw_full[i % rg.nr]), (i / rg.nr) & 1);
+      for (uint32_t i = u > (uint32_t)rg.nu ? u - rg.nu : 0; i < u; ++i)
+        mbar_wait_drain(smem_u32(&sh.u_full[i % rg.nu]), (i / rg.nu) & 1);
+    }
+    __syncwarp();
+  } else if (warp == R::kMma) {
+    // ================================================= MMA issuer
+    if (lane == 0) {
+      Cursor co(rg.no), cu(rg.nu), cb(kAcc);
+      bool ok = true, issued = false;
+      for (Walk w(tab, ts, ninst, total); w.more() && ok; w.next(tab, ts)) {
+        const Geo g = geo<MODE>(w.d);
+        const bool hx = has_x<MODE>(w.d);
+        const int sub0 = w.tn * g.spi, sub1 = min(g.nsub, sub0 + g.spi);
+        const uint32_t idesc = idesc_bf16(kRows, g.bn);
+        for (int kt = 0; kt < g.nkt && ok; ++kt) {
+          if (!mbar_wait(smem_u32(&sh.op_full[co.s]), co.ph, abort_flag)) { ok = false; break; }
+          const uint32_t a_addr = base + off_op + co.s * kOpBytes;
+          const int ksub = min(4, (g.kt - kt * 64) >> 4);
+          for (int sub = sub0; sub < sub1; ++sub) {
+            // (several k-steps go with a single unit an item: cb stays on its accumulator until the last)
+            if (kt == 0 && !mbar_wait(smem_u32(&sh.tempty[cb.s]), cb.ph ^ 1, abort_flag)) { ok = false; break; }
+            if (!mbar_wait(smem_u32(&sh.u_full[cu.s]), cu.ph, abort_flag)) { ok = false; break; }
+            fence_after();
+            const uint32_t b_addr = base + off_u + cu.s * rg.ub;
+            const uint32_t tacc = tmem + cb.s * kAccCols;
+            for (int kk = 0; kk < ksub; ++kk)
+              mma_bf16(tacc, sw128_desc(a_addr + kk * 32), sw128_desc(b_addr + kk * 32), idesc, (kt | kk) ? 1u : 0u);
+            issued = true;
+            if (!(hx && kt == g.nkt - 1)) mbar_arrive_n(smem_u32(&sh.u_empty[cu.s]), 4);
+            mma_commit(smem_u32(&sh.u_empty[cu.s]));
+            cu.next();
+            if (kt == g.nkt - 1) {
+              mma_commit(smem_u32(&sh.tfull[cb.s]));
+              cb.next();
+            }
+          }
+          if (ok) mma_commit(smem_u32(&sh.op_empty[co.s]));
+          co.next();
+        }
+      }
+      if (!ok) {
+        sh.abort_flag = 1;
+        atomicExch(status, 3);
+        if (issued) {
+          mma_commit(smem_u32(&sh.drain));
+          mbar_wait_drain(smem_u32(&sh.drain), 0);
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp < R::kE0) {
+    // ================================================= transform
+    // Every transform thread walks every k-step (they meet at named barrier 1
+    // when the instance changes): a thread whose wait fails stops working but
+    // keeps walking.
+    constexpr int NT = 32 * R::kT;
+    const int t = threadIdx.x - 32 * R::kT0;
+    Cursor cr(rg.nr), co(rg.no);
+    bool ok = true;
+    for (Walk w(tab, ts, ninst, total); w.more(); w.next(tab, ts)) {
+      const ConvDesc* d = w.d;
+      const Geo g = geo<MODE>(d);
+      const bool bn = MODE == FWD && d->x.scale != nullptr;
+      const bool xbf = MODE == FWD && d->x.dt == DT_BF16;
+      const int relu = bn ? d->x.relu : 0;
+      const int lgn = 28 - __clz(min(g.kt, 64));  // log2 of the 8-channel chunks a row
+      if (bn && w.fresh) {
+        asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");  // all are past the previous instance
+        for (int c = t; c < g.kt; c += NT) {
+          sh.scale[c] = __ldg(d->x.scale + c);
+          sh.shift[c] = __ldg(d->x.shift + c);
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+      }
+      for (int kt = 0; kt < g.nkt; ++kt, cr.next(), co.next()) {
+        const int sr = cr.s, so = co.s;
+        if (ok) ok = mbar_wait(smem_u32(&sh.raw_full[sr]), cr.ph, abort_flag);
+        if (ok) ok = mbar_wait(smem_u32(&sh.op_empty[so]), co.ph ^ 1, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) { sh.abort_flag = 1; continue; }
+        const uint8_t* raw = gbase + sr * rg.rawb;
+        uint8_t* op = gbase + off_op + so * kOpBytes;
+        if (MODE == DGRAD) {
+          transform_rows<false, false, NT>(raw, op, lgn, t, nullptr, nullptr, 0);
+        } else if (xbf) {
+          if (bn) transform_rows<true, true, NT>(raw, op, lgn, t, sh.scale + kt * 64, sh.shift + kt * 64, relu);
+          else transform_rows<true, false, NT>(raw, op, lgn, t, nullptr, nullptr, 0);
+        } else {
+          if (bn) transform_rows<false, true, NT>(raw, op, lgn, t, sh.scale + kt * 64, sh.shift + kt * 64, relu);
+          else transform_rows<false, false, NT>(raw, op, lgn, t, nullptr, nullptr, 0);
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(smem_u32(&sh.raw_empty[sr]));
+          mbar_arrive(smem_u32(&sh.op_full[so]));
+        }
+      }
+    }
+    if (!ok) { sh.abort_flag = 1; atomicExch(status, 3); }
+  } else {
+    // ================================================= epilogue
+    const int ew = warp - R::kE0, q = warp & 3, eg = ew >> 2;
+    uint8_t* const st = stage0 + ew * R::kStage;
+    EpiState es{reinterpret_cast<float2*>(red0 + eg * kRedBytes), 0, 2 + eg};
+    Cursor cu(rg.nu), cb(kAcc);
+    int turn = 0, sbuf = 0;
+    bool ok = true;
+    for (Walk w(tab, ts, ninst, total); w.more(); w.next(tab, ts)) {
+      const ConvDesc* d = w.d;
+      const Geo g = geo<MODE>(d);
+      const int m0 = w.tm * kRows, sub0 = w.tn * g.spi, sub1 = min(g.nsub, sub0 + g.spi);
+      float* const part = MODE == FWD ? d->stats : d->bnb_part;
+      const bool stats = part != nullptr, hx = has_x<MODE>(d);
+      const bool acc = MODE == DGRAD && d->accumulate;
+      for (int sub = sub0; sub < sub1; ++sub) {
+        // the unit's last k-step holds X (one unit a k-step: sub1 - sub0 == 1 when nkt > 1)
+        for (int i = 1; i < g.nkt; ++i) cu.next();
+        const int us = cu.s, b = cb.s;
+        const uint32_t uph = cu.ph, bph = cb.ph;
+        cu.next();
+        cb.next();
+        const bool mine = turn == eg;
+        if (++turn == R::kGroups) turn = 0;
+        if (!mine) continue;
+        if (ok) ok = mbar_wait(smem_u32(&sh.tfull[b]), bph, abort_flag);
+        if (ok && hx) ok = mbar_wait(smem_u32(&sh.u_full[us]), uph, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        const int n0 = sub * g.bn;
+        float2* redw = es.red + es.rbuf * 256 + q * 64;
+        if (ok) {
+          fence_after();
+          const uint32_t tacc = tmem + b * kAccCols + ((uint32_t)(q * 32) << 16);
+          const uint8_t* x = gbase + off_u + us * rg.ub + kUnitB;
+          const uint32_t te = smem_u32(&sh.tempty[b]), ue = smem_u32(&sh.u_empty[us]);
+          if (MODE == FWD) {
+            if (g.bn == 64) unit_fwd<64>(d, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue, hx, stats);
+            else if (g.bn == 32) unit_fwd<32>(d, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue, hx, stats);
+            else unit_fwd<16>(d, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue, hx, stats);
+          } else {
+            if (g.bn == 64) unit_dgrad<64>(d, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue, stats, acc);
+            else if (g.bn == 32) unit_dgrad<32>(d, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue, stats, acc);
+            else unit_dgrad<16>(d, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue, stats, acc);
+          }
+        } else {
+          sh.abort_flag = 1;
+        }
+        if (stats) {
+          float* p = part + ((int64_t)w.tm * g.ncols + n0) * 2;
+          if (g.bn == 64) merge_partials<MODE, 64>(es, ok, q, lane, g.rows, m0, p);
+          else if (g.bn == 32) merge_partials<MODE, 32>(es, ok, q, lane, g.rows, m0, p);
+          else merge_partials<MODE, 16>(es, ok, q, lane, g.rows, m0, p);
+        }
+      }
+    }
+    // the output stores must complete before the CTA exits
+    if (lane == 0) bulk_wait_all();
+    __syncwarp();
+    if (!ok) { sh.abort_flag = 1; atomicExch(status, 3); }
+  }
+  fence_before();
+  __syncthreads();
+  if (warp == R::kMma) {
+    fence_after();
+    tmem_dealloc(tmem, kAcc * kAccCols);
+  }
+}
+
+#define PNN_PW_KERNEL(NAME, MODE, W)                                                                                \
+  __global__ void __launch_bounds__(Roles<MODE, W>::kThreads, 1)                                                    \
+      NAME(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int ninst, int total, const Rings rg,      \
+           int32_t* status) {                                                                                       \
+    pw_body<MODE, W>(tab, ts, ninst, total, rg, status);                                                            \
+  }
+PNN_PW_KERNEL(k_pw_fwd, FWD, 0)
+PNN_PW_KERNEL(k_pw_fwd_w, FWD, 1)
+PNN_PW_KERNEL(k_pw_dgrad, DGRAD, 0)
+
+template <int MODE, int W>
+cudaError_t launch(void (*kern)(const ConvDesc*, const int*, int, int, const Rings, int32_t*), int slot,
+                   const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes, int x_bytes,
+                   int32_t* status, cudaStream_t st, int max_ctas) {
+  Rings r;
+  if (!plan_rings<MODE, W>(raw_bytes, x_bytes, r)) return cudaErrorInvalidValue;
+  cudaError_t e = set_smem_attr_once(slot, reinterpret_cast<const void*>(kern), kSmemBudget);
+  if (e != cudaSuccess) return e;
+  const int sms = device_sm_count();
+  int grid = total < sms ? total : sms;
+  if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
+  const int smem = fixed_bytes<MODE, W>() + rings_bytes(r);
+  kern<<<grid, Roles<MODE, W>::kThreads, smem, st>>>(tab, ts, n, total, r, status);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+bool pw_fits(int mode, int raw_bytes, int x_bytes) {
+  Rings r;
+  return mode == FWD ? plan_rings<FWD, 0>(raw_bytes, x_bytes, r) : plan_rings<DGRAD, 0>(raw_bytes, x_bytes, r);
+}
+
+cudaError_t launch_conv_pw(int mode, int wide, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes,
+                           int x_bytes, int32_t* status, cudaStream_t st, int max_ctas) {
+  if (total <= 0) return cudaSuccess;
+  if (raw_bytes <= 0 || (raw_bytes & 1023) || x_bytes < 0 || (x_bytes & 1023)) return cudaErrorInvalidValue;
+  if (mode == DGRAD)
+    return launch<DGRAD, 0>(k_pw_dgrad, 14, tab, ts, n, total, raw_bytes, x_bytes, status, st, max_ctas);
+  return wide ? launch<FWD, 1>(k_pw_fwd_w, 13, tab, ts, n, total, raw_bytes, x_bytes, status, st, max_ctas)
+              : launch<FWD, 0>(k_pw_fwd, 12, tab, ts, n, total, raw_bytes, x_bytes, status, st, max_ctas);
+}
+
+}  // namespace pnn

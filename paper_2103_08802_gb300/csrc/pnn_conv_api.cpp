@@ -62,7 +62,7 @@ int cdv(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 // byte offsets of its scratch in the workspace; the launch-wide kernel
 // parameters.
 struct InstPlan {
-  int P = 0, Q = 0, pad = 0, mtiles = 0, ntiles = 0, splits = 1, pix_per_split = 0, rows = 0;
+  int P = 0, Q = 0, pad = 0, mtiles = 0, ntiles = 0, units = 0, splits = 1, pix_per_split = 0, rows = 0;
   size_t wt = 0, part = 0, stats = 0, gam = 0, bet = 0, scl = 0, shf = 0, coef = 0;
   size_t maps = 0;
   int stat_tiles = 0;
@@ -115,6 +115,15 @@ bool tma_ok(int mode, const pnn_conv_args& g) {
   return tma_wgrad_ok(g.ksize, g.stride, pad, g.c, g.k, g.w, g.x_dtype == PNN_DT_BF16);
 }
 
+// whether k_pw_conv.cu takes this instance
+bool pw_inst(int mode, const pnn_conv_args& g) {
+  if (mode == 0)
+    return pw_ok(g.ksize, g.stride, g.c, g.k) && g.y_dtype == PNN_DT_BF16 && (!g.res || g.res_dtype == PNN_DT_BF16);
+  return mode == 1 && pw_ok(g.ksize, g.stride, g.k, g.c) && (!g.bn_mean || g.x_dtype == PNN_DT_BF16);
+}
+// its second operand: the residual, or the BN input of fused BN-backward sums
+bool pw_has_x(int mode, const pnn_conv_args& g) { return mode == 0 ? g.res != nullptr : g.bn_mean && !g.accumulate; }
+
 // whether instance g of a TMA-fed forward / data-gradient launch takes halo tiles
 bool halo_inst(int mode, const pnn_conv_args& g) {
   if (mode == 2) return false;
@@ -140,6 +149,13 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
   if (mode == 0)
     for (int i = 0; i < n; ++i) auto_tma = auto_tma && ((a[i].k >= 64 && tma_ok(mode, a[i])) || halo_inst(mode, a[i]));
   pl.variant = (impl == 1 || impl == 3) ? 1 : (impl == 2 ? 0 : (auto_tma ? 1 : 0));
+  bool all_pw = impl == 0;
+  int64_t mtiles = 0;
+  for (int i = 0; i < n; ++i) {
+    all_pw = all_pw && pw_inst(mode, a[i]);
+    mtiles += cdv((int64_t)a[i].batch * a[i].h * a[i].w, kTcBM);  // (stride 1)
+  }
+  if (all_pw) pl.variant = 4;
   size_t cur = 0;
   auto take = [&](size_t b) { size_t o = cur; cur = al256(cur + b); return o; };
   pl.tab = take((size_t)n * sizeof(ConvDesc));
@@ -205,7 +221,13 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
       pl.total += base * ip.splits;
     }
     ip.halo = pl.variant == 1 && impl != 3 && halo_inst(mode, g);
-    if (pl.variant == 1) ip.maps = take(4 * 128);
+    if (pl.variant == 4) {
+      ip.units = pw_item_units(ncols, mtiles);
+      pl.total -= ip.mtiles * ip.ntiles;
+      ip.ntiles = cdv(ncols, ip.units * pw_unit_cols(ncols));
+      pl.total += ip.mtiles * ip.ntiles;
+    }
+    if (pl.variant == 1 || pl.variant == 4) ip.maps = take(4 * 128);
   }
   pl.init_bytes = cur;
   for (int i = 0; i < n; ++i) {
@@ -247,6 +269,16 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
   pl.wide = pl.variant == 1 && mode != 2;
   for (int i = 0; i < n; ++i)
     if (a[i].ksize * a[i].ksize * (mode == 0 ? a[i].c : a[i].k) > 64) pl.wide = 0;
+  if (pl.variant == 4) {
+    pl.raw = pl.op = 0;
+    pl.wide = mode == 0;
+    for (int i = 0; i < n; ++i) {
+      const int ch = mode == 1 ? a[i].k : a[i].c, ncols = mode == 1 ? a[i].c : a[i].k;
+      pl.raw = std::max(pl.raw, pw_raw_bytes(ch, mode == 0 && a[i].x_dtype == PNN_DT_BF16 ? 2 : 4));
+      if (pw_has_x(mode, a[i])) pl.op = std::max(pl.op, pw_x_bytes(ncols));
+      if (ch > 64 || ncols < 64) pl.wide = 0;
+    }
+  }
   pl.bytes = cur;
   return PNN_OK;
 }
@@ -356,6 +388,25 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       c.tma_y = mode == 2 ? nullptr : ws + ip.maps + 256;
       c.tma_h = ip.halo ? ws + ip.maps + 384 : nullptr;
     }
+    if (pl.variant == 4) {
+      const char* why = nullptr;
+      uint8_t* m = at(ip.maps);
+      const int ch = mode == 1 ? g.k : g.c, ncols = mode == 1 ? g.c : g.k, bn = pw_unit_cols(ncols);
+      int e = encode_tensor_map_2d(m, mode == 1 ? (const void*)g.dy : g.x, mode == 0 && g.x_dtype == PNN_DT_BF16, ch, Min,
+                                   std::min(ch, 64), kTcBM, 0, &why);
+      if (!e) e = encode_tensor_map_2d(m + 128, c.w, true, ch, ncols, 64, bn, 128, &why);
+      if (!e && mode == 0) e = encode_tensor_map_2d(m + 256, g.y, true, ncols, Min, bn, 32, 2 * bn, &why);
+      if (!e && mode == 1)
+        e = encode_tensor_map_2d(m + 256, g.dx, false, ncols, Min, std::min(bn, 32), 32, 4 * std::min(bn, 32), &why);
+      if (!e && pw_has_x(mode, g))
+        e = encode_tensor_map_2d(m + 384, mode == 0 ? g.res : g.x, true, ncols, Min, bn, kTcBM, 2 * bn, &why);
+      if (e) return set_last_error(PNN_ECUDA, why);
+      c.tma_a = ws + ip.maps;
+      c.tma_b = ws + ip.maps + 128;
+      c.tma_y = ws + ip.maps + 256;
+      c.tma_x = ws + ip.maps + 384;
+      c.ntile_w = ip.units * bn;
+    }
     if (ip.bn && mode == 0) {
       // forward statistics: the epilogue's per-tile partials, then the
       // finalize kernel with gamma = 1, beta = 0 (mean and rstd out)
@@ -389,7 +440,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       // the TMA-fed data gradient forms the sums of its 128-row tiles in its
       // epilogue when it writes the whole gradient; otherwise the separate
       // reduction kernel runs over its own row tiles
-      const bool fused = pl.variant == 1 && !g.accumulate && g.c % 16 == 0;
+      const bool fused = (pl.variant == 1 || pl.variant == 4) && !g.accumulate && g.c % 16 == 0;
       if (fused) {
         c.bn_mean = g.bn_mean; c.bn_rstd = g.bn_rstd; c.bnb_part = b.part;
         b.tiles = ip.mtiles;
@@ -423,6 +474,8 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
   if (e == cudaSuccess && mode == 1)
     e = launch_wtrans(reinterpret_cast<const WtDesc*>(ws + pl.aux_tab), auxts, n, aux_ts.back(), st);
   auto conv_launch = [&]() {
+    if (pl.variant == 4)
+      return launch_conv_pw(mode, pl.wide, tab, tsd, n, pl.total, pl.raw, pl.op, status, st);
     if (pl.variant == 1)
       return launch_conv_tma(mode, pl.wide, tab, tsd, n, pl.total, pl.bnmax, pl.raw, pl.op, status, st);
     if (mode == 0) return launch_conv_fwd_tc(tab, tsd, n, pl.total, pl.bnmax, status, st);

@@ -64,6 +64,10 @@ struct ConvDesc {
   // TMA-fed forward: tensor map over the output y [pixels][K] (box 16
   // columns x 32 rows, 64-byte swizzle for fp32, 32-byte for bf16), or null
   const void* tma_y;
+  // 1x1 kernels of k_pw_conv.cu: tensor map over the unit's second operand
+  // (forward: the residual, data gradient: the BN input h) with box [128 rows x
+  // unit columns] bf16; ntile_w is then the columns of an item
+  const void* tma_x;
   // TMA-fed data gradient of a BN(+ReLU) value (x = that virtual value): when
   // bnb_part is set, the epilogue also writes the BN-backward partial sums of
   // its tile, [m-tile][C][2] = (sum g, sum g * xhat) with g = dA masked by the
@@ -225,6 +229,12 @@ int conv_tma_op_bytes(int mode, int bnmax);
 // whether a halo instance (mode 0 or 1; A source W x ch, N tile bn) leaves
 // two stages even beside per-tap instances of the same launch
 bool conv_halo_fits(int mode, int W, int ch, int bn);
+// 1x1 stride-1 forward (mode 0) / data gradient (mode 1) of k_pw_conv.cu;
+// total: items; raw_bytes, x_bytes: the largest raw A slot and second operand
+// over the launch's instances (multiples of 1024); wide: every instance has one
+// k-step and at least 64 output columns
+cudaError_t launch_conv_pw(int mode, int wide, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes,
+                           int x_bytes, int32_t* status, cudaStream_t st, int max_ctas = 0);
 // record a message for pnn_last_error(NULL) and return `code`
 int set_last_error(int code, const char* msg);
 // streaming multiprocessors of the current device, queried once per device
@@ -336,6 +346,23 @@ PNN_HD inline int halo_op_bytes(int W, int ch, int bn) {
 inline bool tma_shape_ok(int k, int stride, int pad, int ch) {
   const bool geom = stride == 1 && ((k == 1 && pad == 0) || (k == 3 && pad == 1));
   return geom && ch % 8 == 0 && (ch <= 64 ? 64 % ch == 0 : ch % 64 == 0);
+}
+// 1x1 stride-1 forward / data gradient of k_pw_conv.cu (variant 4): ch
+// channels of the A source, ncols GEMM columns.  A unit is 64 columns (or all
+// 16 or 32); several k-steps go with one unit, so that no operand row is
+// transformed twice.
+constexpr int kPwMaxC = 256;
+PNN_HD inline int pw_unit_cols(int ncols) { return ncols % 64 == 0 ? 64 : ncols; }
+inline bool pw_ok(int k, int stride, int ch, int ncols) {
+  return k == 1 && stride == 1 && (ch == 16 || ch == 32 || (ch % 64 == 0 && ch <= kPwMaxC)) &&
+         (ncols == 16 || ncols == 32 || ncols % 64 == 0) && (ch <= 64 || ncols <= 64);
+}
+inline int pw_raw_bytes(int ch, int esz) { return (kTcBM * (ch < 64 ? ch : 64) * esz + 1023) & ~1023; }
+inline int pw_x_bytes(int ncols) { return kTcBM * pw_unit_cols(ncols) * 2; }
+// units of an item: all of an m-tile's (its rows are transformed once), unless
+// the launch has too few m-tiles to occupy the SMs twice over
+inline int pw_item_units(int ncols, int64_t launch_mtiles) {
+  return launch_mtiles >= 2 * (int64_t)device_sm_count() ? ncols / pw_unit_cols(ncols) : 1;
 }
 // N columns of a tile when the layer needs several: 128 for the TMA-fed
 // forward and data gradient (a smaller operand slot leaves room for more

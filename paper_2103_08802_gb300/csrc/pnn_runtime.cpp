@@ -111,7 +111,8 @@ struct Launch {
   int shape[6];         // first op: conv (C_in, C_out, k, stride, H_out, W_out); else (C, H, W, 0, 0, 0)
   int esz = 4;          // TMA-fed conv: largest element size of the A sources
   int raw = 0;          // TMA-fed conv: raw slot bytes of one stage
-  int op = 0;           // TMA-fed conv with halo tiles: operand slot bytes of one stage (0: default)
+  int op = 0;           // TMA-fed conv with halo tiles: operand slot bytes of one stage (0: default);
+                        // variant 4: second-operand bytes of a unit
   int wide = 0;         // TMA-fed forward / data gradient: every tile one k-step (the wide-epilogue variant)
   int block = -1;       // fine forward / backward: position of the layer in its segment
 };
@@ -338,6 +339,9 @@ struct pnn_net {
       // thread-gathered kernel, which is faster there
       const bool halo = use_halo(opt.conv_impl, 0, k, stride, k / 2, iv.H, iv.W, iv.C, tma_bn(0, cout));
       c.variant = tma_impl(opt.conv_impl) && ((cout >= 64 && tma_shape_ok(k, stride, k / 2, iv.C)) || halo) ? 1 : 0;
+      // the 1x1 kernels of k_pw_conv.cu hold bf16 outputs and residuals
+      const bool res_ok = res < 0 || vals[res].dt == DT_BF16;
+      if (tma_impl(opt.conv_impl) && pw_ok(k, stride, iv.C, cout) && out_dt == DT_BF16 && res_ok) c.variant = 4;
       c.mtiles = cdiv(M, kTcBM);
       c.ntiles = cdiv(cout, tc_ntile_w(c.kind, c.variant));
     } else {
@@ -570,6 +574,10 @@ struct pnn_net {
                                                      use_halo(opt.conv_impl, 1, f.k, f.stride, f.pad, ov.H, ov.W, ov.C, bn))
                              ? 1
                              : 0;
+            // the 1x1 kernel of k_pw_conv.cu reads the BN input of its sums as bf16
+            if (tma_impl(opt.conv_impl) && pw_ok(f.k, f.stride, ov.C, iv.C) &&
+                (!iv.virt || vals[iv.src].dt == DT_BF16))
+              dg.variant = 4;
             dg.mtiles = cdiv((int64_t)B * iv.H * iv.W, kTcBM);
             dg.ntiles = cdiv(iv.C, tc_ntile_w(dg.kind, dg.variant));
           } else {
@@ -632,7 +640,8 @@ struct pnn_net {
         // gradient of the BN(+ReLU) value (TMA-fed, stored, sole writer): its
         // epilogue writes the partial sums of each 128-row tile.
         const int wr = vals[vv].gwriter_dgrad;
-        const bool fuse = vals[vv].gwrites == 1 && wr >= 0 && ops[wr].kind == K_DGRAD_TC && ops[wr].variant == 1 &&
+        const bool fuse = vals[vv].gwrites == 1 && wr >= 0 && ops[wr].kind == K_DGRAD_TC &&
+                          (ops[wr].variant == 1 || ops[wr].variant == 4) &&
                           ops[wr].acc == 0 &&
                           ops[wr].in == vv && vals[vv].galias < 0 && vals[vv].pending.empty() && n.C % 16 == 0;
         if (fuse) {
@@ -903,6 +912,11 @@ int pnn_net::plan(const pnn_desc* d) {
   };
   auto fuse_add = [&](int v, int addend, float c) {
     POp& o = ops[vals[v].producer];
+    if (o.variant == 4 && o.kind == K_CONV_FWD_TC) {  // k_pw_conv.cu adds one operand
+      const int cin = vals[o.in].C, cout = vals[o.out].C;
+      o.variant = cout >= 64 && tma_shape_ok(o.k, o.stride, o.pad, cin) ? 1 : 0;
+      o.ntiles = cdiv(cout, tc_ntile_w(o.kind, o.variant));
+    }
     const int e = o.res2[0] < 0 ? 0 : 1;
     o.res2[e] = addend;
     o.rcoef[e] = c;
@@ -1300,6 +1314,8 @@ int pnn_net::build_tables() {
         tstart.push_back(total);
         total += tiles;
       };
+      int64_t group_mtiles = 0;  // m-tiles of the launch
+      for (int id : g.ops) group_mtiles += ops[id].mtiles;
       for (int id : g.ops) {
         const POp& o = ops[id];
         switch (o.kind) {
@@ -1353,6 +1369,35 @@ int pnn_net::build_tables() {
               c.tma_y = ws ? ws + tables_off + mo + 2 * sizeof(CUtensorMap) : nullptr;
               c.tma_h = ws && halo ? ws + tables_off + mo + 3 * sizeof(CUtensorMap) : nullptr;
             }
+            if ((o.kind == K_CONV_FWD_TC || o.kind == K_DGRAD_TC) && o.variant == 4) {
+              // maps: raw A rows, weight units, output staging tiles, second operand
+              const bool fwd = o.kind == K_CONV_FWD_TC;
+              const int ch = fwd ? iv.C : ov.C, ncols = fwd ? ov.C : iv.C, bn = pw_unit_cols(ncols);
+              const int units = pw_item_units(ncols, group_mtiles);
+              const void* a_src = fwd ? c.x.ptr : (const void*)P<float>(gptr(o.out));
+              const int64_t m = (int64_t)B * iv.H * iv.W;
+              CUtensorMap maps[4];
+              memset(maps, 0, sizeof maps);
+              if (ws) {
+                int r = encode_map(&maps[0], a_src, fwd && c.x.dt == DT_BF16, ch, m, std::min(ch, 64), kTcBM, 0);
+                if (!r) r = encode_map(&maps[1], c.w, true, ch, ncols, 64, bn, 128);
+                if (!r && fwd) r = encode_map(&maps[2], ws + ov.off, true, ncols, m, bn, 32, 2 * bn);
+                if (!r && !fwd)
+                  r = encode_map(&maps[2], P<float>(gptr(o.in)), false, ncols, m, std::min(bn, 32), 32,
+                                 4 * std::min(bn, 32));
+                if (!r && fwd && o.res >= 0)
+                  r = encode_map(&maps[3], ws + vals[o.res].off, true, ncols, m, bn, kTcBM, 2 * bn);
+                if (!r && !fwd && o.bn_fuse >= 0) r = encode_map(&maps[3], c.x.ptr, true, ncols, m, bn, kTcBM, 2 * bn);
+                if (r) return r;
+              }
+              const size_t mo = put(maps, sizeof maps);
+              c.tma_a = ws ? ws + tables_off + mo : nullptr;
+              c.tma_b = ws ? ws + tables_off + mo + sizeof(CUtensorMap) : nullptr;
+              c.tma_y = ws ? ws + tables_off + mo + 2 * sizeof(CUtensorMap) : nullptr;
+              c.tma_x = ws ? ws + tables_off + mo + 3 * sizeof(CUtensorMap) : nullptr;
+              c.ntile_w = units * bn;
+              c.ntiles = cdiv(ncols, c.ntile_w);
+            }
             if (o.kind == K_WGRAD_TC && o.variant == 1) {
               // activation halo box [hrows][cwx] (its dtype), gradient box [64][K] fp32
               const WgBoxes bx = wg_boxes(iv.C, ov.C, iv.W, o.pad, c.x.dt == DT_BF16);
@@ -1379,7 +1424,7 @@ int pnn_net::build_tables() {
                   c.res2_c[e] = o.rcoef[e];
                 }
               if (o.stats_norm >= 0) c.stats = P<float>(norms[o.stats_norm].part);
-              add(&c, sizeof c, o.mtiles * o.ntiles);
+              add(&c, sizeof c, c.mtiles * c.ntiles);
             } else if (o.kind == K_DGRAD || o.kind == K_DGRAD_TC) {
               c.dy = P<float>(gptr(o.out));
               c.dx = P<float>(gptr(o.in)); c.accumulate = o.acc;
@@ -1387,7 +1432,7 @@ int pnn_net::build_tables() {
                 const Norm& nf = norms[o.bn_fuse];
                 c.bn_mean = P<float>(nf.mean); c.bn_rstd = P<float>(nf.rstd); c.bnb_part = P<float>(nf.bpart);
               }
-              add(&c, sizeof c, o.tiles);
+              add(&c, sizeof c, c.mtiles * c.ntiles);
             } else {
               c.dy = P<float>(gptr(o.out));
               c.dw_part = P<float>(o.scratch);
@@ -1571,6 +1616,19 @@ int pnn_net::build_tables() {
           if (o.k * o.k * ch > 64) L.wide = 0;
         }
       }
+      if ((g.kind == K_CONV_FWD_TC || g.kind == K_DGRAD_TC) && g.variant == 4) {
+        L.raw = L.op = 0;
+        L.wide = g.kind == K_CONV_FWD_TC;
+        for (int id : g.ops) {
+          const POp& o = ops[id];
+          const bool fwd = o.kind == K_CONV_FWD_TC;
+          const int ch = vals[fwd ? o.in : o.out].C, ncols = vals[fwd ? o.out : o.in].C;
+          const int src = vals[o.in].virt ? vals[o.in].src : o.in;
+          L.raw = std::max(L.raw, pw_raw_bytes(ch, fwd && vals[src].dt == DT_BF16 ? 2 : 4));
+          if (fwd ? o.res >= 0 : o.bn_fuse >= 0) L.op = std::max(L.op, pw_x_bytes(ncols));
+          if (ch > 64 || ncols < 64) L.wide = 0;
+        }
+      }
       for (int id : g.ops) op_cost(ops[id], L.flops, L.bytes);
       tstart.push_back(total);
       L.table_off = put(tab.data(), tab.size());
@@ -1701,12 +1759,22 @@ int pnn_net::run_phase(int p, cudaStream_t st, int cap) {
     switch (L.kind) {
       case K_CONV_FWD: e = launch_conv_fwd_simt((const ConvDesc*)tab, ts, L.count, L.total, L.variant, st); break;
       case K_CONV_FWD_TC:
+        if (L.variant == 4) {
+          e = launch_conv_pw(0, L.wide, (const ConvDesc*)tab, ts, L.count, L.total, L.raw, L.op, P<int32_t>(status_off),
+                             st, cap);
+          break;
+        }
         e = L.variant == 1
                 ? launch_conv_tma(0, L.wide, (const ConvDesc*)tab, ts, L.count, L.total, L.aux, L.raw, L.op,
                                   P<int32_t>(status_off), st, cap)
                 : launch_conv_fwd_tc((const ConvDesc*)tab, ts, L.count, L.total, L.aux, P<int32_t>(status_off), st, cap);
         break;
       case K_DGRAD_TC:
+        if (L.variant == 4) {
+          e = launch_conv_pw(1, 0, (const ConvDesc*)tab, ts, L.count, L.total, L.raw, L.op, P<int32_t>(status_off), st,
+                             cap);
+          break;
+        }
         e = L.variant == 1
                 ? launch_conv_tma(1, L.wide, (const ConvDesc*)tab, ts, L.count, L.total, L.aux, L.raw, L.op,
                                   P<int32_t>(status_off), st, cap)
@@ -2605,7 +2673,7 @@ int pnn_profile_trace(pnn_net* n, int32_t max, pnn_trace* out, int32_t* count) {
     pnn_trace& r = out[i];
     float t = 0.f;
     cudaEventElapsedTime(&t, n->pev[2 * i], n->pev[2 * i + 1]);
-    r.kind = L.kind; r.variant = L.variant + (L.wide ? 1 : (L.op > 0 ? 2 : 0)); r.phase = L.phase; r.instances = L.count;
+    r.kind = L.kind; r.variant = L.variant == 4 ? 4 : L.variant + (L.wide ? 1 : (L.op > 0 ? 2 : 0)); r.phase = L.phase; r.instances = L.count;
     r.tiles = L.total;
     for (int j = 0; j < 6; ++j) r.shape[j] = L.shape[j];
     r.block = L.block;

@@ -1,0 +1,85 @@
+"""The kernels a training step chooses by itself (impl "auto") at the edges of
+their rules: one row, one less and one more than a 128-row tile, more items
+than CTAs, every channel count the rule names, one and several k-steps, one and
+several column units, raw fp32 inputs.  Each launch is held to the oracle and
+the bounds of test_gpu_conv_kernels."""
+import pytest
+
+import test_gpu_conv_kernels as K
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_2103_08802_gb300 import build
+    build.build()
+
+
+def _name(base, kind):
+    """The forward test takes its epilogue from the name's length: 0 bf16 y, 2 bf16 y + bf16 residual."""
+    while len(base) % 3 != kind:
+        base += "_"
+    return base
+
+
+def _pw(batch, h, w, c, k, **kw):
+    return dict(batch=batch, h=h, w=w, c=c, k=k, ksize=1, stride=1, **kw)
+
+
+PW = {
+    "m1": _pw(1, 1, 1, 16, 64, bn=True),
+    "m127": _pw(1, 127, 1, 64, 16, bn=True),
+    "m128": _pw(2, 8, 8, 32, 128, bn=True),
+    "m129": _pw(3, 43, 1, 16, 16, bn=True, relu=False),
+    "m31": _pw(1, 31, 1, 32, 32, bn=False),
+    "c128_k32": _pw(2, 15, 15, 128, 32, bn=True),
+    "c256_k64": _pw(2, 9, 15, 256, 64, bn=True),
+    "c64_k256": _pw(3, 9, 15, 64, 256, bn=True),
+    "c64_k192": _pw(1, 20, 20, 64, 192, bn=True),
+    "c64_k64_fp32x": _pw(2, 15, 15, 64, 64, bn=True, x_fp32=True),
+    "many_k64": _pw(6, 100, 100, 16, 64, bn=True),     # 469 m-tiles: whole rows of units an item
+    "many_k256": _pw(5, 100, 101, 32, 256, bn=True),   # 395 m-tiles, four units each
+    "many_k16": _pw(5, 100, 101, 128, 16, bn=True),
+    "expand": [_pw(2, 16, 16, 16, 64, bn=True), _pw(2, 9, 9, 64, 256, bn=True)],
+    "reduce": [_pw(2, 16, 16, 64, 16, bn=True), _pw(2, 9, 9, 256, 64, bn=False)],
+}
+CASES = [(n, kind) for n in PW for kind in (0, 2)]
+
+
+def _install(monkeypatch, name, spec):
+    if isinstance(spec, list):
+        monkeypatch.setitem(K.GROUPS, name, spec)
+    else:
+        monkeypatch.setitem(K.CASES, name, spec)
+
+
+@pytest.mark.parametrize("base,kind", CASES)
+def test_pointwise_forward(monkeypatch, base, kind):
+    if isinstance(PW[base], list):
+        kind = 2  # the two instances: bf16 y + residual, bf16 y
+    name = _name(base, kind)
+    _install(monkeypatch, name, PW[base])
+    K.test_conv_forward(name, "auto")
+
+
+@pytest.mark.parametrize("base", list(PW))
+def test_pointwise_data_gradient(monkeypatch, base):
+    _install(monkeypatch, base, PW[base])
+    K.test_conv_data_gradient(base, "auto")
+
+
+def test_nonfinite_residual_stays_in_its_element():
+    """An infinite residual element makes that output infinite and no other."""
+    import torch
+    from paper_2103_08802_gb300 import pnn
+    torch.manual_seed(3)
+    d = dict(batch=1, h=16, w=16, c=16, k=64, ksize=1, stride=1)
+    d["x"] = torch.randn(1, 16, 16, 16, device="cuda").bfloat16()
+    d["wt"] = torch.randn(64, 1, 1, 16, device="cuda").bfloat16()
+    d["y"] = torch.empty(1, 16, 16, 64, dtype=torch.bfloat16, device="cuda")
+    d["res"] = torch.randn(1, 16, 16, 64, device="cuda").bfloat16()
+    d["res"][0, 3, 5, 7] = float("inf")
+    pnn.conv_run("forward", [d])
+    bad = ~torch.isfinite(d["y"].float())
+    assert bad.sum().item() == 1 and bad[0, 3, 5, 7].item()
