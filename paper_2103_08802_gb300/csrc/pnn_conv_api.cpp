@@ -155,7 +155,18 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
     all_pw = all_pw && pw_inst(mode, a[i]);
     mtiles += cdv((int64_t)a[i].batch * a[i].h * a[i].w, kTcBM);  // (stride 1)
   }
-  if (all_pw) pl.variant = 4;
+  // the weight gradients of k_wg_conv.cu: one kernel size a launch
+  bool all_wg = impl == 0 && mode == 2;
+  double wg_bytes = 0;
+  auto wg_traffic = [](const pnn_conv_args& g) {
+    return (double)g.batch * g.h * g.w * (g.c * (g.x_dtype == PNN_DT_BF16 ? 2 : 4) + g.k * 4.0);
+  };
+  for (int i = 0; i < n && all_wg; ++i) {
+    all_wg = a[i].ksize == a[0].ksize &&
+             wg_ok(a[i].ksize, a[i].stride, a[i].c, a[i].k, a[i].h, a[i].w, a[i].x_dtype == PNN_DT_BF16);
+    wg_bytes += wg_traffic(a[i]);
+  }
+  if (all_pw || all_wg) pl.variant = 4;
   size_t cur = 0;
   auto take = [&](size_t b) { size_t o = cur; cur = al256(cur + b); return o; };
   pl.tab = take((size_t)n * sizeof(ConvDesc));
@@ -210,6 +221,19 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
     } else {
       ip.rows = tc_tile_rows(2, pl.variant, g.c);
       ip.mtiles = cdv(rsc, ip.rows);
+      if (all_wg) {
+        const WgPlan wp = wg_plan(g.ksize, g.c, g.k, g.h, g.w, g.x_dtype == PNN_DT_BF16);
+        ip.ntiles = wg_ntiles(g.ksize, g.c);
+        const WgSplit sp = wg_split(Mout, wp.kp, ip.ntiles, wg_traffic(g), wg_bytes);
+        ip.mtiles = ip.splits = sp.splits;
+        ip.pix_per_split = sp.pix;
+        pl.raw = std::max(pl.raw, wp.raw);
+        pl.op = std::max(pl.op, wp.op);
+        pl.bnmax = g.ksize;
+        pl.total += ip.splits * ip.ntiles;
+        ip.maps = take(4 * 128);
+        continue;
+      }
       const int base = ip.mtiles * ip.ntiles;
       int splits = std::max(1, std::min(cdv(Mout, 256), cdv(2 * (int64_t)sms, base)));
       ip.pix_per_split = cdv(cdv(Mout, splits), 64) * 64;
@@ -269,7 +293,7 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
   pl.wide = pl.variant == 1 && mode != 2;
   for (int i = 0; i < n; ++i)
     if (a[i].ksize * a[i].ksize * (mode == 0 ? a[i].c : a[i].k) > 64) pl.wide = 0;
-  if (pl.variant == 4) {
+  if (pl.variant == 4 && mode != 2) {
     pl.raw = pl.op = 0;
     pl.wide = mode == 0;
     for (int i = 0; i < n; ++i) {
@@ -388,7 +412,19 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       c.tma_y = mode == 2 ? nullptr : ws + ip.maps + 256;
       c.tma_h = ip.halo ? ws + ip.maps + 384 : nullptr;
     }
-    if (pl.variant == 4) {
+    if (pl.variant == 4 && mode == 2) {
+      const char* why = nullptr;
+      uint8_t* m = at(ip.maps);
+      const bool xbf = g.x_dtype == PNN_DT_BF16;
+      const WgPlan wp = wg_plan(g.ksize, g.c, g.k, g.h, g.w, xbf);
+      int e = encode_tensor_map_2d(m, g.x, xbf, g.c, Min, wp.xch, wp.xrows, 0, &why);
+      if (!e) e = encode_tensor_map_2d(m + 128, g.dy, false, g.k, Mout, g.k, wp.kp, 0, &why);
+      if (e) return set_last_error(PNN_ECUDA, why);
+      c.tma_a = ws + ip.maps;
+      c.tma_b = ws + ip.maps + 128;
+      wrs.back().transposed = wp.x_is_a;
+    }
+    if (pl.variant == 4 && mode != 2) {
       const char* why = nullptr;
       uint8_t* m = at(ip.maps);
       const int ch = mode == 1 ? g.k : g.c, ncols = mode == 1 ? g.c : g.k, bn = pw_unit_cols(ncols);
@@ -454,7 +490,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       bfins.push_back(b);
       fin_ts.push_back(fin_ts.back() + fin_ctas(g.c));
     }
-    ts[i + 1] = ts[i] + (mode == 2 ? ip.mtiles * ip.ntiles * ip.splits : ip.mtiles * ip.ntiles);
+    ts[i + 1] = ts[i] + (mode == 2 && pl.variant != 4 ? ip.mtiles * ip.ntiles * ip.splits : ip.mtiles * ip.ntiles);
   }
   memcpy(at(pl.tab), cds.data(), cds.size() * sizeof(ConvDesc));
   memcpy(at(pl.ts), ts.data(), ts.size() * sizeof(int));
@@ -474,6 +510,8 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
   if (e == cudaSuccess && mode == 1)
     e = launch_wtrans(reinterpret_cast<const WtDesc*>(ws + pl.aux_tab), auxts, n, aux_ts.back(), st);
   auto conv_launch = [&]() {
+    if (pl.variant == 4 && mode == 2)
+      return launch_conv_wg(pl.bnmax, tab, tsd, n, pl.total, pl.raw, pl.op, status, st);
     if (pl.variant == 4)
       return launch_conv_pw(mode, pl.wide, tab, tsd, n, pl.total, pl.raw, pl.op, status, st);
     if (pl.variant == 1)

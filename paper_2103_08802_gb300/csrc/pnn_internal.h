@@ -4,6 +4,7 @@
 // tile_start[i] <= b < tile_start[i+1].  Tensors are NHWC with the batch
 // folded into the row index (row m = (n*H + h)*W + w).
 #pragma once
+#include <algorithm>
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -147,9 +148,8 @@ struct PoolDesc {
   int32_t tiles;
 };
 
-// wgrad split reduction: dw[K*RSC] = sum_s part[s][K*RSC]
 // wgrad split reduction: dw[K*RSC] = sum_s part[s][...]; partials are laid out
-// [s][K][RSC] (CUDA-core wgrad) or [s][RSC][K] (tensor-core wgrad, transposed = 1)
+// [s][K][RSC] or [s][RSC][K] (transposed = 1)
 struct WReduceDesc {
   const float* part;
   float* dw;
@@ -235,6 +235,10 @@ bool conv_halo_fits(int mode, int W, int ch, int bn);
 // k-step and at least 64 output columns
 cudaError_t launch_conv_pw(int mode, int wide, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes,
                            int x_bytes, int32_t* status, cudaStream_t st, int max_ctas = 0);
+// weight gradient of k_wg_conv.cu; raw_bytes, op_bytes: the largest slots over
+// the launch's instances (multiples of 1024)
+cudaError_t launch_conv_wg(int ksize, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes, int op_bytes,
+                           int32_t* status, cudaStream_t st, int max_ctas = 0);
 // record a message for pnn_last_error(NULL) and return `code`
 int set_last_error(int code, const char* msg);
 // streaming multiprocessors of the current device, queried once per device
@@ -363,6 +367,83 @@ inline int pw_x_bytes(int ncols) { return kTcBM * pw_unit_cols(ncols) * 2; }
 // the launch has too few m-tiles to occupy the SMs twice over
 inline int pw_item_units(int ncols, int64_t launch_mtiles) {
   return launch_mtiles >= 2 * (int64_t)device_sm_count() ? ncols / pw_unit_cols(ncols) : 1;
+}
+// Weight gradient of k_wg_conv.cu (variant 4: 1x1, 5: 3x3): the geometry of one instance's
+// k-steps.  1x1: kp pixels; 3x3: krows whole image rows (kp pixels) with the
+// activation rows above and below.  Raw slot: x rows, then dY rows; operand
+// slot: the M side's planes (8 channels each, apitch bytes), then (boff) the N
+// side's.  A plane pitch of 8 / planes (mod 8) 16-byte rows spreads a warp's
+// stores over the banks.
+struct WgPlan {
+  int kp, krows, lgw;
+  int xch, xrows;          // x channels of a tile and raw rows of a k-step
+  int x_is_a, mch, nch;    // M side: x or dY; channels of both sides (3x3: the N side holds three copies)
+  int apitch, bpitch, boff;
+  int yoff, raw, op;
+};
+constexpr int kWgRawMax = 40 * 1024;  // a raw slot: two stages and two operand slots fit
+PNN_HD inline int wg_plane_pad(int ch) { return ch >= 64 ? 1 : 64 / ch; }
+PNN_HD inline WgPlan wg_plan(int ks, int C, int K, int H, int W, bool xbf) {
+  WgPlan p{};
+  const int esz = xbf ? 2 : 4;
+  if (ks == 1) {
+    p.kp = 128;
+    while (p.kp > 32 && p.kp * (C * esz + K * 4) > kWgRawMax) p.kp >>= 1;
+    p.xch = C;
+    p.xrows = p.kp;
+    p.x_is_a = C > K;
+    p.mch = C > K ? C : K;
+    p.nch = C > K ? K : C;
+    p.bpitch = (p.kp + wg_plane_pad(p.nch)) * 16;
+  } else {
+    p.xch = C < 32 ? C : 32;
+    p.mch = K;
+    p.nch = p.xch;
+    p.lgw = W == 8 ? 3 : (W == 16 ? 4 : 5);
+    for (int r = 128 / W; r >= 1; --r) {
+      if (H % r || (r * W) % 16 || (r + 2) * W > 256) continue;
+      if ((r + 2) * W * p.xch * esz + r * W * K * 4 > kWgRawMax) continue;
+      p.krows = r;
+      break;
+    }
+    p.kp = p.krows * W;
+    p.xrows = (p.krows + 2) * W;  // (a multiple of 8)
+    p.bpitch = (p.xrows + wg_plane_pad(p.xch)) * 16;
+  }
+  p.apitch = (p.kp + wg_plane_pad(p.mch)) * 16;
+  p.boff = p.mch / 8 * p.apitch;
+  p.op = (p.boff + (ks == 1 ? 1 : 3) * (p.nch / 8) * p.bpitch + 1023) & ~1023;
+  p.yoff = (p.xrows * p.xch * esz + 127) & ~127;
+  p.raw = (p.yoff + p.kp * K * 4 + 1023) & ~1023;
+  return p;
+}
+bool wg_fits(int raw_bytes, int op_bytes);
+inline bool wg_ok(int k, int stride, int C, int K, int H, int W, bool xbf) {
+  auto pow2 = [](int v, int lo, int hi) { return v >= lo && v <= hi && (v & (v - 1)) == 0; };
+  if (stride != 1 || !pow2(C, 16, 256) || !pow2(K, 16, 256)) return false;
+  if (k == 1) {
+    if (C > 64 && K > 64) return false;
+  } else {
+    if (k != 3 || C > 64 || K > 128 || !pow2(W, 8, 32)) return false;
+  }
+  const WgPlan p = wg_plan(k, C, K, H, W, xbf);
+  return p.kp > 0 && wg_fits(p.raw, p.op);
+}
+// tiles of an instance per split
+PNN_HD inline int wg_ntiles(int ks, int C) { return ks == 3 && C > 32 ? C / 32 : 1; }
+// Splits of the instances of one launch: about two tiles per SM over the
+// launch, each instance in proportion to the bytes it moves, whole k-steps.
+// (With 2 x SMs splits for every instance, as a launch of its own needs, eight
+// instances wrote and reduced eight times the partial sums.)
+struct WgSplit { int splits, pix; };
+inline WgSplit wg_split(int64_t rows, int kp, int ntiles, double bytes, double launch_bytes) {
+  const double share = 2.0 * device_sm_count() * bytes / launch_bytes / ntiles;
+  int64_t s = (int64_t)(share + 0.5);
+  const int64_t steps = (rows + kp - 1) / kp;
+  s = s < 1 ? 1 : (s > steps ? steps : s);
+  // k-steps a split: at least 256 pixels (a partial sum is as large as the layer)
+  const int64_t per = std::max<int64_t>((steps + s - 1) / s, (256 + kp - 1) / kp);
+  return WgSplit{(int)((steps + per - 1) / per), (int)(per * kp)};
 }
 // N columns of a tile when the layer needs several: 128 for the TMA-fed
 // forward and data gradient (a smaller operand slot leaves room for more

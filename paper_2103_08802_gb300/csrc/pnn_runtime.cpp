@@ -112,7 +112,7 @@ struct Launch {
   int esz = 4;          // TMA-fed conv: largest element size of the A sources
   int raw = 0;          // TMA-fed conv: raw slot bytes of one stage
   int op = 0;           // TMA-fed conv with halo tiles: operand slot bytes of one stage (0: default);
-                        // variant 4: second-operand bytes of a unit
+                        // variant 4: second-operand bytes of a unit, or (weight gradient) operand slot bytes
   int wide = 0;         // TMA-fed forward / data gradient: every tile one k-step (the wide-epilogue variant)
   int block = -1;       // fine forward / backward: position of the layer in its segment
 };
@@ -538,6 +538,9 @@ struct pnn_net {
                                                              vals[src].dt == DT_BF16)
                              ? 1
                              : 0;
+            if (tma_impl(opt.conv_impl) && wg_ok(f.k, f.stride, vals[f.in].C, ov.C, vals[f.in].H, vals[f.in].W,
+                                                 vals[src].dt == DT_BF16))
+              wg.variant = f.k == 3 ? 5 : 4;  // (its splits follow from the launch it joins, below)
           }
           wg.mtiles = cdiv(RSC, tc_mtile_rows(wg.kind, wg.variant, vals[f.in].C));
           wg.ntiles = cdiv(ov.C, 256);
@@ -1121,6 +1124,29 @@ int pnn_net::plan(const pnn_desc* d) {
   }
   pre_b.resize(N);
   for (int j = 0; j < N; ++j) backward_list(pre_f[j], pre_b[j]);
+  // splits of the k_wg_conv.cu weight gradients: by the launches they form
+  for (int p = 5; p < 10; ++p)
+    for (const Group& g : phase_groups(p)) {
+      if (g.kind != K_WGRAD_TC || g.variant < 4) continue;
+      auto traffic = [&](const POp& o) {
+        const int src = vals[o.in].virt ? vals[o.in].src : o.in;
+        return (double)rows(o.in) * (vals[o.in].C * (vals[src].dt == DT_BF16 ? 2 : 4) + vals[o.out].C * 4.0);
+      };
+      double all = 0;
+      for (int id : g.ops) all += traffic(ops[id]);
+      for (int id : g.ops) {
+        POp& o = ops[id];
+        const Value& iv = vals[o.in];
+        const int src = iv.virt ? iv.src : o.in;
+        const WgPlan wp = wg_plan(o.k, iv.C, vals[o.out].C, iv.H, iv.W, vals[src].dt == DT_BF16);
+        o.ntiles = wg_ntiles(o.k, iv.C);
+        const WgSplit sp = wg_split(rows(o.in), wp.kp, o.ntiles, traffic(o), all);
+        o.splits = o.mtiles = sp.splits;
+        o.pix_per_split = sp.pix;
+        o.tiles = o.splits * o.ntiles;
+        ops[id + 1].splits = o.splits;  // its reduction, planned right after it
+      }
+    }
   // gradient-accumulating parameters (delta mode: F^j used twice)
   {
     std::vector<int> seen(params.size(), 0);
@@ -1398,6 +1424,21 @@ int pnn_net::build_tables() {
               c.ntile_w = units * bn;
               c.ntiles = cdiv(ncols, c.ntile_w);
             }
+            if (o.kind == K_WGRAD_TC && o.variant >= 4) {
+              const bool xbf = c.x.dt == DT_BF16;
+              const WgPlan wp = wg_plan(o.k, iv.C, ov.C, iv.H, iv.W, xbf);
+              CUtensorMap maps[2];
+              memset(maps, 0, sizeof maps);
+              if (ws) {
+                int r = encode_map(&maps[0], c.x.ptr, xbf, iv.C, (int64_t)B * iv.H * iv.W, wp.xch, wp.xrows, 0);
+                if (!r) r = encode_map(&maps[1], P<float>(gptr(o.out)), false, ov.C, (int64_t)B * ov.H * ov.W, ov.C,
+                                       wp.kp, 0);
+                if (r) return r;
+              }
+              const size_t mo = put(maps, sizeof maps);
+              c.tma_a = ws ? ws + tables_off + mo : nullptr;
+              c.tma_b = ws ? ws + tables_off + mo + sizeof(CUtensorMap) : nullptr;
+            }
             if (o.kind == K_WGRAD_TC && o.variant == 1) {
               // activation halo box [hrows][cwx] (its dtype), gradient box [64][K] fp32
               const WgBoxes bx = wg_boxes(iv.C, ov.C, iv.W, o.pad, c.x.dt == DT_BF16);
@@ -1454,7 +1495,10 @@ int pnn_net::build_tables() {
             r.dw = grad + params[o.w].off;
             r.splits = o.splits;
             r.accumulate = o.acc;
-            r.transposed = wg->kind == K_WGRAD_TC;
+            // [s][RSC][K] unless the gradient is the M side of k_wg_conv.cu
+            r.transposed = wg->kind == K_WGRAD_TC &&
+                           (wg->variant < 4 ||
+                            wg_plan(o.k, vals[o.in].C, vals[o.out].C, vals[o.in].H, vals[o.in].W, true).x_is_a);
             r.kout = vals[o.out].C;
             r.rsc = o.k * o.k * vals[o.in].C;
             r.n = (int64_t)params[o.w].n;
@@ -1629,6 +1673,16 @@ int pnn_net::build_tables() {
           if (ch > 64 || ncols < 64) L.wide = 0;
         }
       }
+      if (g.kind == K_WGRAD_TC && g.variant >= 4) {
+        L.raw = L.op = 0;
+                for (int id : g.ops) {
+          const POp& o = ops[id];
+          const int src = vals[o.in].virt ? vals[o.in].src : o.in;
+          const WgPlan wp = wg_plan(o.k, vals[o.in].C, vals[o.out].C, vals[o.in].H, vals[o.in].W, vals[src].dt == DT_BF16);
+          L.raw = std::max(L.raw, wp.raw);
+          L.op = std::max(L.op, wp.op);
+        }
+      }
       for (int id : g.ops) op_cost(ops[id], L.flops, L.bytes);
       tstart.push_back(total);
       L.table_off = put(tab.data(), tab.size());
@@ -1782,6 +1836,11 @@ int pnn_net::run_phase(int p, cudaStream_t st, int cap) {
                                        st, cap);
         break;
       case K_WGRAD_TC:
+        if (L.variant >= 4) {
+          e = launch_conv_wg(L.variant == 5 ? 3 : 1, (const ConvDesc*)tab, ts, L.count, L.total, L.raw, L.op, P<int32_t>(status_off), st,
+                             cap);
+          break;
+        }
         e = L.variant == 1
                 ? launch_conv_tma(2, L.wide, (const ConvDesc*)tab, ts, L.count, L.total, L.aux, L.raw, L.op,
                                   P<int32_t>(status_off), st, cap)
@@ -2673,7 +2732,7 @@ int pnn_profile_trace(pnn_net* n, int32_t max, pnn_trace* out, int32_t* count) {
     pnn_trace& r = out[i];
     float t = 0.f;
     cudaEventElapsedTime(&t, n->pev[2 * i], n->pev[2 * i + 1]);
-    r.kind = L.kind; r.variant = L.variant == 4 ? 4 : L.variant + (L.wide ? 1 : (L.op > 0 ? 2 : 0)); r.phase = L.phase; r.instances = L.count;
+    r.kind = L.kind; r.variant = L.variant >= 4 ? L.variant : L.variant + (L.wide ? 1 : (L.op > 0 ? 2 : 0)); r.phase = L.phase; r.instances = L.count;
     r.tiles = L.total;
     for (int j = 0; j < 6; ++j) r.shape[j] = L.shape[j];
     r.block = L.block;

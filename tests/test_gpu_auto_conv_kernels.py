@@ -83,3 +83,35 @@ def test_nonfinite_residual_stays_in_its_element():
     pnn.conv_run("forward", [d])
     bad = ~torch.isfinite(d["y"].float())
     assert bad.sum().item() == 1 and bad[0, 3, 5, 7].item()
+
+
+def _wg(batch, h, w, c, k, ks, **kw):
+    return dict(batch=batch, h=h, w=w, c=c, k=k, ksize=ks, stride=1, **kw)
+
+
+WG = {
+    "one_pixel": _wg(1, 1, 1, 16, 64, 1, bn=True),
+    "m127": _wg(1, 127, 1, 64, 16, 1, bn=True),
+    "m129": _wg(3, 43, 1, 32, 32, 1, bn=True, relu=False),
+    "many": _wg(5, 100, 101, 16, 64, 1, bn=True),        # several k-steps a split, a ragged last one
+    "k256": _wg(3, 20, 20, 64, 256, 1, bn=True),         # two halves of the M side, gradient on it
+    "c256": _wg(3, 20, 20, 256, 64, 1, bn=True),         # ... activation on it
+    "c256_fp32x": _wg(2, 15, 15, 256, 16, 1, bn=True, x_fp32=True),
+    "c128_raw": _wg(2, 15, 15, 128, 32, 1, bn=False),
+    "group_1x1": [_wg(2, 16, 16, 64, 16, 1, bn=True), _wg(2, 8, 8, 128, 32, 1, bn=True),
+                  _wg(2, 4, 4, 256, 64, 1, bn=True)],
+    "w32": _wg(3, 32, 32, 16, 16, 3, bn=True),
+    "w32_h6": _wg(2, 6, 32, 16, 32, 3, bn=True),         # k-steps of three rows
+    "w16_h5": _wg(3, 5, 16, 32, 16, 3, bn=True),         # one k-step an image
+    "w8": _wg(3, 8, 8, 64, 64, 3, bn=True),              # two channel halves, row-strided pixel groups
+    "w8_h16_k128": _wg(2, 16, 8, 32, 128, 3, bn=False),
+    "w16_fp32x": _wg(2, 16, 16, 64, 16, 3, bn=True, x_fp32=True, relu=False),
+    "group_3x3": [_wg(4, 32, 32, 16, 16, 3, bn=True), _wg(2, 16, 16, 32, 32, 3, bn=True),
+                  _wg(2, 8, 8, 64, 64, 3, bn=True)],
+}
+
+
+@pytest.mark.parametrize("base", list(WG))
+def test_weight_gradient(monkeypatch, base):
+    _install(monkeypatch, base, WG[base])
+    K.test_conv_weight_gradient(base, "auto")
