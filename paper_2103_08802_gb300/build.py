@@ -19,7 +19,7 @@ CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 NVCC = os.path.join(CUDA, "bin", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
-CU_SOURCES = ["k_simt.cu", "k_tc_conv.cu", "k_pw_conv.cu", "k_wg_conv.cu"]
+CU_SOURCES = ["k_simt.cu", "k_tc_conv.cu", "k_pw_conv.cu", "k_wg_conv.cu", "k_c3_conv.cu"]
 CPP_SOURCES = ["pnn_runtime.cpp", "pnn_conv_api.cpp"]
 
 

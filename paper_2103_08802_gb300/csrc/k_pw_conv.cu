@@ -37,6 +37,7 @@
 
 #include <algorithm>
 
+#include "narrow_epilogue.cuh"
 #include "pnn.h"
 #include "pnn_internal.h"
 #include "tc_pair.cuh"
@@ -47,7 +48,6 @@ namespace {
 
 using namespace tc;
 
-enum { FWD = 0, DGRAD = 1 };
 constexpr int kRows = 128;
 constexpr int kOpBytes = kRows * 128;      // one k-step's A operand (64 bf16 a row)
 constexpr int kUnitB = 64 * 128;           // a unit's weight box: up to 64 rows x 64 bf16
@@ -55,7 +55,6 @@ constexpr int kMaxRing = 4;
 constexpr int kAcc = 4;                    // TMEM accumulators of 64 columns
 constexpr int kAccCols = 64;
 constexpr int kSmemBudget = 227 * 1024;
-constexpr int kRedBytes = 2 * 4 * 64 * 8;  // per epilogue group: [2][4 warps][64 columns] pairs
 
 // W = 1 (forward, every instance one k-step and N >= 64): the epilogue does
 // most of the work, 2 transform + 12 epilogue warps; else 6 + 8.
@@ -66,8 +65,7 @@ struct Roles {
   static constexpr int kProducer = 0, kMma = 1, kT0 = 2, kE0 = 2 + kT;
   static constexpr int kThreads = 32 * (2 + kT + kE);
   static constexpr int kGroups = kE / 4;
-  // per-warp output staging: forward one 32 x 64 bf16 tile, data gradient two of 32 x 32 fp32
-  static constexpr int kStage = MODE == FWD ? 4096 : 8192;
+  static constexpr int kStage = stage_bytes(MODE);
 };
 static_assert(Roles<FWD, 0>::kE0 % 4 == 0 && Roles<FWD, 1>::kE0 % 4 == 0, "epilogue groups start at a TMEM lane quarter");
 
@@ -121,13 +119,6 @@ __device__ __forceinline__ Geo geo(const ConvDesc* d) {
   g.nsub = g.ncols / g.bn;
   g.spi = d->ntile_w / g.bn;
   return g;
-}
-
-// whether a unit has a second operand: the residual (forward), the BN input
-// of the sums (data gradient)
-template <int MODE>
-__device__ __forceinline__ bool has_x(const ConvDesc* d) {
-  return MODE == FWD ? d->res != nullptr : d->bnb_part != nullptr;
 }
 
 // ------------------------------------------------------------ transform
@@ -186,232 +177,14 @@ __device__ __forceinline__ void transform_rows(const uint8_t* __restrict__ raw, 
   }
 }
 
-// ------------------------------------------------------------ epilogue
-// byte offset of 16-byte chunk j of a row in a TMA-swizzled tile of PITCH-byte rows
-template <int PITCH>
-__device__ __forceinline__ uint32_t swp(int row, int j) {
-  if (PITCH == 128) return (uint32_t)(row * 128 + ((j ^ (row & 7)) << 4));
-  if (PITCH == 64) return (uint32_t)(row * 64 + ((j ^ ((row >> 1) & 3)) << 4));
-  return (uint32_t)(row * 32 + ((j ^ ((row >> 2) & 1)) << 4));
-}
-
-struct EpiState {
-  float2* red;  // this group's [2][4][64] pairs
-  int rbuf;     // which half the next unit uses
-  int bar;      // the group's named barrier
+// where a warp's 32 rows of an output tile go
+struct RowDst {
+  int m0;
+  __device__ __forceinline__ void put(const void* map, int n, int q, uint32_t src, bool add) const {
+    if (add) tma_reduce_add_2d(map, n, m0 + q * 32, src);
+    else tma_store_2d(map, n, m0 + q * 32, src);
+  }
 };
-
-// The four warps' column pairs of a unit -> the tile's partial: forward (mean,
-// M2) merged in order, data gradient plain sums.  Every warp of the group
-// calls it (ok: its own values are valid); one barrier, the halves of red
-// alternate.
-template <int MODE, int BN>
-__device__ __forceinline__ void merge_partials(EpiState& es, bool ok, int q, int lane, int rows, int m0, float* part) {
-  float2* red = es.red + es.rbuf * 256;
-  es.rbuf ^= 1;
-  asm volatile("bar.sync %0, 128;" ::"r"(es.bar) : "memory");
-  const int j = q * 32 + lane;
-  if (j < BN && ok) {
-    float a, b;
-    if (MODE == FWD) {
-      float n = 0.f;
-      a = b = 0.f;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int nq = min(32, max(0, rows - (m0 + 32 * i)));
-        const float2 v = red[i * 64 + j];
-        chan_merge(n, a, b, (float)nq, v.x, v.y);
-      }
-    } else {
-      const float2 v0 = red[j], v1 = red[64 + j], v2 = red[128 + j], v3 = red[192 + j];
-      a = v0.x + v1.x + v2.x + v3.x;
-      b = v0.y + v1.y + v2.y + v3.y;
-    }
-    *reinterpret_cast<float2*>(part + 2 * j) = make_float2(a, b);
-  }
-}
-
-// (mean, M2) of the columns of a staged bf16 tile [32][BN] over its first
-// nvalid rows: lane = column pair l % (BN/2) of rows (l / (BN/2)) + RG i, two
-// passes (the sums, then the squared deviations from the warp mean)
-template <int BN, bool FULL>
-__device__ __forceinline__ void staged_moments(const uint8_t* st, int lane, int nvalid, float2* out) {
-  constexpr int PITCH = BN * 2, PAIRS = BN / 2, RG = 32 / PAIRS, IT = 32 / RG;
-  const int p = lane % PAIRS, g = lane / PAIRS;
-  uint32_t w[IT];
-#pragma unroll
-  for (int i = 0; i < IT; ++i)
-    w[i] = *reinterpret_cast<const uint32_t*>(st + swp<PITCH>(RG * i + g, p >> 2) + (p & 3) * 4);
-  uint64_t s[2] = {0ull, 0ull};
-#pragma unroll
-  for (int i = 0; i < IT; ++i) {
-    if (!FULL && RG * i + g >= nvalid) w[i] = 0u;
-    s[i & 1] = add2(s[i & 1], bf2(w[i]));
-  }
-  float2 sum = un2(add2(s[0], s[1]));
-#pragma unroll
-  for (int o = PAIRS; o < 32; o <<= 1) {
-    sum.x += __shfl_xor_sync(0xffffffffu, sum.x, o);
-    sum.y += __shfl_xor_sync(0xffffffffu, sum.y, o);
-  }
-  const float n = (float)nvalid;
-  const float mx = FULL ? sum.x * 0.03125f : (nvalid > 0 ? sum.x / n : 0.f);
-  const float my = FULL ? sum.y * 0.03125f : (nvalid > 0 ? sum.y / n : 0.f);
-  const uint64_t neg = pk2(-mx, -my);
-  s[0] = s[1] = 0ull;
-#pragma unroll
-  for (int i = 0; i < IT; ++i) {
-    const uint64_t d = add2(bf2(w[i]), neg);
-    if (FULL || RG * i + g < nvalid) s[i & 1] = fma2(d, d, s[i & 1]);
-  }
-  float2 m2 = un2(add2(s[0], s[1]));
-#pragma unroll
-  for (int o = PAIRS; o < 32; o <<= 1) {
-    m2.x += __shfl_xor_sync(0xffffffffu, m2.x, o);
-    m2.y += __shfl_xor_sync(0xffffffffu, m2.y, o);
-  }
-  if (g == 0) *reinterpret_cast<float4*>(out + 2 * p) = make_float4(mx, m2.x, my, m2.y);
-}
-
-// Forward unit: accumulator + residual -> bf16 -> staging -> TMA store, statistics.
-template <int BN>
-__device__ __forceinline__ void unit_fwd(const ConvDesc* d, uint32_t tacc, int q, int lane, int rows, int m0, int n0,
-                                         const uint8_t* x, uint8_t* st, float2* redw, uint32_t tempty, uint32_t uempty,
-                                         bool res, bool stats) {
-  uint32_t a[BN];
-#pragma unroll
-  for (int j = 0; j < BN; j += 32) {
-    if (BN >= 32) tmem_ld32(tacc + j, a + j);
-    else tmem_ld16_nowait(tacc + j, a + j);
-  }
-  tmem_wait_ld(a);
-  fence_before();
-  __syncwarp();
-  if (lane == 0) mbar_arrive(tempty);
-  constexpr int PITCH = BN * 2;
-  uint32_t o[BN / 2];
-  if (res) {
-#pragma unroll
-    for (int j = 0; j < BN / 8; ++j) {
-      const uint4 r = *reinterpret_cast<const uint4*>(x + swp<PITCH>(q * 32 + lane, j));
-      const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int c = 8 * j + 2 * i;
-        o[4 * j + i] = pack2(add2(pk2(__uint_as_float(a[c]), __uint_as_float(a[c + 1])), bf2(w[i])));
-      }
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < BN / 2; ++i) o[i] = pack_bf16(__uint_as_float(a[2 * i]), __uint_as_float(a[2 * i + 1]));
-  }
-  // the store issued from this tile for the previous unit must have read it,
-  // and every lane must be done with its statistics
-  if (lane == 0) bulk_wait_read<0>();
-  __syncwarp();
-  if (res && lane == 0) mbar_arrive(uempty);  // X has been read
-#pragma unroll
-  for (int j = 0; j < BN / 8; ++j)
-    *reinterpret_cast<uint4*>(st + swp<PITCH>(lane, j)) = make_uint4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
-  fence_proxy_async();
-  __syncwarp();
-  const int nvalid = min(32, max(0, rows - (m0 + q * 32)));
-  if (lane == 0 && nvalid > 0) {
-    tma_store_2d(d->tma_y, n0, m0 + q * 32, smem_u32(st));
-    bulk_commit();
-  }
-  if (stats) {
-    if (nvalid == 32) staged_moments<BN, true>(st, lane, 32, redw);
-    else staged_moments<BN, false>(st, lane, nvalid, redw);
-  }
-}
-
-// BN-backward sums of HC columns of a staged dX tile [32][HC] fp32 with the
-// unit's h tile [128][BN] bf16: g = dX masked by the ReLU of the forward BN
-// output, xhat = (h - mean) * rstd; (sum g, sum g xhat) over the valid rows.
-template <int BN, bool FULL>
-__device__ __forceinline__ void staged_bn_sums(const uint8_t* st, const uint8_t* h, int c0, const ConvDesc* d, int n0, int q,
-                                               int lane, int nvalid, float2* out) {
-  constexpr int HC = BN < 32 ? BN : 32;
-  constexpr int PAIRS = HC / 2, RG = 32 / PAIRS, IT = 32 / RG;
-  const int p = lane % PAIRS, g = lane / PAIRS;
-  const int c = n0 + c0 + 2 * p;
-  const float2 scv = __ldg(reinterpret_cast<const float2*>(d->x.scale + c));
-  const float2 shv = __ldg(reinterpret_cast<const float2*>(d->x.shift + c));
-  const float2 muv = __ldg(reinterpret_cast<const float2*>(d->bn_mean + c));
-  const float2 rsv = __ldg(reinterpret_cast<const float2*>(d->bn_rstd + c));
-  const uint64_t sc = pk2(scv.x, scv.y), sh = pk2(shv.x, shv.y), nmu = pk2(-muv.x, -muv.y), rs = pk2(rsv.x, rsv.y);
-  const bool relu = d->x.relu != 0;
-  uint64_t s1 = 0ull, s2 = 0ull;
-#pragma unroll
-  for (int i = 0; i < IT; ++i) {
-    // rows r and r + 4 of 128-byte h rows fall into different halves of the banks
-    const int r = BN == 64 ? (i & 3) + 8 * (i >> 2) + 4 * g : RG * i + g;
-    const int hc = c0 / 2 + p;
-    const uint32_t hw =
-        *reinterpret_cast<const uint32_t*>(h + swp<BN * 2>(q * 32 + r, hc >> 2) + (hc & 3) * 4);
-    const float2 dv = *reinterpret_cast<const float2*>(st + swp<HC * 4>(r, p >> 1) + (p & 1) * 8);
-    const uint64_t hv = bf2(hw);
-    const float2 z = un2(fma2(sc, hv, sh));
-    const bool in = FULL || r < nvalid;
-    const uint64_t gv = pk2(in && (!relu || z.x > 0.f) ? dv.x : 0.f, in && (!relu || z.y > 0.f) ? dv.y : 0.f);
-    const uint64_t xh = mul2(add2(hv, nmu), rs);
-    s1 = add2(s1, gv);
-    // (a row past the end adds nothing: its h may be anything)
-    if (in) s2 = fma2(gv, xh, s2);
-  }
-  float2 a = un2(s1), b = un2(s2);
-#pragma unroll
-  for (int o = PAIRS; o < 32; o <<= 1) {
-    a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
-    a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
-    b.x += __shfl_xor_sync(0xffffffffu, b.x, o);
-    b.y += __shfl_xor_sync(0xffffffffu, b.y, o);
-  }
-  if (g == 0) *reinterpret_cast<float4*>(out + c0 + 2 * p) = make_float4(a.x, b.x, a.y, b.y);
-}
-
-// Data-gradient unit: accumulator -> fp32 staging -> TMA store or reduce-add, BN-backward sums.
-template <int BN>
-__device__ __forceinline__ void unit_dgrad(const ConvDesc* d, uint32_t tacc, int q, int lane, int rows, int m0, int n0,
-                                           const uint8_t* h, uint8_t* stage, int& sbuf, float2* redw, uint32_t tempty,
-                                           uint32_t uempty, bool stats, bool acc) {
-  constexpr int HC = BN < 32 ? BN : 32;
-  const int nvalid = min(32, max(0, rows - (m0 + q * 32)));
-#pragma unroll
-  for (int c0 = 0; c0 < BN; c0 += HC) {
-    uint32_t a[HC];
-    if (HC == 32) tmem_ld32(tacc + c0, a);
-    else tmem_ld16_nowait(tacc + c0, a);
-    tmem_wait_ld(a);
-    if (c0 + HC >= BN) {
-      fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tempty);
-    }
-    // the store issued from this buffer two turns ago must have read it
-    if (lane == 0) bulk_wait_read<1>();
-    __syncwarp();
-    uint8_t* st = stage + sbuf * 4096;
-    sbuf ^= 1;
-#pragma unroll
-    for (int j = 0; j < HC / 4; ++j)
-      *reinterpret_cast<uint4*>(st + swp<HC * 4>(lane, j)) = make_uint4(a[4 * j], a[4 * j + 1], a[4 * j + 2], a[4 * j + 3]);
-    fence_proxy_async();
-    __syncwarp();
-    if (lane == 0 && nvalid > 0) {
-      if (acc) tma_reduce_add_2d(d->tma_y, n0 + c0, m0 + q * 32, smem_u32(st));
-      else tma_store_2d(d->tma_y, n0 + c0, m0 + q * 32, smem_u32(st));
-      bulk_commit();
-    }
-    if (stats) {
-      if (nvalid == 32) staged_bn_sums<BN, true>(st, h, c0, d, n0, q, lane, 32, redw);
-      else staged_bn_sums<BN, false>(st, h, c0, d, n0, q, lane, nvalid, redw);
-    }
-  }
-  __syncwarp();
-  if (stats && lane == 0) mbar_arrive(uempty);  // h has been read
-}
 
 template <int MODE, int W>
 __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int ninst,
@@ -461,14 +234,22 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
       Cursor cr(rg.nr), cu(rg.nu);
       uint32_t ka = 0, u = 0;  // k-steps and units issued
       bool ok = true;
+      Geo g{};
+      const void *ma = nullptr, *mb = nullptr, *mx = nullptr;
+      uint32_t abytes = 0;
       for (Walk w(tab, ts, ninst, total); w.more() && ok; w.next(tab, ts)) {
-        const ConvDesc* d = w.d;
-        const Geo g = geo<MODE>(d);
-        const void* ma = d->tma_a;
-        const void* mb = d->tma_b;
-        const void* mx = has_x<MODE>(d) ? d->tma_x : nullptr;
+        if (w.fresh) {
+          const ConvDesc* d = w.d;
+          g = geo<MODE>(d);
+          ma = d->tma_a;
+          mb = d->tma_b;
+          mx = has_x<MODE>(d) ? d->tma_x : nullptr;
+          abytes = (uint32_t)(kRows * min(g.kt, 64) * (MODE == FWD && d->x.dt == DT_BF16 ? 2 : 4));
+          tma_prefetch_map(ma);
+          tma_prefetch_map(mb);
+          if (mx) tma_prefetch_map(mx);
+        }
         const int m0 = w.tm * kRows, sub0 = w.tn * g.spi, sub1 = min(g.nsub, sub0 + g.spi);
-        const uint32_t abytes = (uint32_t)(kRows * min(g.kt, 64) * (MODE == FWD && d->x.dt == DT_BF16 ? 2 : 4));
         for (int kt = 0; kt < g.nkt && ok; ++kt) {
           if (!mbar_wait(smem_u32(&sh.raw_empty[cr.s]), cr.ph ^ 1, abort_flag)) { ok = false; break; }
           const uint32_t full = smem_u32(&sh.raw_full[cr.s]);
@@ -502,11 +283,16 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
     if (lane == 0) {
       Cursor co(rg.no), cu(rg.nu), cb(kAcc);
       bool ok = true, issued = false;
+      Geo g{};
+      bool hx = false;
+      uint32_t idesc = 0;
       for (Walk w(tab, ts, ninst, total); w.more() && ok; w.next(tab, ts)) {
-        const Geo g = geo<MODE>(w.d);
-        const bool hx = has_x<MODE>(w.d);
+        if (w.fresh) {
+          g = geo<MODE>(w.d);
+          hx = has_x<MODE>(w.d);
+          idesc = idesc_bf16(kRows, g.bn);
+        }
         const int sub0 = w.tn * g.spi, sub1 = min(g.nsub, sub0 + g.spi);
-        const uint32_t idesc = idesc_bf16(kRows, g.bn);
         for (int kt = 0; kt < g.nkt && ok; ++kt) {
           if (!mbar_wait(smem_u32(&sh.op_full[co.s]), co.ph, abort_flag)) { ok = false; break; }
           const uint32_t a_addr = base + off_op + co.s * kOpBytes;
@@ -552,13 +338,18 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
     const int t = threadIdx.x - 32 * R::kT0;
     Cursor cr(rg.nr), co(rg.no);
     bool ok = true;
+    Geo g{};
+    bool bn = false, xbf = false;
+    int relu = 0, lgn = 0;
     for (Walk w(tab, ts, ninst, total); w.more(); w.next(tab, ts)) {
       const ConvDesc* d = w.d;
-      const Geo g = geo<MODE>(d);
-      const bool bn = MODE == FWD && d->x.scale != nullptr;
-      const bool xbf = MODE == FWD && d->x.dt == DT_BF16;
-      const int relu = bn ? d->x.relu : 0;
-      const int lgn = 28 - __clz(min(g.kt, 64));  // log2 of the 8-channel chunks a row
+      if (w.fresh) {
+        g = geo<MODE>(d);
+        bn = MODE == FWD && d->x.scale != nullptr;
+        xbf = MODE == FWD && d->x.dt == DT_BF16;
+        relu = bn ? d->x.relu : 0;
+        lgn = 28 - __clz(min(g.kt, 64));  // log2 of the 8-channel chunks a row
+      }
       if (bn && w.fresh) {
         asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");  // all are past the previous instance
         for (int c = t; c < g.kt; c += NT) {
@@ -601,13 +392,14 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
     Cursor cu(rg.nu), cb(kAcc);
     int turn = 0, sbuf = 0;
     bool ok = true;
+    Geo g{};
+    EpiArgs ea{};
     for (Walk w(tab, ts, ninst, total); w.more(); w.next(tab, ts)) {
-      const ConvDesc* d = w.d;
-      const Geo g = geo<MODE>(d);
+      if (w.fresh) {
+        g = geo<MODE>(w.d);
+        ea.load<MODE>(w.d);
+      }
       const int m0 = w.tm * kRows, sub0 = w.tn * g.spi, sub1 = min(g.nsub, sub0 + g.spi);
-      float* const part = MODE == FWD ? d->stats : d->bnb_part;
-      const bool stats = part != nullptr, hx = has_x<MODE>(d);
-      const bool acc = MODE == DGRAD && d->accumulate;
       for (int sub = sub0; sub < sub1; ++sub) {
         // the unit's last k-step holds X (one unit a k-step: sub1 - sub0 == 1 when nkt > 1)
         for (int i = 1; i < g.nkt; ++i) cu.next();
@@ -619,7 +411,7 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
         if (++turn == R::kGroups) turn = 0;
         if (!mine) continue;
         if (ok) ok = mbar_wait(smem_u32(&sh.tfull[b]), bph, abort_flag);
-        if (ok && hx) ok = mbar_wait(smem_u32(&sh.u_full[us]), uph, abort_flag);
+        if (ok && ea.hx) ok = mbar_wait(smem_u32(&sh.u_full[us]), uph, abort_flag);
         ok = __all_sync(0xffffffffu, ok);
         const int n0 = sub * g.bn;
         float2* redw = es.red + es.rbuf * 256 + q * 64;
@@ -628,20 +420,21 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
           const uint32_t tacc = tmem + b * kAccCols + ((uint32_t)(q * 32) << 16);
           const uint8_t* x = gbase + off_u + us * rg.ub + kUnitB;
           const uint32_t te = smem_u32(&sh.tempty[b]), ue = smem_u32(&sh.u_empty[us]);
+          const RowDst dst{m0};
           if (MODE == FWD) {
-            if (g.bn == 64) unit_fwd<64>(d, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue, hx, stats);
-            else if (g.bn == 32) unit_fwd<32>(d, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue, hx, stats);
-            else unit_fwd<16>(d, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue, hx, stats);
+            if (g.bn == 64) unit_fwd<64>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue);
+            else if (g.bn == 32) unit_fwd<32>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue);
+            else unit_fwd<16>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue);
           } else {
-            if (g.bn == 64) unit_dgrad<64>(d, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue, stats, acc);
-            else if (g.bn == 32) unit_dgrad<32>(d, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue, stats, acc);
-            else unit_dgrad<16>(d, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue, stats, acc);
+            if (g.bn == 64) unit_dgrad<64>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue);
+            else if (g.bn == 32) unit_dgrad<32>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue);
+            else unit_dgrad<16>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue);
           }
         } else {
           sh.abort_flag = 1;
         }
-        if (stats) {
-          float* p = part + ((int64_t)w.tm * g.ncols + n0) * 2;
+        if (ea.stats) {
+          float* p = ea.part + ((int64_t)w.tm * g.ncols + n0) * 2;
           if (g.bn == 64) merge_partials<MODE, 64>(es, ok, q, lane, g.rows, m0, p);
           else if (g.bn == 32) merge_partials<MODE, 32>(es, ok, q, lane, g.rows, m0, p);
           else merge_partials<MODE, 16>(es, ok, q, lane, g.rows, m0, p);

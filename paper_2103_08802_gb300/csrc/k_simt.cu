@@ -422,10 +422,21 @@ __global__ void k_wtrans(const WtDesc* __restrict__ tab, const int* __restrict__
   const WtDesc& d = tab[inst];
   const int64_t i = (int64_t)(blockIdx.x - tstart[inst]) * blockDim.x + threadIdx.x;
   if (i >= d.n) return;
-  const int k = (int)(i % d.K);
-  const int64_t t = i / d.K;
-  const int rs = (int)(t % d.RS);
-  const int c = (int)(t / d.RS);
+  // i walks the destination; k, rs, c: its element of the source
+  int k, rs, c;
+  if (d.pack == 0) {
+    k = (int)(i % d.K);
+    const int64_t t = i / d.K;
+    rs = (int)(t % d.RS);
+    c = (int)(t / d.RS);
+  } else {
+    const int rows = d.pack == 1 ? d.K : d.C;
+    const int64_t t = i >> 3;
+    const int row = (int)(t % rows), ch = (int)(t / rows / d.RS) * 8 + (int)(i & 7);
+    rs = (int)(t / rows % d.RS);
+    k = d.pack == 1 ? row : ch;
+    c = d.pack == 1 ? ch : row;
+  }
   reinterpret_cast<__nv_bfloat16*>(d.dst)[i] =
       reinterpret_cast<const __nv_bfloat16*>(d.src)[((int64_t)k * d.RS + rs) * d.C + c];
 }

@@ -18,8 +18,8 @@
 
 namespace pnn {
 
-int encode_tensor_map_2d(void* map, const void* base, bool bf16, int64_t inner, int64_t rows, int box_inner,
-                         int box_rows, int swz, const char** why) {
+int encode_tensor_map_nd(void* map, const void* base, bool bf16, int rank, const int64_t* dims, const int64_t* strides,
+                         const int* box, int swz, const char** why) {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   static std::once_flag once;
   std::call_once(once, []() {
@@ -33,14 +33,17 @@ int encode_tensor_map_2d(void* map, const void* base, bool bf16, int64_t inner, 
     *why = "cuTensorMapEncodeTiled is not available from the driver";
     return 1;
   }
-  const int esz = bf16 ? 2 : 4;
-  const cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)rows};
-  const cuuint64_t pitch[1] = {(cuuint64_t)inner * esz};
-  const cuuint32_t box[2] = {(cuuint32_t)box_inner, (cuuint32_t)box_rows};
-  const cuuint32_t estr[2] = {1, 1};
+  cuuint64_t d[4], pitch[3];
+  cuuint32_t b[4], estr[4];
+  for (int i = 0; i < rank; ++i) {
+    d[i] = (cuuint64_t)dims[i];
+    b[i] = (cuuint32_t)box[i];
+    estr[i] = 1;
+    if (i) pitch[i - 1] = (cuuint64_t)strides[i - 1];
+  }
   const CUresult r = encode(reinterpret_cast<CUtensorMap*>(map),
-                            bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
-                            const_cast<void*>(base), dims, pitch, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, rank,
+                            const_cast<void*>(base), d, pitch, b, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                             swz == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
                             : swz == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
                             : swz == 32 ? CU_TENSOR_MAP_SWIZZLE_32B
@@ -51,6 +54,31 @@ int encode_tensor_map_2d(void* map, const void* base, bool bf16, int64_t inner, 
     return 1;
   }
   return 0;
+}
+int encode_tensor_map_2d(void* map, const void* base, bool bf16, int64_t inner, int64_t rows, int box_inner,
+                         int box_rows, int swz, const char** why) {
+  const int64_t dims[2] = {inner, rows}, strides[1] = {inner * (bf16 ? 2 : 4)};
+  const int box[2] = {box_inner, box_rows};
+  return encode_tensor_map_nd(map, base, bf16, 2, dims, strides, box, swz, why);
+}
+int encode_tensor_map_nhwc(void* map, const void* base, bool bf16, int C, int W, int H, int B, int box_c, int box_w,
+                           int box_h, int box_n, int swz, const char** why) {
+  const int64_t e = bf16 ? 2 : 4;
+  const int64_t dims[4] = {C, W, H, B}, strides[3] = {C * e, W * C * e, (int64_t)H * W * C * e};
+  const int box[4] = {box_c, box_w, box_h, box_n};
+  return encode_tensor_map_nd(map, base, bf16, 4, dims, strides, box, swz, why);
+}
+
+int encode_c3_maps(void* maps, bool fwd, const void* a, bool a_bf16, int ch, void* out, int ncols,
+                   const void* x, int B, int H, int W, const char** why) {
+  char* m = static_cast<char*>(maps);
+  const bool wh = c3_whole(H, W);
+  const int bw = wh ? 8 : 10, bh = wh ? 8 : 18, bi = wh ? 2 : 1;
+  int e = encode_tensor_map_nhwc(m, a, a_bf16, ch, W, H, B, 16, bw, bh, bi, 0, why);
+  const int oc = fwd ? ncols : (ncols < 32 ? ncols : 32);
+  if (!e) e = encode_tensor_map_nhwc(m + 256, out, fwd, ncols, W, H, B, oc, 8, 4, 1, oc * (fwd ? 2 : 4), why);
+  if (!e && x) e = encode_tensor_map_nhwc(m + 384, x, true, ncols, W, H, B, ncols, 8, wh ? 8 : 16, bi, 2 * ncols, why);
+  return e;
 }
 
 namespace {
@@ -72,6 +100,7 @@ struct InstPlan {
 struct Plan {
   int variant = 0;
   int bnmax = 16, raw = 0, op = 0, wide = 0;
+  C3Slots c3{};
   int total = 0;
   size_t tab = 0, ts = 0, status = 0, aux_tab = 0, aux_ts = 0, fin_tab = 0, fin_ts = 0, red_tab = 0, red_ts = 0;
   size_t bytes = 0, init_bytes = 0;  // init_bytes: the prefix copied from the host
@@ -121,7 +150,14 @@ bool pw_inst(int mode, const pnn_conv_args& g) {
     return pw_ok(g.ksize, g.stride, g.c, g.k) && g.y_dtype == PNN_DT_BF16 && (!g.res || g.res_dtype == PNN_DT_BF16);
   return mode == 1 && pw_ok(g.ksize, g.stride, g.k, g.c) && (!g.bn_mean || g.x_dtype == PNN_DT_BF16);
 }
-// its second operand: the residual, or the BN input of fused BN-backward sums
+// whether k_c3_conv.cu takes this instance
+bool c3_inst(int mode, const pnn_conv_args& g) {
+  if (mode == 0)
+    return c3_ok(g.ksize, g.stride, g.h, g.w, g.c, g.k) && g.y_dtype == PNN_DT_BF16 &&
+           (!g.res || g.res_dtype == PNN_DT_BF16);
+  return mode == 1 && c3_ok(g.ksize, g.stride, g.h, g.w, g.k, g.c) && (!g.bn_mean || g.x_dtype == PNN_DT_BF16);
+}
+// their second operand: the residual, or the BN input of fused BN-backward sums
 bool pw_has_x(int mode, const pnn_conv_args& g) { return mode == 0 ? g.res != nullptr : g.bn_mean && !g.accumulate; }
 
 // whether instance g of a TMA-fed forward / data-gradient launch takes halo tiles
@@ -166,7 +202,10 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
              wg_ok(a[i].ksize, a[i].stride, a[i].c, a[i].k, a[i].h, a[i].w, a[i].x_dtype == PNN_DT_BF16);
     wg_bytes += wg_traffic(a[i]);
   }
+  bool all_c3 = impl == 0;
+  for (int i = 0; i < n; ++i) all_c3 = all_c3 && c3_inst(mode, a[i]);
   if (all_pw || all_wg) pl.variant = 4;
+  if (all_c3) pl.variant = 5;
   size_t cur = 0;
   auto take = [&](size_t b) { size_t o = cur; cur = al256(cur + b); return o; };
   pl.tab = take((size_t)n * sizeof(ConvDesc));
@@ -251,13 +290,18 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
       ip.ntiles = cdv(ncols, ip.units * pw_unit_cols(ncols));
       pl.total += ip.mtiles * ip.ntiles;
     }
-    if (pl.variant == 1 || pl.variant == 4) ip.maps = take(4 * 128);
+    if (pl.variant == 5) {
+      c3_add(pl.c3, g.h, g.w, ncols, mode == 0 && g.x_dtype == PNN_DT_BF16 ? 2 : 4, pw_has_x(mode, g));
+      ip.ntiles = 1;
+    }
+    if (pl.variant == 1 || pl.variant == 4 || pl.variant == 5) ip.maps = take(4 * 128);
   }
   pl.init_bytes = cur;
   for (int i = 0; i < n; ++i) {
     const pnn_conv_args& g = a[i];
     InstPlan& ip = pl.in[i];
     const int rsc = g.ksize * g.ksize * g.c;
+    if (mode == 0 && pl.variant == 5) ip.wt = take((size_t)g.k * rsc * 2);
     if (mode == 0 && ip.bn) {
       ip.stats = take((size_t)ip.stat_tiles * g.k * 8);
       ip.scl = take((size_t)g.k * 4);
@@ -363,6 +407,13 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       c.y = g.y; c.y_dt = g.y_dtype;
       if (g.res) { c.res = g.res; c.res_dt = g.res_dtype; }
       if (ip.bn) c.stats = reinterpret_cast<float*>(ws + ip.stats);
+      if (pl.variant == 5) {
+        c.w = ws + ip.wt;  // packed
+        WtDesc w{};
+        w.src = g.wt; w.dst = ws + ip.wt; w.K = g.k; w.RS = 9; w.C = g.c; w.pack = 1; w.n = (int64_t)g.k * rsc;
+        wts.push_back(w);
+        aux_ts.push_back(aux_ts.back() + cdv(w.n, 256));
+      }
     } else if (mode == 1) {
       c.w = ws + ip.wt;  // the transposed bf16 weights Wt[c][r][s][k]
       c.dy = g.dy;
@@ -370,6 +421,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       c.accumulate = g.accumulate ? 1 : 0;
       WtDesc w{};
       w.src = g.wt; w.dst = ws + ip.wt; w.K = g.k; w.RS = g.ksize * g.ksize; w.C = g.c; w.n = (int64_t)g.k * rsc;
+      if (pl.variant == 5) w.pack = 2;
       wts.push_back(w);
       aux_ts.push_back(aux_ts.back() + cdv(w.n, 256));
     } else {
@@ -411,6 +463,17 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       c.tma_b = ws + ip.maps + 128;
       c.tma_y = mode == 2 ? nullptr : ws + ip.maps + 256;
       c.tma_h = ip.halo ? ws + ip.maps + 384 : nullptr;
+    }
+    if (pl.variant == 5) {
+      const char* why = nullptr;
+      const int ch = mode == 1 ? g.k : g.c, ncols = mode == 1 ? g.c : g.k;
+      const int e = encode_c3_maps(at(ip.maps), mode == 0, mode == 1 ? (const void*)g.dy : g.x,
+                                   mode == 0 && g.x_dtype == PNN_DT_BF16, ch, mode == 1 ? (void*)g.dx : g.y, ncols,
+                                   !pw_has_x(mode, g) ? nullptr : (mode == 0 ? g.res : g.x), g.batch, g.h, g.w, &why);
+      if (e) return set_last_error(PNN_ECUDA, why);
+      c.tma_a = ws + ip.maps;
+      c.tma_y = ws + ip.maps + 256;
+      c.tma_x = ws + ip.maps + 384;
     }
     if (pl.variant == 4 && mode == 2) {
       const char* why = nullptr;
@@ -476,7 +539,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       // the TMA-fed data gradient forms the sums of its 128-row tiles in its
       // epilogue when it writes the whole gradient; otherwise the separate
       // reduction kernel runs over its own row tiles
-      const bool fused = (pl.variant == 1 || pl.variant == 4) && !g.accumulate && g.c % 16 == 0;
+      const bool fused = (pl.variant == 1 || pl.variant == 4 || pl.variant == 5) && !g.accumulate && g.c % 16 == 0;
       if (fused) {
         c.bn_mean = g.bn_mean; c.bn_rstd = g.bn_rstd; c.bnb_part = b.part;
         b.tiles = ip.mtiles;
@@ -507,9 +570,10 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
   const auto* tab = reinterpret_cast<const ConvDesc*>(ws + pl.tab);
   const int* tsd = reinterpret_cast<const int*>(ws + pl.ts);
   const int* auxts = reinterpret_cast<const int*>(ws + pl.aux_ts);
-  if (e == cudaSuccess && mode == 1)
+  if (e == cudaSuccess && !wts.empty())
     e = launch_wtrans(reinterpret_cast<const WtDesc*>(ws + pl.aux_tab), auxts, n, aux_ts.back(), st);
   auto conv_launch = [&]() {
+    if (pl.variant == 5) return launch_conv_c3(mode, tab, tsd, n, pl.total, pl.c3, status, st);
     if (pl.variant == 4 && mode == 2)
       return launch_conv_wg(pl.bnmax, tab, tsd, n, pl.total, pl.raw, pl.op, status, st);
     if (pl.variant == 4)

@@ -65,9 +65,9 @@ struct ConvDesc {
   // TMA-fed forward: tensor map over the output y [pixels][K] (box 16
   // columns x 32 rows, 64-byte swizzle for fp32, 32-byte for bf16), or null
   const void* tma_y;
-  // 1x1 kernels of k_pw_conv.cu: tensor map over the unit's second operand
+  // k_pw_conv.cu, k_c3_conv.cu: tensor map over the unit's second operand
   // (forward: the residual, data gradient: the BN input h) with box [128 rows x
-  // unit columns] bf16; ntile_w is then the columns of an item
+  // unit columns] bf16; ntile_w is then (1x1) the columns of an item
   const void* tma_x;
   // TMA-fed data gradient of a BN(+ReLU) value (x = that virtual value): when
   // bnb_part is set, the epilogue also writes the BN-backward partial sums of
@@ -160,11 +160,14 @@ struct WReduceDesc {
   int32_t transposed, kout, rsc;
 };
 
-// bf16 weight transpose for the tensor-core data gradient: dst[c][r][s][k] = src[k][r][s][c]
+// bf16 weight copies from src[K][RS][C].  pack 0: dst[c][r][s][k], for the
+// tensor-core data gradient.  pack 1 (forward: rows n = k, channels ch = c) and 2
+// (data gradient: n = c, ch = k): the operand layout of k_c3_conv.cu,
+// dst[ch / 8][tap][n][ch % 8]
 struct WtDesc {
   const void* src;
   void* dst;
-  int32_t K, RS, C;
+  int32_t K, RS, C, pack;
   int64_t n;
 };
 
@@ -235,6 +238,11 @@ bool conv_halo_fits(int mode, int W, int ch, int bn);
 // k-step and at least 64 output columns
 cudaError_t launch_conv_pw(int mode, int wide, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes,
                            int x_bytes, int32_t* status, cudaStream_t st, int max_ctas = 0);
+// 3x3 stride-1 forward (mode 0) / data gradient (mode 1) of k_c3_conv.cu; s: the
+// largest slots over the launch's instances (c3_add)
+struct C3Slots;
+cudaError_t launch_conv_c3(int mode, const ConvDesc* tab, const int* ts, int n, int total, const C3Slots& s,
+                           int32_t* status, cudaStream_t st, int max_ctas = 0);
 // weight gradient of k_wg_conv.cu; raw_bytes, op_bytes: the largest slots over
 // the launch's instances (multiples of 1024)
 cudaError_t launch_conv_wg(int ksize, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes, int op_bytes,
@@ -368,6 +376,30 @@ inline int pw_x_bytes(int ncols) { return kTcBM * pw_unit_cols(ncols) * 2; }
 inline int pw_item_units(int ncols, int64_t launch_mtiles) {
   return launch_mtiles >= 2 * (int64_t)device_sm_count() ? ncols / pw_unit_cols(ncols) : 1;
 }
+// 3x3 stride-1 forward / data gradient of k_c3_conv.cu (variant 5): ch channels
+// of the A source, ncols GEMM columns; patches of 8 x 16 pixels, or two whole
+// 8 x 8 images a tile.
+struct C3Slots {
+  int raw, op, wt, x;  // bytes of a raw, an operand and a weight slot, and of the second operand
+};
+PNN_HD inline bool c3_whole(int H, int W) { return H == 8 && W == 8; }
+// raw pixels of a k-step; bytes of an operand plane (a halo of 10 x 18 pixels, or
+// three copies of 10 x 16 and four pixels that spread the two planes' stores over the banks)
+PNN_HD inline int c3_raw_px(bool whole) { return whole ? 128 : 180; }
+PNN_HD inline int c3_plane(bool whole) { return (whole ? 484 : 180) * 16; }
+PNN_HD inline int c3_wt_bytes(int ncols) { return 9 * ncols * 32; }  // 16 channels, nine taps
+inline bool c3_ok(int k, int stride, int H, int W, int ch, int ncols) {
+  auto narrow = [](int c) { return c == 16 || c == 32 || c == 64; };
+  return k == 3 && stride == 1 && (c3_whole(H, W) || (W % 8 == 0 && H % 16 == 0)) && narrow(ch) && narrow(ncols);
+}
+inline void c3_add(C3Slots& s, int H, int W, int ncols, int esz, bool x) {
+  const bool wh = c3_whole(H, W);
+  auto most = [](int& a, int b) { if (a < b) a = b; };
+  most(s.raw, c3_raw_px(wh) * 16 * esz);
+  most(s.op, 2 * c3_plane(wh));
+  most(s.wt, (c3_wt_bytes(ncols) + 1023) & ~1023);
+  if (x) most(s.x, kTcBM * ncols * 2);
+}
 // Weight gradient of k_wg_conv.cu (variant 4: 1x1, 5: 3x3): the geometry of one instance's
 // k-steps.  1x1: kp pixels; 3x3: krows whole image rows (kp pixels) with the
 // activation rows above and below.  Raw slot: x rows, then dY rows; operand
@@ -458,6 +490,15 @@ inline int tc_tile_rows(int mode, int variant, int C) { return mode == 2 && vari
 // (bf16 or fp32, row pitch inner * element size) with box
 // [box_rows][box_inner]; swz: swizzle span in bytes (128, 64, 32 or 0).
 // Returns 0, or non-zero with a message in *why.
+// general form: dims, byte strides of dims 1 .., box, innermost first; rank 2 to 4
+int encode_tensor_map_nd(void* map, const void* base, bool bf16, int rank, const int64_t* dims, const int64_t* strides,
+                         const int* box, int swz, const char** why);
+// [images][H][W][C] with a box of box_c channels x box_w x box_h x box_n
+int encode_tensor_map_nhwc(void* map, const void* base, bool bf16, int C, int W, int H, int B, int box_c, int box_w,
+                           int box_h, int box_n, int swz, const char** why);
+// the maps (a, unused, output, second operand; 128 bytes apart) of a k_c3_conv.cu instance
+int encode_c3_maps(void* maps, bool fwd, const void* a, bool a_bf16, int ch, void* out, int ncols,
+                   const void* x, int B, int H, int W, const char** why);
 int encode_tensor_map_2d(void* map, const void* base, bool bf16, int64_t inner, int64_t rows, int box_inner,
                          int box_rows, int swz, const char** why);
 

@@ -113,6 +113,7 @@ struct Launch {
   int raw = 0;          // TMA-fed conv: raw slot bytes of one stage
   int op = 0;           // TMA-fed conv with halo tiles: operand slot bytes of one stage (0: default);
                         // variant 4: second-operand bytes of a unit, or (weight gradient) operand slot bytes
+  C3Slots c3{};         // variant 5: its slots
   int wide = 0;         // TMA-fed forward / data gradient: every tile one k-step (the wide-epilogue variant)
   int block = -1;       // fine forward / backward: position of the layer in its segment
 };
@@ -190,6 +191,7 @@ struct pnn_net {
   size_t export_bytes = 0;
   // memory
   size_t off_master = 0, off_grad = 0, off_mom = 0, off_shadow = 0, off_wt = 0;
+  size_t off_wpf = 0, off_wpd = 0;  // weights packed for k_c3_conv.cu: forward, data gradient
   // weight transpose launch (bf16 mode): Wt[c][r][s][k] for the tensor-core data gradient
   size_t wt_tab = 0, wt_ts = 0;
   int wt_count = 0, wt_total = 0;
@@ -342,6 +344,8 @@ struct pnn_net {
       // the 1x1 kernels of k_pw_conv.cu hold bf16 outputs and residuals
       const bool res_ok = res < 0 || vals[res].dt == DT_BF16;
       if (tma_impl(opt.conv_impl) && pw_ok(k, stride, iv.C, cout) && out_dt == DT_BF16 && res_ok) c.variant = 4;
+      // and the 3x3 kernels of k_c3_conv.cu
+      if (opt.conv_impl == 0 && c3_ok(k, stride, iv.H, iv.W, iv.C, cout) && out_dt == DT_BF16 && res_ok) c.variant = 5;
       c.mtiles = cdiv(M, kTcBM);
       c.ntiles = cdiv(cout, tc_ntile_w(c.kind, c.variant));
     } else {
@@ -581,6 +585,9 @@ struct pnn_net {
             if (tma_impl(opt.conv_impl) && pw_ok(f.k, f.stride, ov.C, iv.C) &&
                 (!iv.virt || vals[iv.src].dt == DT_BF16))
               dg.variant = 4;
+            if (opt.conv_impl == 0 && c3_ok(f.k, f.stride, iv.H, iv.W, ov.C, iv.C) &&
+                (!iv.virt || vals[iv.src].dt == DT_BF16))
+              dg.variant = 5;
             dg.mtiles = cdiv((int64_t)B * iv.H * iv.W, kTcBM);
             dg.ntiles = cdiv(iv.C, tc_ntile_w(dg.kind, dg.variant));
           } else {
@@ -644,7 +651,7 @@ struct pnn_net {
         // epilogue writes the partial sums of each 128-row tile.
         const int wr = vals[vv].gwriter_dgrad;
         const bool fuse = vals[vv].gwrites == 1 && wr >= 0 && ops[wr].kind == K_DGRAD_TC &&
-                          (ops[wr].variant == 1 || ops[wr].variant == 4) &&
+                          ops[wr].variant != 0 &&
                           ops[wr].acc == 0 &&
                           ops[wr].in == vv && vals[vv].galias < 0 && vals[vv].pending.empty() && n.C % 16 == 0;
         if (fuse) {
@@ -915,9 +922,11 @@ int pnn_net::plan(const pnn_desc* d) {
   };
   auto fuse_add = [&](int v, int addend, float c) {
     POp& o = ops[vals[v].producer];
-    if (o.variant == 4 && o.kind == K_CONV_FWD_TC) {  // k_pw_conv.cu adds one operand
-      const int cin = vals[o.in].C, cout = vals[o.out].C;
-      o.variant = cout >= 64 && tma_shape_ok(o.k, o.stride, o.pad, cin) ? 1 : 0;
+    if (o.variant >= 4 && o.kind == K_CONV_FWD_TC) {  // the narrow-layer kernels add one operand
+      const Value& iv = vals[o.in];
+      const int cout = vals[o.out].C;
+      const bool halo = use_halo(opt.conv_impl, 0, o.k, o.stride, o.pad, iv.H, iv.W, iv.C, tma_bn(0, cout));
+      o.variant = (cout >= 64 && tma_shape_ok(o.k, o.stride, o.pad, iv.C)) || halo ? 1 : 0;
       o.ntiles = cdiv(cout, tc_ntile_w(o.kind, o.variant));
     }
     const int e = o.res2[0] < 0 ? 0 : 1;
@@ -1176,6 +1185,11 @@ int pnn_net::plan(const pnn_desc* d) {
   off_mom = opt.inference ? 0 : alloc(nparams * 4);
   off_shadow = act_dt == DT_BF16 ? alloc(nparams * 2) : 0;
   off_wt = act_dt == DT_BF16 ? alloc(nparams * 2) : 0;
+  for (const POp& o : ops) {
+    if (o.variant != 5) continue;
+    if (o.kind == K_CONV_FWD_TC && !off_wpf) off_wpf = alloc(nparams * 2);
+    if (o.kind == K_DGRAD_TC && !off_wpd) off_wpd = alloc(nparams * 2);
+  }
   off_running = alloc(running_floats * 4);
   if (opt.inference) {
     share_activation_buffers();
@@ -1423,6 +1437,27 @@ int pnn_net::build_tables() {
               c.tma_x = ws ? ws + tables_off + mo + 3 * sizeof(CUtensorMap) : nullptr;
               c.ntile_w = units * bn;
               c.ntiles = cdiv(ncols, c.ntile_w);
+            }
+            if ((o.kind == K_CONV_FWD_TC || o.kind == K_DGRAD_TC) && o.variant == 5) {
+              const bool fwd = o.kind == K_CONV_FWD_TC;
+              CUtensorMap maps[4];
+              memset(maps, 0, sizeof maps);
+              if (ws) {
+                const char* why = nullptr;
+                const void* x = fwd ? (o.res >= 0 ? ws + vals[o.res].off : nullptr)
+                                    : (o.bn_fuse >= 0 ? (const char*)c.x.ptr : nullptr);
+                if (encode_c3_maps(maps, fwd, fwd ? c.x.ptr : (const void*)P<float>(gptr(o.out)),
+                                   fwd && c.x.dt == DT_BF16, fwd ? iv.C : ov.C,
+                                   fwd ? (void*)(ws + ov.off) : (void*)P<float>(gptr(o.in)), fwd ? ov.C : iv.C, x, B,
+                                   iv.H, iv.W, &why))
+                  return fail(PNN_ECUDA, why);
+              }
+              const size_t mo = put(maps, sizeof maps);
+              c.tma_a = ws ? ws + tables_off + mo : nullptr;
+              c.tma_y = ws ? ws + tables_off + mo + 2 * sizeof(CUtensorMap) : nullptr;
+              c.tma_x = ws ? ws + tables_off + mo + 3 * sizeof(CUtensorMap) : nullptr;
+              c.w = ws + (fwd ? off_wpf : off_wpd) + params[o.w].off * 2;  // packed by k_wtrans
+              c.ntiles = 1;
             }
             if (o.kind == K_WGRAD_TC && o.variant >= 4) {
               const bool xbf = c.x.dt == DT_BF16;
@@ -1673,6 +1708,17 @@ int pnn_net::build_tables() {
           if (ch > 64 || ncols < 64) L.wide = 0;
         }
       }
+      if ((g.kind == K_CONV_FWD_TC || g.kind == K_DGRAD_TC) && g.variant == 5) {
+        L.c3 = C3Slots{};
+        for (int id : g.ops) {
+          const POp& o = ops[id];
+          const bool fwd = o.kind == K_CONV_FWD_TC;
+          const int src = vals[o.in].virt ? vals[o.in].src : o.in;
+          c3_add(L.c3, vals[o.in].H, vals[o.in].W, vals[fwd ? o.out : o.in].C, fwd && vals[src].dt == DT_BF16 ? 2 : 4,
+                 fwd ? o.res >= 0 : o.bn_fuse >= 0);
+        }
+        L.op = 0;
+      }
       if (g.kind == K_WGRAD_TC && g.variant >= 4) {
         L.raw = L.op = 0;
                 for (int id : g.ops) {
@@ -1709,6 +1755,23 @@ int pnn_net::build_tables() {
         ts.push_back(wt_total);
         wt_total += cdiv(w.n, 256);
       }
+    // the packed copies (a weight used by several ops of a direction once)
+    std::vector<char> done(2 * params.size(), 0);
+    for (const POp& o : ops) {
+      const bool fwd = o.kind == K_CONV_FWD_TC;
+      if (o.variant != 5 || (!fwd && o.kind != K_DGRAD_TC) || done[2 * o.w + fwd]) continue;
+      done[2 * o.w + fwd] = 1;
+      const ParamT& p = params[o.w];
+      WtDesc w{};
+      w.src = ws + off_shadow + p.off * 2;
+      w.dst = ws + (fwd ? off_wpf : off_wpd) + p.off * 2;
+      w.K = p.dims[0]; w.C = p.dims[1]; w.RS = p.dims[2] * p.dims[3];
+      w.pack = fwd ? 1 : 2;
+      w.n = (int64_t)p.n;
+      wt.push_back(w);
+      ts.push_back(wt_total);
+      wt_total += cdiv(w.n, 256);
+    }
     ts.push_back(wt_total);
     wt_count = (int)wt.size();
     wt_tab = put_table(wt.data(), wt.size() * sizeof(WtDesc));
@@ -1813,6 +1876,10 @@ int pnn_net::run_phase(int p, cudaStream_t st, int cap) {
     switch (L.kind) {
       case K_CONV_FWD: e = launch_conv_fwd_simt((const ConvDesc*)tab, ts, L.count, L.total, L.variant, st); break;
       case K_CONV_FWD_TC:
+        if (L.variant == 5) {
+          e = launch_conv_c3(0, (const ConvDesc*)tab, ts, L.count, L.total, L.c3, P<int32_t>(status_off), st, cap);
+          break;
+        }
         if (L.variant == 4) {
           e = launch_conv_pw(0, L.wide, (const ConvDesc*)tab, ts, L.count, L.total, L.raw, L.op, P<int32_t>(status_off),
                              st, cap);
@@ -1824,6 +1891,10 @@ int pnn_net::run_phase(int p, cudaStream_t st, int cap) {
                 : launch_conv_fwd_tc((const ConvDesc*)tab, ts, L.count, L.total, L.aux, P<int32_t>(status_off), st, cap);
         break;
       case K_DGRAD_TC:
+        if (L.variant == 5) {
+          e = launch_conv_c3(1, (const ConvDesc*)tab, ts, L.count, L.total, L.c3, P<int32_t>(status_off), st, cap);
+          break;
+        }
         if (L.variant == 4) {
           e = launch_conv_pw(1, 0, (const ConvDesc*)tab, ts, L.count, L.total, L.raw, L.op, P<int32_t>(status_off), st,
                              cap);

@@ -115,3 +115,31 @@ WG = {
 def test_weight_gradient(monkeypatch, base):
     _install(monkeypatch, base, WG[base])
     K.test_conv_weight_gradient(base, "auto")
+
+
+C3 = {
+    "patch": _wg(1, 16, 8, 16, 16, 3, bn=True),
+    "patches": _wg(3, 32, 32, 16, 16, 3, bn=True),
+    "p48x24": _wg(2, 48, 24, 32, 16, 3, bn=True, relu=False),
+    "p16x40_n64": _wg(2, 16, 40, 16, 64, 3, bn=False),
+    "p16_c64": _wg(2, 16, 16, 64, 64, 3, bn=True),
+    "p16_c64_fp32x": _wg(2, 16, 16, 64, 32, 3, bn=True, x_fp32=True),
+    "whole1": _wg(1, 8, 8, 16, 32, 3, bn=True),           # half a tile
+    "whole5": _wg(5, 8, 8, 64, 64, 3, bn=True),
+    "many": _wg(20, 64, 32, 16, 16, 3, bn=True),          # more tiles than CTAs
+    "stages": [_wg(2, 32, 32, 16, 16, 3, bn=True), _wg(3, 8, 8, 64, 64, 3, bn=True)],
+    "stagex": [_wg(3, 8, 8, 64, 64, 3, bn=True), _wg(2, 16, 16, 32, 32, 3, bn=True)],
+}
+
+
+@pytest.mark.parametrize("base,kind", [(n, kind) for n in C3 for kind in (0, 2)])
+def test_3x3_forward(monkeypatch, base, kind):
+    name = _name(base, 2 if isinstance(C3[base], list) else kind)
+    _install(monkeypatch, name, C3[base])
+    K.test_conv_forward(name, "auto")
+
+
+@pytest.mark.parametrize("base", list(C3))
+def test_3x3_data_gradient(monkeypatch, base):
+    _install(monkeypatch, base, C3[base])
+    K.test_conv_data_gradient(base, "auto")
