@@ -144,6 +144,8 @@ struct Phase { std::vector<Launch> launches; };
 int cdiv(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+constexpr int kAllFineBackward = 11;  // phase_groups: phases 7 and 9 as one
+
 struct Group {
   int kind, variant;
   std::vector<int> ops;
@@ -1133,8 +1135,10 @@ int pnn_net::plan(const pnn_desc* d) {
   }
   pre_b.resize(N);
   for (int j = 0; j < N; ++j) backward_list(pre_f[j], pre_b[j]);
-  // splits of the k_wg_conv.cu weight gradients: by the launches they form
-  for (int p = 5; p < 10; ++p)
+  // splits of the k_wg_conv.cu weight gradients: by the launches they form (all
+  // subnetworks together also when the overlap gives the last one launches of
+  // its own, so that both schedules add the same partial sums)
+  for (int p : {5, 6, kAllFineBackward, 8})
     for (const Group& g : phase_groups(p)) {
       if (g.kind != K_WGRAD_TC || g.variant < 4) continue;
       auto traffic = [&](const POp& o) {
@@ -1321,6 +1325,7 @@ std::vector<Group> pnn_net::phase_groups(int p) const {
     case 7:
       if (overlap_on) return merge(std::vector<std::vector<int>>(fine_b.begin(), fine_b.end() - 1));
       return merge(fine_b);
+    case kAllFineBackward: return merge(fine_b);
     case 8: return merge(pre_b);
     case 9:
       if (overlap_on) return merge(std::vector<std::vector<int>>(fine_b.end() - 1, fine_b.end()));
