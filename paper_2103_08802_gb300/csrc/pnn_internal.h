@@ -188,7 +188,7 @@ cudaError_t launch_conv_fwd_simt(const ConvDesc* tab, const int* tstart, int n, 
                                  int variant, cudaStream_t st);
 cudaError_t launch_conv_dgrad_simt(const ConvDesc* tab, const int* tstart, int n, int total_tiles,
                                    int variant, cudaStream_t st);
-// variant 1: few input channels (R*S*C <= 64), im2col staged per 64-pixel step
+// variant: simt_wgrad_variant
 cudaError_t launch_conv_wgrad_simt(const ConvDesc* tab, const int* tstart, int n, int total_tiles, int variant,
                                    cudaStream_t st);
 cudaError_t launch_wreduce(const WReduceDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
@@ -516,10 +516,30 @@ inline bool tma_wgrad_ok(int k, int stride, int pad, int C, int K, int W, bool x
   const WgBoxes b = wg_boxes(C, K, W, pad, xbf);
   return b.hrows <= 256 && conv_tma_fits(2, 128, wg_raw_bytes(b));
 }
+// CUDA-core forward and data gradient: 64 x 64, 128 x 32 or 64 x 16 tiles by
+// the GEMM's columns (16: a batch of 8 still gives every SM a tile); variant 3,
+// forward only: at most 32 taps x channels (the 3-channel stem and C^j convs),
+// one thread a pixel.
 struct ConvTile { int BM, BN; };
 inline ConvTile simt_tile(int variant) {
-  return variant == 0 ? ConvTile{64, 64} : (variant == 1 ? ConvTile{128, 32} : ConvTile{256, 16});
+  return variant == 0   ? ConvTile{64, 64}
+         : variant == 1 ? ConvTile{128, 32}
+         : variant == 2 ? ConvTile{64, 16}
+                        : ConvTile{256, 16};
 }
+inline int simt_variant(int ncols) { return ncols <= 16 ? 2 : (ncols <= 32 ? 1 : 0); }
+inline int simt_fwd_variant(int k, int C, int K) { return k * k * C <= 32 && C < 8 ? 3 : simt_variant(K); }
+// CUDA-core weight gradient: 64 or 16 output channels a tile (0, 1), few input
+// channels with at most 16 (2) or more (3) output channels, 1x1 stride 1 with at
+// most 4 input channels (4)
+inline int simt_wgrad_variant(int k, int stride, int C, int K) {
+  if (k == 1 && stride == 1 && C <= 4) return 4;
+  return k * k * C <= 32 && C < 8 ? (K <= 16 ? 2 : 3) : (K <= 16 ? 1 : 0);
+}
+inline int simt_wgrad_rows(int variant) { return variant == 1 ? 16 : 64; }
+// CTAs an SM that the splits of a CUDA-core weight gradient aim at (the
+// few-channel kernels' partial sums are small)
+inline int simt_wgrad_ctas(int variant) { return variant >= 2 ? 8 : 2; }
 constexpr int kWgradBM = 64, kWgradBN = 64, kWgradBK = 16;
 
 }  // namespace pnn

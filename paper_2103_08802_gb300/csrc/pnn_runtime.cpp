@@ -351,7 +351,7 @@ struct pnn_net {
       c.mtiles = cdiv(M, kTcBM);
       c.ntiles = cdiv(cout, tc_ntile_w(c.kind, c.variant));
     } else {
-      c.variant = cout <= 16 ? 2 : (cout <= 32 ? 1 : 0);
+      c.variant = simt_fwd_variant(k, iv.C, cout);
       ConvTile t = simt_tile(c.variant);
       c.mtiles = cdiv(M, t.BM);
       c.ntiles = cdiv(cout, t.BN);
@@ -534,7 +534,7 @@ struct pnn_net {
         const int RSC = f.k * f.k * vals[f.in].C;
         const int64_t Mp = (int64_t)B * ov.H * ov.W;
         const bool tc_ok = act_dt == DT_BF16 && opt.conv_impl != 1 && vals[f.in].C % 8 == 0 && ov.C % 8 == 0;
-        int pix_align = kWgradBK;
+        int pix_align = kWgradBK, sm_ctas = 2;
         if (tc_ok) {
           // tensor cores: rows (r,s,c) in 128-row tiles, all k_out per tile, pixels split across CTAs
           wg.kind = K_WGRAD_TC;
@@ -552,14 +552,13 @@ struct pnn_net {
           wg.ntiles = cdiv(ov.C, 256);
           pix_align = 64;
         } else {
-          wg.mtiles = cdiv(ov.C, kWgradBM);
+          wg.variant = simt_wgrad_variant(f.k, f.stride, vals[f.in].C, ov.C);
+          sm_ctas = simt_wgrad_ctas(wg.variant);
+          wg.mtiles = cdiv(ov.C, simt_wgrad_rows(wg.variant));
           wg.ntiles = cdiv(RSC, kWgradBN);
-          // few input channels (the 3-channel stem and C^j convs): the
-          // kernel that stages the im2col operand once per pixel step
-          wg.variant = vals[f.in].C < 8 && RSC <= kWgradBN ? 1 : 0;
         }
         int base = wg.mtiles * wg.ntiles;
-        int splits = std::max(1, std::min(cdiv(Mp, 256), cdiv(2 * (int64_t)device_sm_count(), base)));
+        int splits = std::max(1, std::min(cdiv(Mp, 256), cdiv(sm_ctas * (int64_t)device_sm_count(), base)));
         wg.pix_per_split = cdiv(cdiv(Mp, splits), pix_align) * pix_align;
         wg.splits = cdiv(Mp, wg.pix_per_split);
         wg.tiles = base * wg.splits;
@@ -593,7 +592,7 @@ struct pnn_net {
             dg.mtiles = cdiv((int64_t)B * iv.H * iv.W, kTcBM);
             dg.ntiles = cdiv(iv.C, tc_ntile_w(dg.kind, dg.variant));
           } else {
-            dg.variant = iv.C <= 16 ? 2 : (iv.C <= 32 ? 1 : 0);
+            dg.variant = simt_variant(iv.C);
             ConvTile t = simt_tile(dg.variant);
             dg.mtiles = cdiv((int64_t)B * iv.H * iv.W, t.BM);
             dg.ntiles = cdiv(iv.C, t.BN);
@@ -1081,7 +1080,7 @@ int pnn_net::plan(const pnn_desc* d) {
     if (c.kind != K_CONV_FWD_TC || params[c.w].off % 8 == 0) continue;
     c.kind = K_CONV_FWD;
     const int cout = vals[c.out].C;
-    c.variant = cout <= 16 ? 2 : (cout <= 32 ? 1 : 0);
+    c.variant = simt_fwd_variant(c.k, vals[c.in].C, cout);
     const ConvTile t = simt_tile(c.variant);
     c.mtiles = cdiv(rows(c.out), t.BM);
     c.ntiles = cdiv(cout, t.BN);
