@@ -776,31 +776,57 @@ __global__ void __launch_bounds__(256) k_conv_fwd_few(const ConvDesc* __restrict
   }
 }
 
-// 32 elements per CTA, 8 lanes per element: lane l sums splits l, l+8, ...
-// in order, then a fixed xor-shuffle tree combines the 8 lanes.
-// 32 consecutive partial positions e per CTA; warp w sums splits w, w+8, ..
-// (coalesced 128-byte rows of one split), then the eight warp sums are added
-// in warp order: a fixed order, so the result is deterministic.  Transposed
-// partials ([split][j][k_out], the tensor-core layout) land in dw[k_out][j].
+// 128 consecutive partial positions per CTA, four a lane: warp w sums splits w,
+// w+8, .. (512-byte rows of one split, four in flight), then the eight warp sums
+// are added in warp order: a fixed order, so the result is deterministic.
+// Transposed partials ([split][j][k_out]) land in dw[k_out][j].  (32 positions a
+// CTA and one load in flight read 0.6 TB/s of VGG-16's partials: 876 us a step;
+// now 380.)
 __global__ void __launch_bounds__(256) k_wreduce(const WReduceDesc* __restrict__ tab, const int* __restrict__ tstart,
                                                  int n) {
-  __shared__ float red[8][32];
+  static_assert(kWreduceElems == 128, "four elements a lane");
+  __shared__ float4 red[8][32];
   const int inst = find_instance(tstart, n, blockIdx.x);
   const WReduceDesc d = tab[inst];
-  const int64_t e = (int64_t)(blockIdx.x - tstart[inst]) * 32 + (threadIdx.x & 31);
-  const int w = threadIdx.x >> 5;
-  float s = 0.f;
-  if (e < d.n)
-    for (int k = w; k < d.splits; k += 8) s += d.part[(int64_t)k * d.n + e];
-  red[w][threadIdx.x & 31] = s;
-  __syncthreads();
-  if (w == 0 && e < d.n) {
-    float t = red[0][threadIdx.x];
-#pragma unroll
-    for (int i = 1; i < 8; ++i) t += red[i][threadIdx.x];
-    const int64_t i = d.transposed ? (e % d.kout) * d.rsc + e / d.kout : e;
-    d.dw[i] = d.accumulate ? d.dw[i] + t : t;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t e0 = (int64_t)(blockIdx.x - tstart[inst]) * kWreduceElems + 4 * lane;
+  const bool vec = (d.n & 3) == 0;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto row = [&](int k) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float* p = d.part + (int64_t)k * d.n + e0;
+    if (vec) {
+      if (e0 < d.n) v = __ldg(reinterpret_cast<const float4*>(p));
+    } else {
+      if (e0 < d.n) v.x = __ldg(p);
+      if (e0 + 1 < d.n) v.y = __ldg(p + 1);
+      if (e0 + 2 < d.n) v.z = __ldg(p + 2);
+      if (e0 + 3 < d.n) v.w = __ldg(p + 3);
+    }
+    return v;
+  };
+  auto add = [](float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; };
+  int k = w;
+  for (; k + 24 < d.splits; k += 32) {
+    const float4 v0 = row(k), v1 = row(k + 8), v2 = row(k + 16), v3 = row(k + 24);
+    add(s, v0);
+    add(s, v1);
+    add(s, v2);
+    add(s, v3);
   }
+  for (; k < d.splits; k += 8) add(s, row(k));
+  red[w][lane] = s;
+  __syncthreads();
+  // thread t < 128: element t of the CTA
+  if (threadIdx.x >= kWreduceElems) return;
+  const int64_t e = (int64_t)(blockIdx.x - tstart[inst]) * kWreduceElems + threadIdx.x;
+  if (e >= d.n) return;
+  const float* r = reinterpret_cast<const float*>(&red[0][0]) + threadIdx.x;
+  float t = r[0];
+#pragma unroll
+  for (int i = 1; i < 8; ++i) t += r[i * kWreduceElems];
+  const int64_t i = d.transposed ? (e % d.kout) * d.rsc + e / d.kout : e;
+  d.dw[i] = d.accumulate ? d.dw[i] + t : t;
 }
 
 __global__ void k_wtrans(const WtDesc* __restrict__ tab, const int* __restrict__ tstart, int n) {

@@ -2229,7 +2229,7 @@ extern "C" int pnn_conv_wgrad_noalloc(const float* x, const float* dy, float* dw
   rd.splits = cd.splits;
   rd.accumulate = 0;
   rd.n = (int64_t)nw;
-  rd.tiles = (int)((nw + 31) / 32);
+  rd.tiles = (int)((nw + kWreduceElems - 1) / kWreduceElems);
   rd.transposed = 1;
   rd.kout = k;
   rd.rsc = rsc;

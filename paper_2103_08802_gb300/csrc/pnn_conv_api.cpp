@@ -431,7 +431,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       c.pix_per_split = ip.pix_per_split;
       WReduceDesc w{};
       w.part = c.dw_part; w.dw = g.dw; w.splits = ip.splits; w.accumulate = 0; w.n = (int64_t)g.k * rsc;
-      w.tiles = cdv(w.n, 32); w.transposed = 1; w.kout = g.k; w.rsc = rsc;
+      w.tiles = cdv(w.n, kWreduceElems); w.transposed = 1; w.kout = g.k; w.rsc = rsc;
       wrs.push_back(w);
       aux_ts.push_back(aux_ts.back() + w.tiles);
     }

@@ -150,6 +150,7 @@ struct PoolDesc {
 
 // wgrad split reduction: dw[K*RSC] = sum_s part[s][...]; partials are laid out
 // [s][K][RSC] or [s][RSC][K] (transposed = 1)
+constexpr int kWreduceElems = 128;  // elements a CTA
 struct WReduceDesc {
   const float* part;
   float* dw;

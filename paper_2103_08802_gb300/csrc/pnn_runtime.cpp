@@ -567,7 +567,7 @@ struct pnn_net {
         POp rd;
         rd.kind = K_WREDUCE; rd.w = f.w; rd.splits = wg.splits; rd.out = f.out; rd.in = f.in; rd.k = f.k;
         rd.variant = tc_ok ? 1 : 0;  // partial layout of the matching wgrad
-        rd.tiles = cdiv((int64_t)ov.C * RSC, 32);  // 32 elements per CTA
+        rd.tiles = cdiv((int64_t)ov.C * RSC, kWreduceElems);
         key(rd, 1);
         new_op(L, rd);
         if (vals[f.in].need_grad) {
