@@ -9,6 +9,12 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#ifdef __CUDACC__
+#define PNN_HD __host__ __device__
+#else
+#define PNN_HD
+#endif
+
 namespace pnn {
 
 enum DType : int32_t { DT_F32 = 0, DT_BF16 = 1 };
@@ -139,6 +145,7 @@ struct BnBwdDesc {
   double inv_count;                        // fin: 1 / M
 };
 
+PNN_HD inline int pool_vec(int C) { return C % 4 == 0 ? 4 : 1; }  // channels a thread
 struct PoolDesc {
   Src x;                 // input (maybe virtual)
   void* y; int32_t y_dt; // output
@@ -279,11 +286,6 @@ cudaError_t launch_weight_cast(const float* in, void* out, int32_t out_dt, int64
 
 // tile geometry helpers shared by runtime and kernels
 constexpr int kEwRowsPerTile = 64;
-#ifdef __CUDACC__
-#define PNN_HD __host__ __device__
-#else
-#define PNN_HD
-#endif
 // BN forward statistics are kept as (count, mean, M2 = sum of squared
 // deviations from the mean) and combined with the pairwise update of Chan,
 // Golub & LeVeque ("Updating formulae and a pairwise algorithm for computing

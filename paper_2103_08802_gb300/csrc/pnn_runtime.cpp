@@ -384,7 +384,7 @@ struct pnn_net {
     int out = new_value(iv.C, P, Q, iv.virt ? act_dt : iv.dt, iv.need_grad);
     POp o;
     o.kind = K_POOL_FWD; o.in = in; o.out = out; o.k = k; o.stride = s; o.pad = p;
-    o.tiles = cdiv((int64_t)B * P * Q * iv.C, 256);
+    o.tiles = cdiv((int64_t)B * P * Q * iv.C, 256 * pool_vec(iv.C));
     o.key[0] = key0; o.key[1] = slot;
     int id = new_op(list, o);
     vals[out].producer = id;
@@ -632,7 +632,7 @@ struct pnn_net {
         POp p;
         p.kind = K_POOL_BWD; p.in = f.in; p.out = f.out; p.k = f.k; p.stride = f.stride; p.pad = f.pad;
         p.acc = grad_acc(f.in);
-        p.tiles = cdiv(rows(f.in) * vals[f.in].C, 256);
+        p.tiles = cdiv(rows(f.in) * vals[f.in].C, 256 * pool_vec(vals[f.in].C));
         key(p, 0);
         new_op(L, p);
         break;
