@@ -1831,8 +1831,9 @@ int pnn_net::run_head_fwd() {
   const int* tst = reinterpret_cast<const int*>(tb + head_tstart);
   cudaError_t e = launch_gap(make_src(*this, head_in), P<float>(feat[0]), B, hv.H * hv.W, hv.C, stream);
   for (int l = 0; l < nfc && e == cudaSuccess; ++l) {
-    const int wo = fc_width[l + 1];
-    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_fwd_tab[l]), tst, 1, cdiv(B, 64) * cdiv(wo, 64), stream);
+    const int wi = fc_width[l], wo = fc_width[l + 1];
+    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_fwd_tab[l]), tst, 1, cdiv(B, 64) * cdiv(wo, 64), wi,
+                    stream);
   }
   if (e == cudaSuccess && !opt.inference)
     e = launch_softmax_ce(P<float>(feat[nfc]), labels_dev, B, classes, P<float>(loss_off), P<float>(dfeat[nfc]),
@@ -1848,10 +1849,12 @@ int pnn_net::run_head_bwd(int opid) {
   cudaError_t e = cudaSuccess;
   for (int l = nfc - 1; l >= 0 && e == cudaSuccess; --l) {
     const int wi = fc_width[l], wo = fc_width[l + 1];
-    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_dw_tab[l]), tst, 1, cdiv(wo, 64) * cdiv(wi, 64), stream);
+    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_dw_tab[l]), tst, 1, cdiv(wo, 64) * cdiv(wi, 64), B,
+                    stream);
     if (e == cudaSuccess) e = launch_colsum(P<float>(dfeat[l + 1]), B, wo, grad + params[fc_b[l]].off, stream);
     if (e == cudaSuccess)
-      e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_din_tab[l]), tst, 1, cdiv(B, 64) * cdiv(wi, 64), stream);
+      e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_din_tab[l]), tst, 1, cdiv(B, 64) * cdiv(wi, 64), wo,
+                      stream);
     if (e == cudaSuccess && l > 0) e = launch_relu_mask(P<float>(dfeat[l]), P<float>(feat[l]), (int64_t)B * wi, stream);
   }
   const Value& hv = vals[head_in];
