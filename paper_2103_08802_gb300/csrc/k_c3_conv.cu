@@ -18,7 +18,7 @@
 // producer 200 cycles each and bounded the kernel.
 // Grouped launches of the 8-subnetwork ResNet-1001 (batch 256, 64 px), kernels of
 // k_tc_conv.cu -> now: forward 160 -> 62 us, data gradient (+ BN-backward sums)
-// 133 -> 94 us; bound by per-tile latencies (a tile is 128 x 16 outputs).
+// 133 -> 90 us; bound by per-tile latencies (a tile is 128 x 16 outputs).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -224,7 +224,7 @@ __device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const 
 
   if (warp == kProducer) {
     // ================================================= TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       Cursor cr(rg.nr), cu(rg.nu);
       uint32_t ka = 0, u = 0;  // raw and unit slots issued
       bool ok = true;
@@ -275,7 +275,7 @@ __device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const 
     __syncwarp();
   } else if (warp == kMma) {
     // ================================================= MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       Cursor co(rg.no), cu(rg.nu), cb(kAcc);
       bool ok = true, issued = false;
       Geo g{};
@@ -384,6 +384,7 @@ __device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const 
     EpiState es{reinterpret_cast<float2*>(red0 + eg * kRedBytes), 0, 2 + eg};
     Cursor cu(rg.nu), cb(kAcc);
     int turn = 0, sbuf = 0;
+    const bool leader = elect_one();  // issues and waits for this warp's stores
     bool ok = true;
     Geo g{};
     EpiArgs ea{};
@@ -413,13 +414,13 @@ __device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const 
         const uint32_t te = smem_u32(&sh.tempty[b]), ue = smem_u32(&sh.u_empty[us]);
         const PatchDst dst{patch(g, w.tm), g.whole};
         if (MODE == FWD) {
-          if (g.n == 64) unit_fwd<64>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, redw, te, ue);
-          else if (g.n == 32) unit_fwd<32>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, redw, te, ue);
-          else unit_fwd<16>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, redw, te, ue);
+          if (g.n == 64) unit_fwd<64>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, redw, te, ue, leader);
+          else if (g.n == 32) unit_fwd<32>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, redw, te, ue, leader);
+          else unit_fwd<16>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, redw, te, ue, leader);
         } else {
-          if (g.n == 64) unit_dgrad<64>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, sbuf, redw, te, ue);
-          else if (g.n == 32) unit_dgrad<32>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, sbuf, redw, te, ue);
-          else unit_dgrad<16>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, sbuf, redw, te, ue);
+          if (g.n == 64) unit_dgrad<64>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, sbuf, redw, te, ue, leader);
+          else if (g.n == 32) unit_dgrad<32>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, sbuf, redw, te, ue, leader);
+          else unit_dgrad<16>(ea, dst, tacc, q, lane, g.rows, m0, 0, x, st, sbuf, redw, te, ue, leader);
         }
       } else {
         sh.abort_flag = 1;
@@ -432,7 +433,7 @@ __device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const 
       }
     }
     // the output stores must complete before the CTA exits
-    if (lane == 0) bulk_wait_all();
+    if (leader) bulk_wait_all();
     __syncwarp();
     if (!ok) { sh.abort_flag = 1; atomicExch(status, 3); }
   }

@@ -27,8 +27,8 @@
 // a sixth of the instructions.  Bound by HBM latency and bandwidth, about half
 // of the copy rate: grouped launches of the 8-subnetwork ResNet-1001 (batch
 // 256, 64 px), before -> now: expand forward (16 -> 64 channels + residual +
-// statistics) 218 -> 107 us, reduce forward 117 -> 81, reduce data gradient
-// (+ BN-backward sums) 165 -> 136, expand data gradient 109 -> 98.
+// statistics) 218 -> 105 us, reduce forward 117 -> 75, reduce data gradient
+// (+ BN-backward sums) 165 -> 135, expand data gradient 109 -> 93.
 // Every wait is bounded (2 s); on expiry the CTA records status 3, stops,
 // drains its copies and MMAs (bounded) and frees its TMEM.
 #include <cuda_bf16.h>
@@ -230,7 +230,7 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
 
   if (warp == R::kProducer) {
     // ================================================= TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       Cursor cr(rg.nr), cu(rg.nu);
       uint32_t ka = 0, u = 0;  // k-steps and units issued
       bool ok = true;
@@ -280,7 +280,7 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
     __syncwarp();
   } else if (warp == R::kMma) {
     // ================================================= MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       Cursor co(rg.no), cu(rg.nu), cb(kAcc);
       bool ok = true, issued = false;
       Geo g{};
@@ -391,6 +391,7 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
     EpiState es{reinterpret_cast<float2*>(red0 + eg * kRedBytes), 0, 2 + eg};
     Cursor cu(rg.nu), cb(kAcc);
     int turn = 0, sbuf = 0;
+    const bool leader = elect_one();  // issues and waits for this warp's stores
     bool ok = true;
     Geo g{};
     EpiArgs ea{};
@@ -422,13 +423,13 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
           const uint32_t te = smem_u32(&sh.tempty[b]), ue = smem_u32(&sh.u_empty[us]);
           const RowDst dst{m0};
           if (MODE == FWD) {
-            if (g.bn == 64) unit_fwd<64>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue);
-            else if (g.bn == 32) unit_fwd<32>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue);
-            else unit_fwd<16>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue);
+            if (g.bn == 64) unit_fwd<64>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue, leader);
+            else if (g.bn == 32) unit_fwd<32>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue, leader);
+            else unit_fwd<16>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, redw, te, ue, leader);
           } else {
-            if (g.bn == 64) unit_dgrad<64>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue);
-            else if (g.bn == 32) unit_dgrad<32>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue);
-            else unit_dgrad<16>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue);
+            if (g.bn == 64) unit_dgrad<64>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue, leader);
+            else if (g.bn == 32) unit_dgrad<32>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue, leader);
+            else unit_dgrad<16>(ea, dst, tacc, q, lane, g.rows, m0, n0, x, st, sbuf, redw, te, ue, leader);
           }
         } else {
           sh.abort_flag = 1;
@@ -442,7 +443,7 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
       }
     }
     // the output stores must complete before the CTA exits
-    if (lane == 0) bulk_wait_all();
+    if (leader) bulk_wait_all();
     __syncwarp();
     if (!ok) { sh.abort_flag = 1; atomicExch(status, 3); }
   }

@@ -16,7 +16,7 @@
 //         the three tap rows are descriptor offsets of one image row.  An MMA
 //         costs the read of its M side (128 rows x 16 pixels, 4 KB of shared
 //         memory) whatever its N, so nine MMAs of one tap each (one copy with
-//         zero columns at its sides) took 146 us where three take 67.
+//         zero columns at its sides) took 146 us where three took 67.
 //         (Copying the transformed halo to a plane per tap, as the kernel of
 //         k_tc_conv.cu does, took 80 % of that kernel's 224 us.)
 // Plane pitches are padded so that the eight lanes of a 16-byte store phase
@@ -28,8 +28,8 @@
 // reduced.  Roles: producer (TMA, one thread), MMA (one thread), ten transform
 // warps, four epilogue warps.  Grouped launches of the
 // 8-subnetwork ResNet-1001 (batch 256, 64 px), kernels of k_tc_conv.cu -> now:
-// 3x3 224 -> 67 us, expand (16 -> 64) 159 -> 69 us (two launches before), reduce
-// 141 -> 61 us; the 1x1 are at 0.6 - 0.75 of the copy rate, the 3x3 is bound by
+// 3x3 224 -> 60 us, expand (16 -> 64) 159 -> 65 us (two launches before), reduce
+// 141 -> 56 us; the 1x1 are at 0.6 - 0.75 of the copy rate, the 3x3 is bound by
 // the latency of its k-steps.
 // Every wait is bounded (2 s); on expiry the CTA records status 3, stops,
 // drains its copies and MMAs (bounded) and frees its TMEM.
@@ -228,7 +228,7 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
 
   if (warp == kProducer) {
     // ================================================= TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       Cursor cr(rg.nr);
       uint32_t n = 0;
       bool ok = true;
@@ -256,7 +256,7 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
     __syncwarp();
   } else if (warp == kMma) {
     // ================================================= MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       Cursor co(rg.no), cb(kBufs);
       bool ok = true, issued = false;
       for (Walk w(tab, ts, ninst, total); w.more() && ok; w.next(tab, ts)) {

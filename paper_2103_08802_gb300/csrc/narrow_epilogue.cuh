@@ -137,7 +137,7 @@ __device__ __forceinline__ void staged_moments(const uint8_t* st, int lane, int 
 template <int BN, typename Dst>
 __device__ __forceinline__ void unit_fwd(const EpiArgs& ea, const Dst& dst, uint32_t tacc, int q, int lane, int rows, int m0, int n0,
                                          const uint8_t* x, uint8_t* st, float2* redw, uint32_t tempty,
-                                         uint32_t uempty) {
+                                         uint32_t uempty, bool leader) {
   uint32_t a[BN];
 #pragma unroll
   for (int j = 0; j < BN; j += 32) {
@@ -167,7 +167,7 @@ __device__ __forceinline__ void unit_fwd(const EpiArgs& ea, const Dst& dst, uint
   }
   // the store issued from this tile for the previous unit must have read it,
   // and every lane must be done with its statistics
-  if (lane == 0) bulk_wait_read<0>();
+  if (leader) bulk_wait_read<0>();
   __syncwarp();
   if (ea.hx && lane == 0) mbar_arrive(uempty);  // X has been read
 #pragma unroll
@@ -176,7 +176,7 @@ __device__ __forceinline__ void unit_fwd(const EpiArgs& ea, const Dst& dst, uint
   fence_proxy_async();
   __syncwarp();
   const int nvalid = min(32, max(0, rows - (m0 + q * 32)));
-  if (lane == 0 && nvalid > 0) {
+  if (leader && nvalid > 0) {
     dst.put(ea.y, n0, q, smem_u32(st), false);
     bulk_commit();
   }
@@ -235,7 +235,7 @@ __device__ __forceinline__ void staged_bn_sums(const uint8_t* st, const uint8_t*
 template <int BN, typename Dst>
 __device__ __forceinline__ void unit_dgrad(const EpiArgs& ea, const Dst& dst, uint32_t tacc, int q, int lane, int rows, int m0, int n0,
                                            const uint8_t* h, uint8_t* stage, int& sbuf, float2* redw, uint32_t tempty,
-                                           uint32_t uempty) {
+                                           uint32_t uempty, bool leader) {
   constexpr int HC = BN < 32 ? BN : 32;
   const int nvalid = min(32, max(0, rows - (m0 + q * 32)));
 #pragma unroll
@@ -250,7 +250,7 @@ __device__ __forceinline__ void unit_dgrad(const EpiArgs& ea, const Dst& dst, ui
       if (lane == 0) mbar_arrive(tempty);
     }
     // the store issued from this buffer two turns ago must have read it
-    if (lane == 0) bulk_wait_read<1>();
+    if (leader) bulk_wait_read<1>();
     __syncwarp();
     uint8_t* st = stage + sbuf * 4096;
     sbuf ^= 1;
@@ -259,7 +259,7 @@ __device__ __forceinline__ void unit_dgrad(const EpiArgs& ea, const Dst& dst, ui
       *reinterpret_cast<uint4*>(st + swp<HC * 4>(lane, j)) = make_uint4(a[4 * j], a[4 * j + 1], a[4 * j + 2], a[4 * j + 3]);
     fence_proxy_async();
     __syncwarp();
-    if (lane == 0 && nvalid > 0) {
+    if (leader && nvalid > 0) {
       dst.put(ea.y, n0 + c0, q, smem_u32(st), ea.acc);
       bulk_commit();
     }
