@@ -469,6 +469,7 @@ __device__ __forceinline__ void epilogue(const Tile& T, uint32_t tacc, int q, in
                                          int j_first, int j_step, int etid, int ethreads, uint8_t* ystage, int& ybuf,
                                          int bar_id = 2) {
   const ConvDesc d = *T.d;  // a private copy: stores through other pointers cannot force reloads
+  const bool leader = elect_one();  // issues this warp's output copies
   const int row = q * 32 + lane;
   const int m = T.m0 + row;
   const bool mvalid = m < T.Mrows;
@@ -581,7 +582,7 @@ __device__ __forceinline__ void epilogue(const Tile& T, uint32_t tacc, int q, in
       if (tstore) {
         // the store issued from this buffer two chunks ago must have read it
         RT(const unsigned long long cw = clock64();)
-        if (lane == 0) bulk_wait_read<1>();
+        if (leader) bulk_wait_read<1>();
         __syncwarp();
         RT(e6 += clock64() - cw;)
         uint8_t* st = ystage + ybuf * 2048;
@@ -600,7 +601,7 @@ __device__ __forceinline__ void epilogue(const Tile& T, uint32_t tacc, int q, in
         }
         fence_proxy_async();
         __syncwarp();
-        if (lane == 0 && T.m0 + q * 32 < T.Mrows) {
+        if (leader && T.m0 + q * 32 < T.Mrows) {
           tma_store_2d(d.tma_y, nb, T.m0 + q * 32, smem_u32(st));
           bulk_commit();
         }
@@ -707,7 +708,7 @@ __device__ __forceinline__ void epilogue(const Tile& T, uint32_t tacc, int q, in
       }
       // staged chunk -> TMA store (fresh gradient) or TMA reduce-add (accumulate)
       RT(const unsigned long long cw = clock64();)
-      if (lane == 0) bulk_wait_read<1>();
+      if (leader) bulk_wait_read<1>();
       __syncwarp();
       RT(e6 += clock64() - cw;)
       uint8_t* st = ystage + ybuf * 2048;
@@ -723,7 +724,7 @@ __device__ __forceinline__ void epilogue(const Tile& T, uint32_t tacc, int q, in
       }
       fence_proxy_async();
       __syncwarp();
-      if (lane == 0 && T.m0 + q * 32 < T.Mrows) {
+      if (leader && T.m0 + q * 32 < T.Mrows) {
         if (d.accumulate) tma_reduce_add_2d(d.tma_y, nb, T.m0 + q * 32, smem_u32(st));
         else tma_store_2d(d.tma_y, nb, T.m0 + q * 32, smem_u32(st));
         bulk_commit();
@@ -891,7 +892,7 @@ __device__ __forceinline__ void conv_tc_body(const ConvDesc* __restrict__ tab, c
     })
   } else if (warp == kMmaWarp) {
     // ================================================= MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       uint32_t g = 0;
       int li = 0;
       bool ok = true;
@@ -1572,7 +1573,7 @@ __device__ __forceinline__ void conv_tma_body(const ConvDesc* __restrict__ tab, 
 
   if (warp == R::kProducerWarp) {
     // ================================================= TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       uint32_t g = 0;
       bool ok = true;
       RT(unsigned long long rt_a = 0, rt_b = 0;)
@@ -1780,7 +1781,7 @@ __device__ __forceinline__ void conv_tma_body(const ConvDesc* __restrict__ tab, 
     if (!ok) { sh.abort_flag = 1; atomicExch(status, 3); }
   } else if (warp == R::kMmaWarp) {
     // ================================================= MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       uint32_t g = 0;
       int li = 0;
       bool ok = true;
@@ -1910,7 +1911,7 @@ __device__ __forceinline__ void conv_tma_body(const ConvDesc* __restrict__ tab, 
       RT(rt_b += clock64() - rt1;)
     }
     // the output stores must complete before the CTA exits
-    if (MODE != WGRAD && lane == 0) bulk_wait_all();
+    if (MODE != WGRAD && elect_one()) bulk_wait_all();
     __syncwarp();
     RT(if (threadIdx.x == R::kEpiWarp0 * 32) { atomicAdd(&g_tma_cycles[MODE][8], rt_a); atomicAdd(&g_tma_cycles[MODE][9], rt_b); })
     if (!ok) {
