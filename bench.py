@@ -366,11 +366,13 @@ def retear(args, desc, stream):
     return desc, rec
 
 
-KERNEL_SYMBOL = {("conv_fwd_tc", 0): "k_conv_fwd_tc", ("conv_fwd_tc", 1): "k_conv_fwd_tma",
+# (variant 1 is any TMA-fed kernel without the wide epilogue or halo tiles: those of
+# the shapes that the 1x1, 3x3 and weight-gradient kernels take, else k_conv_*_tma)
+KERNEL_SYMBOL = {("conv_fwd_tc", 0): "k_conv_fwd_tc", ("conv_fwd_tc", 1): "k_pw_fwd|k_c3_fwd|k_conv_fwd_tma",
                  ("conv_fwd_tc", 2): "k_conv_fwd_tma_w", ("conv_dgrad_tc", 0): "k_conv_dgrad_tc",
-                 ("conv_dgrad_tc", 1): "k_conv_dgrad_tma", ("conv_dgrad_tc", 2): "k_conv_dgrad_tma_w",
+                 ("conv_dgrad_tc", 1): "k_pw_dgrad|k_c3_dgrad|k_conv_dgrad_tma", ("conv_dgrad_tc", 2): "k_conv_dgrad_tma_w",
                  ("conv_fwd_tc", 3): "k_conv_fwd_tma_h", ("conv_dgrad_tc", 3): "k_conv_dgrad_tma_h",
-                 ("conv_wgrad_tc", 0): "k_conv_wgrad_tc", ("conv_wgrad_tc", 1): "k_conv_wgrad_tma",
+                 ("conv_wgrad_tc", 0): "k_conv_wgrad_tc", ("conv_wgrad_tc", 1): "k_wg_pw|k_wg_3x3|k_conv_wgrad_tma",
                  ("bn_bwd_apply", 1): "k_bnb_apply8", ("bn_finalize", 0): "k_bn_fin"}
 
 
