@@ -833,24 +833,30 @@ __global__ void k_wtrans(const WtDesc* __restrict__ tab, const int* __restrict__
   const int inst = find_instance(tstart, n, blockIdx.x);
   const WtDesc& d = tab[inst];
   const int64_t i = (int64_t)(blockIdx.x - tstart[inst]) * blockDim.x + threadIdx.x;
-  if (i >= d.n) return;
-  // i walks the destination; k, rs, c: its element of the source
-  int k, rs, c;
+  const uint16_t* src = reinterpret_cast<const uint16_t*>(d.src);
   if (d.pack == 0) {
-    k = (int)(i % d.K);
+    // one element a thread, in the order of the destination
+    if (i >= d.n) return;
+    const int k = (int)(i % d.K);
     const int64_t t = i / d.K;
-    rs = (int)(t % d.RS);
-    c = (int)(t / d.RS);
-  } else {
-    const int rows = d.pack == 1 ? d.K : d.C;
-    const int64_t t = i >> 3;
-    const int row = (int)(t % rows), ch = (int)(t / rows / d.RS) * 8 + (int)(i & 7);
-    rs = (int)(t / rows % d.RS);
-    k = d.pack == 1 ? row : ch;
-    c = d.pack == 1 ? ch : row;
+    const int rs = (int)(t % d.RS), c = (int)(t / d.RS);
+    reinterpret_cast<uint16_t*>(d.dst)[i] = src[((int64_t)k * d.RS + rs) * d.C + c];
+    return;
   }
-  reinterpret_cast<__nv_bfloat16*>(d.dst)[i] =
-      reinterpret_cast<const __nv_bfloat16*>(d.src)[((int64_t)k * d.RS + rs) * d.C + c];
+  // eight channels of one row and tap a thread: a 16-byte store; neighbouring
+  // threads are neighbouring rows (pack 2: of consecutive addresses)
+  if (8 * i >= d.n) return;
+  const int all = d.pack == 1 ? d.K : d.C, rows = c3_block(all);
+  const int64_t per = d.n / all * rows / 8;  // threads of a block of rows
+  const int64_t j = i % per;
+  const int row = (int)(i / per) * rows + (int)(j % rows);
+  const int rs = (int)(j / rows % d.RS), ch = (int)(j / rows / d.RS) * 8;
+  const int64_t step = d.pack == 1 ? 1 : (int64_t)d.RS * d.C;
+  src += d.pack == 1 ? ((int64_t)row * d.RS + rs) * d.C + ch : ((int64_t)ch * d.RS + rs) * d.C + row;
+  uint32_t w[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) w[e] = src[2 * e * step] | (uint32_t)src[(2 * e + 1) * step] << 16;
+  reinterpret_cast<uint4*>(d.dst)[i] = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 // ---------------------------------------------------------------- row-tile geometry

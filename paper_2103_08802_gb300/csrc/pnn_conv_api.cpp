@@ -72,12 +72,16 @@ int encode_tensor_map_nhwc(void* map, const void* base, bool bf16, int C, int W,
 int encode_c3_maps(void* maps, bool fwd, const void* a, bool a_bf16, int ch, void* out, int ncols,
                    const void* x, int B, int H, int W, const char** why) {
   char* m = static_cast<char*>(maps);
-  const bool wh = c3_whole(H, W);
-  const int bw = wh ? 8 : 10, bh = wh ? 8 : 18, bi = wh ? 2 : 1;
-  int e = encode_tensor_map_nhwc(m, a, a_bf16, ch, W, H, B, 16, bw, bh, bi, 0, why);
-  const int oc = fwd ? ncols : (ncols < 32 ? ncols : 32);
-  if (!e) e = encode_tensor_map_nhwc(m + 256, out, fwd, ncols, W, H, B, oc, 8, 4, 1, oc * (fwd ? 2 : 4), why);
-  if (!e && x) e = encode_tensor_map_nhwc(m + 384, x, true, ncols, W, H, B, ncols, 8, wh ? 8 : 16, bi, 2 * ncols, why);
+  const bool patch = c3_kind(H, W) == C3_PATCH, small = c3_kind(H, W) == C3_SMALL;
+  // the M tile's pixels (w x h of n images); a patch is read with its border
+  const int w = patch ? 8 : W, h = patch ? 16 : H, n = patch ? 1 : kTcBM / (H * W), border = patch ? 2 : 0;
+  int e = encode_tensor_map_nhwc(m, a, a_bf16, ch, W, H, B, 16, w + border, h + border, n, 0, why);
+  // a warp's 32 rows of the output
+  const int bn = c3_block(ncols), oc = fwd ? bn : (bn < 32 ? bn : 32);
+  if (!e)
+    e = encode_tensor_map_nhwc(m + 256, out, fwd, ncols, W, H, B, oc, w, small ? H : 4, small ? n / 4 : 1,
+                               oc * (fwd ? 2 : 4), why);
+  if (!e && x) e = encode_tensor_map_nhwc(m + 384, x, true, ncols, W, H, B, bn, w, h, n, 2 * bn, why);
   return e;
 }
 
@@ -292,7 +296,9 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
     }
     if (pl.variant == 5) {
       c3_add(pl.c3, g.h, g.w, ncols, mode == 0 && g.x_dtype == PNN_DT_BF16 ? 2 : 4, pw_has_x(mode, g));
-      ip.ntiles = 1;
+      pl.total -= ip.mtiles * ip.ntiles;
+      ip.ntiles = cdv(ncols, c3_block(ncols));
+      pl.total += ip.mtiles * ip.ntiles;
     }
     if (pl.variant == 1 || pl.variant == 4 || pl.variant == 5) ip.maps = take(4 * 128);
   }
@@ -412,7 +418,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
         WtDesc w{};
         w.src = g.wt; w.dst = ws + ip.wt; w.K = g.k; w.RS = 9; w.C = g.c; w.pack = 1; w.n = (int64_t)g.k * rsc;
         wts.push_back(w);
-        aux_ts.push_back(aux_ts.back() + cdv(w.n, 256));
+        aux_ts.push_back(aux_ts.back() + wtrans_ctas(w));
       }
     } else if (mode == 1) {
       c.w = ws + ip.wt;  // the transposed bf16 weights Wt[c][r][s][k]
@@ -423,7 +429,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       w.src = g.wt; w.dst = ws + ip.wt; w.K = g.k; w.RS = g.ksize * g.ksize; w.C = g.c; w.n = (int64_t)g.k * rsc;
       if (pl.variant == 5) w.pack = 2;
       wts.push_back(w);
-      aux_ts.push_back(aux_ts.back() + cdv(w.n, 256));
+      aux_ts.push_back(aux_ts.back() + wtrans_ctas(w));
     } else {
       c.dy = g.dy;
       c.dw_part = reinterpret_cast<float*>(ws + ip.part);

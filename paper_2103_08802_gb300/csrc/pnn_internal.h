@@ -171,13 +171,15 @@ struct WReduceDesc {
 // bf16 weight copies from src[K][RS][C].  pack 0: dst[c][r][s][k], for the
 // tensor-core data gradient.  pack 1 (forward: rows n = k, channels ch = c) and 2
 // (data gradient: n = c, ch = k): the operand layout of k_c3_conv.cu,
-// dst[ch / 8][tap][n][ch % 8]
+// dst[n / 64][ch / 8][tap][n % 64][ch % 8]
 struct WtDesc {
   const void* src;
   void* dst;
   int32_t K, RS, C, pack;
   int64_t n;
 };
+// CTAs of k_wtrans for it: an element a thread, or (packed) eight
+inline int wtrans_ctas(const WtDesc& w) { return (int)(((w.pack ? w.n / 8 : w.n) + 255) / 256); }
 
 // generic strided fp32 GEMM: C[m][n] = beta*C + sum_k A[m*sam + k*sak] * B[k*sbk + n*sbn] (+ bias[n]) (relu)
 struct GemmDesc {
@@ -381,28 +383,41 @@ inline int pw_item_units(int ncols, int64_t launch_mtiles) {
   return launch_mtiles >= 2 * (int64_t)device_sm_count() ? ncols / pw_unit_cols(ncols) : 1;
 }
 // 3x3 stride-1 forward / data gradient of k_c3_conv.cu (variant 5): ch channels
-// of the A source, ncols GEMM columns; patches of 8 x 16 pixels, or two whole
-// 8 x 8 images a tile.
+// of the A source, ncols GEMM columns in blocks of 64 (or all 16 or 32).  What an
+// M tile is: a patch of 8 x 16 pixels, two whole 8 x 8 images, or 128 / (H W)
+// whole smaller images (H and W powers of two).
 struct C3Slots {
   int raw, op, wt, x;  // bytes of a raw, an operand and a weight slot, and of the second operand
+  // small images or several column blocks somewhere in the launch: the general
+  // form of the kernel (a forward of 16 channels takes 73 us with it, 60 with
+  // the other, which has registers to spare)
+  int any;
 };
-PNN_HD inline bool c3_whole(int H, int W) { return H == 8 && W == 8; }
-// raw pixels of a k-step; bytes of an operand plane (a halo of 10 x 18 pixels, or
-// three copies of 10 x 16 and four pixels that spread the two planes' stores over the banks)
-PNN_HD inline int c3_raw_px(bool whole) { return whole ? 128 : 180; }
-PNN_HD inline int c3_plane(bool whole) { return (whole ? 484 : 180) * 16; }
-PNN_HD inline int c3_wt_bytes(int ncols) { return 9 * ncols * 32; }  // 16 channels, nine taps
+enum { C3_NONE = 0, C3_PATCH, C3_WHOLE, C3_SMALL };
+PNN_HD inline int c3_kind(int H, int W) {
+  if (H == 8 && W == 8) return C3_WHOLE;
+  if (W % 8 == 0 && H % 16 == 0) return C3_PATCH;
+  return H * W <= 32 && (H & (H - 1)) == 0 && (W & (W - 1)) == 0 ? C3_SMALL : C3_NONE;
+}
+// raw pixels of a k-step; bytes of an operand plane: a halo of 10 x 18 pixels,
+// three copies of 10 x 16, or nine copies of 128 pixels (the latter two and four
+// pixels that spread the two planes' stores over the banks)
+PNN_HD inline int c3_raw_px(int kind) { return kind == C3_PATCH ? 180 : 128; }
+PNN_HD inline int c3_plane(int kind) { return (kind == C3_PATCH ? 180 : kind == C3_WHOLE ? 484 : 1156) * 16; }
+PNN_HD inline int c3_block(int ncols) { return ncols < 64 ? ncols : 64; }
+PNN_HD inline int c3_wt_bytes(int block) { return 9 * block * 32; }  // 16 channels, nine taps
 inline bool c3_ok(int k, int stride, int H, int W, int ch, int ncols) {
-  auto narrow = [](int c) { return c == 16 || c == 32 || c == 64; };
-  return k == 3 && stride == 1 && (c3_whole(H, W) || (W % 8 == 0 && H % 16 == 0)) && narrow(ch) && narrow(ncols);
+  auto cols = [](int c) { return c == 16 || c == 32 || (c > 0 && c % 64 == 0); };
+  return k == 3 && stride == 1 && c3_kind(H, W) != C3_NONE && cols(ch) && cols(ncols);
 }
 inline void c3_add(C3Slots& s, int H, int W, int ncols, int esz, bool x) {
-  const bool wh = c3_whole(H, W);
+  const int kind = c3_kind(H, W), block = c3_block(ncols);
   auto most = [](int& a, int b) { if (a < b) a = b; };
-  most(s.raw, c3_raw_px(wh) * 16 * esz);
-  most(s.op, 2 * c3_plane(wh));
-  most(s.wt, (c3_wt_bytes(ncols) + 1023) & ~1023);
-  if (x) most(s.x, kTcBM * ncols * 2);
+  most(s.raw, c3_raw_px(kind) * 16 * esz);
+  most(s.op, 2 * c3_plane(kind));
+  most(s.wt, (c3_wt_bytes(block) + 1023) & ~1023);
+  if (x) most(s.x, kTcBM * block * 2);
+  if (kind == C3_SMALL || ncols > block) s.any = 1;
 }
 // Weight gradient of k_wg_conv.cu (variant 4: 1x1, 5: 3x3): the geometry of one instance's
 // k-steps.  1x1: kp pixels; 3x3: krows whole image rows (kp pixels) with the

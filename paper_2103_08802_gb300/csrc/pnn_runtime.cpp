@@ -1461,7 +1461,7 @@ int pnn_net::build_tables() {
               c.tma_y = ws ? ws + tables_off + mo + 2 * sizeof(CUtensorMap) : nullptr;
               c.tma_x = ws ? ws + tables_off + mo + 3 * sizeof(CUtensorMap) : nullptr;
               c.w = ws + (fwd ? off_wpf : off_wpd) + params[o.w].off * 2;  // packed by k_wtrans
-              c.ntiles = 1;
+              c.ntiles = cdiv(fwd ? ov.C : iv.C, c3_block(fwd ? ov.C : iv.C));
             }
             if (o.kind == K_WGRAD_TC && o.variant >= 4) {
               const bool xbf = c.x.dt == DT_BF16;
@@ -1747,9 +1747,14 @@ int pnn_net::build_tables() {
     std::vector<WtDesc> wt;
     std::vector<int> ts;
     wt_total = 0;
+    // the transposed copies that a data gradient reads
+    std::vector<char> read(params.size(), 0);
+    for (const POp& o : ops)
+      if (o.kind == K_DGRAD_TC && o.variant != 5) read[o.w] = 1;
     if (act_dt == DT_BF16)
-      for (const ParamT& p : params) {
-        if (p.kind != 0) continue;
+      for (size_t id = 0; id < params.size(); ++id) {
+        const ParamT& p = params[id];
+        if (p.kind != 0 || !read[id]) continue;
         WtDesc w{};
         w.src = ws + off_shadow + p.off * 2;
         w.dst = ws + off_wt + p.off * 2;
@@ -1757,7 +1762,7 @@ int pnn_net::build_tables() {
         w.n = (int64_t)p.n;
         wt.push_back(w);
         ts.push_back(wt_total);
-        wt_total += cdiv(w.n, 256);
+        wt_total += wtrans_ctas(w);
       }
     // the packed copies (a weight used by several ops of a direction once)
     std::vector<char> done(2 * params.size(), 0);
@@ -1774,7 +1779,7 @@ int pnn_net::build_tables() {
       w.n = (int64_t)p.n;
       wt.push_back(w);
       ts.push_back(wt_total);
-      wt_total += cdiv(w.n, 256);
+      wt_total += wtrans_ctas(w);
     }
     ts.push_back(wt_total);
     wt_count = (int)wt.size();

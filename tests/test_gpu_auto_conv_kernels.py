@@ -127,6 +127,14 @@ C3 = {
     "whole1": _wg(1, 8, 8, 16, 32, 3, bn=True),           # half a tile
     "whole5": _wg(5, 8, 8, 64, 64, 3, bn=True),
     "many": _wg(20, 64, 32, 16, 16, 3, bn=True),          # more tiles than CTAs
+    "p16_c128_n192": _wg(2, 16, 16, 128, 192, 3, bn=True),   # eight k-steps, three column blocks
+    "whole_c192_n128": _wg(3, 8, 8, 192, 128, 3, bn=True, relu=False),
+    "small4x4": _wg(9, 4, 4, 64, 128, 3, bn=True),        # a full tile and one image
+    "small2x2": _wg(33, 2, 2, 128, 64, 3, bn=True),
+    "small1x1": _wg(129, 1, 1, 16, 32, 3, bn=True),
+    "small2x8_fp32x": _wg(5, 2, 8, 32, 16, 3, bn=True, x_fp32=True),
+    "small_kinds": [_wg(20, 4, 4, 64, 64, 3, bn=True), _wg(2, 16, 16, 32, 128, 3, bn=True)],
+    "small_wholex": [_wg(3, 8, 8, 64, 128, 3, bn=True), _wg(40, 2, 2, 128, 64, 3, bn=False)],
     "stages": [_wg(2, 32, 32, 16, 16, 3, bn=True), _wg(3, 8, 8, 64, 64, 3, bn=True)],
     "stagex": [_wg(3, 8, 8, 64, 64, 3, bn=True), _wg(2, 16, 16, 32, 32, 3, bn=True)],
 }
