@@ -2815,8 +2815,9 @@ int pnn_profile_trace(pnn_net* n, int32_t max, pnn_trace* out, int32_t* count) {
     pnn_trace& r = out[i];
     float t = 0.f;
     cudaEventElapsedTime(&t, n->pev[2 * i], n->pev[2 * i + 1]);
+    const bool tc = L.kind == K_CONV_FWD_TC || L.kind == K_DGRAD_TC || L.kind == K_WGRAD_TC;
     // (k_pw_conv.cu, k_c3_conv.cu, k_wg_conv.cu: 1, fed by TMA)
-    r.variant = L.variant >= 4 ? 1 : L.variant + (L.wide ? 1 : (L.op > 0 ? 2 : 0));
+    r.variant = tc && L.variant >= 4 ? 1 : L.variant + (L.wide ? 1 : (L.op > 0 ? 2 : 0));
     r.kind = L.kind; r.phase = L.phase; r.instances = L.count;
     r.tiles = L.total;
     for (int j = 0; j < 6; ++j) r.shape[j] = L.shape[j];
