@@ -1,5 +1,5 @@
-// Grouped weight gradients of the bottleneck stacks' stride-1 1x1 and 3x3
-// layers with few channels, on the 5th-generation tensor cores:
+// Grouped weight gradients of stride-1 layers, 1x1 with few channels on one side
+// and 3x3, on the 5th-generation tensor cores:
 //
 //   dW[k][r][s][c] = sum_{pixels p} dY[p][k] * act(X)[p + (r-1, s-1)][c]
 //
@@ -18,19 +18,24 @@
 //         memory) whatever its N, so nine MMAs of one tap each (one copy with
 //         zero columns at its sides) took 146 us where three took 67.
 //         (Copying the transformed halo to a plane per tap, as the kernel of
-//         k_tc_conv.cu does, took 80 % of that kernel's 224 us.)
+//         k_tc_conv.cu does, took 80 % of that kernel's 224 us.)  Whole images of
+//         at most 32 pixels have no rows at a uniform distance: theirs are stored
+//         nine times, once a tap.  A tile is a block of 32 by 128 channels: its
+//         nine accumulators of 32 columns fit the tensor memory once.
 // Plane pitches are padded so that the eight lanes of a 16-byte store phase
 // fall into different banks whatever the channel count.
 //
-// Persistent; a tile is one run of pixels of one instance (and, 3x3 with 64
-// input channels, one half of them): the planner cuts the launch into about
+// Persistent; a tile is one run of pixels of one instance (and, 3x3, one block
+// of its channels): the planner cuts the launch into about
 // two tiles per SM of equal traffic, so few partial sums are written and
 // reduced.  Roles: producer (TMA, one thread), MMA (one thread), ten transform
 // warps, four epilogue warps.  Grouped launches of the
 // 8-subnetwork ResNet-1001 (batch 256, 64 px), kernels of k_tc_conv.cu -> now:
 // 3x3 224 -> 60 us, expand (16 -> 64) 159 -> 65 us (two launches before), reduce
 // 141 -> 56 us; the 1x1 are at 0.6 - 0.75 of the copy rate, the 3x3 is bound by
-// the latency of its k-steps.
+// the latency of its k-steps.  VGG-16 (batch 128): 128 -> 128 at 16 x 16, 4
+// instances, 348 -> 74 us; 256 -> 256 at 8 x 8, 3 instances, 232 -> 68; 512 -> 512
+// at 4 x 4 90 -> 55: each block of 32 input channels transforms the gradient again.
 // Every wait is bounded (2 s); on expiry the CTA records status 3, stops,
 // drains its copies and MMAs (bounded) and frees its TMEM.
 #include <cuda_bf16.h>
@@ -143,12 +148,13 @@ __device__ __forceinline__ uint4 chunk8(const uint4 (&q)[2], const Affine& af, i
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-// Rows of one source: raw [nrows][8 << lg channels] -> planes.  HALO: row u is
+// Rows of one source: raw [nrows][8 << lg channels] -> planes.  HALO 1: row u is
 // pixel u of whole image rows of 1 << lgw pixels, zero unless ylo <= u >> lgw <
 // yhi; copy s (2^lg planes after copy s - 1) holds at column x the pixel x + s - 1
 // of its row or zero -- the pixel that falls out of the row at one end marks the
-// zero at the other.
-template <bool XBF, bool BN, bool HALO>
+// zero at the other.  HALO 2: whole images of 1 << (lgw + ylo) pixels, the same in
+// both directions, copy 3 r + s for tap (r, s).
+template <bool XBF, bool BN, int HALO>
 __device__ __forceinline__ void rows_to_planes(const uint8_t* __restrict__ raw, uint8_t* __restrict__ pl, int nrows,
                                                int lg, int pitch, int t, const Affine& af, int relu, int lgw, int ylo,
                                                int yhi) {
@@ -171,7 +177,22 @@ __device__ __forceinline__ void rows_to_planes(const uint8_t* __restrict__ raw, 
       if (e && !two) continue;
       const int u = r + e * step;
       uint4 o = chunk8<XBF, BN>(q[e], af, relu);
-      if (HALO) {
+      if (HALO == 2) {
+        const uint4 zero = make_uint4(0, 0, 0, 0);
+        const int W = 1 << lgw, H = 1 << ylo, x = u & (W - 1), y = (u >> lgw) & (H - 1);
+        const int i0 = u >> (lgw + ylo) << (lgw + ylo);
+#pragma unroll 1
+        for (int r3 = 0; r3 < 9; r3 += 3) {
+          const int dy = y + 1 - r3 / 3;
+          const bool in = dy >= 0 && dy < H;
+          uint8_t* row = dst + (r3 * pitch << lg) + (i0 + ((dy & (H - 1)) << lgw)) * 16;
+#pragma unroll
+          for (int s = 0; s < 3; ++s) {
+            const int c = x + 1 - s;
+            *reinterpret_cast<uint4*>(row + (s * pitch << lg) + (c & (W - 1)) * 16) = in && c >= 0 && c < W ? o : zero;
+          }
+        }
+      } else if (HALO) {
         const uint4 zero = make_uint4(0, 0, 0, 0);
         const int y = u >> lgw, W = 1 << lgw, x = u & (W - 1);
         if (y < ylo || y >= yhi) o = zero;
@@ -187,7 +208,9 @@ __device__ __forceinline__ void rows_to_planes(const uint8_t* __restrict__ raw, 
   }
 }
 
-template <int KS>
+// ANY: a 3x3 launch with small images or several blocks of output channels;
+// without, the code of both folds away
+template <int KS, bool ANY>
 __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int ninst,
                                         int total, const Rings& rg, int32_t* status) {
   extern __shared__ uint8_t smem_raw[];
@@ -236,14 +259,16 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
         const ConvDesc* d = w.d;
         const Geo g = geo<KS>(d);
         const int pbeg = w.tm * d->pix_per_split, pend = min(g.rows, pbeg + d->pix_per_split);
-        const uint32_t bytes = (uint32_t)(g.p.xrows * g.p.xch * (g.xbf ? 2 : 4) + g.p.kp * g.K * 4);
+        const uint32_t bytes = (uint32_t)(g.p.xrows * g.p.xch * (g.xbf ? 2 : 4) + g.p.kp * g.p.ych * 4);
+        const int yb = ANY ? w.tn / wg_xblocks(KS, g.C) : 0, xb = w.tn - (ANY ? yb * wg_xblocks(KS, g.C) : 0);
+        const int up = KS == 3 && !(ANY && g.p.small) ? g.W : 0;  // the row above
         for (int p = pbeg; p < pend; p += g.p.kp) {
           if (!mbar_wait(smem_u32(&sh.raw_empty[cr.s]), cr.ph ^ 1, abort_flag)) { ok = false; break; }
           const uint32_t full = smem_u32(&sh.raw_full[cr.s]);
           const uint32_t slot = base + off_raw + cr.s * rg.rawb;
           mbar_expect_tx(full, bytes);
-          tma_load_2d(slot, d->tma_a, w.tn * g.p.xch, KS == 3 ? p - g.W : p, full);
-          tma_load_2d(slot + g.p.yoff, d->tma_b, 0, p, full);
+          tma_load_2d(slot, d->tma_a, xb * g.p.xch, p - up, full);
+          tma_load_2d(slot + g.p.yoff, d->tma_b, ANY ? yb * g.p.ych : 0, p, full);
           cr.next();
           ++n;
         }
@@ -284,10 +309,11 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
             }
           } else {
             const uint64_t bd = nosw_desc(b_addr, 128, g.p.bpitch);
+            const int rs = ANY && g.p.small ? 3 * (g.p.nch >> 3) * (g.p.bpitch >> 4) : g.W;  // between tap rows
             for (int j = 0; j < steps; ++j)
 #pragma unroll
               for (int r = 0; r < 3; ++r)
-                mma_bf16(tacc + r * 3 * g.p.nch, ad + j * 16, bd + j * 16 + r * g.W, idesc, acc | j ? 1u : 0u);
+                mma_bf16(tacc + r * 3 * g.p.nch, ad + j * 16, bd + j * 16 + r * rs, idesc, acc | j ? 1u : 0u);
           }
           acc = 1;
           issued = true;
@@ -319,9 +345,10 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
       const Geo g = geo<KS>(d);
       const int pbeg = w.tm * d->pix_per_split, pend = min(g.rows, pbeg + d->pix_per_split);
       const int relu = g.bn ? d->x.relu : 0;
-      const int lgx = 28 - __clz(g.p.xch), lgy = 28 - __clz(g.K);  // log2 of the chunks a pixel
+      const int lgx = 28 - __clz(g.p.xch), lgy = 28 - __clz(ANY ? g.p.ych : g.K);  // log2 of the chunks a pixel
+      const int xb = ANY ? w.tn % wg_xblocks(KS, g.C) : w.tn;
       Affine af, none{};
-      if (g.bn) af.load(d->x.scale, d->x.shift, w.tn * g.p.xch + (t & ((1 << lgx) - 1)) * 8);
+      if (g.bn) af.load(d->x.scale, d->x.shift, xb * g.p.xch + (t & ((1 << lgx) - 1)) * 8);
       // which side x and dY are, their planes in the operand slot
       const int xoff = g.p.x_is_a ? 0 : g.p.boff, yoff = g.p.x_is_a ? g.p.boff : 0;
       const int xpitch = g.p.x_is_a ? g.p.apitch : g.p.bpitch, ypitch = g.p.x_is_a ? g.p.bpitch : g.p.apitch;
@@ -333,9 +360,18 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
         if (!ok) { sh.abort_flag = 1; continue; }
         const uint8_t* raw = gbase + off_raw + cr.s * rg.rawb;
         uint8_t* op = gbase + co.s * rg.opb;
-        rows_to_planes<false, false, false>(raw + g.p.yoff, op + yoff, g.p.kp, lgy, ypitch, t, none, 0, 0, 0, 0);
+        rows_to_planes<false, false, 0>(raw + g.p.yoff, op + yoff, g.p.kp, lgy, ypitch, t, none, 0, 0, 0, 0);
         const int ylo = y0 == 0 ? 1 : 0, yhi = y0 + g.p.krows == g.H ? g.p.krows + 1 : g.p.krows + 2;
-        if (g.xbf) {
+        if (ANY && g.p.small) {
+          const int lgh = 31 - __clz(g.H);
+          if (g.xbf) {
+            if (g.bn) rows_to_planes<true, true, 2>(raw, op + xoff, g.p.xrows, lgx, xpitch, t, af, relu, g.p.lgw, lgh, 0);
+            else rows_to_planes<true, false, 2>(raw, op + xoff, g.p.xrows, lgx, xpitch, t, af, 0, g.p.lgw, lgh, 0);
+          } else {
+            if (g.bn) rows_to_planes<false, true, 2>(raw, op + xoff, g.p.xrows, lgx, xpitch, t, af, relu, g.p.lgw, lgh, 0);
+            else rows_to_planes<false, false, 2>(raw, op + xoff, g.p.xrows, lgx, xpitch, t, af, 0, g.p.lgw, lgh, 0);
+          }
+        } else if (g.xbf) {
           if (g.bn)
             rows_to_planes<true, true, KS == 3>(raw, op + xoff, g.p.xrows, lgx, xpitch, t, af, relu, g.p.lgw, ylo, yhi);
           else
@@ -375,6 +411,7 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
       // blocks of 16 accumulator columns: 1x1 (M half, N) rows of nch floats;
       // 3x3 (tap, N) rows of 9 C floats
       const int per = g.p.nch >> 4;
+      const int yb = ANY ? w.tn / wg_xblocks(KS, g.C) : 0, xb = w.tn - (ANY ? yb * wg_xblocks(KS, g.C) : 0);
       const int blocks = (KS == 1 ? (g.p.mch > 128 ? 2 : 1) : 9) * per;
       for (int b = 0; b < blocks; ++b) {
         const int outer = b / per, n = (b - outer * per) * 16;
@@ -385,7 +422,7 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
         tmem_wait_ld(a);
         if (m < g.p.mch) {
           float* out = KS == 1 ? d->dw_part + ((int64_t)w.tm * g.p.mch + m) * g.p.nch + n
-                               : d->dw_part + (((int64_t)w.tm * g.K + m) * 9 + outer) * g.C + w.tn * g.p.nch + n;
+                               : d->dw_part + (((int64_t)w.tm * g.K + yb * 128 + m) * 9 + outer) * g.C + xb * g.p.nch + n;
 #pragma unroll
           for (int i = 0; i < 4; ++i)
             reinterpret_cast<uint4*>(out)[i] = make_uint4(a[4 * i], a[4 * i + 1], a[4 * i + 2], a[4 * i + 3]);
@@ -407,11 +444,12 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
 
 __global__ void __launch_bounds__(kThreads, 1) k_wg_pw(const ConvDesc* __restrict__ tab, const int* __restrict__ ts,
                                                        int ninst, int total, const Rings rg, int32_t* status) {
-  wg_body<1>(tab, ts, ninst, total, rg, status);
+  wg_body<1, false>(tab, ts, ninst, total, rg, status);
 }
+template <bool ANY>
 __global__ void __launch_bounds__(kThreads, 1) k_wg_3x3(const ConvDesc* __restrict__ tab, const int* __restrict__ ts,
                                                         int ninst, int total, const Rings rg, int32_t* status) {
-  wg_body<3>(tab, ts, ninst, total, rg, status);
+  wg_body<3, ANY>(tab, ts, ninst, total, rg, status);
 }
 
 }  // namespace
@@ -421,14 +459,14 @@ bool wg_fits(int raw_bytes, int op_bytes) {
   return plan_rings(raw_bytes, op_bytes, r);
 }
 
-cudaError_t launch_conv_wg(int ksize, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes, int op_bytes,
+cudaError_t launch_conv_wg(int ksize, int any, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes, int op_bytes,
                            int32_t* status, cudaStream_t st, int max_ctas) {
   if (total <= 0) return cudaSuccess;
   Rings r;
   if (raw_bytes <= 0 || op_bytes <= 0 || (raw_bytes & 1023) || (op_bytes & 1023) || !plan_rings(raw_bytes, op_bytes, r))
     return cudaErrorInvalidValue;
-  auto kern = ksize == 3 ? k_wg_3x3 : k_wg_pw;
-  cudaError_t e = set_smem_attr_once(ksize == 3 ? 16 : 15, reinterpret_cast<const void*>(kern), kSmemBudget);
+  auto kern = ksize != 3 ? k_wg_pw : any ? k_wg_3x3<true> : k_wg_3x3<false>;
+  cudaError_t e = set_smem_attr_once(ksize != 3 ? 15 : any ? 21 : 16, reinterpret_cast<const void*>(kern), kSmemBudget);
   if (e != cudaSuccess) return e;
   const int sms = device_sm_count();
   int grid = total < sms ? total : sms;

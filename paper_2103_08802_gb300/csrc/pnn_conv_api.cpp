@@ -105,6 +105,7 @@ struct Plan {
   int variant = 0;
   int bnmax = 16, raw = 0, op = 0, wide = 0;
   C3Slots c3{};
+  int wg_any = 0;  // weight gradient of k_wg_conv.cu: its general form
   int total = 0;
   size_t tab = 0, ts = 0, status = 0, aux_tab = 0, aux_ts = 0, fin_tab = 0, fin_ts = 0, red_tab = 0, red_ts = 0;
   size_t bytes = 0, init_bytes = 0;  // init_bytes: the prefix copied from the host
@@ -266,12 +267,13 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
       ip.mtiles = cdv(rsc, ip.rows);
       if (all_wg) {
         const WgPlan wp = wg_plan(g.ksize, g.c, g.k, g.h, g.w, g.x_dtype == PNN_DT_BF16);
-        ip.ntiles = wg_ntiles(g.ksize, g.c);
+        ip.ntiles = wg_ntiles(g.ksize, g.c, g.k);
         const WgSplit sp = wg_split(Mout, wp.kp, ip.ntiles, wg_traffic(g), wg_bytes);
         ip.mtiles = ip.splits = sp.splits;
         ip.pix_per_split = sp.pix;
         pl.raw = std::max(pl.raw, wp.raw);
         pl.op = std::max(pl.op, wp.op);
+        if (wg_any(g.ksize, g.h, g.w, g.k)) pl.wg_any = 1;
         pl.bnmax = g.ksize;
         pl.total += ip.splits * ip.ntiles;
         ip.maps = take(4 * 128);
@@ -487,7 +489,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       const bool xbf = g.x_dtype == PNN_DT_BF16;
       const WgPlan wp = wg_plan(g.ksize, g.c, g.k, g.h, g.w, xbf);
       int e = encode_tensor_map_2d(m, g.x, xbf, g.c, Min, wp.xch, wp.xrows, 0, &why);
-      if (!e) e = encode_tensor_map_2d(m + 128, g.dy, false, g.k, Mout, g.k, wp.kp, 0, &why);
+      if (!e) e = encode_tensor_map_2d(m + 128, g.dy, false, g.k, Mout, wp.ych, wp.kp, 0, &why);
       if (e) return set_last_error(PNN_ECUDA, why);
       c.tma_a = ws + ip.maps;
       c.tma_b = ws + ip.maps + 128;
@@ -581,7 +583,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
   auto conv_launch = [&]() {
     if (pl.variant == 5) return launch_conv_c3(mode, tab, tsd, n, pl.total, pl.c3, status, st);
     if (pl.variant == 4 && mode == 2)
-      return launch_conv_wg(pl.bnmax, tab, tsd, n, pl.total, pl.raw, pl.op, status, st);
+      return launch_conv_wg(pl.bnmax, pl.wg_any, tab, tsd, n, pl.total, pl.raw, pl.op, status, st);
     if (pl.variant == 4)
       return launch_conv_pw(mode, pl.wide, tab, tsd, n, pl.total, pl.raw, pl.op, status, st);
     if (pl.variant == 1)

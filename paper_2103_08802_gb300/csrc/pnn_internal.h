@@ -254,9 +254,9 @@ cudaError_t launch_conv_pw(int mode, int wide, const ConvDesc* tab, const int* t
 struct C3Slots;
 cudaError_t launch_conv_c3(int mode, const ConvDesc* tab, const int* ts, int n, int total, const C3Slots& s,
                            int32_t* status, cudaStream_t st, int max_ctas = 0);
-// weight gradient of k_wg_conv.cu; raw_bytes, op_bytes: the largest slots over
-// the launch's instances (multiples of 1024)
-cudaError_t launch_conv_wg(int ksize, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes, int op_bytes,
+// weight gradient of k_wg_conv.cu; any: wg_any of some instance; raw_bytes, op_bytes:
+// the largest slots over the launch's instances (multiples of 1024)
+cudaError_t launch_conv_wg(int ksize, int any, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes, int op_bytes,
                            int32_t* status, cudaStream_t st, int max_ctas = 0);
 // record a message for pnn_last_error(NULL) and return `code`
 int set_last_error(int code, const char* msg);
@@ -427,7 +427,8 @@ inline void c3_add(C3Slots& s, int H, int W, int ncols, int esz, bool x) {
 // stores over the banks.
 struct WgPlan {
   int kp, krows, lgw;
-  int xch, xrows;          // x channels of a tile and raw rows of a k-step
+  int small;               // 3x3, whole images of at most 32 pixels: the N side holds a copy a tap
+  int xch, ych, xrows;     // x and dY channels of a tile and raw rows of a k-step
   int x_is_a, mch, nch;    // M side: x or dY; channels of both sides (3x3: the N side holds three copies)
   int apitch, bpitch, boff;
   int yoff, raw, op;
@@ -441,6 +442,7 @@ PNN_HD inline WgPlan wg_plan(int ks, int C, int K, int H, int W, bool xbf) {
     p.kp = 128;
     while (p.kp > 32 && p.kp * (C * esz + K * 4) > kWgRawMax) p.kp >>= 1;
     p.xch = C;
+    p.ych = K;
     p.xrows = p.kp;
     p.x_is_a = C > K;
     p.mch = C > K ? C : K;
@@ -448,40 +450,51 @@ PNN_HD inline WgPlan wg_plan(int ks, int C, int K, int H, int W, bool xbf) {
     p.bpitch = (p.kp + wg_plane_pad(p.nch)) * 16;
   } else {
     p.xch = C < 32 ? C : 32;
-    p.mch = K;
+    p.ych = K < 128 ? K : 128;
+    p.mch = p.ych;
     p.nch = p.xch;
-    p.lgw = W == 8 ? 3 : (W == 16 ? 4 : 5);
-    for (int r = 128 / W; r >= 1; --r) {
-      if (H % r || (r * W) % 16 || (r + 2) * W > 256) continue;
-      if ((r + 2) * W * p.xch * esz + r * W * K * 4 > kWgRawMax) continue;
-      p.krows = r;
-      break;
+    p.small = c3_kind(H, W) == C3_SMALL;
+    while (1 << p.lgw < W) ++p.lgw;
+    if (p.small) {
+      p.kp = p.xrows = 64;
+    } else {
+      for (int r = 128 / W; r >= 1; --r) {
+        if (H % r || (r * W) % 16 || (r + 2) * W > 256) continue;
+        if ((r + 2) * W * p.xch * esz + r * W * p.ych * 4 > kWgRawMax) continue;
+        p.krows = r;
+        break;
+      }
+      p.kp = p.krows * W;
+      p.xrows = (p.krows + 2) * W;  // (a multiple of 8)
     }
-    p.kp = p.krows * W;
-    p.xrows = (p.krows + 2) * W;  // (a multiple of 8)
     p.bpitch = (p.xrows + wg_plane_pad(p.xch)) * 16;
   }
   p.apitch = (p.kp + wg_plane_pad(p.mch)) * 16;
   p.boff = p.mch / 8 * p.apitch;
-  p.op = (p.boff + (ks == 1 ? 1 : 3) * (p.nch / 8) * p.bpitch + 1023) & ~1023;
+  p.op = (p.boff + (ks == 1 ? 1 : p.small ? 9 : 3) * (p.nch / 8) * p.bpitch + 1023) & ~1023;
   p.yoff = (p.xrows * p.xch * esz + 127) & ~127;
-  p.raw = (p.yoff + p.kp * K * 4 + 1023) & ~1023;
+  p.raw = (p.yoff + p.kp * p.ych * 4 + 1023) & ~1023;
   return p;
 }
 bool wg_fits(int raw_bytes, int op_bytes);
 inline bool wg_ok(int k, int stride, int C, int K, int H, int W, bool xbf) {
   auto pow2 = [](int v, int lo, int hi) { return v >= lo && v <= hi && (v & (v - 1)) == 0; };
-  if (stride != 1 || !pow2(C, 16, 256) || !pow2(K, 16, 256)) return false;
+  if (stride != 1) return false;
   if (k == 1) {
-    if (C > 64 && K > 64) return false;
+    if (!pow2(C, 16, 256) || !pow2(K, 16, 256) || (C > 64 && K > 64)) return false;
   } else {
-    if (k != 3 || C > 64 || K > 128 || !pow2(W, 8, 32)) return false;
+    // blocks of 32 x 128 channels, or all of a narrower layer's
+    if (k != 3 || (C != 16 && (C <= 0 || C % 32 != 0)) || (!pow2(K, 16, 128) && (K <= 0 || K % 128 != 0))) return false;
+    if (c3_kind(H, W) != C3_SMALL && !pow2(W, 8, 32)) return false;
   }
   const WgPlan p = wg_plan(k, C, K, H, W, xbf);
   return p.kp > 0 && wg_fits(p.raw, p.op);
 }
-// tiles of an instance per split
-PNN_HD inline int wg_ntiles(int ks, int C) { return ks == 3 && C > 32 ? C / 32 : 1; }
+// tiles of an instance per split: blocks of x channels and of dY channels
+PNN_HD inline int wg_xblocks(int ks, int C) { return ks == 3 && C > 32 ? C / 32 : 1; }
+PNN_HD inline int wg_ntiles(int ks, int C, int K) { return wg_xblocks(ks, C) * (ks == 3 && K > 128 ? K / 128 : 1); }
+// whether a layer needs the general form of the 3x3 kernel
+inline bool wg_any(int ks, int H, int W, int K) { return ks == 3 && (c3_kind(H, W) == C3_SMALL || K > 128); }
 // Splits of the instances of one launch: about two tiles per SM over the
 // launch, each instance in proportion to the bytes it moves, whole k-steps.
 // (With 2 x SMs splits for every instance, as a launch of its own needs, eight

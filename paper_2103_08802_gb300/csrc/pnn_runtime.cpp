@@ -114,6 +114,7 @@ struct Launch {
   int op = 0;           // TMA-fed conv with halo tiles: operand slot bytes of one stage (0: default);
                         // variant 4: second-operand bytes of a unit, or (weight gradient) operand slot bytes
   C3Slots c3{};         // variant 5: its slots
+  int wg_any = 0;       // k_wg_conv.cu: the general form
   int wide = 0;         // TMA-fed forward / data gradient: every tile one k-step (the wide-epilogue variant)
   int block = -1;       // fine forward / backward: position of the layer in its segment
 };
@@ -1151,7 +1152,7 @@ int pnn_net::plan(const pnn_desc* d) {
         const Value& iv = vals[o.in];
         const int src = iv.virt ? iv.src : o.in;
         const WgPlan wp = wg_plan(o.k, iv.C, vals[o.out].C, iv.H, iv.W, vals[src].dt == DT_BF16);
-        o.ntiles = wg_ntiles(o.k, iv.C);
+        o.ntiles = wg_ntiles(o.k, iv.C, vals[o.out].C);
         const WgSplit sp = wg_split(rows(o.in), wp.kp, o.ntiles, traffic(o), all);
         o.splits = o.mtiles = sp.splits;
         o.pix_per_split = sp.pix;
@@ -1470,7 +1471,7 @@ int pnn_net::build_tables() {
               memset(maps, 0, sizeof maps);
               if (ws) {
                 int r = encode_map(&maps[0], c.x.ptr, xbf, iv.C, (int64_t)B * iv.H * iv.W, wp.xch, wp.xrows, 0);
-                if (!r) r = encode_map(&maps[1], P<float>(gptr(o.out)), false, ov.C, (int64_t)B * ov.H * ov.W, ov.C,
+                if (!r) r = encode_map(&maps[1], P<float>(gptr(o.out)), false, ov.C, (int64_t)B * ov.H * ov.W, wp.ych,
                                        wp.kp, 0);
                 if (r) return r;
               }
@@ -1724,13 +1725,14 @@ int pnn_net::build_tables() {
         L.op = 0;
       }
       if (g.kind == K_WGRAD_TC && g.variant >= 4) {
-        L.raw = L.op = 0;
-                for (int id : g.ops) {
+        L.raw = L.op = L.wg_any = 0;
+        for (int id : g.ops) {
           const POp& o = ops[id];
           const int src = vals[o.in].virt ? vals[o.in].src : o.in;
           const WgPlan wp = wg_plan(o.k, vals[o.in].C, vals[o.out].C, vals[o.in].H, vals[o.in].W, vals[src].dt == DT_BF16);
           L.raw = std::max(L.raw, wp.raw);
           L.op = std::max(L.op, wp.op);
+          if (wg_any(o.k, vals[o.in].H, vals[o.in].W, vals[o.out].C)) L.wg_any = 1;
         }
       }
       for (int id : g.ops) op_cost(ops[id], L.flops, L.bytes);
@@ -1920,7 +1922,7 @@ int pnn_net::run_phase(int p, cudaStream_t st, int cap) {
         break;
       case K_WGRAD_TC:
         if (L.variant >= 4) {
-          e = launch_conv_wg(L.variant == 5 ? 3 : 1, (const ConvDesc*)tab, ts, L.count, L.total, L.raw, L.op, P<int32_t>(status_off), st,
+          e = launch_conv_wg(L.variant == 5 ? 3 : 1, L.wg_any, (const ConvDesc*)tab, ts, L.count, L.total, L.raw, L.op, P<int32_t>(status_off), st,
                              cap);
           break;
         }

@@ -106,6 +106,13 @@ WG = {
     "w8": _wg(3, 8, 8, 64, 64, 3, bn=True),              # two channel halves, row-strided pixel groups
     "w8_h16_k128": _wg(2, 16, 8, 32, 128, 3, bn=False),
     "w16_fp32x": _wg(2, 16, 16, 64, 16, 3, bn=True, x_fp32=True, relu=False),
+    "w16_c128_k128": _wg(2, 16, 16, 128, 128, 3, bn=True),   # four blocks of input channels
+    "w8_c96_k256": _wg(3, 8, 8, 96, 256, 3, bn=True, relu=False),  # three by two blocks
+    "small4x4": _wg(9, 4, 4, 64, 128, 3, bn=True),           # whole images, a ragged last k-step
+    "small2x2": _wg(70, 2, 2, 32, 256, 3, bn=True),
+    "small1x1": _wg(130, 1, 1, 16, 32, 3, bn=True),
+    "small2x8_fp32x": _wg(5, 2, 8, 32, 16, 3, bn=True, x_fp32=True),
+    "group_kinds": [_wg(20, 4, 4, 64, 64, 3, bn=True), _wg(2, 16, 16, 32, 128, 3, bn=True)],
     "group_3x3": [_wg(4, 32, 32, 16, 16, 3, bn=True), _wg(2, 16, 16, 32, 32, 3, bn=True),
                   _wg(2, 8, 8, 64, 64, 3, bn=True)],
 }
