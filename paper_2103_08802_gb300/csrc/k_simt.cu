@@ -15,6 +15,7 @@
 #include <mutex>
 
 #include "pnn_internal.h"
+#include "tc_pair.cuh"
 
 namespace pnn {
 
@@ -1486,108 +1487,168 @@ __global__ void __launch_bounds__(256) k_pool_bwd(const PoolDesc* __restrict__ t
 
 // ---------------------------------------------------------------- GEMM (head)
 // C[m][n] = sum_k A[m][k] B[k][n] (+ bias[n]) (+ beta C[m][n]) (ReLU), fp32.
-// 64 x 64 tiles; 256 threads with 4 x 4 consecutive outputs each read both
-// operands as float4 from shared memory; 16-wide K steps, the next step's
-// operands loaded into registers meanwhile.  Each operand is read along
-// whichever of its two indices is contiguous in memory.  KS groups of 256
-// threads share a tile's K range (a head has 128 tiles and K = 4096: one group
-// leaves an SM with eight warps); their sums are added in group order.  (Scalar
-// shared-memory reads and one group: VGG-16's head 0.57 / 0.77 ms forward /
-// backward at batch 128; now 0.50 / 0.73.)
-template <int KS>
-__global__ void __launch_bounds__(256 * KS) k_gemm(const GemmDesc* __restrict__ tab, const int* __restrict__ tstart,
-                                                   int n) {
-  constexpr int BM = 64, BN = 64, BK = 16, PER = BM * BK / 256;
-  __shared__ __align__(16) float As[KS][2][BK][BM + 4];
-  __shared__ __align__(16) float Bs[KS][2][BK][BN + 4];
-  const int inst = find_instance(tstart, n, blockIdx.x);
-  const GemmDesc d = tab[inst];
-  const int t = blockIdx.x - tstart[inst];
-  const int tm = t % d.mtiles, tn = t / d.mtiles;
-  const int m0 = tm * BM, n0 = tn * BN;
-  const int grp = threadIdx.x / 256, tid = threadIdx.x % 256, tx = tid % 16, ty = tid / 16;
-  const int kper = (d.K + KS * BK - 1) / (KS * BK) * BK;  // this group's share: whole steps
-  const int kb0 = grp * kper, kb1 = min(d.K, kb0 + kper);
+// BM x BN tiles by 128 threads of TM x TN outputs, 16-wide K steps, the next
+// step's operands loaded into registers meanwhile, as float4 along whichever of
+// an operand's two indices is contiguous (single elements at the edges and
+// where the alignment does not allow it).  Bound by the fp32 FMA rate: with 8 x 8
+// outputs a thread reads 64 bytes of shared memory for 64 FMAs -- with 4 x 4, as
+// before, 32 for 16 -- and two FMAs are one packed instruction, which leaves the
+// issue slots for the rest.  The K range of a tile is split over the CTAs of a
+// cluster, so that a layer of 64 tiles still occupies every SM; the partial
+// tiles meet in distributed shared memory and are added in rank order, each CTA
+// finishing its share of the rows.  VGG-16's head at batch 128 (512 -> 4096 -> 4096
+// -> 10): forward 0.50 -> 0.19 ms, backward 0.73 -> 0.37, about half of the FMA rate.
+template <int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__(128, 4) k_gemm(const GemmDesc* __restrict__ desc) {
+  constexpr int BK = 16, VM = TM < 4 ? TM : 4, VN = TN < 4 ? TN : 4;  // outputs in runs of VM rows, VN columns
+  constexpr int TX = BN / TN;
+  constexpr int UA = (BM * 4 + 127) / 128, UB = (BN * 4 + 127) / 128;  // float4 loads a thread and step
+  static_assert(BM / TM * TX == 128, "128 threads");
+  constexpr int PA = BM + 4, PB = BN + 4, PC = BN + 4;
+  constexpr int kOperands = 2 * BK * (PA + PB), kTile = BM * PC;
+  __shared__ __align__(16) float sm[kOperands > kTile ? kOperands : kTile];
+  float* const As = sm;
+  float* const Bs = sm + 2 * BK * PA;
+  const GemmDesc d = *desc;
+  uint32_t rank, splits;
+  asm("mov.u32 %0, %cluster_ctarank;" : "=r"(rank));
+  asm("mov.u32 %0, %cluster_nctarank;" : "=r"(splits));
+  const int tile = blockIdx.x / splits, mt = (d.M + BM - 1) / BM;
+  const int m0 = tile % mt * BM, n0 = tile / mt * BN;
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const int kper = (d.K + (int)splits * BK - 1) / ((int)splits * BK) * BK;  // this CTA's share: whole steps
+  const int kb0 = (int)rank * kper, kb1 = min(d.K, kb0 + kper);
   const bool a_k = d.sak == 1, b_k = d.sbk == 1;  // k contiguous in A / in B
-  float ra[PER], rb[PER];
-  auto slot = [&](int e, bool k_fast, int W, int& kk, int& x) {
-    if (k_fast) { kk = e % BK; x = e / BK; } else { x = e % W; kk = e / W; }
+  const bool a_v = ((a_k ? d.sam : d.sak) & 3) == 0 && (a_k || d.sam == 1) && (reinterpret_cast<uintptr_t>(d.A) & 15) == 0;
+  const bool b_v = ((b_k ? d.sbn : d.sbk) & 3) == 0 && (b_k || d.sbn == 1) && (reinterpret_cast<uintptr_t>(d.Bm) & 15) == 0;
+  float4 ra[UA], rb[UB];
+  // four elements from (x, k) along k or along x
+  auto load4 = [&](const float* p, int64_t sx, int64_t sk, int x, int X, int k, bool k_fast, bool vec) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (x >= X || k >= kb1) return v;
+    p += x * sx + k * sk;
+    if (vec && (k_fast ? k + 4 <= kb1 : x + 4 <= X)) return __ldg(reinterpret_cast<const float4*>(p));
+    const int left = k_fast ? kb1 - k : X - x;
+    const int64_t step = k_fast ? sk : sx;
+    v.x = __ldg(p);
+    if (left > 1) v.y = __ldg(p + step);
+    if (left > 2) v.z = __ldg(p + 2 * step);
+    if (left > 3) v.w = __ldg(p + 3 * step);
+    return v;
   };
   auto load = [&](int k0) {
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      int kk, x;
-      slot(tid + 256 * q, a_k, BM, kk, x);
-      const int m = m0 + x, k = k0 + kk;
-      ra[q] = (m < d.M && k < kb1) ? __ldg(d.A + (int64_t)m * d.sam + (int64_t)k * d.sak) : 0.f;
-      slot(tid + 256 * q, b_k, BN, kk, x);
-      const int nc = n0 + x, kb = k0 + kk;
-      rb[q] = (nc < d.N && kb < kb1) ? __ldg(d.Bm + (int64_t)kb * d.sbk + (int64_t)nc * d.sbn) : 0.f;
+    for (int q = 0; q < UA; ++q) {
+      const int u = tid + 128 * q;
+      if (u < BM * 4)
+        ra[q] = a_k ? load4(d.A, d.sam, d.sak, m0 + u / 4, d.M, k0 + u % 4 * 4, true, a_v)
+                    : load4(d.A, d.sam, d.sak, m0 + u % (BM / 4) * 4, d.M, k0 + u / (BM / 4), false, a_v);
+    }
+#pragma unroll
+    for (int q = 0; q < UB; ++q) {
+      const int u = tid + 128 * q;
+      if (u < BN * 4)
+        rb[q] = b_k ? load4(d.Bm, d.sbn, d.sbk, n0 + u / 4, d.N, k0 + u % 4 * 4, true, b_v)
+                    : load4(d.Bm, d.sbn, d.sbk, n0 + u % (BN / 4) * 4, d.N, k0 + u / (BN / 4), false, b_v);
+    }
+  };
+  auto put = [&](float* s, int pitch, int W, int u, const float4& v, bool k_fast) {
+    if (k_fast) {
+      float* c = s + u % 4 * 4 * pitch + u / 4;
+      c[0] = v.x; c[pitch] = v.y; c[2 * pitch] = v.z; c[3 * pitch] = v.w;
+    } else {
+      *reinterpret_cast<float4*>(s + u / (W / 4) * pitch + u % (W / 4) * 4) = v;
     }
   };
   auto store = [&](int buf) {
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      int kk, x;
-      slot(tid + 256 * q, a_k, BM, kk, x);
-      As[grp][buf][kk][x] = ra[q];
-      slot(tid + 256 * q, b_k, BN, kk, x);
-      Bs[grp][buf][kk][x] = rb[q];
-    }
+    for (int q = 0; q < UA; ++q)
+      if (tid + 128 * q < BM * 4) put(As + buf * BK * PA, PA, BM, tid + 128 * q, ra[q], a_k);
+#pragma unroll
+    for (int q = 0; q < UB; ++q)
+      if (tid + 128 * q < BN * 4) put(Bs + buf * BK * PB, PB, BN, tid + 128 * q, rb[q], b_k);
   };
-  float acc[4][4] = {};
+  // output i of a thread is row BM / (TM / VM) * (i / VM) + VM ty + i % VM of the tile
+  auto row = [&](int i) { return BM / (TM / VM) * (i / VM) + VM * ty + i % VM; };
+  auto col = [&](int j) { return BN / (TN / VN) * (j / VN) + VN * tx + j % VN; };
+  uint64_t acc[TM][TN / 2] = {};
   load(kb0);
   store(0);
   __syncthreads();
   int buf = 0;
-  // every group runs the same number of steps (the last group's tail is zeros)
-  for (int k0 = kb0; k0 < kb0 + kper; k0 += BK) {
-    const bool more = k0 + BK < kb0 + kper;
+  for (int k0 = kb0; k0 < kb1; k0 += BK) {
+    const bool more = k0 + BK < kb1;
     if (more) load(k0 + BK);
+    const float* a0 = As + buf * BK * PA;
+    const float* b0 = Bs + buf * BK * PB;
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      const float4 a = *reinterpret_cast<const float4*>(&As[grp][buf][kk][4 * ty]);
-      const float4 b = *reinterpret_cast<const float4*>(&Bs[grp][buf][kk][4 * tx]);
-      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+      float av[TM];
+      uint64_t bv[TN / 2];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TM; i += VM) {
+        if (VM == 4) *reinterpret_cast<float4*>(av + i) = *reinterpret_cast<const float4*>(a0 + kk * PA + row(i));
+        else *reinterpret_cast<float2*>(av + i) = *reinterpret_cast<const float2*>(a0 + kk * PA + row(i));
+      }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+      for (int j = 0; j < TN; j += VN) {
+        if (VN == 4) {
+          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(b0 + kk * PB + col(j));
+          bv[j / 2] = v.x;
+          bv[j / 2 + (VN == 4)] = v.y;
+        } else {
+          bv[j / 2] = *reinterpret_cast<const uint64_t*>(b0 + kk * PB + col(j));
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const uint64_t aa = tc::pk2(av[i], av[i]);
+#pragma unroll
+        for (int j = 0; j < TN / 2; ++j) acc[i][j] = tc::fma2(aa, bv[j], acc[i][j]);
+      }
     }
     if (more) store(buf ^ 1);
     __syncthreads();
     buf ^= 1;
   }
-  if (KS > 1) {
-    // groups 1 .. KS - 1 leave their sums in the (consumed) operand buffers
-    float4* sum = reinterpret_cast<float4*>(&As[0][0][0][0]);
-    static_assert(KS == 1 || sizeof(As) >= (KS - 1) * 256 * 64, "room for the groups' sums");
-    if (grp > 0)
+  // (a share past the end of K has read nothing and holds zeros)
+  __syncthreads();
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        sum[((grp - 1) * 4 + i) * 256 + tid] = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; j += 2) *reinterpret_cast<uint64_t*>(sm + row(i) * PC + col(j)) = acc[i][j / 2];
+  // every CTA of the cluster has left its sums; no one returns before this
+  if (splits > 1) {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  } else {
     __syncthreads();
-    if (grp > 0) return;
-    for (int g = 0; g < KS - 1; ++g)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float4 v = sum[(g * 4 + i) * 256 + tid];
-        acc[i][0] += v.x; acc[i][1] += v.y; acc[i][2] += v.z; acc[i][3] += v.w;
-      }
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int m = m0 + 4 * ty + i, nc = n0 + 4 * tx + j;
-      if (m < d.M && nc < d.N) {
-        float v = acc[i][j];
-        if (d.bias) v += d.bias[nc];
-        if (d.beta != 0.f) v += d.beta * d.Cm[(int64_t)m * d.scm + nc];
-        if (d.relu) v = fmaxf(v, 0.f);
-        d.Cm[(int64_t)m * d.scm + nc] = v;
-      }
+  const int rows = BM / (int)splits, r0 = (int)rank * rows;
+  const uint32_t mine = (uint32_t)__cvta_generic_to_shared(sm);
+  for (int e = tid; e < rows * BN; e += 128) {
+    const int r = r0 + e / BN, c = e % BN;
+    const int m = m0 + r, nc = n0 + c;
+    if (m >= d.M || nc >= d.N) continue;
+    float v = 0.f;
+    for (uint32_t p = 0; p < splits; ++p) {
+      uint32_t at;
+      float x;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(mine + (uint32_t)(r * PC + c) * 4u), "r"(p));
+      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(at));
+      v += x;
     }
+    if (d.bias) v += d.bias[nc];
+    if (d.beta != 0.f) v += d.beta * d.Cm[(int64_t)m * d.scm + nc];
+    if (d.relu) v = fmaxf(v, 0.f);
+    d.Cm[(int64_t)m * d.scm + nc] = v;
+  }
+  if (splits > 1) {
+    // a CTA's shared memory stays until its peers have read it
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
 }
 
 // ---------------------------------------------------------------- head + misc
@@ -1886,12 +1947,31 @@ cudaError_t launch_pool_bwd(const PoolDesc* tab, const int* tstart, int n, int t
   k_pool_bwd<<<total, 256, 0, st>>>(tab, tstart, n);
   return cudaGetLastError();
 }
-cudaError_t launch_gemm(const GemmDesc* tab, const int* tstart, int n, int total, int kmax, cudaStream_t st) {
-  if (total <= 0) return cudaSuccess;
-  // two groups of threads a tile while the tiles do not give every SM two CTAs and K is long enough
-  if (total < 2 * device_sm_count() && kmax >= 256) k_gemm<2><<<total, 512, 0, st>>>(tab, tstart, n);
-  else k_gemm<1><<<total, 256, 0, st>>>(tab, tstart, n);
-  return cudaGetLastError();
+cudaError_t launch_gemm(const GemmDesc* desc, int M, int N, int K, cudaStream_t st) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  // 32 x 16 tiles where a 128 x 64 tile would be mostly padding (a classifier's
+  // few columns)
+  const bool small = M <= 32 || N <= 16;
+  const int BM = small ? 32 : 128, BN = small ? 16 : 64;
+  const int64_t tiles = (int64_t)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+  // CTAs of a tile: while the launch fits the chip at once (four CTAs an SM) and
+  // each keeps at least 128 of K
+  int splits = 1;
+  while (splits < 8 && tiles * splits * 2 <= 4 * (int64_t)device_sm_count() && K / (splits * 2) >= 128) splits *= 2;
+  if (tiles * splits > 0x7fffffff) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(tiles * splits));
+  cfg.blockDim = dim3(128);
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = splits;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = small ? cudaLaunchKernelEx(&cfg, k_gemm<32, 16, 2, 2>, desc)
+                              : cudaLaunchKernelEx(&cfg, k_gemm<128, 64, 8, 8>, desc);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 cudaError_t launch_pack_input(const float* x, void* out, int32_t dt, int B, int C, int H, int W, cudaStream_t st) {
   const int64_t total = (int64_t)B * C * H * W;

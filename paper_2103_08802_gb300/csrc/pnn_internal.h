@@ -189,7 +189,6 @@ struct GemmDesc {
   int64_t sam, sak, sbk, sbn, scm;
   float beta;
   int32_t relu;
-  int32_t mtiles, ntiles;
 };
 
 // ------------------------------------------------------------ launchers
@@ -216,7 +215,8 @@ cudaError_t launch_bnb_apply8(const BnBwdDesc* tab, const int* tstart, int n, in
 cudaError_t launch_pool_fwd(const PoolDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_pool_bwd(const PoolDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 // kmax: the largest K of the launch
-cudaError_t launch_gemm(const GemmDesc* tab, const int* tstart, int n, int total_tiles, int kmax, cudaStream_t st);
+// desc (device memory) of an M x N x K product
+cudaError_t launch_gemm(const GemmDesc* desc, int M, int N, int K, cudaStream_t st);
 // tcgen05 implicit-GEMM convolution (bf16 operands, fp32 accumulate in TMEM);
 // instances need C % 8 == 0; bnmax = largest N tile (multiple of 16, <= 256)
 // (max_ctas > 0 caps the persistent grid below the SM count, leaving SMs to

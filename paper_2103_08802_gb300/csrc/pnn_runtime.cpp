@@ -722,7 +722,6 @@ struct pnn_net {
   }
   // head GEMM tables: per FC layer l: forward, dW, dIn descriptors
   std::vector<size_t> head_fwd_tab, head_dw_tab, head_din_tab;
-  size_t head_tstart = 0;
   void build_head_tables();
   int run_head_fwd();
   int run_head_bwd(int opid);
@@ -1801,7 +1800,6 @@ void pnn_net::build_head_tables() {
   float* master = P<float>(off_master);
   float* grad = P<float>(off_grad);
   head_fwd_tab.clear(); head_dw_tab.clear(); head_din_tab.clear();
-  int ts[2];
   for (int l = 0; l < nfc; ++l) {
     const int wi = fc_width[l], wo = fc_width[l + 1];
     GemmDesc f{};  // feat[l+1][b][o] = sum_i feat[l][b][i] W[o][i] + bias[o]
@@ -1810,37 +1808,30 @@ void pnn_net::build_head_tables() {
     f.Cm = P<float>(feat[l + 1]); f.scm = wo;
     f.bias = master + params[fc_b[l]].off;
     f.M = B; f.N = wo; f.K = wi; f.relu = l + 1 < nfc;
-    f.mtiles = cdiv(B, 64); f.ntiles = cdiv(wo, 64);
     head_fwd_tab.push_back(put_table(&f, sizeof f));
     GemmDesc g{};  // dW[o][i] = sum_b dfeat[l+1][b][o] feat[l][b][i]
     g.A = P<float>(dfeat[l + 1]); g.sam = 1; g.sak = wo;
     g.Bm = P<float>(feat[l]); g.sbk = wi; g.sbn = 1;
     g.Cm = grad + params[fc_w[l]].off; g.scm = wi;
     g.M = wo; g.N = wi; g.K = B;
-    g.mtiles = cdiv(wo, 64); g.ntiles = cdiv(wi, 64);
     head_dw_tab.push_back(put_table(&g, sizeof g));
     GemmDesc h{};  // dfeat[l][b][i] = sum_o dfeat[l+1][b][o] W[o][i]
     h.A = P<float>(dfeat[l + 1]); h.sam = wo; h.sak = 1;
     h.Bm = master + params[fc_w[l]].off; h.sbk = wi; h.sbn = 1;
     h.Cm = P<float>(dfeat[l]); h.scm = wi;
     h.M = B; h.N = wi; h.K = wo;
-    h.mtiles = cdiv(B, 64); h.ntiles = cdiv(wi, 64);
     head_din_tab.push_back(put_table(&h, sizeof h));
   }
-  ts[0] = 0; ts[1] = 1 << 30;
-  head_tstart = put_table(ts, sizeof ts);
 }
 
 int pnn_net::run_head_fwd() {
   const int nfc = (int)fc_width.size() - 1;
   const Value& hv = vals[head_in];
   const char* tb = ws + tables_off;
-  const int* tst = reinterpret_cast<const int*>(tb + head_tstart);
   cudaError_t e = launch_gap(make_src(*this, head_in), P<float>(feat[0]), B, hv.H * hv.W, hv.C, stream);
   for (int l = 0; l < nfc && e == cudaSuccess; ++l) {
     const int wi = fc_width[l], wo = fc_width[l + 1];
-    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_fwd_tab[l]), tst, 1, cdiv(B, 64) * cdiv(wo, 64), wi,
-                    stream);
+    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_fwd_tab[l]), B, wo, wi, stream);
   }
   if (e == cudaSuccess && !opt.inference)
     e = launch_softmax_ce(P<float>(feat[nfc]), labels_dev, B, classes, P<float>(loss_off), P<float>(dfeat[nfc]),
@@ -1851,17 +1842,14 @@ int pnn_net::run_head_fwd() {
 int pnn_net::run_head_bwd(int opid) {
   const int nfc = (int)fc_width.size() - 1;
   const char* tb = ws + tables_off;
-  const int* tst = reinterpret_cast<const int*>(tb + head_tstart);
   float* grad = P<float>(off_grad);
   cudaError_t e = cudaSuccess;
   for (int l = nfc - 1; l >= 0 && e == cudaSuccess; --l) {
     const int wi = fc_width[l], wo = fc_width[l + 1];
-    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_dw_tab[l]), tst, 1, cdiv(wo, 64) * cdiv(wi, 64), B,
-                    stream);
+    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_dw_tab[l]), wo, wi, B, stream);
     if (e == cudaSuccess) e = launch_colsum(P<float>(dfeat[l + 1]), B, wo, grad + params[fc_b[l]].off, stream);
     if (e == cudaSuccess)
-      e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_din_tab[l]), tst, 1, cdiv(B, 64) * cdiv(wi, 64), wo,
-                      stream);
+      e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_din_tab[l]), B, wi, wo, stream);
     if (e == cudaSuccess && l > 0) e = launch_relu_mask(P<float>(dfeat[l]), P<float>(feat[l]), (int64_t)B * wi, stream);
   }
   const Value& hv = vals[head_in];

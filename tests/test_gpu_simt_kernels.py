@@ -33,6 +33,9 @@ NETS = {
     "seven_in": _net("seven_in", 5, 7, 12, 8, [C(40, k=1)], [C(64, stride=2), C(65)], hidden=(300,)),
     "seven_in_3x3": _net("seven_in_3x3", 2, 7, 8, 8, [C(12)], [C(16), C(32, pool=2)]),
     "three_in_64": _net("three_in_64", 9, 3, 20, 20, [C(64)], [C(16, k=1)]),
+    # the head's K over the CTAs of a cluster (1030: a short last share), ragged tiles
+    "wide_head": _net("wide_head", 33, 3, 8, 8, [C(16)], [C(32, k=1)], hidden=(1030, 517)),
+    "wide_head_130": _net("wide_head_130", 130, 3, 4, 4, [C(16)], [C(260, k=1)], hidden=(640,), classes=17),
     "one_image": W.tiny_resnet(batch=1),
     "torn": W.tiny_resnet(batch=5),
     "torn_delta": W.tiny_resnet(batch=3, correction="delta"),
