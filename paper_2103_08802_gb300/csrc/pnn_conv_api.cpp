@@ -258,7 +258,7 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
       ip.bn = g.bn_mean != nullptr;
       if (ip.bn) {
         // the fused sums use 128-row tiles; the separate reduction its own
-        ip.stat_tiles = std::max(ip.mtiles, cdv(Min, bnb_rows_per_tile(g.c)));
+        ip.stat_tiles = std::max(ip.mtiles, cdv(Min, bnb_rows_per_tile(g.c, Min)));
         ip.gam = take((size_t)g.c * 4);
       }
       pl.total += ip.mtiles * ip.ntiles;
@@ -542,7 +542,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       b.dgamma = g.dgamma; b.dbeta = g.dbeta;
       b.coef = reinterpret_cast<float*>(ws + ip.coef);
       b.M = Min; b.C = g.c;
-      b.rows_per_tile = bnb_rows_per_tile(g.c);
+      b.rows_per_tile = bnb_rows_per_tile(g.c, Min);
       b.inv_count = 1.0 / (double)Min;
       // the TMA-fed data gradient forms the sums of its 128-row tiles in its
       // epilogue when it writes the whole gradient; otherwise the separate
@@ -553,7 +553,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
         b.tiles = ip.mtiles;
       } else {
         if (g.c % 8 != 0 || g.c > 2048) return set_last_error(PNN_EINVAL, "pnn_conv_run: BN sums need c % 8 == 0");
-        b.tiles = cdv(Min, bnb_rows_per_tile(g.c));
+        b.tiles = cdv(Min, bnb_rows_per_tile(g.c, Min));
         breds.push_back(b);
         red_ts.push_back(red_ts.back() + b.tiles);
       }

@@ -534,9 +534,18 @@ int encode_c3_maps(void* maps, bool fwd, const void* a, bool a_bf16, int ch, voi
 int encode_tensor_map_2d(void* map, const void* base, bool bf16, int64_t inner, int64_t rows, int box_inner,
                          int box_rows, int swz, const char** why);
 
-constexpr int kBnbRowsPerTile = 256;  // BN backward reduce/apply tiles: at least this many rows
-// rows of a BN-backward tile for C channels: about 32K elements a CTA
-inline int bnb_rows_per_tile(int C) { return C > 0 && 32768 / C > kBnbRowsPerTile ? 32768 / C : kBnbRowsPerTile; }
+constexpr int kBnbRowsPerTile = 256;  // BN backward reduce/apply tiles: at most this many rows of a wide layer
+// rows of a BN-backward tile of M rows x C channels: about 32K elements a CTA; a
+// layer with few rows gets 16 tiles, of at least 2K elements (a batch of 8 at 32 x
+// 32 x 16 had 4 tiles, the 512 x 512 gradient of VGG-16's last layer 2).  More do
+// not pay: a launch holds several instances, and every CTA loads seven parameters a
+// channel (two tiles an SM for each instance: ResNet-1001 with 4 subnetworks 26.6 ->
+// 28.8 ms; 32 tiles: 26.5 -> 26.7).
+inline int bnb_rows_per_tile(int C, int64_t M) {
+  int rows = C > 0 && 32768 / C > kBnbRowsPerTile ? 32768 / C : kBnbRowsPerTile;
+  while (rows > 8 && (int64_t)rows * C > 2048 && M < 16 * (int64_t)rows) rows /= 2;
+  return rows;
+}
 // The TMA-fed weight gradient loads a k-step's activation rows for all taps
 // as one halo box and the output-gradient rows as another: channels 8..64
 // (dividing 64) or multiples of 128 up to 512, at most 128 output channels

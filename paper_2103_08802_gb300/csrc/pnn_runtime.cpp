@@ -646,7 +646,7 @@ struct pnn_net {
         POp r;
         r.kind = K_BNB_RED; r.norm = f.norm; r.in = vv;
         r.variant = (n.C % 8 == 0 && n.C <= 2048) ? 1 : 0;  // 1: 8 channels per thread
-        r.tiles = cdiv(n.count, bnb_rows_per_tile(n.C));
+        r.tiles = cdiv(n.count, bnb_rows_per_tile(n.C, n.count));
         key(r, 0);
         // The reduction is fused into the data gradient that wrote the whole
         // gradient of the BN(+ReLU) value (TMA-fed, stored, sole writer): its
@@ -669,7 +669,7 @@ struct pnn_net {
         new_op(L, fi);
         POp ap = r;
         ap.kind = K_BNB_APPLY;
-        ap.tiles = cdiv(n.count, bnb_rows_per_tile(n.C));
+        ap.tiles = cdiv(n.count, bnb_rows_per_tile(n.C, n.count));
         if (vals[n.h].need_grad) {
           ap.acc = grad_acc(n.h);
           ap.out = n.h;
@@ -1207,7 +1207,7 @@ int pnn_net::plan(const pnn_desc* d) {
     n.mean = alloc(n.C * 4); n.rstd = alloc(n.C * 4); n.scale = alloc(n.C * 4); n.shift = alloc(n.C * 4);
     n.run = off_running + run_at[n.gamma] * 4;
     if (opt.inference) continue;
-    n.btiles = cdiv(n.count, bnb_rows_per_tile(n.C));
+    n.btiles = cdiv(n.count, bnb_rows_per_tile(n.C, n.count));
     // room for the reduce kernel's tiles or a fused data gradient's 128-row tiles
     const int bt = std::max(n.btiles, cdiv(n.count, kTcBM));
     n.bpart = alloc((size_t)bt * n.C * 8);
@@ -1602,7 +1602,7 @@ int pnn_net::build_tables() {
             b.dgamma = grad + params[n.gamma].off; b.dbeta = grad + params[n.beta].off;
             b.coef = P<float>(n.coef);
             b.M = n.count; b.C = n.C;
-            b.rows_per_tile = bnb_rows_per_tile(n.C); b.tiles = n.fused_tiles ? n.fused_tiles : n.btiles;
+            b.rows_per_tile = bnb_rows_per_tile(n.C, n.count); b.tiles = n.fused_tiles ? n.fused_tiles : n.btiles;
             b.inv_count = 1.0 / (double)n.count;
             if (o.kind == K_BNB_FIN) b.accumulate = o.acc_in[0];
             if (o.kind == K_BNB_APPLY) {
