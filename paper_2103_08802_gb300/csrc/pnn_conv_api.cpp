@@ -173,7 +173,24 @@ bool halo_inst(int mode, const pnn_conv_args& g) {
   return halo_ok(g.ksize, g.stride, g.ksize / 2, g.h, g.w, ch) && conv_halo_fits(mode, g.w, ch, bn);
 }
 
-int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
+// Whether the caller's pointers suit k_pw_conv.cu, k_c3_conv.cu and k_wg_conv.cu:
+// tensor maps want 16 bytes, the pairwise reads of the per-channel values 8.  (The
+// other kernels read those one at a time; slices at an odd offset stay with them.)
+bool narrow_pointers(int n, const pnn_conv_args* a) {
+  auto on = [](const void* p, uintptr_t bytes) { return reinterpret_cast<uintptr_t>(p) % bytes == 0; };
+  for (int i = 0; i < n; ++i) {
+    const pnn_conv_args& g = a[i];
+    for (const void* p : {(const void*)g.x, (const void*)g.wt, (const void*)g.y, (const void*)g.res, (const void*)g.dy,
+                          (const void*)g.dx})
+      if (!on(p, 16)) return false;
+    for (const void* p : {(const void*)g.bn_scale, (const void*)g.bn_shift, (const void*)g.bn_mean, (const void*)g.bn_rstd})
+      if (!on(p, 8)) return false;
+  }
+  return true;
+}
+
+// narrow: the kernels of k_pw_conv.cu, k_c3_conv.cu and k_wg_conv.cu may be chosen
+int make_plan(int mode, int impl, int n, const pnn_conv_args* a, bool narrow, Plan& pl) {
   int r = check_args(mode, impl, n, a);
   if (r) return r;
   // (an instance with halo tiles needs no per-tap boxes)
@@ -190,14 +207,14 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
   if (mode == 0)
     for (int i = 0; i < n; ++i) auto_tma = auto_tma && ((a[i].k >= 64 && tma_ok(mode, a[i])) || halo_inst(mode, a[i]));
   pl.variant = (impl == 1 || impl == 3) ? 1 : (impl == 2 ? 0 : (auto_tma ? 1 : 0));
-  bool all_pw = impl == 0;
+  bool all_pw = impl == 0 && narrow;
   int64_t mtiles = 0;
   for (int i = 0; i < n; ++i) {
     all_pw = all_pw && pw_inst(mode, a[i]);
     mtiles += cdv((int64_t)a[i].batch * a[i].h * a[i].w, kTcBM);  // (stride 1)
   }
   // the weight gradients of k_wg_conv.cu: one kernel size a launch
-  bool all_wg = impl == 0 && mode == 2;
+  bool all_wg = impl == 0 && narrow && mode == 2;
   double wg_bytes = 0;
   auto wg_traffic = [](const pnn_conv_args& g) {
     return (double)g.batch * g.h * g.w * (g.c * (g.x_dtype == PNN_DT_BF16 ? 2 : 4) + g.k * 4.0);
@@ -207,7 +224,7 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, Plan& pl) {
              wg_ok(a[i].ksize, a[i].stride, a[i].c, a[i].k, a[i].h, a[i].w, a[i].x_dtype == PNN_DT_BF16);
     wg_bytes += wg_traffic(a[i]);
   }
-  bool all_c3 = impl == 0;
+  bool all_c3 = impl == 0 && narrow;
   for (int i = 0; i < n; ++i) all_c3 = all_c3 && c3_inst(mode, a[i]);
   if (all_pw || all_wg) pl.variant = 4;
   if (all_c3) pl.variant = 5;
@@ -366,10 +383,12 @@ using namespace pnn;
 
 extern "C" int pnn_conv_workspace_bytes(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* args, size_t* bytes) {
   if (!bytes) return set_last_error(PNN_EINVAL, "pnn_conv_workspace_bytes: null output");
-  Plan pl;
-  const int r = make_plan(mode, impl, n, args, pl);
+  // enough for either choice, so that the answer does not depend on the pointers' alignment
+  Plan narrow, other;
+  int r = make_plan(mode, impl, n, args, true, narrow);
+  if (!r) r = make_plan(mode, impl, n, args, false, other);
   if (r) return r;
-  *bytes = pl.bytes;
+  *bytes = std::max(narrow.bytes, other.bytes);
   return PNN_OK;
 }
 
@@ -377,7 +396,8 @@ namespace {
 int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void* workspace, size_t workspace_bytes,
              void* stream, int repeat, float* ms_out) {
   Plan pl;
-  int r = make_plan(mode, impl, n, a, pl);
+  // (a null array is refused by the plan's own checks)
+  int r = make_plan(mode, impl, n, a, a && n > 0 && narrow_pointers(n, a), pl);
   if (r) return r;
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255))
     return set_last_error(PNN_EINVAL, "pnn_conv_run: workspace must be a 256-byte aligned device pointer");

@@ -158,3 +158,32 @@ def test_3x3_forward(monkeypatch, base, kind):
 def test_3x3_data_gradient(monkeypatch, base):
     _install(monkeypatch, base, C3[base])
     K.test_conv_data_gradient(base, "auto")
+
+
+@pytest.mark.parametrize("mode,c,k,ks", [("forward", 16, 64, 1), ("forward", 16, 16, 3), ("wgrad", 16, 64, 1),
+                                         ("wgrad", 16, 16, 3)])
+def test_per_channel_values_at_odd_offsets(mode, c, k, ks):
+    """BN scale and shift may be slices at any float offset: such a call keeps the
+    kernels that read them one at a time, whose result is that of impl "tma"."""
+    import torch
+    from paper_2103_08802_gb300 import pnn
+    torch.manual_seed(5)
+    b, h = 3, 32
+    base = dict(batch=b, h=h, w=h, c=c, k=k, ksize=ks, stride=1, relu=1)
+    base["x"] = torch.randn(b, h, h, c, device="cuda").bfloat16()
+    base["wt"] = torch.randn(k, ks, ks, c, device="cuda").bfloat16()
+    base["dy"] = torch.randn(b, h, h, k, device="cuda")
+    buf = torch.rand(2, c + 1, device="cuda") + 0.5
+    results = []
+    for impl, odd in (("tma", False), ("auto", True)):
+        d = dict(base)
+        for i, name in enumerate(("bn_scale", "bn_shift")):
+            t = torch.empty(c + 1, device="cuda")[1:] if odd else torch.empty(c, device="cuda")
+            t.copy_(buf[i, 1:])
+            assert t.data_ptr() % 8 == (4 if odd else 0)
+            d[name] = t
+        d["y"] = torch.zeros(b, h, h, k, device="cuda", dtype=torch.bfloat16)
+        d["dw"] = torch.zeros(k, ks, ks, c, device="cuda")
+        pnn.conv_run(mode, [d], impl=impl)
+        results.append(d["y"] if mode == "forward" else d["dw"])
+    assert results[0].abs().max() > 0 and torch.equal(results[0], results[1])
