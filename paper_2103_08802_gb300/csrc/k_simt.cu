@@ -874,82 +874,81 @@ struct RowTile {
   }
 };
 
-// Rows are taken kEwBatch at a time, all loads of a batch first: with a store
-// between two rows' loads the kernel waited for memory once a row (100 us for
-// the 512 x 512 sums of VGG-16's last interface; now 91, and 41 -> 21 us for the
-// gradient's).
+// A CTA takes a tile's rows of a slice of 64 channels (fewer: all), so that four
+// or more threads share a channel's rows.  Rows are taken kEwBatch at a time, all
+// loads of a batch first.  (All channels of the rows a CTA and one thread a
+// channel left VGG-16's last interface, 512 x 512, eight CTAs with a chain of 64
+// rows: 98 us,
+// 91 with the batches; 36 now, of which an event-timed launch is about 8.)
 constexpr int kEwBatch = 8;
 __global__ void __launch_bounds__(256) k_ew(const EwDesc* __restrict__ tab, const int* __restrict__ tstart, int n) {
   __shared__ float red[256][2];
   const int inst = find_instance(tstart, n, blockIdx.x);
   const EwDesc& d = tab[inst];
-  const int tile = blockIdx.x - tstart[inst];
   const int C = d.C;
-  const RowTile rt(C, threadIdx.x);
+  int tile = blockIdx.x - tstart[inst], cb = 0;
+  if (C > kEwSlice) {
+    const int slices = ew_slices(C), item = tile;
+    tile = item / slices;
+    cb = (item - tile * slices) * kEwSlice;
+  }
+  const int Cs = min(C - cb, kEwSlice);
+  const int G = 256 / Cs;                                        // row groups
+  const int g = threadIdx.x / Cs, c = cb + threadIdx.x % Cs;     // (g >= G: an idle thread)
   const int64_t r0 = (int64_t)tile * d.rows_per_tile;
   const int64_t r1 = min((int64_t)d.M, r0 + d.rows_per_tile);
   // BN partials of the output: Welford's update over this thread's rows
   // (count, mean, M2), then chan_merge over the row groups in order
-  for (int ci = 0; ci < rt.cpt; ++ci) {
-    const int c = rt.c0 + 256 * ci;
-    float n = 0.f, mean = 0.f, m2 = 0.f;
-    if (c < C) {
-      for (int64_t r = r0 + rt.g; r < r1; r += (int64_t)kEwBatch * rt.G) {
-        float v[kEwBatch];
+  float cnt = 0.f, mean = 0.f, m2 = 0.f;
+  if (g < G) {
+    for (int64_t r = r0 + g; r < r1; r += (int64_t)kEwBatch * G) {
+      float v[kEwBatch];
 #pragma unroll
-        for (int u = 0; u < kEwBatch; ++u) v[u] = 0.f;
-        for (int i = 0; i < d.nin; ++i) {
-          const Src src = d.in[i];
-          float x[kEwBatch];
-#pragma unroll
-          for (int u = 0; u < kEwBatch; ++u) {
-            const int64_t rr = r + (int64_t)u * rt.G;
-            x[u] = rr < r1 ? ld_src(src, rr * C + c, c) : 0.f;
-          }
-#pragma unroll
-          for (int u = 0; u < kEwBatch; ++u) v[u] = fmaf(d.coef[i], x[u], v[u]);
-        }
+      for (int u = 0; u < kEwBatch; ++u) v[u] = 0.f;
+      for (int i = 0; i < d.nin; ++i) {
+        const Src src = d.in[i];
+        float x[kEwBatch];
 #pragma unroll
         for (int u = 0; u < kEwBatch; ++u) {
-          const int64_t rr = r + (int64_t)u * rt.G;
-          if (rr >= r1) break;
-          float y = v[u];
-          if (d.relu) y = fmaxf(y, 0.f);
-          if (d.out) {
-            y = rnd(d.out_dt, y);
-            stv(d.out, d.out_dt, rr * C + c, y);
-          }
-          if (d.stats) {
-            n += 1.f;
-            const float delta = y - mean;
-            mean += delta / n;
-            m2 = fmaf(delta, y - mean, m2);
-          }
+          const int64_t rr = r + (int64_t)u * G;
+          x[u] = rr < r1 ? ld_src(src, rr * C + c, c) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < kEwBatch; ++u) v[u] = fmaf(d.coef[i], x[u], v[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < kEwBatch; ++u) {
+        const int64_t rr = r + (int64_t)u * G;
+        if (rr >= r1) break;
+        float y = v[u];
+        if (d.relu) y = fmaxf(y, 0.f);
+        if (d.out) {
+          y = rnd(d.out_dt, y);
+          stv(d.out, d.out_dt, rr * C + c, y);
+        }
+        if (d.stats) {
+          cnt += 1.f;
+          const float delta = y - mean;
+          mean += delta / cnt;
+          m2 = fmaf(delta, y - mean, m2);
         }
       }
     }
-    if (d.stats) {
-      if (rt.G == 1) {
-        if (c < C) {
-          d.stats[((int64_t)tile * C + c) * 2] = mean;
-          d.stats[((int64_t)tile * C + c) * 2 + 1] = m2;
-        }
-      } else {
-        red[threadIdx.x][0] = mean;
-        red[threadIdx.x][1] = m2;
-        __syncthreads();
-        if ((int)threadIdx.x < C) {
-          float a = 0.f, am = 0.f, a2 = 0.f;
-          for (int g = 0; g < rt.G; ++g) {
-            // rows r0 + g, r0 + g + G, ... below r1
-            const float cg = r1 > r0 + g ? (float)((r1 - r0 - g + rt.G - 1) / rt.G) : 0.f;
-            chan_merge(a, am, a2, cg, red[g * C + threadIdx.x][0], red[g * C + threadIdx.x][1]);
-          }
-          d.stats[((int64_t)tile * C + threadIdx.x) * 2] = am;
-          d.stats[((int64_t)tile * C + threadIdx.x) * 2 + 1] = a2;
-        }
-        __syncthreads();
+  }
+  if (d.stats) {
+    red[threadIdx.x][0] = mean;
+    red[threadIdx.x][1] = m2;
+    __syncthreads();
+    if ((int)threadIdx.x < Cs) {
+      float a = 0.f, am = 0.f, a2 = 0.f;
+      for (int q = 0; q < G; ++q) {
+        // rows r0 + q, r0 + q + G, ... below r1
+        const float cq = r1 > r0 + q ? (float)((r1 - r0 - q + G - 1) / G) : 0.f;
+        chan_merge(a, am, a2, cq, red[q * Cs + threadIdx.x][0], red[q * Cs + threadIdx.x][1]);
       }
+      float* out = d.stats + ((int64_t)tile * C + cb + threadIdx.x) * 2;
+      out[0] = am;
+      out[1] = a2;
     }
   }
 }
@@ -960,8 +959,9 @@ __global__ void __launch_bounds__(256) k_ew_bwd(const EwBwdDesc* __restrict__ ta
   const int inst = find_instance(tstart, n, blockIdx.x);
   const EwBwdDesc& d = tab[inst];
   const int tile = blockIdx.x - tstart[inst];
-  const int64_t base = (int64_t)tile * d.rows_per_tile * d.C;
-  const int64_t end = min((int64_t)d.M * d.C, base + (int64_t)d.rows_per_tile * d.C);
+  const int elems = ew_bwd_elems(d.C);
+  const int64_t base = (int64_t)tile * elems;
+  const int64_t end = min((int64_t)d.M * d.C, base + elems);
   for (int64_t o = base + threadIdx.x; o < end; o += U * 256) {
     float g[U];
 #pragma unroll

@@ -1555,7 +1555,7 @@ int pnn_net::build_tables() {
             if (o.stats_norm >= 0) e.stats = P<float>(norms[o.stats_norm].part);
             e.M = rows(ref); e.C = vals[ref].C;
             e.rows_per_tile = kEwRowsPerTile; e.tiles = o.tiles;
-            add(&e, sizeof e, o.tiles);
+            add(&e, sizeof e, o.tiles * ew_slices(e.C));
             break;
           }
           case K_EW_BWD: {
@@ -1570,8 +1570,7 @@ int pnn_net::build_tables() {
             }
             e.nin = o.nin;
             e.M = rows(o.in); e.C = vals[o.in].C;
-            e.rows_per_tile = kEwRowsPerTile; e.tiles = o.tiles;
-            add(&e, sizeof e, o.tiles);
+            add(&e, sizeof e, cdiv((int64_t)e.M * e.C, ew_bwd_elems(e.C)));
             break;
           }
           case K_BN_FIN: {
