@@ -7,6 +7,17 @@
 // instances (typically the same layer position of all N fine subnetworks,
 // Algorithm 1's parallel loop), each CTA finds its instance from a tile prefix.
 // All reductions run in a fixed order so that results are bit-reproducible.
+//
+// Fixed order: an fp32 network (check mode) further keeps the order of its sums
+// from version to version, whatever the tiles and splits of the kernels are.
+// The last bit of a BN statistic decides whether a pre-activation next to zero
+// passes the ReLU, and one that flips moves the gradients by 1e-5 to 1e-3, far
+// above the 1e-7 of a rounding.  The order: conv and FC outputs one fused
+// multiply-add after another; BN partials over 256, 128 or 64 rows (layers of at
+// most 16, at most 32, more channels) in 16 row groups, or of an elementwise sum
+// over 64 rows in 256 / C; their combination as in tile_moments_fixed; weight
+// gradients over the pixels of a split, BN-backward sums over the rows of tiles of
+// bnb_fixed_rows, average pool and bias gradients over pixels and images.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -85,14 +96,59 @@ struct TapStep {  // contraction index k = (r * S + s) * C + c
 };
 constexpr int kRowOutside = -0x4000;  // a row coordinate no tap brings into an image
 
+// BN partial (mean, M2) of a thread's rows m0 + 16 i < M, i < tm: two passes
+template <typename Get>
+__device__ __forceinline__ float2 row_moments(int tm, int m0, int M, Get v) {
+  int cnt = 0;
+  float s1 = 0.f, m2 = 0.f;
+#pragma unroll
+  for (int i = 0; i < tm; ++i)
+    if (m0 + 16 * i < M) {
+      s1 += v(i);
+      ++cnt;
+    }
+  const float mean = cnt > 0 ? s1 / (float)cnt : 0.f;
+#pragma unroll
+  for (int i = 0; i < tm; ++i)
+    if (m0 + 16 * i < M) m2 = fmaf(v(i) - mean, v(i) - mean, m2);
+  return make_float2(mean, m2);
+}
+// the partial of the rows m0 .. m0 + 16 tm - 1 from its 16 row groups, in order
+template <typename Get>
+__device__ __forceinline__ void merge_row_groups(int tm, int m0, int M, Get red, float* out) {
+  float n = 0.f, mean = 0.f, m2 = 0.f;
+  for (int r = 0; r < 16; ++r) {
+    int cr = 0;
+    for (int i = 0; i < tm; ++i) cr += m0 + r + 16 * i < M ? 1 : 0;
+    const float2 v = red(r);
+    chan_merge(n, mean, m2, (float)cr, v.x, v.y);
+  }
+  out[0] = mean;
+  out[1] = m2;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// *p of CTA `rank` of the cluster (p: this CTA's shared memory)
+__device__ __forceinline__ float ld_cluster(const float* p, uint32_t rank) {
+  uint32_t at;
+  float x;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(at));
+  return x;
+}
+
 // Y[m][k] = sum_{r,s,c} act(X)[n, p*st+r-pad, q*st+s-pad, c] * W[k][r][s][c] (+ res[m][k])
-template <int BM, int BN>
-__global__ void __launch_bounds__(256) k_conv_fwd(const ConvDesc* __restrict__ tab,
-                                                  const int* __restrict__ tstart, int n) {
+// CL: CTAs of a cluster, whose rows form one partial of the BN statistics.  (With 256
+// rows a CTA, as the fixed order wants them, a batch of 8 at 32 x 32 occupies 32 SMs.)
+template <int BM, int BN, int CL>
+__device__ __forceinline__ void conv_fwd_body(const ConvDesc* __restrict__ tab, const int* __restrict__ tstart, int n) {
   constexpr int BK = 16, TM = BM / 16, TN = BN / 16;
   __shared__ float As[2][BK][BM + 4];
   __shared__ float Bs[2][BK][BN + 4];
   __shared__ float red[16][BN][2];
+  __shared__ float quad[CL == 1 ? 1 : BM][CL == 1 ? 1 : BN + 1];
   __shared__ int rowp[BM], rowh[BM], roww[BM];  // pixel index of tap (0, 0), its row and column
   const int inst = find_instance(tstart, n, blockIdx.x);
   const ConvDesc d = tab[inst];
@@ -182,16 +238,10 @@ __global__ void __launch_bounds__(256) k_conv_fwd(const ConvDesc* __restrict__ t
     __syncthreads();
     buf ^= 1;
   }
-  // epilogue: residual, store, BN partials (mean, M2) of the stored value:
-  // two passes over each thread's TM rows, then chan_merge over the 16 row
-  // groups in order
-  int cnt = 0;  // rows of this thread inside the layer
-#pragma unroll
-  for (int i = 0; i < TM; ++i) cnt += m0 + ty + 16 * i < M ? 1 : 0;
+  // epilogue: residual, store, BN partials of the stored value
 #pragma unroll
   for (int j = 0; j < TN; ++j) {
     const int co = n0 + tx + 16 * j;
-    float s1 = 0.f;
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
       const int m = m0 + ty + 16 * i;
@@ -204,33 +254,52 @@ __global__ void __launch_bounds__(256) k_conv_fwd(const ConvDesc* __restrict__ t
         v = rnd(d.y_dt, v);
         stv(d.y, d.y_dt, o, v);
         acc[i][j] = v;
-        s1 += v;
       }
     }
-    const float mean = cnt > 0 ? s1 / (float)cnt : 0.f;
-    float m2 = 0.f;
+  }
+  if (!d.stats) return;
+  if (CL == 1) {
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
-      if (m0 + ty + 16 * i < M) m2 = fmaf(acc[i][j] - mean, acc[i][j] - mean, m2);
-    red[ty][tx + 16 * j][0] = mean;
-    red[ty][tx + 16 * j][1] = m2;
-  }
-  if (d.stats) {
-    __syncthreads();
-    for (int nn = tid; nn < BN; nn += 256) {
-      const int co = n0 + nn;
-      if (co < d.K) {
-        float n = 0.f, mean = 0.f, m2 = 0.f;
-        for (int r = 0; r < 16; ++r) {
-          int cr = 0;
-          for (int i = 0; i < TM; ++i) cr += m0 + r + 16 * i < M ? 1 : 0;
-          chan_merge(n, mean, m2, (float)cr, red[r][nn][0], red[r][nn][1]);
-        }
-        d.stats[((int64_t)tm * d.K + co) * 2 + 0] = mean;
-        d.stats[((int64_t)tm * d.K + co) * 2 + 1] = m2;
-      }
+    for (int j = 0; j < TN; ++j) {
+      const float2 v = row_moments(TM, m0 + ty, M, [&](int i) { return acc[i][j]; });
+      red[ty][tx + 16 * j][0] = v.x;
+      red[ty][tx + 16 * j][1] = v.y;
     }
+    __syncthreads();
+    for (int nn = tid; nn < BN; nn += 256)
+      if (n0 + nn < d.K)
+        merge_row_groups(TM, m0, M, [&](int r) { return make_float2(red[r][nn][0], red[r][nn][1]); },
+                         d.stats + ((int64_t)tm * d.K + n0 + nn) * 2);
+  } else {
+    // the cluster's first CTA reads the others' rows
+    static_assert(CL == 1 || BN == 16, "a column a thread");
+#pragma unroll
+    for (int i = 0; i < TM; ++i) quad[CL == 1 ? 0 : ty + 16 * i][CL == 1 ? 0 : tx] = acc[i][0];
+    cluster_sync();
+    if (tm % CL == 0) {
+      float v[TM * CL];
+#pragma unroll
+      for (int i = 0; i < TM * CL; ++i)
+        v[i] = i < TM ? acc[i % TM][0] : ld_cluster(&quad[CL == 1 ? 0 : ty + 16 * (i % TM)][CL == 1 ? 0 : tx], i / TM);
+      const float2 s = row_moments(TM * CL, m0 + ty, M, [&](int i) { return v[i]; });
+      red[ty][tx][0] = s.x;
+      red[ty][tx][1] = s.y;
+      __syncthreads();
+      if (tid < BN && n0 + tid < d.K)
+        merge_row_groups(TM * CL, m0, M, [&](int r) { return make_float2(red[r][tid][0], red[r][tid][1]); },
+                         d.stats + ((int64_t)(tm / CL) * d.K + n0 + tid) * 2);
+    }
+    cluster_sync();  // a CTA's shared memory stays until it has been read
   }
+}
+template <int BM, int BN>
+__global__ void __launch_bounds__(256) k_conv_fwd(const ConvDesc* __restrict__ tab,
+                                                  const int* __restrict__ tstart, int n) {
+  conv_fwd_body<BM, BN, 1>(tab, tstart, n);
+}
+__global__ void __cluster_dims__(kQuad, 1, 1) __launch_bounds__(256)
+    k_conv_fwd_quad(const ConvDesc* __restrict__ tab, const int* __restrict__ tstart, int n) {
+  conv_fwd_body<64, 16, kQuad>(tab, tstart, n);
 }
 
 // ---------------------------------------------------------------- conv dgrad
@@ -754,7 +823,19 @@ __global__ void __launch_bounds__(256) k_conv_fwd_few(const ConvDesc* __restrict
     const int r = e / BN, j = e % BN;
     if (n0 + j < d.K) stv(d.y, d.y_dt, (int64_t)(m0 + r) * d.K + n0 + j, st[r][j]);
   }
-  if (d.stats) {
+  if (d.stats && d.stat_rows) {
+    // partials of stat_rows rows in 16 row groups, as k_conv_fwd forms them
+    __shared__ float2 red[16][BN];
+    const int j = tid % BN, ty = tid / BN, tmr = d.stat_rows / 16;
+    for (int r0 = 0; r0 < rows; r0 += d.stat_rows) {
+      red[ty][j] = row_moments(tmr, m0 + r0 + ty, M, [&](int i) { return st[r0 + ty + 16 * i][j]; });
+      __syncthreads();
+      if (tid < BN && n0 + tid < d.K)
+        merge_row_groups(tmr, m0 + r0, M, [&](int r) { return red[r][tid]; },
+                         d.stats + ((int64_t)((m0 + r0) / d.stat_rows) * d.K + n0 + tid) * 2);
+      __syncthreads();
+    }
+  } else if (d.stats) {
     // warp w: columns 2 w and 2 w + 1; lane l: rows l, l + 32, ...
     const int lane = tid & 31, warp = tid >> 5;
 #pragma unroll
@@ -893,7 +974,7 @@ __global__ void __launch_bounds__(256) k_ew(const EwDesc* __restrict__ tab, cons
     cb = (item - tile * slices) * kEwSlice;
   }
   const int Cs = min(C - cb, kEwSlice);
-  const int G = 256 / Cs;                                        // row groups
+  const int G = d.groups ? d.groups : 256 / Cs;                  // row groups
   const int g = threadIdx.x / Cs, c = cb + threadIdx.x % Cs;     // (g >= G: an idle thread)
   const int64_t r0 = (int64_t)tile * d.rows_per_tile;
   const int64_t r1 = min((int64_t)d.M, r0 + d.rows_per_tile);
@@ -1088,6 +1169,60 @@ __device__ __forceinline__ void tile_sums(const float* __restrict__ part, int C,
   }
 }
 
+// The moments in the fixed order of an fp32 network (see the top): eight tiles of a
+// chunk of 64, w + 8 k, in fp32; the chunk's eight sums in order; the chunks w,
+// w + 8, ... and then the eight sums of chunks, all in fp64.  Tile lane l of a CTA is
+// sum l & 7 of chunk l >> 3 of the 512 tiles of a round.
+__device__ __forceinline__ void tile_moments_fixed(const float* __restrict__ part, int C, int tiles, int64_t M, int rpt,
+                                                   int cg, double& s1, double& s2, float& K) {
+  constexpr int Q = 2 * kFinChannels;
+  __shared__ double red[kFinLanes][Q + 1];
+  __shared__ double tot[8][Q];
+  const int tid = threadIdx.x, ch = tid % kFinChannels, l = tid / kFinChannels;
+  const int c = cg * kFinChannels + ch;
+  K = c < C && tiles > 0 ? __ldg(part + (int64_t)c * 2) : 0.f;
+  double acc = 0.0;  // thread 16 j + q: quantity q of the chunks j, j + 8, ...
+  for (int t0 = 0; t0 < tiles; t0 += 8 * kFinLanes) {
+    const int b = t0 + (l >> 3) * 64 + (l & 7);
+    float2 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      v[k] = c < C && b + 8 * k < tiles ? __ldg(reinterpret_cast<const float2*>(part) + (int64_t)(b + 8 * k) * C + c)
+                                        : make_float2(0.f, 0.f);
+    float fa = 0.f, fb = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int64_t t = b + 8 * k;
+      if (t < tiles) {
+        const int64_t r1 = (t + 1) * rpt < M ? (t + 1) * rpt : M;
+        const float n = (float)(r1 - t * rpt);
+        const float d = v[k].x - K;
+        const float nd = n * d;
+        fa += nd;
+        fb += v[k].y + nd * d;
+      }
+    }
+    red[l][2 * ch] = fa;
+    red[l][2 * ch + 1] = fb;
+    __syncthreads();
+    if (tid < 8 * Q) {
+      double s = 0.0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) s += red[tid / Q * 8 + w][tid % Q];
+      acc += s;
+    }
+    __syncthreads();
+  }
+  if (tid < 8 * Q) tot[tid / Q][tid % Q] = acc;
+  __syncthreads();
+  s1 = s2 = 0.0;
+  if (tid < kFinChannels)
+    for (int j = 0; j < 8; ++j) {
+      s1 += tot[j][2 * tid];
+      s2 += tot[j][2 * tid + 1];
+    }
+}
+
 // scale and shift of a BN layer from the statistics it normalises with
 __device__ __forceinline__ void bn_affine(const BnFinDesc& d, int c, float gamma, float beta, float mean, float var) {
   const float rstd = 1.f / sqrtf(var + 1e-5f);
@@ -1098,6 +1233,7 @@ __device__ __forceinline__ void bn_affine(const BnFinDesc& d, int c, float gamma
   d.shift[c] = fmaf(-mean, sc, beta);
 }
 
+template <bool FIXED>
 __global__ void __launch_bounds__(kFinThreads) k_bn_fin(const BnFinDesc* __restrict__ tab,
                                                         const int* __restrict__ tstart, int n) {
   const int inst = find_instance(tstart, n, blockIdx.x);
@@ -1114,7 +1250,8 @@ __global__ void __launch_bounds__(kFinThreads) k_bn_fin(const BnFinDesc* __restr
   }
   double s1, s2;
   float K;
-  tile_sums<true>(d.part, d.C, d.tiles, d.count, d.rows_per_tile, cg, s1, s2, K);
+  if (FIXED) tile_moments_fixed(d.part, d.C, d.tiles, d.count, d.rows_per_tile, cg, s1, s2, K);
+  else tile_sums<true>(d.part, d.C, d.tiles, d.count, d.rows_per_tile, cg, s1, s2, K);
   if (!fin) return;
   // (1 / count comes from the host: no fp64 division here; from the moments on
   // fp32 holds every quantity to 2^-24)
@@ -1126,8 +1263,8 @@ __global__ void __launch_bounds__(kFinThreads) k_bn_fin(const BnFinDesc* __restr
     // running statistics follow the batch mean and the unbiased variance
     const float m = d.momentum;
     const float unbiased = d.count > 1 ? var * ((float)d.count / (float)(d.count - 1)) : var;
-    d.run_mean[c] = (1.f - m) * rm + m * mean;
-    d.run_var[c] = (1.f - m) * rv + m * unbiased;
+    d.run_mean[c] = fmaf(m, mean, (1.f - m) * rm);
+    d.run_var[c] = fmaf(m, unbiased, (1.f - m) * rv);
   }
   bn_affine(d, c, gamma, beta, mean, var);
 }
@@ -1255,6 +1392,10 @@ __device__ __forceinline__ void ld8any(const void* base, int dt, int64_t i, floa
   }
 }
 
+// U rows of a thread in flight: 8 in an fp32 network, whose tiles are the tall ones of
+// bnb_fixed_rows (16 rows a thread at 16 channels), and 1 where the tiles are cut to
+// fill the SMs.
+template <int U>
 __global__ void __launch_bounds__(256) k_bnb_reduce8(const BnBwdDesc* __restrict__ tab,
                                                      const int* __restrict__ tstart, int n) {
   __shared__ float red[16][256];  // [quantity x channel][thread]: a warp touches 32 consecutive words
@@ -1276,16 +1417,24 @@ __global__ void __launch_bounds__(256) k_bnb_reduce8(const BnBwdDesc* __restrict
     for (int k = 0; k < 8; ++k) {
       mean[k] = d.mean[c0 + k]; rstd[k] = d.rstd[c0 + k]; sc[k] = d.scale[c0 + k]; sh[k] = d.shift[c0 + k];
     }
-    for (int64_t r = r0 + g; r < r1; r += G) {
-      const int64_t o = r * C + c0;
-      float h[8], dz[8];
-      ld8any(d.h, d.h_dt, o, h);
-      ld8f(d.da + o, dz);
+    for (int64_t r = r0 + g; r < r1; r += U * G) {
+      float h[U][8], dz[U][8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        if (d.relu && !(fmaf(sc[k], h[k], sh[k]) > 0.f)) dz[k] = 0.f;
-        s1[k] += dz[k];
-        s2[k] += dz[k] * ((h[k] - mean[k]) * rstd[k]);
+      for (int u = 0; u < U; ++u) {
+        if (u && r + u * G >= r1) break;
+        const int64_t o = (r + u * G) * C + c0;
+        ld8any(d.h, d.h_dt, o, h[u]);
+        ld8f(d.da + o, dz[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (u && r + u * G >= r1) break;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          if (d.relu && !(fmaf(sc[k], h[u][k], sh[k]) > 0.f)) dz[u][k] = 0.f;
+          s1[k] += dz[u][k];
+          s2[k] += dz[u][k] * ((h[u][k] - mean[k]) * rstd[k]);
+        }
       }
     }
   }
@@ -1619,26 +1768,15 @@ __global__ void __launch_bounds__(128, 4) k_gemm(const GemmDesc* __restrict__ de
 #pragma unroll
     for (int j = 0; j < TN; j += 2) *reinterpret_cast<uint64_t*>(sm + row(i) * PC + col(j)) = acc[i][j / 2];
   // every CTA of the cluster has left its sums; no one returns before this
-  if (splits > 1) {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  } else {
-    __syncthreads();
-  }
+  if (splits > 1) cluster_sync();
+  else __syncthreads();
   const int rows = BM / (int)splits, r0 = (int)rank * rows;
-  const uint32_t mine = (uint32_t)__cvta_generic_to_shared(sm);
   for (int e = tid; e < rows * BN; e += 128) {
     const int r = r0 + e / BN, c = e % BN;
     const int m = m0 + r, nc = n0 + c;
     if (m >= d.M || nc >= d.N) continue;
     float v = 0.f;
-    for (uint32_t p = 0; p < splits; ++p) {
-      uint32_t at;
-      float x;
-      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(mine + (uint32_t)(r * PC + c) * 4u), "r"(p));
-      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(at));
-      v += x;
-    }
+    for (uint32_t p = 0; p < splits; ++p) v += ld_cluster(sm + r * PC + c, p);
     if (d.bias) v += d.bias[nc];
     if (d.beta != 0.f) v += d.beta * d.Cm[(int64_t)m * d.scm + nc];
     if (d.relu) v = fmaxf(v, 0.f);
@@ -1647,8 +1785,7 @@ __global__ void __launch_bounds__(128, 4) k_gemm(const GemmDesc* __restrict__ de
   if (splits > 1) {
     // a CTA's shared memory stays until its peers have read it
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_sync();
   }
 }
 
@@ -1682,6 +1819,51 @@ __global__ void __launch_bounds__(256) k_gap(Src x, float* feat, int B, int HW, 
     for (int i = 1; i < 8; ++i) t += red[i][lane];
     feat[b * C + c] = t / (float)HW;
   }
+}
+
+// Sums over the rows of a group of HW, one after another (fp32 networks: average pool,
+// bias gradients): out[b][c] = sum of x[b HW + k][c] / div.  32 columns a CTA; all
+// warps bring 256 rows at a time to shared memory, the next ones in registers while one
+// warp adds.  (One thread per sum with a load a row: 149 us for eight 32 x 32 x 16
+// images.)
+__global__ void __launch_bounds__(256) k_rowsum_fixed(Src x, float* out, int HW, int C, float div) {
+  constexpr int R = 256, U = R / 8;
+  __shared__ float tile[R][32];
+  const int groups = (C + 31) / 32;
+  const int b = blockIdx.x / groups, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = (blockIdx.x - b * groups) * 32 + lane;
+  float v[U], s = 0.f;
+  const float* p = static_cast<const float*>(x.ptr) + (int64_t)b * HW * C + c;  // (fp32 networks: DT_F32)
+  const bool bn = c < C && x.scale != nullptr;
+  const float sc = bn ? __ldg(x.scale + c) : 1.f, sf = bn ? __ldg(x.shift + c) : 0.f;
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = k0 + warp + 8 * u;
+      v[u] = c < C && k < HW ? __ldg(p + (int64_t)k * C) : 0.f;
+    }
+  };
+  load(0);
+  for (int k0 = 0; k0 < HW; k0 += R) {
+    __syncthreads();  // the previous rows have been added
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      float y = v[u];
+      if (bn) {
+        y = fmaf(sc, y, sf);
+        if (x.relu) y = fmaxf(y, 0.f);
+      }
+      tile[warp + 8 * u][lane] = y;
+    }
+    __syncthreads();
+    if (k0 + R < HW) load(k0 + R);
+    if (warp == 0) {
+      const int rows = min(R, HW - k0);
+#pragma unroll 16
+      for (int k = 0; k < rows; ++k) s += tile[k][lane];
+    }
+  }
+  if (warp == 0 && c < C) out[(int64_t)b * C + c] = s / div;
 }
 
 __global__ void k_gap_bwd(const float* dfeat, float* dx, int B, int HW, int C) {
@@ -1862,6 +2044,7 @@ cudaError_t launch_conv_fwd_simt(const ConvDesc* tab, const int* tstart, int n, 
   if (variant == 0) k_conv_fwd<64, 64><<<total, 256, 0, st>>>(tab, tstart, n);
   else if (variant == 1) k_conv_fwd<128, 32><<<total, 256, 0, st>>>(tab, tstart, n);
   else if (variant == 2) k_conv_fwd<64, 16><<<total, 256, 0, st>>>(tab, tstart, n);
+  else if (variant == 4) k_conv_fwd_quad<<<total, 256, 0, st>>>(tab, tstart, n);
   else k_conv_fwd_few<<<total, 256, 0, st>>>(tab, tstart, n);
   return cudaGetLastError();
 }
@@ -1903,9 +2086,10 @@ cudaError_t launch_ew_bwd(const EwBwdDesc* tab, const int* tstart, int n, int to
   k_ew_bwd<<<total, 256, 0, st>>>(tab, tstart, n);
   return cudaGetLastError();
 }
-cudaError_t launch_bn_fin(const BnFinDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {
+cudaError_t launch_bn_fin(const BnFinDesc* tab, const int* tstart, int n, int total, int fixed_order, cudaStream_t st) {
   if (total <= 0) return cudaSuccess;
-  k_bn_fin<<<total, kFinThreads, 0, st>>>(tab, tstart, n);
+  if (fixed_order) k_bn_fin<true><<<total, kFinThreads, 0, st>>>(tab, tstart, n);
+  else k_bn_fin<false><<<total, kFinThreads, 0, st>>>(tab, tstart, n);
   return cudaGetLastError();
 }
 cudaError_t launch_bn_eval(const BnFinDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {
@@ -1918,9 +2102,11 @@ cudaError_t launch_bnb_reduce(const BnBwdDesc* tab, const int* tstart, int n, in
   k_bnb_reduce<<<total, 256, 0, st>>>(tab, tstart, n);
   return cudaGetLastError();
 }
-cudaError_t launch_bnb_reduce8(const BnBwdDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {
+cudaError_t launch_bnb_reduce8(const BnBwdDesc* tab, const int* tstart, int n, int total, int fixed_order,
+                               cudaStream_t st) {
   if (total <= 0) return cudaSuccess;
-  k_bnb_reduce8<<<total, 256, 0, st>>>(tab, tstart, n);
+  if (fixed_order) k_bnb_reduce8<8><<<total, 256, 0, st>>>(tab, tstart, n);
+  else k_bnb_reduce8<1><<<total, 256, 0, st>>>(tab, tstart, n);
   return cudaGetLastError();
 }
 cudaError_t launch_bnb_fin(const BnBwdDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {
@@ -1948,17 +2134,21 @@ cudaError_t launch_pool_bwd(const PoolDesc* tab, const int* tstart, int n, int t
   k_pool_bwd<<<total, 256, 0, st>>>(tab, tstart, n);
   return cudaGetLastError();
 }
-cudaError_t launch_gemm(const GemmDesc* desc, int M, int N, int K, cudaStream_t st) {
+cudaError_t launch_gemm(const GemmDesc* desc, int M, int N, int K, int fixed_order, cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   // 32 x 16 tiles where a 128 x 64 tile would be mostly padding (a classifier's
   // few columns)
   const bool small = M <= 32 || N <= 16;
-  const int BM = small ? 32 : 128, BN = small ? 16 : 64;
-  const int64_t tiles = (int64_t)((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+  int BM = small ? 32 : 128, BN = small ? 16 : 64;
+  auto count = [&]() { return (int64_t)((M + BM - 1) / BM) * ((N + BN - 1) / BN); };
+  // a sum of an fp32 network is not split: smaller tiles where the large ones leave SMs idle
+  const bool mid = fixed_order && !small && count() < device_sm_count();
+  if (mid) BM = 64, BN = 32;
+  const int64_t tiles = count();
   // CTAs of a tile: while the launch fits the chip at once (four CTAs an SM) and
   // each keeps at least 128 of K
   int splits = 1;
-  while (splits < 8 && tiles * splits * 2 <= 4 * (int64_t)device_sm_count() && K / (splits * 2) >= 128) splits *= 2;
+  while (!fixed_order && splits < 8 && tiles * splits * 2 <= 4 * (int64_t)device_sm_count() && K / (splits * 2) >= 128) splits *= 2;
   if (tiles * splits > 0x7fffffff) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(tiles * splits));
@@ -1971,6 +2161,7 @@ cudaError_t launch_gemm(const GemmDesc* desc, int M, int N, int K, cudaStream_t 
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   const cudaError_t e = small ? cudaLaunchKernelEx(&cfg, k_gemm<32, 16, 2, 2>, desc)
+                        : mid ? cudaLaunchKernelEx(&cfg, k_gemm<64, 32, 4, 4>, desc)
                               : cudaLaunchKernelEx(&cfg, k_gemm<128, 64, 8, 8>, desc);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1979,8 +2170,9 @@ cudaError_t launch_pack_input(const float* x, void* out, int32_t dt, int B, int 
   k_pack_input<<<cdiv64(total, 256), 256, 0, st>>>(x, out, dt, B, C, H, W);
   return cudaGetLastError();
 }
-cudaError_t launch_gap(Src x, float* feat, int B, int HW, int C, cudaStream_t st) {
-  k_gap<<<B * cdiv64(C, 32), 256, 0, st>>>(x, feat, B, HW, C);
+cudaError_t launch_gap(Src x, float* feat, int B, int HW, int C, int fixed_order, cudaStream_t st) {
+  if (fixed_order) k_rowsum_fixed<<<B * cdiv64(C, 32), 256, 0, st>>>(x, feat, HW, C, (float)HW);
+  else k_gap<<<B * cdiv64(C, 32), 256, 0, st>>>(x, feat, B, HW, C);
   return cudaGetLastError();
 }
 cudaError_t launch_gap_bwd(const float* dfeat, float* dx, int B, int HW, int C, cudaStream_t st) {
@@ -1993,8 +2185,9 @@ cudaError_t launch_softmax_ce(const float* logits, const int32_t* labels, int B,
   k_softmax_ce<<<1, kCeThreads, 0, st>>>(logits, labels, B, m, loss, dlogits, status);
   return cudaGetLastError();
 }
-cudaError_t launch_colsum(const float* A, int rows, int cols, float* out, cudaStream_t st) {
-  k_colsum<<<cdiv64(cols, 32), 256, 0, st>>>(A, rows, cols, out);
+cudaError_t launch_colsum(const float* A, int rows, int cols, float* out, int fixed_order, cudaStream_t st) {
+  if (fixed_order) k_rowsum_fixed<<<cdiv64(cols, 32), 256, 0, st>>>(Src{A, nullptr, nullptr, DT_F32, 0}, out, rows, cols, 1.f);
+  else k_colsum<<<cdiv64(cols, 32), 256, 0, st>>>(A, rows, cols, out);
   return cudaGetLastError();
 }
 cudaError_t launch_relu_mask(float* g, const float* pre, int64_t n, cudaStream_t st) {

@@ -633,10 +633,10 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
     e = launch_wreduce(reinterpret_cast<const WReduceDesc*>(ws + pl.aux_tab), auxts, n, aux_ts.back(), st);
   if (e == cudaSuccess && !fins.empty())
     e = launch_bn_fin(reinterpret_cast<const BnFinDesc*>(ws + pl.fin_tab), reinterpret_cast<const int*>(ws + pl.fin_ts),
-                      (int)fins.size(), fin_ts.back(), st);
+                      (int)fins.size(), fin_ts.back(), 0, st);
   if (e == cudaSuccess && !breds.empty())
     e = launch_bnb_reduce8(reinterpret_cast<const BnBwdDesc*>(ws + pl.red_tab),
-                           reinterpret_cast<const int*>(ws + pl.red_ts), (int)breds.size(), red_ts.back(), st);
+                           reinterpret_cast<const int*>(ws + pl.red_ts), (int)breds.size(), red_ts.back(), 0, st);
   if (e == cudaSuccess && !bfins.empty())
     e = launch_bnb_fin(reinterpret_cast<const BnBwdDesc*>(ws + pl.fin_tab), reinterpret_cast<const int*>(ws + pl.fin_ts),
                        (int)bfins.size(), fin_ts.back(), st);

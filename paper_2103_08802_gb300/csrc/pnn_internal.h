@@ -45,6 +45,7 @@ struct ConvDesc {
   // (r_j = y_j - x_{j+1}, rt_{j+1} = r_{j+1} + F^j(rt_j), ytilde = y_N + rt_N)
   const void* res2[2]; int32_t res2_dt[2]; float res2_c[2];
   float* stats;                       // per-tile BN partials [mtiles][K][2] = (mean, M2) or null
+  int32_t stat_rows;                  // k_conv_fwd_few: rows of a partial (fp32 networks), or 0: the CTA's
   // dgrad: dx[B*H*W][C] (fp32) = (accumulate ? dx : 0) + W^T * dy
   float* dx; int32_t accumulate;
   // dgrad / wgrad operand dy[B*P*Q][K] (fp32)
@@ -95,7 +96,7 @@ struct EwDesc {
   int64_t M;
   int32_t C;
   int32_t rows_per_tile;
-  int32_t tiles;
+  int32_t groups;        // row groups of a channel's partials, or 0: as many as the CTA's threads give
 };
 
 // backward of EW: g = dout * [out > 0 if relu]; grad_i (+)= coef_i * g
@@ -202,20 +203,21 @@ cudaError_t launch_conv_wgrad_simt(const ConvDesc* tab, const int* tstart, int n
 cudaError_t launch_wreduce(const WReduceDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_ew(const EwDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_ew_bwd(const EwBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
-cudaError_t launch_bn_fin(const BnFinDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
+cudaError_t launch_bn_fin(const BnFinDesc* tab, const int* tstart, int n, int total_tiles, int fixed_order,
+                          cudaStream_t st);
 // eval mode: scale and shift from the running statistics (total: CTAs of kFinEvalChannels channels)
 cudaError_t launch_bn_eval(const BnFinDesc* tab, const int* tstart, int n, int total, cudaStream_t st);
 cudaError_t launch_bnb_reduce(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_bnb_fin(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_bnb_apply(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 // 8 channels per thread; every instance needs C % 8 == 0 and C <= 2048
-cudaError_t launch_bnb_reduce8(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
+cudaError_t launch_bnb_reduce8(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, int fixed_order,
+                               cudaStream_t st);
 cudaError_t launch_bnb_apply8(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_pool_fwd(const PoolDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_pool_bwd(const PoolDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
-// kmax: the largest K of the launch
 // desc (device memory) of an M x N x K product
-cudaError_t launch_gemm(const GemmDesc* desc, int M, int N, int K, cudaStream_t st);
+cudaError_t launch_gemm(const GemmDesc* desc, int M, int N, int K, int fixed_order, cudaStream_t st);
 // tcgen05 implicit-GEMM convolution (bf16 operands, fp32 accumulate in TMEM);
 // instances need C % 8 == 0; bnmax = largest N tile (multiple of 16, <= 256)
 // (max_ctas > 0 caps the persistent grid below the SM count, leaving SMs to
@@ -274,11 +276,11 @@ constexpr int kTcBM = 128;
 // single-instance helpers
 cudaError_t launch_pack_input(const float* x_nchw, void* out, int32_t out_dt, int B, int C, int H, int W,
                               cudaStream_t st);
-cudaError_t launch_gap(Src x, float* feat, int B, int HW, int C, cudaStream_t st);
+cudaError_t launch_gap(Src x, float* feat, int B, int HW, int C, int fixed_order, cudaStream_t st);
 cudaError_t launch_gap_bwd(const float* dfeat, float* dx, int B, int HW, int C, cudaStream_t st);
 cudaError_t launch_softmax_ce(const float* logits, const int32_t* labels, int B, int m, float* loss,
                               float* dlogits, int32_t* status, cudaStream_t st);
-cudaError_t launch_colsum(const float* A, int rows, int cols, float* out, cudaStream_t st);
+cudaError_t launch_colsum(const float* A, int rows, int cols, float* out, int fixed_order, cudaStream_t st);
 cudaError_t launch_relu_mask(float* g, const float* pre, int64_t n, cudaStream_t st);
 cudaError_t launch_sgd(float* w, const float* g, float* v, void* shadow, int32_t shadow_dt, int64_t n,
                        float lr, float mu, float wd, int nesterov, int first, cudaStream_t st);
@@ -291,6 +293,8 @@ constexpr int kEwRowsPerTile = 64;
 // channels of a CTA of the elementwise sum, and its CTAs a row tile
 constexpr int kEwSlice = 64;
 PNN_HD inline int ew_slices(int C) { return (C + kEwSlice - 1) / kEwSlice; }
+// row groups of its BN partials in an fp32 network (see "Fixed order", k_simt.cu)
+inline int ew_fixed_groups(int C) { return C <= 256 ? 256 / C : 1; }
 // elements of a CTA of its gradient: 64 rows, of a wide layer fewer (with 64 rows of
 // 512 channels the six launches of a VGG-16 step took 124 us, now 56)
 PNN_HD inline int ew_bwd_elems(int C) { return C < 64 ? kEwRowsPerTile * C : 4096; }
@@ -545,9 +549,11 @@ constexpr int kBnbRowsPerTile = 256;  // BN backward reduce/apply tiles: at most
 // 32 x 16 had 4 tiles, the 512 x 512 gradient of VGG-16's last layer 2).  More do
 // not pay: a launch holds several instances, and every CTA loads seven parameters a
 // channel (two tiles an SM for each instance: ResNet-1001 with 4 subnetworks 26.6 ->
-// 28.8 ms; 32 tiles: 26.5 -> 26.7).
+// 28.8 ms; 32 tiles: 26.5 -> 26.7).  (bnb_fixed_rows: the reduction of an fp32
+// network, see "Fixed order" in k_simt.cu.)
+inline int bnb_fixed_rows(int C) { return C > 0 && 32768 / C > kBnbRowsPerTile ? 32768 / C : kBnbRowsPerTile; }
 inline int bnb_rows_per_tile(int C, int64_t M) {
-  int rows = C > 0 && 32768 / C > kBnbRowsPerTile ? 32768 / C : kBnbRowsPerTile;
+  int rows = bnb_fixed_rows(C);
   while (rows > 8 && (int64_t)rows * C > 2048 && M < 16 * (int64_t)rows) rows /= 2;
   return rows;
 }
@@ -563,22 +569,38 @@ inline bool tma_wgrad_ok(int k, int stride, int pad, int C, int K, int W, bool x
   return b.hrows <= 256 && conv_tma_fits(2, 128, wg_raw_bytes(b));
 }
 // CUDA-core forward and data gradient: 64 x 64, 128 x 32 or 64 x 16 tiles by
-// the GEMM's columns (16: a batch of 8 still gives every SM a tile); variant 3,
-// forward only: at most 32 taps x channels (the 3-channel stem and C^j convs),
-// one thread a pixel.
+// the GEMM's columns (16: a batch of 8 still gives every SM a tile); forward
+// only: variant 3, at most 32 taps x channels (the 3-channel stem and C^j
+// convs), one thread a pixel; variant 4, 64 x 16 tiles of an fp32 network in
+// clusters of four, which form one partial of the BN statistics.
 struct ConvTile { int BM, BN; };
 inline ConvTile simt_tile(int variant) {
-  return variant == 0   ? ConvTile{64, 64}
-         : variant == 1 ? ConvTile{128, 32}
-         : variant == 2 ? ConvTile{64, 16}
-                        : ConvTile{256, 16};
+  return variant == 0                   ? ConvTile{64, 64}
+         : variant == 1                 ? ConvTile{128, 32}
+         : variant == 2 || variant == 4 ? ConvTile{64, 16}
+                                        : ConvTile{256, 16};
 }
 inline int simt_variant(int ncols) { return ncols <= 16 ? 2 : (ncols <= 32 ? 1 : 0); }
-inline int simt_fwd_variant(int k, int C, int K) { return k * k * C <= 32 && C < 8 ? 3 : simt_variant(K); }
+inline int simt_fwd_variant(int k, int C, int K, bool fp32) {
+  const int v = k * k * C <= 32 && C < 8 ? 3 : simt_variant(K);
+  return fp32 && v == 2 ? 4 : v;
+}
+constexpr int kQuad = 4;  // CTAs of a cluster of variant 4
+inline int simt_fwd_mtiles(int variant, int64_t M) {
+  const int bm = simt_tile(variant).BM, group = variant == 4 ? kQuad : 1;
+  return (int)((M + bm * group - 1) / (bm * group)) * group;
+}
+// rows of a partial of the BN statistics: the kernel's tile, or, of an fp32
+// network, fixed by the layer's width ("Fixed order", k_simt.cu)
+inline int simt_stat_rows(int variant, int K, bool fp32) {
+  return !fp32 ? simt_tile(variant).BM : K <= 16 ? 256 : K <= 32 ? 128 : 64;
+}
 // CUDA-core weight gradient: 64 or 16 output channels a tile (0, 1), few input
 // channels with at most 16 (2) or more (3) output channels, 1x1 stride 1 with at
-// most 4 input channels (4)
-inline int simt_wgrad_variant(int k, int stride, int C, int K) {
+// most 4 input channels (4).  An fp32 network takes 0 and 1, which add a split's
+// pixels one after another.
+inline int simt_wgrad_variant(int k, int stride, int C, int K, bool fp32) {
+  if (fp32) return K <= 16 ? 1 : 0;
   if (k == 1 && stride == 1 && C <= 4) return 4;
   return k * k * C <= 32 && C < 8 ? (K <= 16 ? 2 : 3) : (K <= 16 ? 1 : 0);
 }

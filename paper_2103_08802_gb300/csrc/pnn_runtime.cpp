@@ -276,6 +276,10 @@ struct pnn_net {
     vals.push_back(v);
     return (int)vals.size() - 1;
   }
+  // rows of a tile of the separate BN-backward reduction
+  int bnb_reduce_rows(const Norm& n) const {
+    return act_dt == DT_F32 ? bnb_fixed_rows(n.C) : bnb_rows_per_tile(n.C, n.count);
+  }
   int64_t rows(int v) const { return (int64_t)B * vals[v].H * vals[v].W; }
   int new_op(std::vector<int>& list, const POp& op) {
     ops.push_back(op);
@@ -291,7 +295,7 @@ struct pnn_net {
         p.stats_norm = nid;
         norms[nid].tiles = p.tiles;
         norms[nid].stat_rows = p.kind == K_CONV_FWD_TC ? kTcBM
-                               : p.kind == K_CONV_FWD  ? simt_tile(p.variant).BM
+                               : p.kind == K_CONV_FWD  ? simt_stat_rows(p.variant, hv.C, act_dt == DT_F32)
                                                        : kEwRowsPerTile;
         return;
       }
@@ -352,12 +356,12 @@ struct pnn_net {
       c.mtiles = cdiv(M, kTcBM);
       c.ntiles = cdiv(cout, tc_ntile_w(c.kind, c.variant));
     } else {
-      c.variant = simt_fwd_variant(k, iv.C, cout);
-      ConvTile t = simt_tile(c.variant);
-      c.mtiles = cdiv(M, t.BM);
-      c.ntiles = cdiv(cout, t.BN);
+      c.variant = simt_fwd_variant(k, iv.C, cout, act_dt == DT_F32);
+      c.mtiles = simt_fwd_mtiles(c.variant, M);
+      c.ntiles = cdiv(cout, simt_tile(c.variant).BN);
     }
-    c.tiles = c.mtiles;  // stats partial rows
+    // partials of the BN statistics
+    c.tiles = c.kind == K_CONV_FWD_TC ? c.mtiles : cdiv(M, simt_stat_rows(c.variant, cout, act_dt == DT_F32));
     int id = new_op(list, c);
     vals[out].producer = id;
     return out;
@@ -553,7 +557,7 @@ struct pnn_net {
           wg.ntiles = cdiv(ov.C, 256);
           pix_align = 64;
         } else {
-          wg.variant = simt_wgrad_variant(f.k, f.stride, vals[f.in].C, ov.C);
+          wg.variant = simt_wgrad_variant(f.k, f.stride, vals[f.in].C, ov.C, act_dt == DT_F32);
           sm_ctas = simt_wgrad_ctas(wg.variant);
           wg.mtiles = cdiv(ov.C, simt_wgrad_rows(wg.variant));
           wg.ntiles = cdiv(RSC, kWgradBN);
@@ -646,7 +650,7 @@ struct pnn_net {
         POp r;
         r.kind = K_BNB_RED; r.norm = f.norm; r.in = vv;
         r.variant = (n.C % 8 == 0 && n.C <= 2048) ? 1 : 0;  // 1: 8 channels per thread
-        r.tiles = cdiv(n.count, bnb_rows_per_tile(n.C, n.count));
+        r.tiles = cdiv(n.count, bnb_reduce_rows(n));
         key(r, 0);
         // The reduction is fused into the data gradient that wrote the whole
         // gradient of the BN(+ReLU) value (TMA-fed, stored, sole writer): its
@@ -1080,7 +1084,7 @@ int pnn_net::plan(const pnn_desc* d) {
     if (c.kind != K_CONV_FWD_TC || params[c.w].off % 8 == 0) continue;
     c.kind = K_CONV_FWD;
     const int cout = vals[c.out].C;
-    c.variant = simt_fwd_variant(c.k, vals[c.in].C, cout);
+    c.variant = simt_fwd_variant(c.k, vals[c.in].C, cout, false);  // (a bf16 network)
     const ConvTile t = simt_tile(c.variant);
     c.mtiles = cdiv(rows(c.out), t.BM);
     c.ntiles = cdiv(cout, t.BN);
@@ -1207,7 +1211,7 @@ int pnn_net::plan(const pnn_desc* d) {
     n.mean = alloc(n.C * 4); n.rstd = alloc(n.C * 4); n.scale = alloc(n.C * 4); n.shift = alloc(n.C * 4);
     n.run = off_running + run_at[n.gamma] * 4;
     if (opt.inference) continue;
-    n.btiles = cdiv(n.count, bnb_rows_per_tile(n.C, n.count));
+    n.btiles = cdiv(n.count, bnb_reduce_rows(n));
     // room for the reduce kernel's tiles or a fused data gradient's 128-row tiles
     const int bt = std::max(n.btiles, cdiv(n.count, kTcBM));
     n.bpart = alloc((size_t)bt * n.C * 8);
@@ -1504,6 +1508,7 @@ int pnn_net::build_tables() {
                   c.res2_c[e] = o.rcoef[e];
                 }
               if (o.stats_norm >= 0) c.stats = P<float>(norms[o.stats_norm].part);
+              if (act_dt == DT_F32 && o.variant == 3) c.stat_rows = simt_stat_rows(o.variant, ov.C, true);
               add(&c, sizeof c, c.mtiles * c.ntiles);
             } else if (o.kind == K_DGRAD || o.kind == K_DGRAD_TC) {
               c.dy = P<float>(gptr(o.out));
@@ -1554,7 +1559,8 @@ int pnn_net::build_tables() {
             e.relu = o.relu;
             if (o.stats_norm >= 0) e.stats = P<float>(norms[o.stats_norm].part);
             e.M = rows(ref); e.C = vals[ref].C;
-            e.rows_per_tile = kEwRowsPerTile; e.tiles = o.tiles;
+            e.rows_per_tile = kEwRowsPerTile;
+            e.groups = act_dt == DT_F32 ? ew_fixed_groups(e.C) : 0;
             add(&e, sizeof e, o.tiles * ew_slices(e.C));
             break;
           }
@@ -1601,7 +1607,8 @@ int pnn_net::build_tables() {
             b.dgamma = grad + params[n.gamma].off; b.dbeta = grad + params[n.beta].off;
             b.coef = P<float>(n.coef);
             b.M = n.count; b.C = n.C;
-            b.rows_per_tile = bnb_rows_per_tile(n.C, n.count); b.tiles = n.fused_tiles ? n.fused_tiles : n.btiles;
+            b.rows_per_tile = o.kind == K_BNB_RED ? bnb_reduce_rows(n) : bnb_rows_per_tile(n.C, n.count);
+            b.tiles = n.fused_tiles ? n.fused_tiles : n.btiles;
             b.inv_count = 1.0 / (double)n.count;
             if (o.kind == K_BNB_FIN) b.accumulate = o.acc_in[0];
             if (o.kind == K_BNB_APPLY) {
@@ -1827,10 +1834,10 @@ int pnn_net::run_head_fwd() {
   const int nfc = (int)fc_width.size() - 1;
   const Value& hv = vals[head_in];
   const char* tb = ws + tables_off;
-  cudaError_t e = launch_gap(make_src(*this, head_in), P<float>(feat[0]), B, hv.H * hv.W, hv.C, stream);
+  cudaError_t e = launch_gap(make_src(*this, head_in), P<float>(feat[0]), B, hv.H * hv.W, hv.C, act_dt == DT_F32, stream);
   for (int l = 0; l < nfc && e == cudaSuccess; ++l) {
     const int wi = fc_width[l], wo = fc_width[l + 1];
-    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_fwd_tab[l]), B, wo, wi, stream);
+    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_fwd_tab[l]), B, wo, wi, act_dt == DT_F32, stream);
   }
   if (e == cudaSuccess && !opt.inference)
     e = launch_softmax_ce(P<float>(feat[nfc]), labels_dev, B, classes, P<float>(loss_off), P<float>(dfeat[nfc]),
@@ -1842,13 +1849,14 @@ int pnn_net::run_head_bwd(int opid) {
   const int nfc = (int)fc_width.size() - 1;
   const char* tb = ws + tables_off;
   float* grad = P<float>(off_grad);
+  const int fixed = act_dt == DT_F32;
   cudaError_t e = cudaSuccess;
   for (int l = nfc - 1; l >= 0 && e == cudaSuccess; --l) {
     const int wi = fc_width[l], wo = fc_width[l + 1];
-    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_dw_tab[l]), wo, wi, B, stream);
-    if (e == cudaSuccess) e = launch_colsum(P<float>(dfeat[l + 1]), B, wo, grad + params[fc_b[l]].off, stream);
+    e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_dw_tab[l]), wo, wi, B, fixed, stream);
+    if (e == cudaSuccess) e = launch_colsum(P<float>(dfeat[l + 1]), B, wo, grad + params[fc_b[l]].off, fixed, stream);
     if (e == cudaSuccess)
-      e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_din_tab[l]), B, wi, wo, stream);
+      e = launch_gemm(reinterpret_cast<const GemmDesc*>(tb + head_din_tab[l]), B, wi, wo, fixed, stream);
     if (e == cudaSuccess && l > 0) e = launch_relu_mask(P<float>(dfeat[l]), P<float>(feat[l]), (int64_t)B * wi, stream);
   }
   const Value& hv = vals[head_in];
@@ -1926,10 +1934,10 @@ int pnn_net::run_phase(int p, cudaStream_t st, int cap) {
       case K_EW_BWD: e = launch_ew_bwd((const EwBwdDesc*)tab, ts, L.count, L.total, st); break;
       case K_BN_FIN:
         e = opt.inference ? launch_bn_eval((const BnFinDesc*)tab, ts, L.count, L.total, st)
-                          : launch_bn_fin((const BnFinDesc*)tab, ts, L.count, L.total, st);
+                          : launch_bn_fin((const BnFinDesc*)tab, ts, L.count, L.total, act_dt == DT_F32, st);
         break;
       case K_BNB_RED:
-        e = L.variant ? launch_bnb_reduce8((const BnBwdDesc*)tab, ts, L.count, L.total, st)
+        e = L.variant ? launch_bnb_reduce8((const BnBwdDesc*)tab, ts, L.count, L.total, act_dt == DT_F32, st)
                       : launch_bnb_reduce((const BnBwdDesc*)tab, ts, L.count, L.total, st);
         break;
       case K_BNB_FIN: e = launch_bnb_fin((const BnBwdDesc*)tab, ts, L.count, L.total, st); break;
