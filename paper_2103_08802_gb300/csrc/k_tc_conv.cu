@@ -580,7 +580,8 @@ __device__ __forceinline__ void epilogue(const Tile& T, uint32_t tacc, int q, in
         }
       }
       if (tstore) {
-        // the store issued from this buffer two chunks ago must have read it
+        // the store issued from this buffer two chunks ago must have read it: every
+        // chunk commits a group, an empty one where the warp's rows lie past the end
         RT(const unsigned long long cw = clock64();)
         if (leader) bulk_wait_read<1>();
         __syncwarp();
@@ -601,8 +602,8 @@ __device__ __forceinline__ void epilogue(const Tile& T, uint32_t tacc, int q, in
         }
         fence_proxy_async();
         __syncwarp();
-        if (leader && T.m0 + q * 32 < T.Mrows) {
-          tma_store_2d(d.tma_y, nb, T.m0 + q * 32, smem_u32(st));
+        if (leader) {
+          if (T.m0 + q * 32 < T.Mrows) tma_store_2d(d.tma_y, nb, T.m0 + q * 32, smem_u32(st));
           bulk_commit();
         }
         ybuf ^= 1;
@@ -706,7 +707,8 @@ __device__ __forceinline__ void epilogue(const Tile& T, uint32_t tacc, int q, in
           red[q][j0 + (lane >> 1)][1] = b;
         }
       }
-      // staged chunk -> TMA store (fresh gradient) or TMA reduce-add (accumulate)
+      // staged chunk -> TMA store (fresh gradient) or TMA reduce-add (accumulate);
+      // a group every chunk, as in the forward
       RT(const unsigned long long cw = clock64();)
       if (leader) bulk_wait_read<1>();
       __syncwarp();
@@ -724,9 +726,11 @@ __device__ __forceinline__ void epilogue(const Tile& T, uint32_t tacc, int q, in
       }
       fence_proxy_async();
       __syncwarp();
-      if (leader && T.m0 + q * 32 < T.Mrows) {
-        if (d.accumulate) tma_reduce_add_2d(d.tma_y, nb, T.m0 + q * 32, smem_u32(st));
-        else tma_store_2d(d.tma_y, nb, T.m0 + q * 32, smem_u32(st));
+      if (leader) {
+        if (T.m0 + q * 32 < T.Mrows) {
+          if (d.accumulate) tma_reduce_add_2d(d.tma_y, nb, T.m0 + q * 32, smem_u32(st));
+          else tma_store_2d(d.tma_y, nb, T.m0 + q * 32, smem_u32(st));
+        }
         bulk_commit();
       }
       if (sst) {

@@ -249,7 +249,8 @@ __device__ __forceinline__ void unit_dgrad(const EpiArgs& ea, const Dst& dst, ui
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty);
     }
-    // the store issued from this buffer two turns ago must have read it
+    // the store issued from this buffer two turns ago must have read it: every turn
+    // commits a group, an empty one where the warp's rows lie past the layer's end
     if (leader) bulk_wait_read<1>();
     __syncwarp();
     uint8_t* st = stage + sbuf * 4096;
@@ -259,8 +260,8 @@ __device__ __forceinline__ void unit_dgrad(const EpiArgs& ea, const Dst& dst, ui
       *reinterpret_cast<uint4*>(st + swp<HC * 4>(lane, j)) = make_uint4(a[4 * j], a[4 * j + 1], a[4 * j + 2], a[4 * j + 3]);
     fence_proxy_async();
     __syncwarp();
-    if (leader && nvalid > 0) {
-      dst.put(ea.y, n0 + c0, q, smem_u32(st), ea.acc);
+    if (leader) {
+      if (nvalid > 0) dst.put(ea.y, n0 + c0, q, smem_u32(st), ea.acc);
       bulk_commit();
     }
     if (ea.stats) {

@@ -187,3 +187,59 @@ def test_per_channel_values_at_odd_offsets(mode, c, k, ks):
         pnn.conv_run(mode, [d], impl=impl)
         results.append(d["y"] if mode == "forward" else d["dw"])
     assert results[0].abs().max() > 0 and torch.equal(results[0], results[1])
+
+
+def _flat(rows, c, k):
+    return dict(batch=1, h=rows, w=1, c=c, k=k, ksize=1)
+
+
+# layers whose last tile leaves whole warps without rows (rows % 128 in 1 .. 96), after full tiles of the
+# same warps: 64 columns (two staged blocks a unit), and 16 or 32 (one) in groups of more tiles than CTAs,
+# where a CTA goes from such a tile to another layer's
+RAGGED = {
+    "dgrad_1x1_c64": ("dgrad", "auto", [_flat(60000, 64, 16)]),
+    "dgrad_1x1_c256": ("dgrad", "auto", [_flat(20000 + 33, 256, 64)]),
+    "dgrad_1x1_group": ("dgrad", "auto", [_flat(257, 16 * (1 + i % 2), 16) for i in range(150)]),
+    "dgrad_3x3_c64": ("dgrad", "auto", [dict(batch=401, h=8, w=8, c=64, k=16, ksize=3)]),
+    "dgrad_3x3_group": ("dgrad", "auto", [dict(batch=5, h=8, w=8, c=16 * (1 + i % 2), k=16, ksize=3) for i in range(120)]),
+    "dgrad_3x3_small": ("dgrad", "auto", [dict(batch=8 * 40 + 1, h=4, w=4, c=128, k=64, ksize=3)]),
+    "dgrad_tma": ("dgrad", "tma", [_flat(60000, 64, 64)]),
+    "dgrad_tma_group": ("dgrad", "tma", [_flat(257, 16, 64) for i in range(150)]),
+    "dgrad_tma_tap": ("dgrad", "tma_tap", [dict(batch=401, h=8, w=8, c=64, k=64, ksize=3)]),
+    "forward_1x1_k64": ("forward", "auto", [_flat(60000, 16, 64)]),
+    "forward_tma": ("forward", "tma", [_flat(60000, 64, 128)]),
+    "forward_tma_group": ("forward", "tma", [_flat(257, 64, 64) for i in range(150)]),
+}
+
+
+@pytest.mark.parametrize("name,accumulate", [(n, a) for n in RAGGED for a in ([0, 1] if n.startswith("dgrad") else [0])])
+def test_staged_tiles_next_to_empty_rows(name, accumulate):
+    """Small whole numbers, so every sum is exact; no BN sums between a staged tile and the next."""
+    import torch
+    import torch.nn.functional as F
+    from paper_2103_08802_gb300 import pnn
+    mode, impl, geo = RAGGED[name]
+    torch.manual_seed(7)
+    ints = lambda *s: torch.randint(-1, 2, s, device="cuda").float()  # noqa: E731
+    insts, want = [], []
+    for g in geo:
+        d = dict(g, stride=1)
+        b, h, w, c, k, ks = (d[n] for n in ("batch", "h", "w", "c", "k", "ksize"))
+        wt, src = ints(k, ks, ks, c), ints(b, h, w, c if mode == "forward" else k)
+        d["wt"] = wt.bfloat16()
+        kern = wt.double().permute(0, 3, 1, 2)
+        x = src.double().permute(0, 3, 1, 2)
+        if mode == "forward":
+            d["x"], d["y"] = src.bfloat16(), torch.empty(b, h, w, k, device="cuda", dtype=torch.bfloat16)
+            want.append(F.conv2d(x, kern, padding=ks // 2).permute(0, 2, 3, 1))
+        else:
+            d["dy"], d["dx"], d["accumulate"] = src, torch.empty(b, h, w, c, device="cuda"), accumulate
+            want.append(F.conv_transpose2d(x, kern, padding=ks // 2).permute(0, 2, 3, 1))
+        insts.append(d)
+    for _ in range(8):
+        for d in insts:
+            d["y" if mode == "forward" else "dx"].fill_(3.0)
+        pnn.conv_run(mode, insts, impl=impl)
+        for d, e in zip(insts, want):
+            got = d["y" if mode == "forward" else "dx"].double()
+            assert torch.equal(got, e + 3.0 if accumulate else e)
