@@ -1076,28 +1076,56 @@ __global__ void __launch_bounds__(256) k_ew_bwd(const EwBwdDesc* __restrict__ ta
 // a single level -- thread = (channel t & 7, tile lane t >> 3), 64 tile lanes,
 // 16 loads in flight a thread, one pass through shared memory.  There is no
 // second level (the former 32 channels x 64 tiles a CTA met in global scratch
-// behind an atomic count: five dependent trips to L2).  Sums run as
-// unevaluated pairs of floats (Knuth's TwoSum), about 48 bits: this part's
-// fp64 pipe would take longer than the loads.  The training step of the
+// behind an atomic count: five dependent trips to L2).  Sums run as unevaluated
+// sums of floats (Knuth's TwoSum) -- two, about 48 bits, for the forward's fp32
+// terms; three, more than the 53 bits of fp64, for the backward's -- since this
+// part's fp64 pipe would take longer than the loads.  The training step of the
 // 8-subnetwork ResNet-1001 (batch 256, 64 px; 340 such launches of up to 2048
-// tiles a layer): 81.94 -> 81.36 ms.
-__device__ __forceinline__ void pair_add(float& hi, float& lo, float x) {
-  const float s = __fadd_rn(hi, x);
-  const float bb = __fsub_rn(s, hi);
-  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
-  hi = s;
+// tiles a layer): 81.94 -> 81.36 ms with two floats, one quantity at a time.  Both
+// quantities of a partial packed, with the third float: 4-subnetwork ResNet-1001
+// (batch 128, 32 px) 26.27 -> 26.01 ms; unpacked, the third float had cost 0.17 ms, and
+// with 4 channels a CTA 0.5 ms (three such networks at once).
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+  return tc::fma2(b, tc::pk2(-1.f, -1.f), a);  // (one rounding: a - b)
 }
-__device__ __forceinline__ void pair_merge(float& hi, float& lo, float hi2, float lo2) {
-  pair_add(hi, lo, hi2);
-  lo = __fadd_rn(lo, lo2);
+// a + b -> its fp32 rounding, e: what that leaves out
+__device__ __forceinline__ uint64_t two_sum(uint64_t a, uint64_t b, uint64_t& e) {
+  const uint64_t s = tc::add2(a, b), bb = sub2(s, a);
+  e = tc::add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+  return s;
 }
-// the value of a pair (an overflowed or NaN sum has no meaningful low part)
-__device__ __forceinline__ double pair_value(float2 p) { return isfinite(p.x) ? (double)p.x + (double)p.y : (double)p.x; }
+template <int N>
+struct FloatSum {
+  uint64_t v[N] = {};  // decreasing
+  // x into part `from` and its remainders into the following ones
+  __device__ __forceinline__ void add(uint64_t x, int from = 0) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      if (i < from) continue;
+      if (i == N - 1) v[i] = tc::add2(v[i], x);
+      else v[i] = two_sum(v[i], x, x);
+    }
+  }
+  __device__ __forceinline__ void add(const FloatSum& o) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) add(o.v[i], i);
+  }
+  // (an overflowed or NaN sum has no meaningful low parts)
+  __device__ __forceinline__ double2 value() const {
+    double x = 0.0, y = 0.0;
+#pragma unroll
+    for (int i = N - 1; i > 0; --i) {
+      x += (double)tc::un2(v[i]).x;
+      y += (double)tc::un2(v[i]).y;
+    }
+    const float2 h = tc::un2(v[0]);
+    return make_double2(isfinite(h.x) ? (double)h.x + x : (double)h.x, isfinite(h.y) ? (double)h.y + y : (double)h.y);
+  }
+};
 
 constexpr int kFinThreads = 512;
 constexpr int kFinLanes = kFinThreads / kFinChannels;  // tile lanes
 constexpr int kFinUnroll = 16;                         // loads in flight a thread
-static_assert(kFinThreads / 32 == 2 * kFinChannels, "one warp per (channel, quantity) sum");
 
 // Sums over all tiles for the 8 channels of group cg.  MOMENTS false: of the
 // two partial quantities.  MOMENTS true: the tiles hold (mean_t, M2_t) of
@@ -1112,15 +1140,18 @@ static_assert(kFinThreads / 32 == 2 * kFinChannels, "one warp per (channel, quan
 template <bool MOMENTS>
 __device__ __forceinline__ void tile_sums(const float* __restrict__ part, int C, int tiles, int64_t M, int rpt, int cg,
                                           double& s1, double& s2, float& K) {
-  __shared__ float2 red[kFinLanes][2 * kFinChannels + 1];
-  __shared__ float2 tot[2 * kFinChannels];
+  constexpr int N = MOMENTS ? 2 : 3;
+  using Sum = FloatSum<N>;
+  __shared__ uint64_t red[N][kFinLanes][kFinChannels + 1];
+  __shared__ double2 tot[kFinChannels];
   const int ch = threadIdx.x % kFinChannels, tl = threadIdx.x / kFinChannels;
   const int c = cg * kFinChannels + ch;
-  float ah = 0.f, al = 0.f, bh = 0.f, bl = 0.f;
+  Sum a;
   K = 0.f;
   if (c < C) {
     const float2* p = reinterpret_cast<const float2*>(part) + c;
     if (MOMENTS && tiles > 0) K = __ldg(part + (int64_t)c * 2);
+    const float full = (float)rpt, last = (float)(M - (int64_t)(tiles - 1) * rpt);  // rows of a tile
     for (int t0 = tl; t0 < tiles; t0 += kFinLanes * kFinUnroll) {
       float2 v[kFinUnroll];
 #pragma unroll
@@ -1133,39 +1164,46 @@ __device__ __forceinline__ void tile_sums(const float* __restrict__ part, int C,
         const int t = t0 + k * kFinLanes;
         if (t >= tiles) continue;
         if (MOMENTS) {
-          const int64_t r1 = (int64_t)(t + 1) * rpt < M ? (int64_t)(t + 1) * rpt : M;
-          const float n = (float)(r1 - (int64_t)t * rpt);
+          const float n = t + 1 < tiles ? full : last;
           const float d = v[k].x - K;
           const float nd = n * d;
-          pair_add(ah, al, nd);
-          pair_add(bh, bl, fmaf(nd, d, v[k].y));
+          a.add(tc::pk2(nd, fmaf(nd, d, v[k].y)));
         } else {
-          pair_add(ah, al, v[k].x);
-          pair_add(bh, bl, v[k].y);
+          a.add(tc::pk2(v[k].x, v[k].y));
         }
       }
     }
   }
-  red[tl][2 * ch] = make_float2(ah, al);
-  red[tl][2 * ch + 1] = make_float2(bh, bl);
-  __syncthreads();
-  {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float2 a = red[lane][w];
 #pragma unroll
-    for (int i = 32; i < kFinLanes; i += 32) pair_merge(a.x, a.y, red[lane + i][w].x, red[lane + i][w].y);
+  for (int i = 0; i < N; ++i) red[i][tl][ch] = a.v[i];
+  __syncthreads();
+  if (const int w = threadIdx.x >> 5, lane = threadIdx.x & 31; w < kFinChannels) {
+    Sum s;
+#pragma unroll
+    for (int i = 0; i < N; ++i) s.v[i] = red[i][lane][w];
+#pragma unroll
+    for (int l = 32; l < kFinLanes; l += 32) {
+      if (l >= tiles) break;  // (a lane without a tile holds zero)
+      Sum o;
+#pragma unroll
+      for (int i = 0; i < N; ++i) o.v[i] = red[i][lane + l][w];
+      s.add(o);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const float h = __shfl_xor_sync(0xffffffffu, a.x, o), l = __shfl_xor_sync(0xffffffffu, a.y, o);
-      pair_merge(a.x, a.y, h, l);
+      if (o >= tiles) continue;
+      Sum t;
+#pragma unroll
+      for (int i = 0; i < N; ++i) t.v[i] = __shfl_xor_sync(0xffffffffu, s.v[i], o);
+      s.add(t);
     }
-    if (lane == 0) tot[w] = a;
+    if (lane == 0) tot[w] = s.value();
   }
   __syncthreads();
   s1 = s2 = 0.0;
   if (threadIdx.x < kFinChannels) {
-    s1 = pair_value(tot[2 * threadIdx.x]);
-    s2 = pair_value(tot[2 * threadIdx.x + 1]);
+    s1 = tot[threadIdx.x].x;
+    s2 = tot[threadIdx.x].y;
   }
 }
 

@@ -74,3 +74,25 @@ def test_backward_sums(rows, c):
     for got, term in ((d["dbeta"], g), (d["dgamma"], g * xh)):
         err = (got.double() - term.sum(0)).abs()
         assert (err <= 160 * U * term.abs().sum(0) + 1e-30).all(), float((err / term.abs().sum(0)).max())
+
+
+def test_backward_sums_keep_fp64_bits():
+    """Partials of one column that need 53 bits together and cancel to the last of them: the tiles that one
+    thread of the finalisation adds (128 apart) hold 2^30, 8, 2^-22, -8, -2^30."""
+    import torch
+    from paper_2103_08802_gb300 import pnn
+    rows, c = 513 * 128, 16
+    d = dict(batch=1, h=rows, w=1, c=c, k=c, ksize=1, stride=1, relu=0)
+    d["x"] = torch.ones(1, rows, 1, c, device="cuda").bfloat16()
+    d["wt"] = torch.eye(c, device="cuda").view(c, 1, 1, c).bfloat16()
+    for n, v in (("bn_scale", 1.0), ("bn_shift", 0.0), ("bn_mean", 0.0), ("bn_rstd", 1.0)):
+        d[n] = torch.full((c,), v, device="cuda")
+    d["dy"] = torch.zeros(1, rows, 1, c, device="cuda")
+    for i, v in enumerate((2.0 ** 30, 8.0, 2.0 ** -22, -8.0, -2.0 ** 30)):
+        d["dy"][0, i * 128 * 128, 0, 3] = v
+    d["dx"] = torch.empty(1, rows, 1, c, device="cuda")
+    d["dgamma"], d["dbeta"] = torch.empty(c, device="cuda"), torch.empty(c, device="cuda")
+    pnn.conv_run("dgrad", [d])
+    want = torch.zeros(c, device="cuda")
+    want[3] = 2.0 ** -22
+    assert torch.equal(d["dbeta"], want) and torch.equal(d["dgamma"], want)
