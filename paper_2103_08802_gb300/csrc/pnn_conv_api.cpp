@@ -383,12 +383,15 @@ using namespace pnn;
 
 extern "C" int pnn_conv_workspace_bytes(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* args, size_t* bytes) {
   if (!bytes) return set_last_error(PNN_EINVAL, "pnn_conv_workspace_bytes: null output");
-  // enough for either choice, so that the answer does not depend on the pointers' alignment
-  Plan narrow, other;
-  int r = make_plan(mode, impl, n, args, true, narrow);
-  if (!r) r = make_plan(mode, impl, n, args, false, other);
+  Plan pl;
+  const int r = make_plan(mode, impl, n, args, true, pl);
   if (r) return r;
-  *bytes = std::max(narrow.bytes, other.bytes);
+  *bytes = pl.bytes;
+  if (pl.variant < 4) return PNN_OK;  // (the plan whatever the pointers)
+  // enough for the other choice too, so that the answer does not depend on the pointers' alignment
+  Plan other;
+  make_plan(mode, impl, n, args, false, other);
+  *bytes = std::max(pl.bytes, other.bytes);
   return PNN_OK;
 }
 

@@ -178,6 +178,33 @@ def test_single_conv_call_checks_its_arguments(pnn):
     assert lib.pnn_conv_run(0, 0, 1, args(), C.c_void_p(256), 256, None) == 2
 
 
+@pytest.mark.parametrize("geometry", [dict(h=32, w=32, c=16, k=64, ksize=1, stride=1), dict(h=16, w=16, c=16, k=32, ksize=3, stride=1),
+                                      dict(h=27, w=27, c=24, k=40, ksize=3, stride=2)])
+def test_conv_workspace_does_not_depend_on_alignment(pnn, geometry):
+    """The kernel choice of impl 0 looks at the pointers' alignment; the workspace size covers either choice."""
+    lib = pnn.load()
+
+    def args(off):
+        a = pnn.ConvArgs()
+        for key, v in dict(geometry, batch=3).items():
+            setattr(a, key, v)
+        a.x = a.wt = a.y = a.dy = a.dx = a.dw = 256
+        a.x_dtype = a.y_dtype = a.res_dtype = 1
+        a.bn_scale = a.bn_shift = a.bn_mean = a.bn_rstd = 256 + off
+        a.y_mean = a.y_rstd = a.dgamma = a.dbeta = 256
+        return (pnn.ConvArgs * 1)(a)
+
+    for mode in range(3):
+        size = []
+        for off in (0, 4):
+            nb = C.c_size_t()
+            assert lib.pnn_conv_workspace_bytes(mode, 0, 1, args(off), C.byref(nb)) == 0
+            size.append(nb.value)
+            # one region less is refused before any launch, whatever the alignment
+            assert lib.pnn_conv_run(mode, 0, 1, args(off), C.c_void_p(256), 256, None) == 2
+        assert size[0] == size[1]
+
+
 def test_halo_tiles_kernel_choice(pnn):
     """The TMA-fed 3x3 forward / data gradient take halo tiles (one box per
     128-pixel tile) where 128 divides h*w, w <= 63 and the A source has 16 |
