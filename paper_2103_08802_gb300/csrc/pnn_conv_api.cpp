@@ -173,20 +173,30 @@ bool halo_inst(int mode, const pnn_conv_args& g) {
   return halo_ok(g.ksize, g.stride, g.ksize / 2, g.h, g.w, ch) && conv_halo_fits(mode, g.w, ch, bn);
 }
 
+bool aligned(const void* p, uintptr_t bytes) { return reinterpret_cast<uintptr_t>(p) % bytes == 0; }
+bool bn_values_aligned(const pnn_conv_args& g, uintptr_t bytes) {
+  return aligned(g.bn_scale, bytes) && aligned(g.bn_shift, bytes) && aligned(g.bn_mean, bytes) && aligned(g.bn_rstd, bytes);
+}
 // Whether the caller's pointers suit k_pw_conv.cu, k_c3_conv.cu and k_wg_conv.cu:
-// tensor maps want 16 bytes, the pairwise reads of the per-channel values 8.  (The
-// other kernels read those one at a time; slices at an odd offset stay with them.)
+// tensor maps want 16 bytes, the pairwise reads of the per-channel values 8.
+// (Slices at an odd offset stay with the other kernels, which read them one at a
+// time but for the BN sums of a data gradient: bn_sums_fused.)
 bool narrow_pointers(int n, const pnn_conv_args* a) {
-  auto on = [](const void* p, uintptr_t bytes) { return reinterpret_cast<uintptr_t>(p) % bytes == 0; };
   for (int i = 0; i < n; ++i) {
     const pnn_conv_args& g = a[i];
     for (const void* p : {(const void*)g.x, (const void*)g.wt, (const void*)g.y, (const void*)g.res, (const void*)g.dy,
                           (const void*)g.dx})
-      if (!on(p, 16)) return false;
-    for (const void* p : {(const void*)g.bn_scale, (const void*)g.bn_shift, (const void*)g.bn_mean, (const void*)g.bn_rstd})
-      if (!on(p, 8)) return false;
+      if (!aligned(p, 16)) return false;
+    if (!bn_values_aligned(g, 8)) return false;
   }
   return true;
+}
+// Whether a data gradient forms its BN sums in its epilogue: TMA-fed, writing the
+// whole gradient, and (k_conv_dgrad_tma) the per-channel values on 16 bytes, which
+// it reads four at a time.  Otherwise the separate reduction runs over its own row
+// tiles and reads them one at a time.
+bool bn_sums_fused(int variant, const pnn_conv_args& g) {
+  return variant != 0 && !g.accumulate && g.c % 16 == 0 && (variant != 1 || bn_values_aligned(g, 16));
 }
 
 // narrow: the kernels of k_pw_conv.cu, k_c3_conv.cu and k_wg_conv.cu may be chosen
@@ -567,11 +577,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
       b.M = Min; b.C = g.c;
       b.rows_per_tile = bnb_rows_per_tile(g.c, Min);
       b.inv_count = 1.0 / (double)Min;
-      // the TMA-fed data gradient forms the sums of its 128-row tiles in its
-      // epilogue when it writes the whole gradient; otherwise the separate
-      // reduction kernel runs over its own row tiles
-      const bool fused = (pl.variant == 1 || pl.variant == 4 || pl.variant == 5) && !g.accumulate && g.c % 16 == 0;
-      if (fused) {
+      if (bn_sums_fused(pl.variant, g)) {
         c.bn_mean = g.bn_mean; c.bn_rstd = g.bn_rstd; c.bnb_part = b.part;
         b.tiles = ip.mtiles;
       } else {

@@ -189,6 +189,40 @@ def test_per_channel_values_at_odd_offsets(mode, c, k, ks):
     assert results[0].abs().max() > 0 and torch.equal(results[0], results[1])
 
 
+@pytest.mark.parametrize("ks,c,k", [(1, 64, 16), (3, 16, 16)])
+@pytest.mark.parametrize("odd", ["bn_scale", "bn_shift", "bn_mean", "bn_rstd"])
+def test_data_gradient_sums_with_values_at_odd_offsets(odd, ks, c, k):
+    """Each of the BN values of a data gradient's sums in turn at an odd float offset: dx is that of impl "tma",
+    the sums (of another kernel, in another order) within the bound of any order of the same fp32 terms."""
+    import torch
+    from paper_2103_08802_gb300 import pnn
+    torch.manual_seed(6)
+    b, h = 3, 32
+    rows = b * h * h
+    base = dict(batch=b, h=h, w=h, c=c, k=k, ksize=ks, stride=1, relu=1)
+    base["x"] = torch.randn(b, h, h, c, device="cuda").bfloat16()
+    base["wt"] = torch.randn(k, ks, ks, c, device="cuda").bfloat16()
+    base["dy"] = torch.randn(b, h, h, k, device="cuda")
+    values = {n: torch.rand(c, device="cuda") + 0.5 for n in ("bn_scale", "bn_shift", "bn_mean", "bn_rstd")}
+    dx = []
+    for impl, shifted in (("tma", None), ("auto", odd)):
+        d = dict(base, dx=torch.zeros(b, h, h, c, device="cuda"))
+        for n, v in values.items():
+            d[n] = torch.empty(c + 1, device="cuda")[1:] if n == shifted else torch.empty(c, device="cuda")
+            d[n].copy_(v)
+            assert d[n].data_ptr() % 8 == (4 if n == shifted else 0)
+        d["dgamma"], d["dbeta"] = torch.empty(c, device="cuda"), torch.empty(c, device="cuda")
+        pnn.conv_run("dgrad", [d], impl=impl)
+        dx.append(d["dx"])
+        x = base["x"].view(-1, c)
+        pre = (values["bn_scale"].double() * x.double() + values["bn_shift"].double()).float()
+        g = torch.where(pre > 0, d["dx"].view(-1, c), torch.zeros((), device="cuda")).double()
+        xh = ((x.float() - values["bn_mean"]) * values["bn_rstd"]).double()
+        for got, term in ((d["dbeta"], g), (d["dgamma"], g * xh)):
+            assert ((got.double() - term.sum(0)).abs() <= rows * K.U * term.abs().sum(0)).all()
+    assert torch.equal(dx[0], dx[1])
+
+
 def _flat(rows, c, k):
     return dict(batch=1, h=rows, w=1, c=c, k=k, ksize=1)
 
