@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(256) k_conv_wgrad_few(const ConvDesc* __restri
   constexpr int BM = kWgradBM, BP = 64, JG = 32 / KL;        // JG lane groups share the columns
   constexpr int KPL = KL == 16 ? 1 : BM / 32;                // output channels a lane
   constexpr int JV = kFewCols / 4 / JG;                      // float4 columns a lane
-  __shared__ float As[BP][BM];                               // dY[pixel][k_out]
+  __shared__ __align__(16) float As[BP][BM];                 // dY[pixel][k_out]; at the end the sums, as float4
   __shared__ __align__(16) float Bs[BP][kFewCols + 4];       // im2col[pixel][j]
   const int inst = find_instance(tstart, n, blockIdx.x);
   const ConvDesc d = tab[inst];
