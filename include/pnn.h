@@ -395,6 +395,15 @@ typedef struct pnn_conv_args {
   float* dw;                     /* weight gradient output, k x ksize x ksize x c float32 */
 } pnn_conv_args;
 int pnn_conv_workspace_bytes(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* args, size_t* bytes);
+/* Which kernels pnn_conv_run takes for these arguments (host only): impl 0
+ * chooses the last three by shape, storage type and alignment. */
+typedef enum {
+  PNN_CONV_KERNEL_GATHERED = 0, PNN_CONV_KERNEL_TMA = 1, /* k_tc_conv.cu */
+  PNN_CONV_KERNEL_1X1 = 2,   /* k_pw_conv.cu: forward, data gradient */
+  PNN_CONV_KERNEL_3X3 = 3,   /* k_c3_conv.cu: forward, data gradient */
+  PNN_CONV_KERNEL_WGRAD = 4  /* k_wg_conv.cu */
+} pnn_conv_kernel_kind;
+int pnn_conv_kernel(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* args, int32_t* kernel);
 int pnn_conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* args, void* workspace,
                  size_t workspace_bytes, void* stream);
 /* pnn_conv_run, then `repeat` (> 0) further launches of the convolution

@@ -391,6 +391,19 @@ int make_plan(int mode, int impl, int n, const pnn_conv_args* a, bool narrow, Pl
 
 using namespace pnn;
 
+extern "C" int pnn_conv_kernel(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* args, int32_t* kernel) {
+  if (!kernel) return set_last_error(PNN_EINVAL, "pnn_conv_kernel: null output");
+  Plan pl;
+  const int r = make_plan(mode, impl, n, args, args && n > 0 && narrow_pointers(n, args), pl);
+  if (r) return r;
+  *kernel = pl.variant == 5                ? PNN_CONV_KERNEL_3X3
+            : pl.variant == 4 && mode == 2 ? PNN_CONV_KERNEL_WGRAD
+            : pl.variant == 4              ? PNN_CONV_KERNEL_1X1
+            : pl.variant == 1              ? PNN_CONV_KERNEL_TMA
+                                           : PNN_CONV_KERNEL_GATHERED;
+  return PNN_OK;
+}
+
 extern "C" int pnn_conv_workspace_bytes(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* args, size_t* bytes) {
   if (!bytes) return set_last_error(PNN_EINVAL, "pnn_conv_workspace_bytes: null output");
   Plan pl;

@@ -127,6 +127,7 @@ def load():
         "pnn_conv_wgrad_noalloc": (C.c_int, [P, P, P, I32, I32, I32, I32, I32, I32, I32, P]),
         "pnn_selftest_wait_timeout": (C.c_int, [C.c_int64, P]),
         "pnn_conv_workspace_bytes": (C.c_int, [I32, I32, I32, C.POINTER(ConvArgs), C.POINTER(SZ)]),
+        "pnn_conv_kernel": (C.c_int, [I32, I32, I32, C.POINTER(ConvArgs), C.POINTER(I32)]),
         "pnn_conv_run": (C.c_int, [I32, I32, I32, C.POINTER(ConvArgs), P, SZ, P]),
         "pnn_conv_time": (C.c_int, [I32, I32, I32, C.POINTER(ConvArgs), P, SZ, P, I32, C.POINTER(C.c_float)]),
         "pnn_last_error": (C.c_char_p, [P]),

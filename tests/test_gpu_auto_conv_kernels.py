@@ -2,7 +2,8 @@
 their rules: one row, one less and one more than a 128-row tile, more items
 than CTAs, every channel count the rule names, one and several k-steps, one and
 several column units, raw fp32 inputs.  Each launch is held to the oracle and
-the bounds of test_gpu_conv_kernels."""
+the bounds of test_gpu_conv_kernels; test_conv_choice_cpu asserts that these are
+the cases the rules take."""
 import pytest
 
 import test_gpu_conv_kernels as K
@@ -14,13 +15,6 @@ pytestmark = pytest.mark.gpu
 def _lib():
     from paper_2103_08802_gb300 import build
     build.build()
-
-
-def _name(base, kind):
-    """The forward test takes its epilogue from the name's length: 0 bf16 y, 2 bf16 y + bf16 residual."""
-    while len(base) % 3 != kind:
-        base += "_"
-    return base
 
 
 def _pw(batch, h, w, c, k, **kw):
@@ -44,7 +38,9 @@ PW = {
     "expand": [_pw(2, 16, 16, 16, 64, bn=True), _pw(2, 9, 9, 64, 256, bn=True)],
     "reduce": [_pw(2, 16, 16, 64, 16, bn=True), _pw(2, 9, 9, 256, 64, bn=False)],
 }
-CASES = [(n, kind) for n in PW for kind in (0, 2)]
+# epilogues: 0 bf16 y, 2 bf16 y + bf16 residual; a group's second instance takes the next of three, so 2 gives
+# both (1, fp32 y and residual, is not these kernels')
+CASES = [(n, kind) for n in PW for kind in ([2] if isinstance(PW[n], list) else [0, 2])]
 
 
 def _install(monkeypatch, name, spec):
@@ -56,11 +52,8 @@ def _install(monkeypatch, name, spec):
 
 @pytest.mark.parametrize("base,kind", CASES)
 def test_pointwise_forward(monkeypatch, base, kind):
-    if isinstance(PW[base], list):
-        kind = 2  # the two instances: bf16 y + residual, bf16 y
-    name = _name(base, kind)
-    _install(monkeypatch, name, PW[base])
-    K.test_conv_forward(name, "auto")
+    _install(monkeypatch, base, PW[base])
+    K.check_forward(base, "auto", kind)
 
 
 @pytest.mark.parametrize("base", list(PW))
@@ -141,17 +134,16 @@ C3 = {
     "small1x1": _wg(129, 1, 1, 16, 32, 3, bn=True),
     "small2x8_fp32x": _wg(5, 2, 8, 32, 16, 3, bn=True, x_fp32=True),
     "small_kinds": [_wg(20, 4, 4, 64, 64, 3, bn=True), _wg(2, 16, 16, 32, 128, 3, bn=True)],
-    "small_wholex": [_wg(3, 8, 8, 64, 128, 3, bn=True), _wg(40, 2, 2, 128, 64, 3, bn=False)],
+    "small_whole": [_wg(3, 8, 8, 64, 128, 3, bn=True), _wg(40, 2, 2, 128, 64, 3, bn=False)],
     "stages": [_wg(2, 32, 32, 16, 16, 3, bn=True), _wg(3, 8, 8, 64, 64, 3, bn=True)],
-    "stagex": [_wg(3, 8, 8, 64, 64, 3, bn=True), _wg(2, 16, 16, 32, 32, 3, bn=True)],
+    "stages_reversed": [_wg(3, 8, 8, 64, 64, 3, bn=True), _wg(2, 16, 16, 32, 32, 3, bn=True)],
 }
 
 
-@pytest.mark.parametrize("base,kind", [(n, kind) for n in C3 for kind in (0, 2)])
+@pytest.mark.parametrize("base,kind", [(n, kind) for n in C3 for kind in ([2] if isinstance(C3[n], list) else [0, 2])])
 def test_3x3_forward(monkeypatch, base, kind):
-    name = _name(base, 2 if isinstance(C3[base], list) else kind)
-    _install(monkeypatch, name, C3[base])
-    K.test_conv_forward(name, "auto")
+    _install(monkeypatch, base, C3[base])
+    K.check_forward(base, "auto", kind)
 
 
 @pytest.mark.parametrize("base", list(C3))
