@@ -87,6 +87,16 @@ bool plan_rings(const C3Slots& s, Rings& r) {
   return true;
 }
 
+// two slots of each ring and one second operand fit for the largest instances of c3_ok
+// together (fp32 patches, small images, 64 columns), so the launch of a planned group
+// cannot fail
+template <int MODE>
+constexpr bool fits() {
+  return fixed_bytes<MODE>() + 2 * (c3_raw_px(C3_PATCH) * 16 * 4 + 2 * c3_plane(C3_SMALL) + c3_wt_bytes(64)) +
+             kTcBM * 64 * 2 <= kSmemBudget;
+}
+static_assert(fits<FWD>() && fits<DGRAD>(), "two slots of each ring");
+
 struct Geo {
   int rows, n, nt, nk, H, W, tx, tpi;  // GEMM M, columns of a block and in all; 16-channel k-steps; patches a row and an image
   int kind, lw, li;                    // C3_PATCH, C3_WHOLE or C3_SMALL; log2 W, log2 H W (whole images)
@@ -226,8 +236,8 @@ __device__ __forceinline__ void transform_kind(const uint8_t* raw, uint8_t* op, 
 }
 
 template <int MODE, bool ANY>
-__device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int ninst,
-                                        int total, const Rings& rg, int32_t* status) {
+__device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int total,
+                                        const Rings& rg, int32_t* status) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw0 = smem_u32(smem_raw);
   const uint32_t base = (raw0 + 1023u) & ~1023u;
@@ -281,7 +291,7 @@ __device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const 
       const uint8_t* wt = nullptr;
       uint32_t abytes = 0;
       int off = 0;
-      for (Walk w(tab, ts, ninst, total); w.more() && ok; w.next(tab, ts)) {
+      for (Walk w(tab, ts, total); w.more() && ok; w.next(tab, ts)) {
         if (w.fresh) {
           const ConvDesc* d = w.d;
           g = geo<MODE, ANY>(d);
@@ -339,7 +349,7 @@ __device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const 
       bool hx = false;
       uint32_t idesc = 0;
       int rs = 0, ss = 1;  // pixels between the starts of tap rows and of taps
-      for (Walk w(tab, ts, ninst, total); w.more() && ok; w.next(tab, ts), cb.next()) {
+      for (Walk w(tab, ts, total); w.more() && ok; w.next(tab, ts), cb.next()) {
         if (w.fresh) {
           g = geo<MODE, ANY>(w.d);
           hx = has_x<MODE>(w.d);
@@ -396,7 +406,7 @@ __device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const 
     Geo g{};
     bool bn = false, xbf = false;
     int relu = 0;
-    for (Walk w(tab, ts, ninst, total); w.more(); w.next(tab, ts)) {
+    for (Walk w(tab, ts, total); w.more(); w.next(tab, ts)) {
       const ConvDesc* d = w.d;
       if (w.fresh) {
         g = geo<MODE, ANY>(d);
@@ -452,7 +462,7 @@ __device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const 
     bool ok = true;
     Geo g{};
     EpiArgs ea{};
-    for (Walk w(tab, ts, ninst, total); w.more(); w.next(tab, ts)) {
+    for (Walk w(tab, ts, total); w.more(); w.next(tab, ts)) {
       if (w.fresh) {
         g = geo<MODE, ANY>(w.d);
         ea.load<MODE>(w.d);
@@ -510,18 +520,18 @@ __device__ __forceinline__ void c3_body(const ConvDesc* __restrict__ tab, const 
 
 template <bool ANY>
 __global__ void __launch_bounds__(kThreads, 1) k_c3_fwd(const ConvDesc* __restrict__ tab, const int* __restrict__ ts,
-                                                        int ninst, int total, const Rings rg, int32_t* status) {
-  c3_body<FWD, ANY>(tab, ts, ninst, total, rg, status);
+                                                        int total, const Rings rg, int32_t* status) {
+  c3_body<FWD, ANY>(tab, ts, total, rg, status);
 }
 template <bool ANY>
 __global__ void __launch_bounds__(kThreads, 1) k_c3_dgrad(const ConvDesc* __restrict__ tab, const int* __restrict__ ts,
-                                                          int ninst, int total, const Rings rg, int32_t* status) {
-  c3_body<DGRAD, ANY>(tab, ts, ninst, total, rg, status);
+                                                          int total, const Rings rg, int32_t* status) {
+  c3_body<DGRAD, ANY>(tab, ts, total, rg, status);
 }
 
 }  // namespace
 
-cudaError_t launch_conv_c3(int mode, const ConvDesc* tab, const int* ts, int n, int total, const C3Slots& s,
+cudaError_t launch_conv_c3(int mode, const ConvDesc* tab, const int* ts, int total, const C3Slots& s,
                            int32_t* status, cudaStream_t st, int max_ctas) {
   if (total <= 0) return cudaSuccess;
   if ((s.raw & 127) || (s.op & 127) || (s.wt & 1023) || (s.x & 1023) || s.raw <= 0 || s.op <= 0 || s.wt <= 0)
@@ -535,7 +545,7 @@ cudaError_t launch_conv_c3(int mode, const ConvDesc* tab, const int* ts, int n, 
   int grid = total < sms ? total : sms;
   if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
   const int smem = (mode == FWD ? fixed_bytes<FWD>() : fixed_bytes<DGRAD>()) + rings_bytes(r);
-  kern<<<grid, kThreads, smem, st>>>(tab, ts, n, total, r, status);
+  kern<<<grid, kThreads, smem, st>>>(tab, ts, total, r, status);
   return cudaGetLastError();
 }
 

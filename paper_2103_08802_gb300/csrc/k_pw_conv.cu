@@ -104,6 +104,14 @@ bool plan_rings(int rawb, int xb, Rings& r) {
   return true;
 }
 
+// two slots of each ring fit for the largest instance of pw_ok (64 fp32 channels a
+// k-step, a second operand), so the launch of a planned group cannot fail
+template <int MODE, int W>
+constexpr bool fits() {
+  return fixed_bytes<MODE, W>() + 2 * (pw_raw_bytes(kPwMaxC, 4) + kOpBytes + kUnitB + pw_x_bytes(64)) <= kSmemBudget;
+}
+static_assert(fits<FWD, 0>() && fits<FWD, 1>() && fits<DGRAD, 0>(), "two slots of each ring");
+
 // what the roles need of an instance
 struct Geo {
   int rows, ncols, kt, nkt, bn, spi, nsub;  // GEMM M, N, K; k-steps; unit columns; units an item, in all
@@ -187,8 +195,8 @@ struct RowDst {
 };
 
 template <int MODE, int W>
-__device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int ninst,
-                                        int total, const Rings& rg, int32_t* status) {
+__device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int total,
+                                        const Rings& rg, int32_t* status) {
   using R = Roles<MODE, W>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw0 = smem_u32(smem_raw);
@@ -237,7 +245,7 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
       Geo g{};
       const void *ma = nullptr, *mb = nullptr, *mx = nullptr;
       uint32_t abytes = 0;
-      for (Walk w(tab, ts, ninst, total); w.more() && ok; w.next(tab, ts)) {
+      for (Walk w(tab, ts, total); w.more() && ok; w.next(tab, ts)) {
         if (w.fresh) {
           const ConvDesc* d = w.d;
           g = geo<MODE>(d);
@@ -286,7 +294,7 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
       Geo g{};
       bool hx = false;
       uint32_t idesc = 0;
-      for (Walk w(tab, ts, ninst, total); w.more() && ok; w.next(tab, ts)) {
+      for (Walk w(tab, ts, total); w.more() && ok; w.next(tab, ts)) {
         if (w.fresh) {
           g = geo<MODE>(w.d);
           hx = has_x<MODE>(w.d);
@@ -341,7 +349,7 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
     Geo g{};
     bool bn = false, xbf = false;
     int relu = 0, lgn = 0;
-    for (Walk w(tab, ts, ninst, total); w.more(); w.next(tab, ts)) {
+    for (Walk w(tab, ts, total); w.more(); w.next(tab, ts)) {
       const ConvDesc* d = w.d;
       if (w.fresh) {
         g = geo<MODE>(d);
@@ -395,7 +403,7 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
     bool ok = true;
     Geo g{};
     EpiArgs ea{};
-    for (Walk w(tab, ts, ninst, total); w.more(); w.next(tab, ts)) {
+    for (Walk w(tab, ts, total); w.more(); w.next(tab, ts)) {
       if (w.fresh) {
         g = geo<MODE>(w.d);
         ea.load<MODE>(w.d);
@@ -457,17 +465,17 @@ __device__ __forceinline__ void pw_body(const ConvDesc* __restrict__ tab, const 
 
 #define PNN_PW_KERNEL(NAME, MODE, W)                                                                                \
   __global__ void __launch_bounds__(Roles<MODE, W>::kThreads, 1)                                                    \
-      NAME(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int ninst, int total, const Rings rg,      \
+      NAME(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int total, const Rings rg,                 \
            int32_t* status) {                                                                                       \
-    pw_body<MODE, W>(tab, ts, ninst, total, rg, status);                                                            \
+    pw_body<MODE, W>(tab, ts, total, rg, status);                                                                   \
   }
 PNN_PW_KERNEL(k_pw_fwd, FWD, 0)
 PNN_PW_KERNEL(k_pw_fwd_w, FWD, 1)
 PNN_PW_KERNEL(k_pw_dgrad, DGRAD, 0)
 
 template <int MODE, int W>
-cudaError_t launch(void (*kern)(const ConvDesc*, const int*, int, int, const Rings, int32_t*), int slot,
-                   const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes, int x_bytes,
+cudaError_t launch(void (*kern)(const ConvDesc*, const int*, int, const Rings, int32_t*), int slot,
+                   const ConvDesc* tab, const int* ts, int total, int raw_bytes, int x_bytes,
                    int32_t* status, cudaStream_t st, int max_ctas) {
   Rings r;
   if (!plan_rings<MODE, W>(raw_bytes, x_bytes, r)) return cudaErrorInvalidValue;
@@ -477,25 +485,20 @@ cudaError_t launch(void (*kern)(const ConvDesc*, const int*, int, int, const Rin
   int grid = total < sms ? total : sms;
   if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
   const int smem = fixed_bytes<MODE, W>() + rings_bytes(r);
-  kern<<<grid, Roles<MODE, W>::kThreads, smem, st>>>(tab, ts, n, total, r, status);
+  kern<<<grid, Roles<MODE, W>::kThreads, smem, st>>>(tab, ts, total, r, status);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-bool pw_fits(int mode, int raw_bytes, int x_bytes) {
-  Rings r;
-  return mode == FWD ? plan_rings<FWD, 0>(raw_bytes, x_bytes, r) : plan_rings<DGRAD, 0>(raw_bytes, x_bytes, r);
-}
-
-cudaError_t launch_conv_pw(int mode, int wide, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes,
+cudaError_t launch_conv_pw(int mode, int wide, const ConvDesc* tab, const int* ts, int total, int raw_bytes,
                            int x_bytes, int32_t* status, cudaStream_t st, int max_ctas) {
   if (total <= 0) return cudaSuccess;
   if (raw_bytes <= 0 || (raw_bytes & 1023) || x_bytes < 0 || (x_bytes & 1023)) return cudaErrorInvalidValue;
   if (mode == DGRAD)
-    return launch<DGRAD, 0>(k_pw_dgrad, 14, tab, ts, n, total, raw_bytes, x_bytes, status, st, max_ctas);
-  return wide ? launch<FWD, 1>(k_pw_fwd_w, 13, tab, ts, n, total, raw_bytes, x_bytes, status, st, max_ctas)
-              : launch<FWD, 0>(k_pw_fwd, 12, tab, ts, n, total, raw_bytes, x_bytes, status, st, max_ctas);
+    return launch<DGRAD, 0>(k_pw_dgrad, 14, tab, ts, total, raw_bytes, x_bytes, status, st, max_ctas);
+  return wide ? launch<FWD, 1>(k_pw_fwd_w, 13, tab, ts, total, raw_bytes, x_bytes, status, st, max_ctas)
+              : launch<FWD, 0>(k_pw_fwd, 12, tab, ts, total, raw_bytes, x_bytes, status, st, max_ctas);
 }
 
 }  // namespace pnn

@@ -211,8 +211,8 @@ __device__ __forceinline__ void rows_to_planes(const uint8_t* __restrict__ raw, 
 // ANY: a 3x3 launch with small images or several blocks of output channels;
 // without, the code of both folds away
 template <int KS, bool ANY>
-__device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int ninst,
-                                        int total, const Rings& rg, int32_t* status) {
+__device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const int* __restrict__ ts, int total,
+                                        const Rings& rg, int32_t* status) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw0 = smem_u32(smem_raw);
   const uint32_t base = (raw0 + 1023u) & ~1023u;
@@ -255,7 +255,7 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
       Cursor cr(rg.nr);
       uint32_t n = 0;
       bool ok = true;
-      for (Walk w(tab, ts, ninst, total); w.more() && ok; w.next(tab, ts)) {
+      for (Walk w(tab, ts, total); w.more() && ok; w.next(tab, ts)) {
         const ConvDesc* d = w.d;
         const Geo g = geo<KS>(d);
         const int pbeg = w.tm * d->pix_per_split, pend = min(g.rows, pbeg + d->pix_per_split);
@@ -284,7 +284,7 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
     if (elect_one()) {
       Cursor co(rg.no), cb(kBufs);
       bool ok = true, issued = false;
-      for (Walk w(tab, ts, ninst, total); w.more() && ok; w.next(tab, ts)) {
+      for (Walk w(tab, ts, total); w.more() && ok; w.next(tab, ts)) {
         const ConvDesc* d = w.d;
         const Geo g = geo<KS>(d);
         const int pbeg = w.tm * d->pix_per_split, pend = min(g.rows, pbeg + d->pix_per_split);
@@ -340,7 +340,7 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
     const int t = threadIdx.x - 32 * kT0;
     Cursor cr(rg.nr), co(rg.no);
     bool ok = true;
-    for (Walk w(tab, ts, ninst, total); w.more(); w.next(tab, ts)) {
+    for (Walk w(tab, ts, total); w.more(); w.next(tab, ts)) {
       const ConvDesc* d = w.d;
       const Geo g = geo<KS>(d);
       const int pbeg = w.tm * d->pix_per_split, pend = min(g.rows, pbeg + d->pix_per_split);
@@ -400,7 +400,7 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
     const int q = warp & 3;
     Cursor cb(kBufs);
     bool ok = true;
-    for (Walk w(tab, ts, ninst, total); w.more(); w.next(tab, ts), cb.next()) {
+    for (Walk w(tab, ts, total); w.more(); w.next(tab, ts), cb.next()) {
       const ConvDesc* d = w.d;
       const Geo g = geo<KS>(d);
       if (ok) ok = mbar_wait(smem_u32(&sh.tfull[cb.s]), cb.ph, abort_flag);
@@ -443,13 +443,13 @@ __device__ __forceinline__ void wg_body(const ConvDesc* __restrict__ tab, const 
 }
 
 __global__ void __launch_bounds__(kThreads, 1) k_wg_pw(const ConvDesc* __restrict__ tab, const int* __restrict__ ts,
-                                                       int ninst, int total, const Rings rg, int32_t* status) {
-  wg_body<1, false>(tab, ts, ninst, total, rg, status);
+                                                       int total, const Rings rg, int32_t* status) {
+  wg_body<1, false>(tab, ts, total, rg, status);
 }
 template <bool ANY>
 __global__ void __launch_bounds__(kThreads, 1) k_wg_3x3(const ConvDesc* __restrict__ tab, const int* __restrict__ ts,
-                                                        int ninst, int total, const Rings rg, int32_t* status) {
-  wg_body<3, ANY>(tab, ts, ninst, total, rg, status);
+                                                        int total, const Rings rg, int32_t* status) {
+  wg_body<3, ANY>(tab, ts, total, rg, status);
 }
 
 }  // namespace
@@ -459,7 +459,7 @@ bool wg_fits(int raw_bytes, int op_bytes) {
   return plan_rings(raw_bytes, op_bytes, r);
 }
 
-cudaError_t launch_conv_wg(int ksize, int any, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes, int op_bytes,
+cudaError_t launch_conv_wg(int ksize, int any, const ConvDesc* tab, const int* ts, int total, int raw_bytes, int op_bytes,
                            int32_t* status, cudaStream_t st, int max_ctas) {
   if (total <= 0) return cudaSuccess;
   Rings r;
@@ -471,7 +471,7 @@ cudaError_t launch_conv_wg(int ksize, int any, const ConvDesc* tab, const int* t
   const int sms = device_sm_count();
   int grid = total < sms ? total : sms;
   if (max_ctas > 0 && grid > max_ctas) grid = max_ctas;
-  kern<<<grid, kThreads, kFixed + rings_bytes(r), st>>>(tab, ts, n, total, r, status);
+  kern<<<grid, kThreads, kFixed + rings_bytes(r), st>>>(tab, ts, total, r, status);
   return cudaGetLastError();
 }
 

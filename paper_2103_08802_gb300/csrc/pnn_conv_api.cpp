@@ -623,11 +623,11 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
   if (e == cudaSuccess && !wts.empty())
     e = launch_wtrans(reinterpret_cast<const WtDesc*>(ws + pl.aux_tab), auxts, n, aux_ts.back(), st);
   auto conv_launch = [&]() {
-    if (pl.variant == 5) return launch_conv_c3(mode, tab, tsd, n, pl.total, pl.c3, status, st);
+    if (pl.variant == 5) return launch_conv_c3(mode, tab, tsd, pl.total, pl.c3, status, st);
     if (pl.variant == 4 && mode == 2)
-      return launch_conv_wg(pl.bnmax, pl.wg_any, tab, tsd, n, pl.total, pl.raw, pl.op, status, st);
+      return launch_conv_wg(pl.bnmax, pl.wg_any, tab, tsd, pl.total, pl.raw, pl.op, status, st);
     if (pl.variant == 4)
-      return launch_conv_pw(mode, pl.wide, tab, tsd, n, pl.total, pl.raw, pl.op, status, st);
+      return launch_conv_pw(mode, pl.wide, tab, tsd, pl.total, pl.raw, pl.op, status, st);
     if (pl.variant == 1)
       return launch_conv_tma(mode, pl.wide, tab, tsd, n, pl.total, pl.bnmax, pl.raw, pl.op, status, st);
     if (mode == 0) return launch_conv_fwd_tc(tab, tsd, n, pl.total, pl.bnmax, status, st);

@@ -248,16 +248,16 @@ bool conv_halo_fits(int mode, int W, int ch, int bn);
 // total: items; raw_bytes, x_bytes: the largest raw A slot and second operand
 // over the launch's instances (multiples of 1024); wide: every instance has one
 // k-step and at least 64 output columns
-cudaError_t launch_conv_pw(int mode, int wide, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes,
+cudaError_t launch_conv_pw(int mode, int wide, const ConvDesc* tab, const int* ts, int total, int raw_bytes,
                            int x_bytes, int32_t* status, cudaStream_t st, int max_ctas = 0);
 // 3x3 stride-1 forward (mode 0) / data gradient (mode 1) of k_c3_conv.cu; s: the
 // largest slots over the launch's instances (c3_add)
 struct C3Slots;
-cudaError_t launch_conv_c3(int mode, const ConvDesc* tab, const int* ts, int n, int total, const C3Slots& s,
+cudaError_t launch_conv_c3(int mode, const ConvDesc* tab, const int* ts, int total, const C3Slots& s,
                            int32_t* status, cudaStream_t st, int max_ctas = 0);
 // weight gradient of k_wg_conv.cu; any: wg_any of some instance; raw_bytes, op_bytes:
 // the largest slots over the launch's instances (multiples of 1024)
-cudaError_t launch_conv_wg(int ksize, int any, const ConvDesc* tab, const int* ts, int n, int total, int raw_bytes, int op_bytes,
+cudaError_t launch_conv_wg(int ksize, int any, const ConvDesc* tab, const int* ts, int total, int raw_bytes, int op_bytes,
                            int32_t* status, cudaStream_t st, int max_ctas = 0);
 // record a message for pnn_last_error(NULL) and return `code`
 int set_last_error(int code, const char* msg);
@@ -379,13 +379,13 @@ inline bool tma_shape_ok(int k, int stride, int pad, int ch) {
 // 16 or 32); several k-steps go with one unit, so that no operand row is
 // transformed twice.
 constexpr int kPwMaxC = 256;
-PNN_HD inline int pw_unit_cols(int ncols) { return ncols % 64 == 0 ? 64 : ncols; }
+PNN_HD constexpr int pw_unit_cols(int ncols) { return ncols % 64 == 0 ? 64 : ncols; }
 inline bool pw_ok(int k, int stride, int ch, int ncols) {
   return k == 1 && stride == 1 && (ch == 16 || ch == 32 || (ch % 64 == 0 && ch <= kPwMaxC)) &&
          (ncols == 16 || ncols == 32 || ncols % 64 == 0) && (ch <= 64 || ncols <= 64);
 }
-inline int pw_raw_bytes(int ch, int esz) { return (kTcBM * (ch < 64 ? ch : 64) * esz + 1023) & ~1023; }
-inline int pw_x_bytes(int ncols) { return kTcBM * pw_unit_cols(ncols) * 2; }
+constexpr int pw_raw_bytes(int ch, int esz) { return (kTcBM * (ch < 64 ? ch : 64) * esz + 1023) & ~1023; }
+constexpr int pw_x_bytes(int ncols) { return kTcBM * pw_unit_cols(ncols) * 2; }
 // units of an item: all of an m-tile's (its rows are transformed once), unless
 // the launch has too few m-tiles to occupy the SMs twice over
 inline int pw_item_units(int ncols, int64_t launch_mtiles) {
@@ -411,10 +411,10 @@ PNN_HD inline int c3_kind(int H, int W) {
 // raw pixels of a k-step; bytes of an operand plane: a halo of 10 x 18 pixels,
 // three copies of 10 x 16, or nine copies of 128 pixels (the latter two and four
 // pixels that spread the two planes' stores over the banks)
-PNN_HD inline int c3_raw_px(int kind) { return kind == C3_PATCH ? 180 : 128; }
-PNN_HD inline int c3_plane(int kind) { return (kind == C3_PATCH ? 180 : kind == C3_WHOLE ? 484 : 1156) * 16; }
+PNN_HD constexpr int c3_raw_px(int kind) { return kind == C3_PATCH ? 180 : 128; }
+PNN_HD constexpr int c3_plane(int kind) { return (kind == C3_PATCH ? 180 : kind == C3_WHOLE ? 484 : 1156) * 16; }
 PNN_HD inline int c3_block(int ncols) { return ncols < 64 ? ncols : 64; }
-PNN_HD inline int c3_wt_bytes(int block) { return 9 * block * 32; }  // 16 channels, nine taps
+PNN_HD constexpr int c3_wt_bytes(int block) { return 9 * block * 32; }  // 16 channels, nine taps
 inline bool c3_ok(int k, int stride, int H, int W, int ch, int ncols) {
   auto cols = [](int c) { return c == 16 || c == 32 || (c > 0 && c % 64 == 0); };
   return k == 3 && stride == 1 && c3_kind(H, W) != C3_NONE && cols(ch) && cols(ncols);
@@ -428,7 +428,7 @@ inline void c3_add(C3Slots& s, int H, int W, int ncols, int esz, bool x) {
   if (x) most(s.x, kTcBM * block * 2);
   if (kind == C3_SMALL || ncols > block) s.any = 1;
 }
-// Weight gradient of k_wg_conv.cu (variant 4: 1x1, 5: 3x3): the geometry of one instance's
+// Weight gradient of k_wg_conv.cu (a network's variant 4: 1x1, 5: 3x3): the geometry of one instance's
 // k-steps.  1x1: kp pixels; 3x3: krows whole image rows (kp pixels) with the
 // activation rows above and below.  Raw slot: x rows, then dY rows; operand
 // slot: the M side's planes (8 channels each, apitch bytes), then (boff) the N

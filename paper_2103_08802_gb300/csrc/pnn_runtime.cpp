@@ -668,7 +668,6 @@ struct pnn_net {
         }
         POp fi = r;
         fi.kind = K_BNB_FIN;
-        fi.tiles = n.C;  // one CTA per channel
         key(fi, 1);
         new_op(L, fi);
         POp ap = r;
@@ -1886,11 +1885,11 @@ int pnn_net::run_phase(int p, cudaStream_t st, int cap) {
       case K_CONV_FWD: e = launch_conv_fwd_simt((const ConvDesc*)tab, ts, L.count, L.total, L.variant, st); break;
       case K_CONV_FWD_TC:
         if (L.variant == 5) {
-          e = launch_conv_c3(0, (const ConvDesc*)tab, ts, L.count, L.total, L.c3, P<int32_t>(status_off), st, cap);
+          e = launch_conv_c3(0, (const ConvDesc*)tab, ts, L.total, L.c3, P<int32_t>(status_off), st, cap);
           break;
         }
         if (L.variant == 4) {
-          e = launch_conv_pw(0, L.wide, (const ConvDesc*)tab, ts, L.count, L.total, L.raw, L.op, P<int32_t>(status_off),
+          e = launch_conv_pw(0, L.wide, (const ConvDesc*)tab, ts, L.total, L.raw, L.op, P<int32_t>(status_off),
                              st, cap);
           break;
         }
@@ -1901,11 +1900,11 @@ int pnn_net::run_phase(int p, cudaStream_t st, int cap) {
         break;
       case K_DGRAD_TC:
         if (L.variant == 5) {
-          e = launch_conv_c3(1, (const ConvDesc*)tab, ts, L.count, L.total, L.c3, P<int32_t>(status_off), st, cap);
+          e = launch_conv_c3(1, (const ConvDesc*)tab, ts, L.total, L.c3, P<int32_t>(status_off), st, cap);
           break;
         }
         if (L.variant == 4) {
-          e = launch_conv_pw(1, 0, (const ConvDesc*)tab, ts, L.count, L.total, L.raw, L.op, P<int32_t>(status_off), st,
+          e = launch_conv_pw(1, 0, (const ConvDesc*)tab, ts, L.total, L.raw, L.op, P<int32_t>(status_off), st,
                              cap);
           break;
         }
@@ -1917,7 +1916,7 @@ int pnn_net::run_phase(int p, cudaStream_t st, int cap) {
         break;
       case K_WGRAD_TC:
         if (L.variant >= 4) {
-          e = launch_conv_wg(L.variant == 5 ? 3 : 1, L.wg_any, (const ConvDesc*)tab, ts, L.count, L.total, L.raw, L.op, P<int32_t>(status_off), st,
+          e = launch_conv_wg(L.variant == 5 ? 3 : 1, L.wg_any, (const ConvDesc*)tab, ts, L.total, L.raw, L.op, P<int32_t>(status_off), st,
                              cap);
           break;
         }

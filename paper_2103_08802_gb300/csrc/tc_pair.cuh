@@ -90,14 +90,13 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[N]) {
 // found by stepping forward, so an item costs no division and no descriptor
 // reload unless the instance changes.
 struct Walk {
-  int item, total, ninst, inst, t0, t1;  // instance inst owns items t0 .. t1 - 1
+  int item, total, inst, t0, t1;         // instance inst owns items t0 .. t1 - 1
   int tm, tn, mt;                        // m-tile and N item within the instance, its m-tiles
   bool fresh;                            // the instance changed with this item
   const ConvDesc* d;
-  __device__ __forceinline__ Walk(const ConvDesc* tab, const int* ts, int n, int tot) {
+  __device__ __forceinline__ Walk(const ConvDesc* tab, const int* ts, int tot) {
     item = blockIdx.x;
     total = tot;
-    ninst = n;
     inst = -1;
     t0 = 0;
     t1 = 0;
