@@ -366,14 +366,19 @@ def retear(args, desc, stream):
     return desc, rec
 
 
-# (variant 1 is any TMA-fed kernel without the wide epilogue or halo tiles: those of
-# the shapes that the 1x1, 3x3 and weight-gradient kernels take, else k_conv_*_tma)
-KERNEL_SYMBOL = {("conv_fwd_tc", 0): "k_conv_fwd_tc", ("conv_fwd_tc", 1): "k_pw_fwd|k_c3_fwd|k_conv_fwd_tma",
+# (for trace records that do not name their kernel)
+KERNEL_SYMBOL = {("conv_fwd_tc", 0): "k_conv_fwd_tc", ("conv_fwd_tc", 1): "k_conv_fwd_tma",
                  ("conv_fwd_tc", 2): "k_conv_fwd_tma_w", ("conv_dgrad_tc", 0): "k_conv_dgrad_tc",
-                 ("conv_dgrad_tc", 1): "k_pw_dgrad|k_c3_dgrad|k_conv_dgrad_tma", ("conv_dgrad_tc", 2): "k_conv_dgrad_tma_w",
+                 ("conv_dgrad_tc", 1): "k_conv_dgrad_tma", ("conv_dgrad_tc", 2): "k_conv_dgrad_tma_w",
                  ("conv_fwd_tc", 3): "k_conv_fwd_tma_h", ("conv_dgrad_tc", 3): "k_conv_dgrad_tma_h",
-                 ("conv_wgrad_tc", 0): "k_conv_wgrad_tc", ("conv_wgrad_tc", 1): "k_wg_pw|k_wg_3x3|k_conv_wgrad_tma",
+                 ("conv_wgrad_tc", 0): "k_conv_wgrad_tc", ("conv_wgrad_tc", 1): "k_conv_wgrad_tma",
                  ("bn_bwd_apply", 1): "k_bnb_apply8", ("bn_finalize", 0): "k_bn_fin"}
+
+
+def group_key(r):
+    """(kind, variant, first-instance shape, instances, kernel) of a trace record."""
+    name = r.get("kernel") or KERNEL_SYMBOL.get((r["kind"], r["variant"]), r["kind"])
+    return r["kind"], r["variant"], r["shape"], r["instances"], name
 
 
 def dram_traffic(symbol):
@@ -399,41 +404,38 @@ def dram_traffic(symbol):
 
 
 def launch_groups(trace, steps, n=14):
-    """The n launch groups (kind, variant, first-instance shape, instances)
-    with the most device time per step, with their algorithmic GB/s against
-    the measured HBM peak."""
+    """The n launch groups (kernel, first-instance shape, instances) with the
+    most device time per step, with their algorithmic GB/s against the measured
+    HBM peak."""
     pk, _ = peaks()
     groups = {}
     for r in trace or []:
-        k = (r["kind"], r["variant"], r["shape"], r["instances"])
-        g = groups.setdefault(k, [0.0, 0, 0.0])
+        g = groups.setdefault(group_key(r), [0.0, 0, 0.0])
         g[0] += r["ms"]; g[1] += 1; g[2] += r["bytes"]
     out = []
-    for (kind, variant, shape, inst), (ms, cnt, by) in sorted(groups.items(), key=lambda kv: -kv[1][0])[:n]:
+    for (_, _, shape, inst, name), (ms, cnt, by) in sorted(groups.items(), key=lambda kv: -kv[1][0])[:n]:
         gbs = by / (ms / 1e3) / 1e9 if ms else 0.0
-        out.append({"kernel": KERNEL_SYMBOL.get((kind, variant), kind), "shape": list(shape), "instances": inst,
+        out.append({"kernel": name, "shape": list(shape), "instances": inst,
                     "launches_per_step": cnt / steps, "ms_per_step": ms / steps, "us_per_launch": 1e3 * ms / cnt,
                     "gbs": gbs, "frac_of_hbm": gbs / pk["hbm_gbs"]})
     return out
 
 
 def roofline_of(prof, steps, trace=None):
-    """Roofline record of the dominant kernel: the launch group (kind,
-    variant, first-instance shape, instances) with the largest device time in
+    """Roofline record of the dominant kernel: the launch group (kernel,
+    first-instance shape, instances) with the largest device time in
     a profiled window of `steps` steps, from the per-launch trace; without a
     trace, the dominant kind ({kind: (ms, launches, flops, bytes)})."""
     pk, src = peaks()
     if trace:
         groups = {}
         for r in trace:
-            k = (r["kind"], r["variant"], r["shape"], r["instances"])
-            g = groups.setdefault(k, [0.0, 0, 0.0, 0.0])
+            g = groups.setdefault(group_key(r), [0.0, 0, 0.0, 0.0])
             g[0] += r["ms"]; g[1] += 1; g[2] += r["flops"]; g[3] += r["bytes"]
         # (a group with no algorithmic bytes or FLOPs -- the per-channel BN
         # finalisation, the head -- has no roof to be measured against)
         cand = {k: g for k, g in groups.items() if g[2] > 0 or g[3] > 0} or groups
-        (kind, variant, shape, inst), (kms, kn, kfl, kby) = max(cand.items(), key=lambda kv: kv[1][0])
-        name = KERNEL_SYMBOL.get((kind, variant), kind)
+        (kind, variant, shape, inst, name), (kms, kn, kfl, kby) = max(cand.items(), key=lambda kv: kv[1][0])
         what = {"kind": kind, "variant": variant, "first_instance_shape": list(shape), "instances": inst}
     else:
         cand = {k: v for k, v in prof.items() if v[2] > 0 or v[3] > 0} or prof

@@ -326,6 +326,10 @@ typedef struct pnn_trace {
   double ms, flops, bytes;
 } pnn_trace;
 int pnn_profile_trace(pnn_net* net, int32_t max, pnn_trace* out, int32_t* count);
+/* The kernel of trace record i of a tensor-core convolution (the variant field
+ * calls every TMA-fed kernel without halo tiles or the wide epilogue 1); NULL for
+ * other records and bad i. */
+const char* pnn_profile_kernel_name(const pnn_net* net, int32_t i);
 int32_t pnn_num_kernel_kinds(void);
 const char* pnn_kernel_kind_name(int32_t kind); /* NULL for a bad kind */
 

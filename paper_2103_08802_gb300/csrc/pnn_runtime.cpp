@@ -2824,6 +2824,26 @@ int pnn_profile_trace(pnn_net* n, int32_t max, pnn_trace* out, int32_t* count) {
   return PNN_OK;
 }
 
+const char* pnn_profile_kernel_name(const pnn_net* n, int32_t i) {
+  if (!n || i < 0 || (size_t)i >= n->pnext / 2) return nullptr;
+  const Launch& L = *n->plaunch[i];
+  const bool general = L.c3.any;
+  switch (L.kind) {
+    case K_CONV_FWD_TC:
+      if (L.variant == 5) return general ? "k_c3_fwd<true>" : "k_c3_fwd<false>";
+      if (L.variant == 4) return L.wide ? "k_pw_fwd_w" : "k_pw_fwd";
+      return L.variant == 0 ? "k_conv_fwd_tc" : L.wide ? "k_conv_fwd_tma_w" : L.op > 0 ? "k_conv_fwd_tma_h" : "k_conv_fwd_tma";
+    case K_DGRAD_TC:
+      if (L.variant == 5) return general ? "k_c3_dgrad<true>" : "k_c3_dgrad<false>";
+      if (L.variant == 4) return "k_pw_dgrad";
+      return L.variant == 0 ? "k_conv_dgrad_tc" : L.wide ? "k_conv_dgrad_tma_w" : L.op > 0 ? "k_conv_dgrad_tma_h" : "k_conv_dgrad_tma";
+    case K_WGRAD_TC:
+      if (L.variant == 5) return L.wg_any ? "k_wg_3x3<true>" : "k_wg_3x3<false>";
+      return L.variant == 4 ? "k_wg_pw" : L.variant == 0 ? "k_conv_wgrad_tc" : "k_conv_wgrad_tma";
+    default: return nullptr;
+  }
+}
+
 const char* pnn_kernel_kind_name(int32_t kind) {
   return (kind >= 0 && kind < K_NKINDS) ? kKindName[kind] : nullptr;
 }

@@ -121,6 +121,7 @@ def load():
         "pnn_profile_read": (C.c_int, [P, I32, C.POINTER(C.c_double), C.POINTER(C.c_int64),
                                        C.POINTER(C.c_double), C.POINTER(C.c_double)]),
         "pnn_profile_trace": (C.c_int, [P, I32, C.POINTER(Trace), C.POINTER(I32)]),
+        "pnn_profile_kernel_name": (C.c_char_p, [P, I32]),
         "pnn_num_kernel_kinds": (I32, []),
         "pnn_debug_word": (C.c_uint64, []),
         "pnn_kernel_kind_name": (C.c_char_p, [I32]),
@@ -414,9 +415,13 @@ class ParaNet:
         self._check(self.lib.pnn_profile_trace(self.h, 0, None, C.byref(n)))
         buf = (Trace * max(1, n.value))()
         self._check(self.lib.pnn_profile_trace(self.h, n.value, buf, C.byref(n)))
-        return [{"kind": self.lib.pnn_kernel_kind_name(r.kind).decode(), "variant": r.variant, "phase": r.phase,
+        def kernel(i):
+            name = self.lib.pnn_profile_kernel_name(self.h, i)
+            return name.decode() if name else None
+        return [{"kind": self.lib.pnn_kernel_kind_name(r.kind).decode(), "kernel": kernel(i), "variant": r.variant,
+                 "phase": r.phase,
                  "instances": r.instances, "tiles": r.tiles, "shape": tuple(r.shape), "block": r.block,
-                 "ms": r.ms, "flops": r.flops, "bytes": r.bytes} for r in buf[:n.value]]
+                 "ms": r.ms, "flops": r.flops, "bytes": r.bytes} for i, r in enumerate(buf[:n.value])]
 
     def launch_counts(self):
         c = (C.c_int32 * 3)()

@@ -269,3 +269,23 @@ def test_staged_tiles_next_to_empty_rows(name, accumulate):
         for d, e in zip(insts, want):
             got = d["y" if mode == "forward" else "dx"].double()
             assert torch.equal(got, e + 3.0 if accumulate else e)
+
+
+def test_trace_names_the_kernels_of_a_network():
+    import torch
+    import workloads as W
+    from paper_2103_08802_gb300 import pnn
+    desc = W.parareal_resnet1001(n_seg=2, batch=16, per_stage=2)
+    net = pnn.ParaNet(desc, seed=1, lr=0.002)
+    x, labels = W.make_batch(desc, seed=3)
+    net.profile(True)
+    net.forward(torch.from_numpy(x).cuda(), torch.from_numpy(labels).cuda())
+    net.backward()
+    trace = net.profile_trace()
+    net.close()
+    tc = ("conv_fwd_tc", "conv_dgrad_tc", "conv_wgrad_tc")
+    assert all((r["kernel"] is not None) == (r["kind"] in tc) for r in trace)
+    # 1x1 and 3x3 layers, the stride-2 ones, and the last convolution of a subnetwork (a correction addend)
+    assert {r["kernel"] for r in trace} >= {"k_pw_fwd", "k_pw_fwd_w", "k_pw_dgrad", "k_c3_fwd<false>", "k_c3_dgrad<false>",
+                                            "k_wg_pw", "k_wg_3x3<false>", "k_conv_fwd_tc", "k_conv_dgrad_tc"}
+    assert any(r["kernel"].startswith("k_conv_fwd_tma") for r in trace if r["kind"] == "conv_fwd_tc")
