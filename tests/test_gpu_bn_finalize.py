@@ -4,8 +4,10 @@ of loads, a ragged last tile, channels that do not fill the CTA's group.
 
 The statistics are compared with float64 ones of the values the kernel stored.
 Bounds: a tile's mean and M2 are fp32 sums of 128 terms (at most 32 in a row,
-merged in fours), so each is within 64 u of its sum of absolute terms; the
-tiles are combined to about 48 bits and rounded once."""
+merged in fours), so each is within 40 u of its sum of absolute terms; the
+finalisation forms d = mean_t - mean_0, n d and M2 + n d^2 in fp32, one rounding
+each (the forward's terms have 24 bits), and adds them to about 48 bits, the
+backward's sums to more than 53.  64 u covers the forward's."""
 import numpy as np
 import pytest
 
