@@ -1083,8 +1083,8 @@ __global__ void __launch_bounds__(256) k_ew_bwd(const EwBwdDesc* __restrict__ ta
 // 8-subnetwork ResNet-1001 (batch 256, 64 px; 340 such launches of up to 2048
 // tiles a layer): 81.94 -> 81.36 ms with two floats, one quantity at a time.  Both
 // quantities of a partial packed, with the third float: 4-subnetwork ResNet-1001
-// (batch 128, 32 px) 26.27 -> 26.01 ms; unpacked, the third float had cost 0.17 ms, and
-// with 4 channels a CTA 0.5 ms (three such networks at once).
+// (batch 128, 32 px) 26.27 -> 26.01 ms a step; unpacked, the third float had cost 0.17 ms, and
+// with 4 channels a CTA 0.5 ms.
 __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
   return tc::fma2(b, tc::pk2(-1.f, -1.f), a);  // (one rounding: a - b)
 }
@@ -1430,10 +1430,6 @@ __device__ __forceinline__ void ld8any(const void* base, int dt, int64_t i, floa
   }
 }
 
-// U rows of a thread in flight: 8 in an fp32 network, whose tiles are the tall ones of
-// bnb_fixed_rows (16 rows a thread at 16 channels), and 1 where the tiles are cut to
-// fill the SMs.
-template <int U>
 __global__ void __launch_bounds__(256) k_bnb_reduce8(const BnBwdDesc* __restrict__ tab,
                                                      const int* __restrict__ tstart, int n) {
   __shared__ float red[16][256];  // [quantity x channel][thread]: a warp touches 32 consecutive words
@@ -1455,24 +1451,16 @@ __global__ void __launch_bounds__(256) k_bnb_reduce8(const BnBwdDesc* __restrict
     for (int k = 0; k < 8; ++k) {
       mean[k] = d.mean[c0 + k]; rstd[k] = d.rstd[c0 + k]; sc[k] = d.scale[c0 + k]; sh[k] = d.shift[c0 + k];
     }
-    for (int64_t r = r0 + g; r < r1; r += U * G) {
-      float h[U][8], dz[U][8];
+    for (int64_t r = r0 + g; r < r1; r += G) {
+      const int64_t o = r * C + c0;
+      float h[8], dz[8];
+      ld8any(d.h, d.h_dt, o, h);
+      ld8f(d.da + o, dz);
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (u && r + u * G >= r1) break;
-        const int64_t o = (r + u * G) * C + c0;
-        ld8any(d.h, d.h_dt, o, h[u]);
-        ld8f(d.da + o, dz[u]);
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (u && r + u * G >= r1) break;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          if (d.relu && !(fmaf(sc[k], h[u][k], sh[k]) > 0.f)) dz[u][k] = 0.f;
-          s1[k] += dz[u][k];
-          s2[k] += dz[u][k] * ((h[u][k] - mean[k]) * rstd[k]);
-        }
+      for (int k = 0; k < 8; ++k) {
+        if (d.relu && !(fmaf(sc[k], h[k], sh[k]) > 0.f)) dz[k] = 0.f;
+        s1[k] += dz[k];
+        s2[k] += dz[k] * ((h[k] - mean[k]) * rstd[k]);
       }
     }
   }
@@ -1502,6 +1490,81 @@ __global__ void __launch_bounds__(256) k_bnb_reduce8(const BnBwdDesc* __restrict
     for (int k = 0; k < 8; ++k) {
       d.part[((int64_t)tile * C + threadIdx.x * 8 + k) * 2] = a[k];
       d.part[((int64_t)tile * C + threadIdx.x * 8 + k) * 2 + 1] = b[k];
+    }
+  }
+}
+
+// The same sums for an fp32 network, in the fixed order: the tall tiles of
+// bnb_fixed_rows, G = 256 / (C / 8) row groups one row after another, the groups in
+// k_bnb_reduce8's tree.  A CTA takes half of a tile's channels, a thread four of them
+// with all its rows in flight (16 a thread up to 128 channels).  (8 channels a thread,
+// eight rows in flight, one CTA a tile: 10.4 us a launch of the tiny network under
+// ncu, now 8.1; its step 255 -> 251 us.)
+__global__ void __launch_bounds__(256) k_bnb_reduce_fixed(const BnBwdDesc* __restrict__ tab,
+                                                          const int* __restrict__ tstart, int n) {
+  constexpr int U = 16;
+  __shared__ float red[8][256];
+  const int inst = find_instance(tstart, n, blockIdx.x);
+  const BnBwdDesc d = tab[inst];
+  const int t = blockIdx.x - tstart[inst], tile = t >> 1;
+  const int C = d.C, CG = C / 8, G = 256 / CG;  // CG quads of channels a CTA
+  const int q = threadIdx.x % CG, g = threadIdx.x / CG, c0 = ((t & 1) * CG + q) * 4;
+  const int64_t r0 = (int64_t)tile * d.rows_per_tile;
+  const int64_t r1 = min((int64_t)d.M, r0 + d.rows_per_tile);
+  const float* hp = static_cast<const float*>(d.h);
+  float s1[4] = {}, s2[4] = {};
+  if (g < G) {
+    float mean[4], rstd[4], sc[4], sh[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      mean[k] = d.mean[c0 + k]; rstd[k] = d.rstd[c0 + k]; sc[k] = d.scale[c0 + k]; sh[k] = d.shift[c0 + k];
+    }
+    for (int64_t r = r0 + g; r < r1; r += U * G) {
+      float4 hv[U], dv[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (r + u * G >= r1) break;
+        const int64_t o = (r + u * G) * C + c0;
+        hv[u] = *reinterpret_cast<const float4*>(hp + o);
+        dv[u] = *reinterpret_cast<const float4*>(d.da + o);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (r + u * G >= r1) break;
+        const float h[4] = {hv[u].x, hv[u].y, hv[u].z, hv[u].w};
+        float dz[4] = {dv[u].x, dv[u].y, dv[u].z, dv[u].w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (d.relu && !(fmaf(sc[k], h[k], sh[k]) > 0.f)) dz[k] = 0.f;
+          s1[k] += dz[k];
+          s2[k] += dz[k] * ((h[k] - mean[k]) * rstd[k]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) { red[k][threadIdx.x] = s1[k]; red[4 + k][threadIdx.x] = s2[k]; }
+  __syncthreads();
+  int groups = G;
+  if ((G & (G - 1)) == 0) {
+    for (int st = G >> 1; st > 0; st >>= 1) {
+      if (g < st) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + st * CG];
+      }
+      __syncthreads();
+    }
+    groups = 1;
+  }
+  if ((int)threadIdx.x < CG) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      float a = 0.f, b = 0.f;
+      for (int gg = 0; gg < groups; ++gg) {
+        a += red[k][gg * CG + q];
+        b += red[4 + k][gg * CG + q];
+      }
+      reinterpret_cast<float2*>(d.part)[(int64_t)tile * C + c0 + k] = make_float2(a, b);
     }
   }
 }
@@ -2140,11 +2203,14 @@ cudaError_t launch_bnb_reduce(const BnBwdDesc* tab, const int* tstart, int n, in
   k_bnb_reduce<<<total, 256, 0, st>>>(tab, tstart, n);
   return cudaGetLastError();
 }
-cudaError_t launch_bnb_reduce8(const BnBwdDesc* tab, const int* tstart, int n, int total, int fixed_order,
-                               cudaStream_t st) {
+cudaError_t launch_bnb_reduce8(const BnBwdDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {
   if (total <= 0) return cudaSuccess;
-  if (fixed_order) k_bnb_reduce8<8><<<total, 256, 0, st>>>(tab, tstart, n);
-  else k_bnb_reduce8<1><<<total, 256, 0, st>>>(tab, tstart, n);
+  k_bnb_reduce8<<<total, 256, 0, st>>>(tab, tstart, n);
+  return cudaGetLastError();
+}
+cudaError_t launch_bnb_reduce_fixed(const BnBwdDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {
+  if (total <= 0) return cudaSuccess;
+  k_bnb_reduce_fixed<<<total, 256, 0, st>>>(tab, tstart, n);
   return cudaGetLastError();
 }
 cudaError_t launch_bnb_fin(const BnBwdDesc* tab, const int* tstart, int n, int total, cudaStream_t st) {

@@ -658,7 +658,7 @@ int conv_run(int32_t mode, int32_t impl, int32_t n, const pnn_conv_args* a, void
                       (int)fins.size(), fin_ts.back(), 0, st);
   if (e == cudaSuccess && !breds.empty())
     e = launch_bnb_reduce8(reinterpret_cast<const BnBwdDesc*>(ws + pl.red_tab),
-                           reinterpret_cast<const int*>(ws + pl.red_ts), (int)breds.size(), red_ts.back(), 0, st);
+                           reinterpret_cast<const int*>(ws + pl.red_ts), (int)breds.size(), red_ts.back(), st);
   if (e == cudaSuccess && !bfins.empty())
     e = launch_bnb_fin(reinterpret_cast<const BnBwdDesc*>(ws + pl.fin_tab), reinterpret_cast<const int*>(ws + pl.fin_ts),
                        (int)bfins.size(), fin_ts.back(), st);

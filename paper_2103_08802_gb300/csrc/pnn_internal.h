@@ -211,8 +211,9 @@ cudaError_t launch_bnb_reduce(const BnBwdDesc* tab, const int* tstart, int n, in
 cudaError_t launch_bnb_fin(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_bnb_apply(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 // 8 channels per thread; every instance needs C % 8 == 0 and C <= 2048
-cudaError_t launch_bnb_reduce8(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, int fixed_order,
-                               cudaStream_t st);
+cudaError_t launch_bnb_reduce8(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
+// fp32 networks; total: two CTAs a tile
+cudaError_t launch_bnb_reduce_fixed(const BnBwdDesc* tab, const int* tstart, int n, int total, cudaStream_t st);
 cudaError_t launch_bnb_apply8(const BnBwdDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_pool_fwd(const PoolDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);
 cudaError_t launch_pool_bwd(const PoolDesc* tab, const int* tstart, int n, int total_tiles, cudaStream_t st);

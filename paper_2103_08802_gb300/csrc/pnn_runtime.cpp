@@ -1618,7 +1618,9 @@ int pnn_net::build_tables() {
               b.add_c[0] = o.addc[0];
               b.add_c[1] = o.addc[1];
             }
-            add(&b, sizeof b, o.kind == K_BNB_FIN ? fin_ctas(n.C) : o.tiles);
+            // (k_bnb_reduce_fixed: two CTAs a tile)
+            const int ctas = o.kind == K_BNB_RED && o.variant && act_dt == DT_F32 ? 2 : 1;
+            add(&b, sizeof b, o.kind == K_BNB_FIN ? fin_ctas(n.C) : o.tiles * ctas);
             break;
           }
           case K_POOL_FWD:
@@ -1936,8 +1938,9 @@ int pnn_net::run_phase(int p, cudaStream_t st, int cap) {
                           : launch_bn_fin((const BnFinDesc*)tab, ts, L.count, L.total, act_dt == DT_F32, st);
         break;
       case K_BNB_RED:
-        e = L.variant ? launch_bnb_reduce8((const BnBwdDesc*)tab, ts, L.count, L.total, act_dt == DT_F32, st)
-                      : launch_bnb_reduce((const BnBwdDesc*)tab, ts, L.count, L.total, st);
+        e = L.variant && act_dt == DT_F32 ? launch_bnb_reduce_fixed((const BnBwdDesc*)tab, ts, L.count, L.total, st)
+            : L.variant ? launch_bnb_reduce8((const BnBwdDesc*)tab, ts, L.count, L.total, st)
+                        : launch_bnb_reduce((const BnBwdDesc*)tab, ts, L.count, L.total, st);
         break;
       case K_BNB_FIN: e = launch_bnb_fin((const BnBwdDesc*)tab, ts, L.count, L.total, st); break;
       case K_BNB_APPLY:
