@@ -19,10 +19,10 @@
 // contiguous copy brings them: as 18 boxes of 16-byte rows they cost the
 // producer 200 cycles each and bounded the kernel.
 // Grouped launches of the 8-subnetwork ResNet-1001 (batch 256, 64 px), kernels of
-// k_tc_conv.cu -> now: forward 160 -> 60 us, data gradient (+ BN-backward sums)
-// 133 -> 76 us; bound by per-tile latencies (a tile is 128 x 16 outputs).  VGG-16
+// k_tc_conv.cu -> now: forward 160 -> 58 us, data gradient (+ BN-backward sums)
+// 133 -> 74 us; bound by per-tile latencies (a tile is 128 x 16 outputs).  VGG-16
 // (batch 128), kernels of k_tc_conv.cu -> now: 128 -> 128 channels at 16 x 16, 4
-// instances, forward 204 -> 68 us, data gradient 152 -> 72; 256 -> 256 at 8 x 8, 3
+// instances, forward 204 -> 70 us, data gradient 152 -> 74; 256 -> 256 at 8 x 8, 3
 // instances, 171 -> 54 and 120 -> 55; 512 -> 512 at 2 x 2, 116 -> 29 and 80 -> 27.
 // Those are 9 MMAs a k-step of N = 64 (about 300 cycles: the read of the M side)
 // beside a transform of 400 - 500 by six warps.

@@ -27,8 +27,8 @@
 // a sixth of the instructions.  Bound by HBM latency and bandwidth, about half
 // of the copy rate: grouped launches of the 8-subnetwork ResNet-1001 (batch
 // 256, 64 px), before -> now: expand forward (16 -> 64 channels + residual +
-// statistics) 218 -> 105 us, reduce forward 117 -> 75, reduce data gradient
-// (+ BN-backward sums) 165 -> 135, expand data gradient 109 -> 93.
+// statistics) 218 -> 107 us, reduce forward 117 -> 73, reduce data gradient
+// (+ BN-backward sums) 165 -> 128, expand data gradient 109 -> 88.
 // Every wait is bounded (2 s); on expiry the CTA records status 3, stops,
 // drains its copies and MMAs (bounded) and frees its TMEM.
 #include <cuda_bf16.h>

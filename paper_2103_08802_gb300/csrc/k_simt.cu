@@ -117,9 +117,9 @@ __device__ __forceinline__ float2 row_moments(int tm, int m0, int M, Get v) {
 template <typename Get>
 __device__ __forceinline__ void merge_row_groups(int tm, int m0, int M, Get red, float* out) {
   float n = 0.f, mean = 0.f, m2 = 0.f;
+#pragma unroll
   for (int r = 0; r < 16; ++r) {
-    int cr = 0;
-    for (int i = 0; i < tm; ++i) cr += m0 + r + 16 * i < M ? 1 : 0;
+    const int cr = min(tm, max(0, (M - m0 - r + 15) >> 4));  // rows m0 + r + 16 i < M, i < tm
     const float2 v = red(r);
     chan_merge(n, mean, m2, (float)cr, v.x, v.y);
   }
@@ -1110,18 +1110,23 @@ struct FloatSum {
 #pragma unroll
     for (int i = 0; i < N; ++i) add(o.v[i], i);
   }
-  // (an overflowed or NaN sum has no meaningful low parts)
-  __device__ __forceinline__ double2 value() const {
-    double x = 0.0, y = 0.0;
-#pragma unroll
-    for (int i = N - 1; i > 0; --i) {
-      x += (double)tc::un2(v[i]).x;
-      y += (double)tc::un2(v[i]).y;
-    }
-    const float2 h = tc::un2(v[0]);
-    return make_double2(isfinite(h.x) ? (double)h.x + x : (double)h.x, isfinite(h.y) ? (double)h.y + y : (double)h.y);
+  // as two floats: nothing cancels any more, and 48 bits are to become an fp32
+  // (an overflowed or NaN sum is its first part)
+  __device__ __forceinline__ void pair(uint64_t& hi, uint64_t& lo) const {
+    hi = v[0];
+    lo = v[1];
+    if (N == 2) return;
+    hi = two_sum(v[0], v[1], lo);
+    lo = tc::add2(lo, v[N - 1]);
+    hi = two_sum(hi, lo, lo);
+    const float2 a = tc::un2(v[0]), b = tc::un2(hi);
+    hi = tc::pk2(isfinite(a.x) ? b.x : a.x, isfinite(a.y) ? b.y : a.y);
   }
 };
+// (an overflowed or NaN sum has no meaningful low part)
+__device__ __forceinline__ double pair_value(float hi, float lo) {
+  return isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+}
 
 constexpr int kFinThreads = 512;
 constexpr int kFinLanes = kFinThreads / kFinChannels;  // tile lanes
@@ -1143,7 +1148,7 @@ __device__ __forceinline__ void tile_sums(const float* __restrict__ part, int C,
   constexpr int N = MOMENTS ? 2 : 3;
   using Sum = FloatSum<N>;
   __shared__ uint64_t red[N][kFinLanes][kFinChannels + 1];
-  __shared__ double2 tot[kFinChannels];
+  __shared__ uint64_t tot[kFinChannels][2];
   const int ch = threadIdx.x % kFinChannels, tl = threadIdx.x / kFinChannels;
   const int c = cg * kFinChannels + ch;
   Sum a;
@@ -1197,13 +1202,14 @@ __device__ __forceinline__ void tile_sums(const float* __restrict__ part, int C,
       for (int i = 0; i < N; ++i) t.v[i] = __shfl_xor_sync(0xffffffffu, s.v[i], o);
       s.add(t);
     }
-    if (lane == 0) tot[w] = s.value();
+    if (lane == 0) s.pair(tot[w][0], tot[w][1]);
   }
   __syncthreads();
   s1 = s2 = 0.0;
   if (threadIdx.x < kFinChannels) {
-    s1 = tot[threadIdx.x].x;
-    s2 = tot[threadIdx.x].y;
+    const float2 h = tc::un2(tot[threadIdx.x][0]), l = tc::un2(tot[threadIdx.x][1]);
+    s1 = pair_value(h.x, l.x);
+    s2 = pair_value(h.y, l.y);
   }
 }
 

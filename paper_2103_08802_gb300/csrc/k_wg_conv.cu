@@ -31,10 +31,10 @@
 // reduced.  Roles: producer (TMA, one thread), MMA (one thread), ten transform
 // warps, four epilogue warps.  Grouped launches of the
 // 8-subnetwork ResNet-1001 (batch 256, 64 px), kernels of k_tc_conv.cu -> now:
-// 3x3 224 -> 60 us, expand (16 -> 64) 159 -> 65 us (two launches before), reduce
-// 141 -> 56 us; the 1x1 are at 0.6 - 0.75 of the copy rate, the 3x3 is bound by
+// 3x3 224 -> 59 us, expand (16 -> 64) 159 -> 63 us (two launches before), reduce
+// 141 -> 52 us; the 1x1 are at 0.68 - 0.84 of the copy rate, the 3x3 is bound by
 // the latency of its k-steps.  VGG-16 (batch 128): 128 -> 128 at 16 x 16, 4
-// instances, 348 -> 74 us; 256 -> 256 at 8 x 8, 3 instances, 232 -> 68; 512 -> 512
+// instances, 348 -> 76 us; 256 -> 256 at 8 x 8, 3 instances, 232 -> 68; 512 -> 512
 // at 4 x 4 90 -> 55: each block of 32 input channels transforms the gradient again.
 // Every wait is bounded (2 s); on expiry the CTA records status 3, stops,
 // drains its copies and MMAs (bounded) and frees its TMEM.
